@@ -334,8 +334,8 @@ int zorth(cudaStream_t s, int64_t n, int64_t m, zd *V, int64_t ldv, zd *R, int64
 size_t zorth_work_elems(int64_t n, int64_t m);
 
 // Batched projected eigensolve: alpha / beta eigenvalue pairs and unit right
-// eigenvectors V of (A, B), B upper triangular.  m <= 64: QZ, one warp per
-// pencil (A, B overwritten by the Schur form); m > 64: standard-form path
+// eigenvectors V of (A, B), B upper triangular.  m <= 64: zeig_refined, then
+// QZ for the pencils it leaves (A, B overwritten by their Schur form); m > 64: standard-form path
 // of k_zeig.cu, pencil by pencil (A, B overwritten).  work: batch *
 // zqz_work_bytes(m) bytes.  timeout (may be null): set if a grid barrier
 // of the large path gave up.
@@ -343,6 +343,13 @@ size_t zqz_work_bytes(int m);
 int zqz_batched(cudaStream_t s, int m, int batch, zd *A, int64_t lda, int64_t sA, zd *B,
                 int64_t ldb, int64_t sB, zd *alpha, zd *beta, zd *V, int64_t ldv, int64_t sV,
                 void *work, int *fail, int *timeout, int *stats = nullptr, double defl = 0.0);
+
+// The same for 3 <= m <= 64 by an FP32 Schur form and an FP64 Newton
+// iteration alone (A, B kept): the int at work + 16 b m^2 bytes is 0 when
+// pencil b was solved (beta = 1), 1 when it needs another method (its
+// alpha, beta and V are then not written).
+int zeig_refined(cudaStream_t s, int m, int batch, const zd *A, int64_t lda, int64_t sA, const zd *B, int64_t ldb,
+                 int64_t sB, zd *alpha, zd *beta, zd *V, int64_t ldv, int64_t sV, void *work);
 
 // Large projected problems (k_zeig.cu): standard form, Hessenberg
 // reduction and chunked QR; alpha = eigenvalue, beta = 1.

@@ -149,7 +149,7 @@ constexpr int kZeigMinM = 8;         // smallest projected problem on the standa
 // skinny blocks were faster: at n = 16384, m0 = 64 the orthonormalisation
 // took 9.8 ms per pass in FP64 and 16.8 ms on the digit slices)
 constexpr int kBandOzMinM = 256;
-constexpr double kZeigSmallEpsMin = 1e-10;   // ... when m0 <= 64: the strictest eps it serves
+constexpr double kZeigSmallEpsMin = 1e-10;   // double-single QR at m0 <= 64: the strictest eps it serves
 
 struct Carver {
     char *base;
@@ -935,18 +935,29 @@ static int iterate_impl(feast_ctx *c, feast_iter_info *info)
         const double defl = (c->c_prev > 0 || final_pass) ? 0.0 : 1e-8;
         FEAST_CUDA_TRY(cudaMemcpyAsync(c->Q, c->P, sizeof(zd) * 2 * m * m, cudaMemcpyDeviceToDevice, s));
         if (rr && (e = triangularise_bt(c))) return e;
-        // B~ is upper triangular here (R2, or made so for Rayleigh-Ritz):
-        // the standard-form QR on the FP32 pipe (double-single) from m =
-        // kZeigMinM up (GB300's FP64 pipe made the FP64 QZ ~50 ms at m0 =
-        // 64); a small problem keeps the FP64 QZ when eps is within ~1000x
-        // of the double-single QR's backward error (2^-44 of ||C||), so
+        // B~ is upper triangular here (R2, or made so for Rayleigh-Ritz).
+        // Up to 64 rows one CTA solves the pencil to FP64 accuracy (an FP32
+        // Schur form and an FP64 Newton iteration, k_zqz.cu: 3.6 ms at m0 =
+        // 64).  What it leaves goes to the double-single standard-form QR
+        // (~7 ms) from m = kZeigMinM up, or to the FP64 QZ (~70 ms) when eps
+        // is within ~1000x of that QR's backward error (2^-44 of ||C||), so
         // that e(k) can still fall below eps
-        if (m > 64 || (m >= kZeigMinM && c->eps >= kZeigSmallEpsMin))
-            e = zeig_large(s, (int)m, c->Q, c->Q + m * m, c->alpha, c->beta, c->Yv, c->qz_work, &c->st->qz_fail,
+        zd *Bq = c->Q + m * m;
+        int left = 1;
+        if (m >= 3 && m <= 64) {
+            if ((e = zeig_refined(s, (int)m, 1, c->Q, m, 0, Bq, m, 0, c->alpha, c->beta, c->Yv, m, 0, c->qz_work)))
+                return e;
+            FEAST_CUDA_TRY(cudaMemcpyAsync(&left, c->qz_work, sizeof(int), cudaMemcpyDeviceToHost, s));
+            FEAST_CUDA_TRY(cudaStreamSynchronize(s));
+        }
+        if (!left)
+            e = FEAST_OK;
+        else if (m > 64 || (m >= kZeigMinM && c->eps >= kZeigSmallEpsMin))
+            e = zeig_large(s, (int)m, c->Q, Bq, c->alpha, c->beta, c->Yv, c->qz_work, &c->st->qz_fail,
                            &c->st->timeout, &c->st->qz_sweeps, defl);
         else
-            e = zqz_batched(s, (int)m, 1, c->Q, m, 0, c->Q + m * m, m, 0, c->alpha, c->beta, c->Yv, m, 0,
-                            c->qz_work, &c->st->qz_fail, &c->st->timeout, &c->st->qz_sweeps, defl);
+            e = zqz_batched(s, (int)m, 1, c->Q, m, 0, Bq, m, 0, c->alpha, c->beta, c->Yv, m, 0, c->qz_work,
+                            &c->st->qz_fail, &c->st->timeout, &c->st->qz_sweeps, defl);
         if (e) return e;
     }
     FEAST_CUDA_TRY(cudaEventRecord(c->ev[2], s));

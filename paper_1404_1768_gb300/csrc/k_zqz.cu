@@ -153,7 +153,7 @@ template <int NT>
 __global__ void __launch_bounds__(NT) k_qz(int m, zd *A, int64_t lda, int64_t sA, zd *B,
                                            int64_t ldb, int64_t sB, zd *alpha, zd *beta, zd *V,
                                            int64_t ldv, int64_t sV, zd *work, int use_smem,
-                                           int *fail)
+                                           int *fail, int only_redo)
 {
     extern __shared__ zd smem[];
     __shared__ double red[32];
@@ -165,6 +165,8 @@ __global__ void __launch_bounds__(NT) k_qz(int m, zd *A, int64_t lda, int64_t sA
     beta += (int64_t)b * m;
     zd *Wk = work + (int64_t)b * m * m;
     const int tid = threadIdx.x;
+    if (only_redo && *(volatile int *)Wk == 0) return;   // k_eig_refined has solved this pencil
+    Team<NT>::bar();
     const double eps = 2.220446049250313e-16;
 
     Mat H, T, Z, Yh;
@@ -271,10 +273,9 @@ __global__ void __launch_bounds__(NT) k_qz(int m, zd *A, int64_t lda, int64_t sA
     // eigenvalues
     for (int k = tid; k < m; k += NT) { alpha[k] = H(k, k); beta[k] = T(k, k); }
     // y_hat_k by back-substitution, one thread per eigenvector
-    const double small = eps * (hn + tn);
     for (int k = tid; k < m; k += NT) {
         const zd al = H(k, k), be = T(k, k);
-        const double g = small * (zabs(al) + zabs(be));
+        const double g = eps * (hn * zabs(be) + tn * zabs(al));   // rounding level of be S - al P, whatever their scales
         for (int i = k + 1; i < m; ++i) Yh(i, k) = zmake(0.0, 0.0);
         Yh(k, k) = zmake(1.0, 0.0);
         for (int i = k - 1; i >= 0; --i) {
@@ -320,6 +321,689 @@ __global__ void __launch_bounds__(NT) k_qz(int m, zd *A, int64_t lda, int64_t sA
         }
     }
 }
+
+// ---------------------------------------------------------------- refined
+// Eigenpairs of (A, B), B upper triangular, from an FP32 Schur form made
+// exact by an FP64 Newton iteration on the pencil itself; one CTA per pencil.
+//
+// GB300 issues one warp-wide FP64 instruction per 64 clocks on each SM
+// quarter, whatever the number of active lanes, and a QZ rotation is a chain
+// of ~80 of them (three hypot, two divisions): k_qz spent ~10 us per rotation
+// pair, 70 ms at m = 64.  In FP32 the same chain is ~0.2 us, and what FP32
+// leaves is small enough for Newton's iteration to remove: with approximate
+// eigenvectors V and L^H = (B V)^{-1},
+//     R = A V - B V Lambda  (FP64),  W = L^H R,  lambda_j += W_jj,
+//     G_ij = W_ij / (lambda_j - lambda_i),  V += V G,
+// where only R carries FP64 products (8 m^3 DFMA on the tile grid); L, W, G
+// and V G multiply something small, so FP32 is enough for them and sets the
+// rate of convergence, not the limit.  The error left by a step is about
+// |G| (m |G| + delta), delta = ||I - L^H B V||_F measured at the start and
+// bounded from then on; the iteration ends when that, or the contraction
+// seen from step to step, leaves less than EZ_DONE.  B is only inverted in
+// FP32, so the limit is the residual's FP64 rounding, as for QZ.
+// Two eigenvalues closer than FP32 resolves (|W_ij| > EZ_PAIR |lambda_j - lambda_i|)
+// are separated by the eigenvectors of their own 2 x 2 block of Lambda + W,
+// which the FP64 residual determines, before the iteration goes on.
+// Pencils it does not fit (B singular or cond(B) beyond FP32's reach, three
+// or more eigenvalues that close, non-finite entries) raise *redo; the caller
+// then takes the QZ (k_qz) or the double-single QR.  Measured on GB300, see
+// zqz_batched.
+constexpr int EZ_T = 256;            // threads per CTA
+constexpr int EZ_Q = 128;            // of them in the QR iteration (one warp per SM quarter)
+constexpr int EZ_MIN_M = 3;          // smallest pencil
+constexpr int EZ_STEPS = 10;         // most Newton steps
+constexpr float EZ_PAIR = 1.f / 16;  // largest G_ij of a Newton step
+constexpr double EZ_DONE = 4e-15;    // error bound at which the iteration ends
+
+struct RotF {
+    float c;
+    cf s;
+};
+
+// 1 / sqrt(x) with one Newton step: rsqrtf alone is off by up to 2^-22.9
+// with a bias, which thousands of rotations would add up
+__device__ __forceinline__ float ez_rsqrt(float x)
+{
+    const float y = rsqrtf(x);
+    return y * fmaf(-0.5f * x * y, y, 1.5f);
+}
+
+// G = [c s; -conj(s) c] with G [x; y] = [r; 0]
+__device__ __forceinline__ RotF ez_rot(cf x, cf y)
+{
+    RotF g;
+    const float mx = fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(y.x), fabsf(y.y)));
+    // bring the larger entry into [1, 2): squares neither overflow nor vanish
+    int ex = (int)(__float_as_uint(mx) >> 23);
+    ex = ex < 1 ? 1 : (ex > 253 ? 253 : ex);
+    const float f = __uint_as_float((unsigned)(254 - ex) << 23);
+    x = cmakef(x.x * f, x.y * f);
+    y = cmakef(y.x * f, y.y * f);
+    const float ax2 = cabs2(x), ay2 = cabs2(y);
+    if (ay2 == 0.f) { g.c = 1.f; g.s = cmakef(0.f, 0.f); return g; }
+    if (ax2 < 1e-36f) { g.c = 0.f; const float ia = ez_rsqrt(ay2); g.s = cmakef(y.x * ia, -y.y * ia); return g; }
+    const float k = ez_rsqrt(ax2) * ez_rsqrt(ax2 + ay2);
+    g.c = ax2 * k;
+    g.s = cmakef((x.x * y.x + x.y * y.y) * k, (x.y * y.x - x.x * y.y) * k);   // x conj(y) k
+    return g;
+}
+__device__ __forceinline__ void ez_rot_pair(const RotF &g, cf &a, cf &b)          // G [a; b]
+{
+    const cf s = g.s;
+    const cf na = cmakef(fmaf(g.c, a.x, fmaf(s.x, b.x, -s.y * b.y)), fmaf(g.c, a.y, fmaf(s.x, b.y, s.y * b.x)));
+    b = cmakef(fmaf(g.c, b.x, -fmaf(s.x, a.x, s.y * a.y)), fmaf(g.c, b.y, -fmaf(s.x, a.y, -s.y * a.x)));
+    a = na;
+}
+__device__ __forceinline__ void ez_rot_pair_h(const RotF &g, cf &a, cf &b)        // [a b] G^H
+{
+    RotF h;
+    h.c = g.c;
+    h.s = cmakef(g.s.x, -g.s.y);
+    ez_rot_pair(h, a, b);
+}
+
+__device__ __forceinline__ void ez_bar() { asm volatile("bar.sync 1, %0;" ::"n"(EZ_Q) : "memory"); }
+
+__device__ __forceinline__ float ez_absf(cf a) { return sqrtf(cabs2(a)); }
+
+// Sum over the CTA of one float per thread, in a fixed order.
+__device__ __forceinline__ float ez_sum(float v, float *red)
+{
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    float r = 0.f;
+    for (int w = 0; w < EZ_T / 32; ++w) r += red[w];
+    return r;
+}
+__device__ __forceinline__ float ez_max(float v, float *red)
+{
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    float r = red[0];
+    for (int w = 1; w < EZ_T / 32; ++w) r = fmaxf(r, red[w]);
+    return r;
+}
+
+// C <- op(X) op(Y) (m x m in shared memory, row-major, ld), 4 x 4 entries per
+// thread with interleaved rows and columns; HY: Y^H.  C is neither X nor Y.
+template <bool HY>
+__device__ void ez_mul(int m, int ld, const cf *X, const cf *Y, cf *C)
+{
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    cf acc[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = cmakef(0.f, 0.f);
+    for (int p = 0; p < m; ++p) {
+        cf x[4], y[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) x[i] = (ty + 16 * i < m) ? X[(ty + 16 * i) * ld + p] : cmakef(0.f, 0.f);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int c = tx + 16 * j;
+            y[j] = (c < m) ? (HY ? cconj(Y[c * ld + p]) : Y[p * ld + c]) : cmakef(0.f, 0.f);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) cfma(acc[i][j], x[i], y[j]);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (ty + 16 * i < m && tx + 16 * j < m) C[(ty + 16 * i) * ld + tx + 16 * j] = acc[i][j];
+    __syncthreads();
+}
+
+// Rows of X (and X2, when given) <- U^{-1} X by back-substitution, U upper
+// triangular (UNIT: unit diagonal); row-major, ld.
+template <bool UNIT>
+__device__ void ez_back_solve(int m, int ld, const cf *U, cf *X, cf *X2)
+{
+    const int cols = X2 ? 2 * m : m;
+    for (int i = m - 1; i >= 0; --i) {
+        if (!UNIT) {
+            const cf d = U[i * ld + i];
+            for (int c = threadIdx.x; c < cols; c += EZ_T) {
+                cf *x = (c < m) ? X + i * ld + c : X2 + i * ld + (c - m);
+                *x = cdiv(*x, d);
+            }
+            __syncthreads();
+        }
+        for (int e = threadIdx.x; e < i * cols; e += EZ_T) {
+            const int r = e / cols, c = e - r * cols;
+            cf *x = (c < m) ? X + c : X2 + (c - m);
+            cf v = x[r * ld];
+            cfma(v, cneg(U[r * ld + i]), x[i * ld]);
+            x[r * ld] = v;
+        }
+        __syncthreads();
+    }
+}
+
+// Hessenberg form of H by Householder reflectors, Z <- product (both m x m
+// row-major, ld); hv: m entries.
+__device__ void ez_hess(int m, int ld, cf *H, cf *Z, cf *hv)
+{
+    const int t = threadIdx.x, lane = t & 31;
+    for (int e = t; e < m * m; e += EZ_T) Z[(e / m) * ld + e % m] = cmakef(e / m == e % m ? 1.f : 0.f, 0.f);
+    __syncthreads();
+    for (int j = 0; j + 2 < m; ++j) {
+        const int len = m - j - 1;
+        // every warp forms the same reflector
+        float s = 0.f;
+        for (int i = lane; i < len; i += 32) s += cabs2(H[(j + 1 + i) * ld + j]);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        const cf x0 = H[(j + 1) * ld + j];
+        const float nrm = sqrtf(s), a0 = ez_absf(x0);
+        const cf ph = a0 > 0.f ? cmakef(x0.x / a0, x0.y / a0) : cmakef(1.f, 0.f);
+        const float vv = 2.f * nrm * (nrm + a0), tau = vv > 0.f ? 2.f / vv : 0.f;
+        for (int i = t; i < len; i += EZ_T)
+            hv[i] = (i == 0) ? cmakef(x0.x + ph.x * nrm, x0.y + ph.y * nrm) : H[(j + 1 + i) * ld + j];
+        __syncthreads();
+        // left: four threads per column j+1 .. m-1
+        {
+            const int c = j + 1 + (t >> 2), part = t & 3;
+            cf acc = cmakef(0.f, 0.f);
+            if (c < m)
+                for (int i = part; i < len; i += 4) cfma(acc, cconj(hv[i]), H[(j + 1 + i) * ld + c]);
+            acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 1);
+            acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 1);
+            acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 2);
+            acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 2);
+            const cf f = cmakef(-tau * acc.x, -tau * acc.y);
+            if (c < m)
+                for (int i = part; i < len; i += 4) cfma(H[(j + 1 + i) * ld + c], hv[i], f);
+        }
+        if (t < len) H[(j + 1 + t) * ld + j] = (t == 0) ? cmakef(-ph.x * nrm, -ph.y * nrm) : cmakef(0.f, 0.f);
+        __syncthreads();
+        // right: two threads per row of H and of Z
+        {
+            const int r = t >> 1, part = t & 1;
+            cf *row = (r < m) ? H + r * ld : Z + (r - m) * ld;
+            const bool on = r < 2 * m;
+            cf acc = cmakef(0.f, 0.f);
+            if (on)
+                for (int i = part; i < len; i += 2) cfma(acc, row[j + 1 + i], hv[i]);
+            acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 1);
+            acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 1);
+            const cf f = cmakef(-tau * acc.x, -tau * acc.y);
+            if (on)
+                for (int i = part; i < len; i += 2) cfma(row[j + 1 + i], f, cconj(hv[i]));
+        }
+        __syncthreads();
+    }
+}
+
+// Single-shift QR of the Hessenberg H to triangular form, Z <- Z Q (row-major,
+// ld), by the first EZ_Q threads: threads 0 .. 63 own a column of H in the
+// left half of a rotation and a row in the right half, threads 64 .. 127 a row
+// of Z; every warp forms each rotation from the same two entries (redundantly:
+// that costs no barrier), two barriers per rotation.  false: budget spent.
+__device__ bool ez_qr(int m, int ld, cf *H, cf *Z, float tol_abs)
+{
+    const int t = threadIdx.x, lane = t & 31;
+    const float tol_rel = 2.4e-7f;
+    int hi = m - 1, it = 0, tot = 0;
+    while (hi > 0) {
+        int lo = 0;
+        for (int base = hi; base >= 1 && lo == 0; base -= 32) {
+            const int p = base - lane;
+            bool neg = false;
+            if (p >= 1) {
+                const float sub = ez_absf(H[p * ld + p - 1]);
+                const float loc = ez_absf(H[(p - 1) * ld + p - 1]) + ez_absf(H[p * ld + p]);
+                neg = !(sub > tol_rel * loc) || !(sub > tol_abs);
+            }
+            const unsigned b = __ballot_sync(0xffffffffu, neg);
+            if (b) lo = base - (__ffs(b) - 1);
+        }
+        if (lo == hi) { --hi; it = 0; continue; }
+        if (++tot > 40 * m) return false;
+        ++it;
+        cf sigma;
+        {
+            const cf h00 = H[(hi - 1) * ld + hi - 1], h01 = H[(hi - 1) * ld + hi];
+            const cf h10 = H[hi * ld + hi - 1], h11 = H[hi * ld + hi];
+            if (it % 11 == 10) {
+                const float a = ez_absf(h10);
+                sigma = cmakef(h11.x + a, h11.y + 0.5f * a);
+            } else {
+                // Wilkinson shift: h11 + the smaller root of z^2 - 2 d z - h01 h10, d = (h00 - h11) / 2
+                const cf d = cmakef(0.5f * (h00.x - h11.x), 0.5f * (h00.y - h11.y));
+                const cf bc = cmul(h01, h10);
+                cf w = cadd(cmul(d, d), bc);
+                const float aw = ez_absf(w);
+                // principal square root of w, on the side of d
+                float re = sqrtf(0.5f * (aw + fabsf(w.x))), im = re > 0.f ? 0.5f * w.y / re : 0.f;
+                if (w.x < 0.f) { const float q = re; re = fabsf(im); im = copysignf(q, w.y); }
+                if (re * d.x + im * d.y < 0.f) { re = -re; im = -im; }
+                const cf den = cmakef(d.x + re, d.y + im);
+                const cf corr = cis_zero(den) ? cmakef(0.f, 0.f) : cdiv(bc, den);
+                sigma = cmakef(h11.x - corr.x, h11.y - corr.y);
+            }
+        }
+        for (int k = lo; k < hi; ++k) {
+            cf x, y;
+            if (k == lo) {
+                x = H[k * ld + k];
+                x = cmakef(x.x - sigma.x, x.y - sigma.y);
+                y = H[(k + 1) * ld + k];
+            } else {
+                x = H[k * ld + k - 1];
+                y = H[(k + 1) * ld + k - 1];
+            }
+            const RotF g = ez_rot(x, y);
+            // (the sweep's first x, y come from column k, which the left half
+            // writes: every warp has read them, the shift and the scan's entries)
+            if (k == lo) ez_bar();
+            if (t < 64) {
+                if (t >= k && t < m) {
+                    cf a = H[k * ld + t], b = H[(k + 1) * ld + t];
+                    ez_rot_pair(g, a, b);
+                    H[k * ld + t] = a;
+                    H[(k + 1) * ld + t] = b;
+                }
+            } else if (t - 64 < m) {
+                cf *z = Z + (t - 64) * ld + k;
+                cf a = z[0], b = z[1];
+                ez_rot_pair_h(g, a, b);
+                z[0] = a;
+                z[1] = b;
+            }
+            ez_bar();
+            if (t < 64) {
+                if (t <= ((k + 2 < hi) ? k + 2 : hi)) {
+                    cf a = H[t * ld + k], b = H[t * ld + k + 1];
+                    ez_rot_pair_h(g, a, b);
+                    H[t * ld + k] = a;
+                    H[t * ld + k + 1] = b;
+                }
+            } else if (t == 64 && k > lo) {
+                // column k - 1: (r, 0), now that every warp has read x and y
+                cf a = x, b = y;
+                ez_rot_pair(g, a, b);
+                H[k * ld + k - 1] = a;
+                H[(k + 1) * ld + k - 1] = cmakef(0.f, 0.f);
+            }
+            ez_bar();
+        }
+    }
+    return true;
+}
+
+// Eigenvector columns of the upper triangle of T into Y (upper triangular,
+// unit diagonal), one warp per eigenvector; row-major, ld.  An entry whose
+// eigenvalue is within small of the column's is left at zero: FP32 cannot
+// tell the two apart, the quotient would make the columns parallel, and the
+// pair's own block settles it in the iteration.
+__device__ void ez_vectors(int m, int ld, const cf *T, cf *Y, float small)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int e = threadIdx.x; e < m * m; e += EZ_T) Y[(e / m) * ld + e % m] = cmakef(0.f, 0.f);
+    __syncthreads();
+    for (int k = warp; k < m; k += EZ_T / 32) {
+        const cf lam = T[k * ld + k];
+        // lane l holds entries l and l + 32 of the vector
+        cf y0 = cmakef(lane == k ? 1.f : 0.f, 0.f), y1 = cmakef(lane + 32 == k ? 1.f : 0.f, 0.f);
+        for (int i = k - 1; i >= 0; --i) {
+            cf acc = cmakef(0.f, 0.f);
+            if (lane > i && lane <= k) cfma(acc, T[i * ld + lane], y0);
+            if (lane + 32 > i && lane + 32 <= k) cfma(acc, T[i * ld + lane + 32], y1);
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+                acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
+                acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
+            }
+            cf d = T[i * ld + i];
+            d = cmakef(lam.x - d.x, lam.y - d.y);
+            const cf q = cabs2(d) < small * small ? cmakef(0.f, 0.f) : cdiv(acc, d);
+            if (lane == i) y0 = q;
+            if (lane + 32 == i) y1 = q;
+        }
+        if (lane <= k) Y[lane * ld + k] = y0;
+        if (lane + 32 <= k) Y[(lane + 32) * ld + k] = y1;
+    }
+    __syncthreads();
+}
+
+// exponent bits of the largest |component| (0x7ff: a non-finite entry)
+__device__ __forceinline__ unsigned ez_hi(zd v)
+{
+    const unsigned a = (unsigned)__double2hiint(v.x) & 0x7fffffffu, b = (unsigned)__double2hiint(v.y) & 0x7fffffffu;
+    return a > b ? a : b;
+}
+__device__ __forceinline__ double ez_pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
+
+__host__ __device__ inline int ez_ld(int m) { return m | 1; }   // odd: rows fall on different banks
+__host__ inline size_t ez_smem_bytes(int m)
+{
+    return sizeof(zd) * (size_t)m * m + 4 * sizeof(cf) * (size_t)m * ez_ld(m) + sizeof(cf) * (size_t)m +
+           sizeof(zd) * (size_t)m + 4 * sizeof(float) * (size_t)m + 2 * sizeof(zd) * (size_t)m + sizeof(int) * (size_t)m;
+}
+
+__global__ void __launch_bounds__(EZ_T) k_eig_refined(int m, const zd *__restrict__ A, int64_t lda, int64_t sA,
+                                                      const zd *__restrict__ B, int64_t ldb, int64_t sB,
+                                                      zd *__restrict__ alpha, zd *__restrict__ beta,
+                                                      zd *__restrict__ V, int64_t ldv, int64_t sV, zd *work)
+{
+    extern __shared__ zd smem[];
+    __shared__ float red[EZ_T / 32];
+    __shared__ unsigned s_ea, s_eb;
+    __shared__ int s_bad;
+    const int b = blockIdx.x, t = threadIdx.x, ld = ez_ld(m);
+    A += (int64_t)b * sA;
+    B += (int64_t)b * sB;
+    V += (int64_t)b * sV;
+    alpha += (int64_t)b * m;
+    beta += (int64_t)b * m;
+    int *redo = (int *)(work + (int64_t)b * m * m);
+    zd *Vd = smem;                                  // V, column-major, ld m
+    zd *lam = Vd + (size_t)m * m;
+    zd *pu = lam + m;                               // pair (i, j): U = [1 pu_i; pu_j 1], and det U
+    zd *pd = pu + m;
+    cf *H = (cf *)(pd + m), *Z = H + m * ld, *W = Z + m * ld, *L = W + m * ld, *hv = L + m * ld;
+    float *lf = (float *)(hv + m);                  // lambda as double-single pairs: 4 floats each
+    int *part = (int *)(lf + 4 * m);                // the index this one is too close to, or -1
+    const cf zero = cmakef(0.f, 0.f);
+    if (t == 0) { s_ea = 0; s_eb = 0; s_bad = 0; *redo = 1; }
+    __syncthreads();
+    {
+        unsigned ha = 0, hb = 0;
+        for (int e = t; e < m * m; e += EZ_T) {
+            const int r = e % m, c = e / m;
+            ha = max(ha, ez_hi(A[r + c * lda]));
+            if (r <= c) hb = max(hb, ez_hi(B[r + c * ldb]));
+        }
+        atomicMax(&s_ea, ha);
+        atomicMax(&s_eb, hb);
+    }
+    __syncthreads();
+    // A' = 2^-ea A, B' = 2^-eb B have entries below 1; lambda' = 2^(eb - ea) lambda
+    const int xa = (int)(s_ea >> 20), xb = (int)(s_eb >> 20);
+    if (xa < 523 || xa > 1523 || xb < 523 || xb > 1523) return;   // zero, non-finite or far out of range: QZ
+    const double fa = ez_pow2(1022 - xa), fb = ez_pow2(1022 - xb), fl = ez_pow2(xa - xb);
+    for (int e = t; e < m * m; e += EZ_T) {
+        const int r = e % m, c = e / m;
+        const zd a = A[r + c * lda];
+        H[r * ld + c] = cmakef((float)(a.x * fa), (float)(a.y * fa));
+        cf v = zero;
+        if (r <= c) {
+            const zd w = B[r + c * ldb];
+            v = cmakef((float)(w.x * fb), (float)(w.y * fb));
+        }
+        W[r * ld + c] = v;
+        if (r == c && !(cabs2(v) > 1e-14f)) s_bad = 1;            // |B_ii| <= 1e-7 max|B|
+        L[r * ld + c] = cmakef(r == c ? 1.f : 0.f, 0.f);
+    }
+    __syncthreads();
+    if (s_bad) return;
+    // H = C = B'^{-1} A', L = B'^{-1}
+    ez_back_solve<false>(m, ld, W, H, L);
+    float cn = 0.f;
+    for (int e = t; e < m * m; e += EZ_T) {
+        const float a = cabs2(H[(e / m) * ld + e % m]);
+        cn = fmaxf(cn, a == a ? a : __int_as_float(0x7f800000));   // (fmaxf drops a NaN)
+    }
+    cn = sqrtf(ez_max(cn, red));
+    if (!(cn > 0.f && cn < 1e15f)) return;
+    ez_hess(m, ld, H, Z, hv);
+    if (t < EZ_Q && !ez_qr(m, ld, H, Z, 6e-8f * cn) && t == 0) s_bad = 1;
+    __syncthreads();
+    if (s_bad) return;
+    // Y into W; V = Z Y with unit columns; L^H = (B' V)^{-1} = D Y^{-1} Z^H B'^{-1}
+    ez_vectors(m, ld, H, W, 1e-5f * cn);
+    for (int j = t; j < m; j += EZ_T) lam[j] = zmake((double)H[j * ld + j].x, (double)H[j * ld + j].y);
+    __syncthreads();
+    for (int e = t; e < m * m; e += EZ_T) H[(e / m) * ld + e % m] = cmakef(e / m == e % m ? 1.f : 0.f, 0.f);
+    __syncthreads();
+    ez_back_solve<true>(m, ld, W, H, nullptr);      // H = Y^{-1}
+    {
+        cf *T1 = (cf *)Vd;                          // (V is not there yet)
+        ez_mul<true>(m, ld, H, Z, T1);              // needs m ld entries: ld <= 2 m
+        ez_mul<false>(m, ld, T1, L, H);             // H = Y^{-1} Z^H B'^{-1}
+        ez_mul<false>(m, ld, Z, W, L);              // L = Z Y
+    }
+    for (int j = t; j < m; j += EZ_T) {
+        float s = 0.f;
+        for (int r = 0; r < m; ++r) s += cabs2(L[r * ld + j]);
+        lf[j] = sqrtf(s);
+    }
+    __syncthreads();
+    for (int e = t; e < m * m; e += EZ_T) {
+        const int r = e % m, c = e / m;
+        const float d = lf[c], di = 1.f / d;
+        cf v = L[r * ld + c];
+        v = cmakef(v.x * di, v.y * di);
+        L[r * ld + c] = v;                          // V in FP32
+        Vd[r + c * m] = zmake((double)v.x, (double)v.y);
+    }
+    for (int e = t; e < m * m; e += EZ_T) {
+        const int r = e / m, c = e % m;
+        cf v = H[r * ld + c];
+        H[r * ld + c] = cmakef(v.x * lf[r], v.y * lf[r]);
+    }
+    // delta = || I - L^H B' V ||_F (B' again into W, B' V into Z, the product into W)
+    for (int e = t; e < m * m; e += EZ_T) {
+        const int r = e % m, c = e / m;
+        cf v = zero;
+        if (r <= c) {
+            const zd w = B[r + c * ldb];
+            v = cmakef((float)(w.x * fb), (float)(w.y * fb));
+        }
+        W[r * ld + c] = v;
+    }
+    __syncthreads();
+    ez_mul<false>(m, ld, W, L, Z);
+    ez_mul<false>(m, ld, H, Z, W);
+    float dl = 0.f;
+    for (int e = t; e < m * m; e += EZ_T) {
+        const int r = e / m, c = e % m;
+        cf v = W[r * ld + c];
+        if (r == c) v.x -= 1.f;
+        dl += cabs2(v);
+    }
+    dl = sqrtf(ez_sum(dl, red));
+    if (!(dl < 0.05f)) return;
+    bool done = false;
+    float gprev = 0.f;
+    for (int step = 0; step < EZ_STEPS && !done; ++step) {
+        for (int j = t; j < m; j += EZ_T) {
+            const zd l = lam[j];
+            const float hx = (float)l.x, hy = (float)l.y;
+            lf[4 * j] = hx;
+            lf[4 * j + 1] = (float)(l.x - (double)hx);
+            lf[4 * j + 2] = hy;
+            lf[4 * j + 3] = (float)(l.y - (double)hy);
+            part[j] = -1;
+        }
+        // R' = 2^-ea (A V - B V Lambda), a 4 x 4 tile per thread, into W (FP32)
+        {
+            const int tx = t & 15, ty = t >> 4;
+            zd ra[4][4], rb[4][4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) ra[i][j] = rb[i][j] = zmake(0.0, 0.0);
+            const int ilo = ty;   // B's rows ty, ty + 16, ...: nothing left of column ty
+            for (int p = 0; p < m; ++p) {
+                zd a[4], v[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) a[i] = (ty + 16 * i < m) ? A[ty + 16 * i + p * lda] : zmake(0.0, 0.0);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) v[j] = (tx + 16 * j < m) ? Vd[p + (tx + 16 * j) * m] : zmake(0.0, 0.0);
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (16 * i < m)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if (16 * j < m) zfma(ra[i][j], a[i], v[j]);
+                if (p < ilo) continue;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    // (uniform over a warp's two rows but for the diagonal's neighbour, where B is zero)
+                    if (16 * i < m && p >= 16 * i) {
+                        const zd w = (ty + 16 * i <= p) ? B[ty + 16 * i + p * ldb] : zmake(0.0, 0.0);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if (16 * j < m) zfma(rb[i][j], w, v[j]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int c = tx + 16 * j;
+                if (c >= m) continue;
+                const zd l = zscale(lam[c], fl);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int r = ty + 16 * i;
+                    if (r >= m) continue;
+                    const zd d = zscale(zsub(ra[i][j], zmul(l, rb[i][j])), fa);
+                    W[r * ld + c] = cmakef((float)d.x, (float)d.y);
+                }
+            }
+        }
+        __syncthreads();
+        ez_mul<false>(m, ld, H, W, Z);              // Z = L^H R'
+        float gm = 0.f;
+        bool paired = false;
+        for (int e = t; e < m * m; e += EZ_T) {
+            const int i = e / m, j = e % m;
+            if (i == j) continue;
+            const cf w = Z[i * ld + j];
+            const cf d = cmakef((lf[4 * j] - lf[4 * i]) + (lf[4 * j + 1] - lf[4 * i + 1]),
+                                (lf[4 * j + 2] - lf[4 * i + 2]) + (lf[4 * j + 3] - lf[4 * i + 3]));
+            const float w2 = cabs2(w), d2 = cabs2(d);
+            cf gg = zero;
+            if (sqrtf(w2) <= 1e-14f * cn) {
+                // coupling at rounding level: converged.  (For a close pair G
+                // may still be large, and V G in FP32 would put FP32 errors
+                // back into V: only a small one is applied.)
+                if (w2 <= 1e-16f * d2 && d2 > 1e-30f) W[i * ld + j] = cdiv(w, d);
+                else W[i * ld + j] = zero;
+                continue;
+            } else if (w2 <= EZ_PAIR * EZ_PAIR * d2 && d2 > 1e-30f) {
+                gg = cdiv(w, d);
+            } else {
+                const int pi = atomicCAS(part + i, -1, j), pj = atomicCAS(part + j, -1, i);
+                if ((pi != -1 && pi != j) || (pj != -1 && pj != i)) s_bad = 1;
+                paired = true;
+            }
+            gm = fmaxf(gm, cabs2(gg));
+            W[i * ld + j] = gg;
+        }
+        gm = sqrtf(ez_max(gm, red));                // (a barrier: s_bad, the pairs and G are out)
+        paired = __syncthreads_or(paired);
+        if (s_bad) return;
+        if (t < m) {
+            const int i = t, j = part[t];
+            const cf w = Z[i * ld + i];
+            const zd li = zmake(lam[i].x + (double)w.x, lam[i].y + (double)w.y);
+            if (j > i) {
+                // the block [a b; c d] of Lambda + W: eigenvectors (1, c / g) and (-b / g, 1),
+                // g = h + s, h = (a - d) / 2, s = sqrt(h^2 + b c) on the side of h
+                const cf wj = Z[j * ld + j], wb = Z[i * ld + j], wc = Z[j * ld + i];
+                const zd lj = zmake(lam[j].x + (double)wj.x, lam[j].y + (double)wj.y);
+                const zd bb = zmake((double)wb.x, (double)wb.y), cc = zmake((double)wc.x, (double)wc.y);
+                const zd h = zscale(zsub(li, lj), 0.5);
+                zd r = zsqrt_d(zadd(zmul(h, h), zmul(bb, cc)));
+                if (r.x * h.x + r.y * h.y < 0.0) r = zscale(r, -1.0);
+                const zd g = zadd(h, r), mid = zscale(zadd(li, lj), 0.5);
+                if (g.x == 0.0 && g.y == 0.0) {
+                    s_bad = 1;
+                } else {
+                    pu[i] = zscale(zdiv(bb, g), -1.0);
+                    pu[j] = zdiv(cc, g);
+                    const zd det = zsub(zmake(1.0, 0.0), zmul(pu[i], pu[j]));
+                    if (!(zabs2(det) > 2.5e-3)) s_bad = 1;   // nearly parallel: not for this iteration
+                    pd[i] = pd[j] = det;
+                }
+                lam[i] = zadd(mid, r);
+                lam[j] = zsub(mid, r);
+                W[i * ld + j] = W[j * ld + i] = zero;
+            } else if (j < 0) {
+                lam[i] = li;
+            }
+            W[i * ld + i] = zero;
+        }
+        __syncthreads();
+        if (s_bad) return;
+        ez_mul<false>(m, ld, L, W, Z);              // V G
+        for (int e = t; e < m * m; e += EZ_T) {
+            const int r = e % m, c = e / m;
+            const cf g = Z[r * ld + c];
+            Vd[e] = zmake(Vd[e].x + (double)g.x, Vd[e].y + (double)g.y);
+        }
+        __syncthreads();
+        if (paired || gm > 1e-6f) {
+            // L^H <- (I - G) L^H (to be (B V)^{-1} of the new V up to |G|^2)
+            ez_mul<false>(m, ld, W, H, Z);
+            for (int e = t; e < m * m; e += EZ_T) {
+                const int o = (e / m) * ld + e % m;
+                H[o] = cmakef(H[o].x - Z[o].x, H[o].y - Z[o].y);
+            }
+            __syncthreads();
+            dl += (float)m * gm * gm;
+        } else {
+            dl += (float)m * gm;
+        }
+        // V[:, (i j)] <- V[:, (i j)] U, rows (i j) of L^H <- U^{-1} L^H
+        for (int e = t; e < m * m; e += EZ_T) {
+            const int r = e % m, i = e / m, j = part[i];
+            if (j <= i) continue;
+            zd vi = Vd[r + i * m], vj = Vd[r + j * m];
+            Vd[r + i * m] = zadd(vi, zmul(vj, pu[j]));
+            Vd[r + j * m] = zadd(vj, zmul(vi, pu[i]));
+            const zd di = zdiv(zmake(1.0, 0.0), pd[i]);
+            const cf hi = H[i * ld + r], hj = H[j * ld + r];
+            const zd xi = zmake((double)hi.x, (double)hi.y), xj = zmake((double)hj.x, (double)hj.y);
+            const zd yi = zmul(di, zsub(xi, zmul(pu[i], xj))), yj = zmul(di, zsub(xj, zmul(pu[j], xi)));
+            H[i * ld + r] = cmakef((float)yi.x, (float)yi.y);
+            H[j * ld + r] = cmakef((float)yj.x, (float)yj.y);
+        }
+        __syncthreads();
+        for (int e = t; e < m * m; e += EZ_T) {
+            const int r = e % m, c = e / m;
+            const zd v = Vd[e];
+            L[r * ld + c] = cmakef((float)v.x, (float)v.y);
+        }
+        __syncthreads();
+        // what this step leaves, by the bound on delta or by the contraction
+        // seen (|G| over the step before's, at least delta); a pair's block is
+        // followed by another step
+        const double seen = 8.0 * fmax((double)gm, (double)gm / (double)gprev), bnd = (double)m * (double)gm + (double)dl;
+        done = !paired && (double)gm * fmin(seen, bnd) <= EZ_DONE;
+        gprev = gm;
+    }
+    if (!done) return;
+    // unit columns, the eigenvalues on their own scale
+    {
+        const int j = t >> 2;                       // four threads per column
+        double s = 0.0;
+        if (j < m)
+            for (int r = t & 3; r < m; r += 4) s += zabs2(Vd[r + j * m]);
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        const double inv = 1.0 / sqrt(s);
+        if (j < m)
+            for (int r = t & 3; r < m; r += 4) V[r + j * ldv] = zscale(Vd[r + j * m], inv);
+        if (j < m && (t & 3) == 0) {
+            alpha[j] = zscale(lam[j], fl);
+            beta[j] = zmake(1.0, 0.0);
+        }
+    }
+    if (t == 0) *redo = 0;
+}
 }  // namespace
 
 size_t zqz_work_bytes(int m)
@@ -330,6 +1014,16 @@ size_t zqz_work_bytes(int m)
     return (big + 255) & ~(size_t)255;
 }
 
+int zeig_refined(cudaStream_t s, int m, int batch, const zd *A, int64_t lda, int64_t sA, const zd *B, int64_t ldb,
+                 int64_t sB, zd *alpha, zd *beta, zd *V, int64_t ldv, int64_t sV, void *work)
+{
+    if (m < EZ_MIN_M || m > 64 || batch <= 0) return FEAST_EINVAL;
+    FEAST_CUDA_TRY(ensure_dyn_smem(k_eig_refined, ez_smem_bytes(m)));
+    k_eig_refined<<<batch, EZ_T, ez_smem_bytes(m), s>>>(m, A, lda, sA, B, ldb, sB, alpha, beta, V, ldv, sV, (zd *)work);
+    FEAST_LAUNCH_CHECK();
+    return FEAST_OK;
+}
+
 int zqz_batched(cudaStream_t s, int m, int batch, zd *A, int64_t lda, int64_t sA, zd *B,
                 int64_t ldb, int64_t sB, zd *alpha, zd *beta, zd *V, int64_t ldv, int64_t sV,
                 void *work, int *fail, int *timeout, int *stats, double defl)
@@ -337,8 +1031,17 @@ int zqz_batched(cudaStream_t s, int m, int batch, zd *A, int64_t lda, int64_t sA
     if (m <= 0 || batch <= 0) return FEAST_OK;
     if (m <= 64) {
         size_t sm = 3 * (size_t)m * m * sizeof(zd);
+        // refined FP32 Schur form first (GB300, one pencil per SM: 0.61 ms at
+        // m = 24 and 3.6 ms at m = 64, against 10.5 and 67 ms for k_qz, whose
+        // every rotation is a chain of FP64 instructions); k_qz then solves
+        // the pencils that it left (its CTAs return at once on the others).
+        // Up to two rows there is nothing to iterate: k_qz alone.
+        const int refined = m >= EZ_MIN_M;
+        int e;
+        if (refined && (e = zeig_refined(s, m, batch, A, lda, sA, B, ldb, sB, alpha, beta, V, ldv, sV, work))) return e;
         FEAST_CUDA_TRY(ensure_dyn_smem(k_qz<128>, sm));
-        k_qz<128><<<batch, 128, sm, s>>>(m, A, lda, sA, B, ldb, sB, alpha, beta, V, ldv, sV, (zd *)work, 1, fail);
+        k_qz<128><<<batch, 128, sm, s>>>(m, A, lda, sA, B, ldb, sB, alpha, beta, V, ldv, sV, (zd *)work, 1, fail,
+                                         refined);
         FEAST_LAUNCH_CHECK();
         return FEAST_OK;
     }
