@@ -371,12 +371,11 @@ int schur_large(cudaStream_t s, int m, zd *C, zd *Q, void *work, int *fail, int 
 // back-substitution; unit 2-norm columns.
 // scratch: m x m (T transposed, for contiguous row reads).
 int schur_vectors(cudaStream_t s, int m, const zd *T, zd *Y, double snorm, zd *scratch);
-// The same Schur form with the QR in plain FP32 (k_zeig32.cu): Q unitary
-// and T triangular to ~1e-6 relative -- a start for an FP64 polish.
-// work: schur_large_work_bytes_fp32(m) (= schur_large_work_bytes(m)).
-size_t schur_large_work_bytes_fp32(int m);
-int schur_large_fp32(cudaStream_t s, int m, zd *C, zd *Q, void *work, int *fail, int *timeout, int *stats,
-                     double *hn_out, double defl);
+// Schur form of a complex64 m x m matrix in plain FP32 (k_zeig32.cu): C <- T
+// = Q^H C Q, Q unitary to FP32; cmax: max |C_ij|.  *fail is raised when the
+// iteration's budget runs out.  work: schur32_work_bytes(m).
+size_t schur32_work_bytes(int m);
+int schur32(cudaStream_t s, int m, cf *C, cf *Q, float cmax, void *work, int *fail, int *timeout, int *stats);
 int normalise_cols(cudaStream_t s, int m, zd *V);
 
 // SEARCH (k_search.cu): out = sum_j Re(y_j^H u_j) over p columns; the
@@ -393,26 +392,22 @@ size_t rrqr_work_bytes(int64_t n, int m);
 int rrqr_basis(cudaStream_t s, int64_t n, int m, const zd *U, zd *Q, double rank_tol, void *work, int *timeout,
                int *t_out);
 
-// Warm-started projected eigensolve (k_warm.cu).
-struct WarmParams {
-    int min_m;          // smallest m that tries it
-    int min_tail;       // smallest trailing block given to the QR
-    double tau;         // column of C counted converged: ||C[j+1:, j]|| <= tau max|C|
-    double accept_tol;  // largest relative eigen-residual accepted
-    double tail_defl;   // relative deflation tolerance of the tail QR (0: the floor)
-    int cold_fp32;      // 1: no converged block assumed -- the whole matrix
-                        // through the FP32 QR, its Schur vectors made unitary
-                        // in FP64 (BCGS2), then the Newton step
+// Projected eigensolve by an FP32 Schur form and a Newton iteration with an
+// FP64 residual, cold or warm-started (k_warm.cu).
+struct RefineParams {
+    int warm;           // 1: C's leading columns may have converged (ordered Ritz pairs)
+    double target;      // error of the eigenvectors at which the iteration may end
 };
-struct WarmResult {
+struct RefineResult {
     int accepted;   // 1: alpha, beta, V hold the eigenpairs
     int k;          // converged leading columns found
     int tail;       // rows of the block given to the QR
-    double resid;   // largest relative eigen-residual of the Newton step
+    int steps;      // Newton steps taken
+    double resid;   // estimated error left by the last step
 };
-size_t zeig_warm_work_bytes(int m);
-// Events around the warm solve's FP64 product segments (GEMMs and
-// triangular inverses), for the per-kernel roofline: pairs (begin, end) in
+size_t zeig_refined_large_work_bytes(int m);
+// Events around the projected solve's FP64 product segments, for the
+// per-kernel roofline: pairs (begin, end) in
 // ev[0 .. used), with the segments' algorithmic flops (complex MAC = 8).
 struct GemmTimer {
     static constexpr int kMax = 10;
@@ -420,11 +415,12 @@ struct GemmTimer {
     int used;
     double flops;
 };
-// A, Bt as zeig_large (both overwritten whether accepted or not).  qz_work:
-// zeig_large_work_bytes(m) bytes.  gt (may be null): segment timer.
-int zeig_warm(cudaStream_t s, int m, zd *A, zd *Bt, zd *alpha, zd *beta, zd *V, void *warm_work, void *qz_work,
-              const WarmParams &prm, WarmResult *res, int *fail, int *timeout, int *stats, GemmTimer *gt = nullptr,
-              const OzScratch *oz = nullptr);
+// A, Bt as zeig_large, kept; V is overwritten whether accepted or not.  gt (may
+// be null): segment timer; oz (may be null): digit-plane scratch.  Synchronises
+// the stream.
+int zeig_refined_large(cudaStream_t s, int m, const zd *A, const zd *Bt, zd *alpha, zd *beta, zd *V, void *work,
+                       const RefineParams &prm, RefineResult *res, int *timeout, int *stats,
+                       GemmTimer *gt = nullptr, const OzScratch *oz = nullptr);
 // Line 16 on Ritz pairs in defect form (k_defect.cu):
 // U = X rho(Lambda) + sum_j w_j M_j^{-1} (R D_j), R = A X - B X Lambda.
 struct DefectScratch {

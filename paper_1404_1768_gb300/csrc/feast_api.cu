@@ -86,7 +86,7 @@ struct feast_ctx {
     void *chol_work;    // Cholesky QR (dense precision form)
     void *search_work;  // SEARCH's rank-revealing factorisation
     void *qz_work;
-    void *warm_work;    // warm-started projected eigensolve (m0 >= kWarmMinM)
+    void *warm_work;    // refined projected eigensolve (m0 > 64)
     int *pair_perm;     // m0: order of the Ritz pairs (most converged next pass first)
     zd *ord_x, *ord_ab; // gather targets for X (n x m0) and [A X | B X] (n x 2 m0)
     DevStatus *st;
@@ -119,9 +119,9 @@ struct feast_ctx {
     double *zw_host;    // nodes and weights (2 q complex), for rho(lambda)
     int ritz_filter;    // line 16 of this pass filters the Ritz vectors
     int warm_ready;     // U1 comes from ordered Ritz vectors: line 6 may start warm
-    WarmResult last_warm;
+    RefineResult last_warm;
     int warm_tried;
-    int cold_fp32;      // this pass: 1 FP32 QR + Newton accepted, -1 tried and not accepted
+    int cold_fp32;      // this pass, started cold: 1 FP32 QR + Newton accepted, -1 tried and not accepted
     int k, c_prev, done, cur;
     double e_prev;
     int out_count, out_flag, out_k;
@@ -133,16 +133,10 @@ struct feast_ctx {
 
 namespace {
 
-// Projected problems this large take the warm-started solve (k_warm.cu)
-// once a pass has ordered its Ritz pairs.
+// Projected problems this large are solved warm (k_warm.cu) once a pass has
+// ordered its Ritz pairs.
 constexpr int kWarmMinM = 96;
-constexpr int kWarmMinTail = 65;     // the QR's own size range (m > 64)
-constexpr double kWarmTauMin = 1e-8; // converged column: strictly lower part <= tau max|C|
-constexpr double kWarmAccMin = 1e-12;  // the cold double-single QR's own backward error (2^-44 of ||H||)
-// A cold pass whose pairs are needed to at least this (relative eigen-
-// residual) tries the FP32 QR polished by the Newton step first: from an
-// FP32 Schur form (~1e-6 remainder) one Newton step reaches ~1e-10.
-constexpr double kColdFp32AccMin = 1e-8;
+constexpr double kWarmAccMin = 1e-12;  // the double-single QR's own backward error (2^-44 of ||H||)
 constexpr int kZeigMinM = 8;         // smallest projected problem on the standard-form QR
 // banded precision form: the n x m0 products go to the digit-sliced
 // tensor-core GEMM from this width on (below it the FP64 GEMMs of the tall,
@@ -295,8 +289,8 @@ void carve(feast_ctx *c, Carver &cv)
     c->orth_work = cv.take<zd>(zorth_work_elems((int64_t)n, (int64_t)m));
     c->qz_work = cv.take<char>(std::max(zqz_work_bytes((int)m), (zeig_large_work_bytes((int)m) + 255) & ~(size_t)255));
     c->search_work = cv.take<char>(rrqr_work_bytes((int64_t)n, (int)m));
+    if ((int)m > 64) c->warm_work = cv.take<char>(zeig_refined_large_work_bytes((int)m));
     if ((int)m >= kWarmMinM) {
-        c->warm_work = cv.take<char>(zeig_warm_work_bytes((int)m));
         c->pair_perm = cv.take<int>(m);
         c->ord_x = cv.take<zd>(n * m);
         c->ord_ab = cv.take<zd>(2 * n * m);
@@ -879,7 +873,7 @@ static int iterate_impl(feast_ctx *c, feast_iter_info *info)
     FEAST_CUDA_TRY(cudaEventRecord(c->ev[1], s));
     // line 6: projected eigenpairs, x_i = U1 y_i
     FEAST_CUDA_TRY(cudaMemsetAsync(&c->st->qz_sweeps, 0, 3 * sizeof(int), s));
-    c->last_warm = WarmResult{};
+    c->last_warm = RefineResult{};
     c->gt.used = 0;
     c->gt.flops = 0.0;
     c->warm_tried = c->warm_ready;
@@ -891,39 +885,25 @@ static int iterate_impl(feast_ctx *c, feast_iter_info *info)
     // accuracy, as at any pass that may stop)
     const bool final_pass = c->k >= c->max_iter && !c->no_stop;
     const double acc = final_pass ? kWarmAccMin : fmax(kWarmAccMin, 1e-3 * eref);
-    if (c->warm_ready) {
-        // the previous pass filtered its |rho|-ordered Ritz vectors: C is
-        // block upper triangular up to a remainder of the size of its
-        // residuals.  A converged column's remainder enters the Newton step
-        // squared over an eigenvalue gap (~1e-3 of max|C| and up):
-        // tau^2 / 1e-3 <= tol
-        const double tau = fmin(1e-5, fmax(kWarmTauMin, sqrt(1e-3 * acc)));
-        // the tail QR deflates at 1e-3 of the acceptance tolerance, and at
-        // most at 1e-2 eps: its backward error (~ the deflation times
-        // max|C|) then stays far below the residual a stop needs
-        const WarmParams prm{kWarmMinM, kWarmMinTail, tau, acc, fmin(1e-3 * acc, 1e-2 * c->eps), 0};
-        FEAST_CUDA_TRY(cudaMemcpyAsync(c->Q, c->P, sizeof(zd) * 2 * m * m, cudaMemcpyDeviceToDevice, s));
-        // (the Newton step's defect-form products on the digit-sliced
-        // tensor-core GEMM where the context has its scratch)
-        if ((e = zeig_warm(s, (int)m, c->Q, c->Q + m * m, c->alpha, c->beta, c->Yv, c->warm_work, c->qz_work, prm,
-                           &c->last_warm, &c->st->qz_fail, &c->st->timeout, &c->st->qz_sweeps, &c->gt, orth_oz(c))))
+    if (m > 64) {
+        // FP32 Schur form (of the unconverged trailing block, when the
+        // previous pass filtered its ordered Ritz vectors) and Newton steps
+        // until the eigenvectors are two decades below that accuracy; their
+        // residuals' products run on the digit-sliced tensor-core GEMM where
+        // the context has its scratch, as far as its resolution goes
+        const zd *Ap = c->P, *Bp = c->P + m * m;
+        if (rr) {
+            FEAST_CUDA_TRY(cudaMemcpyAsync(c->Q, c->P, sizeof(zd) * 2 * m * m, cudaMemcpyDeviceToDevice, s));
+            if ((e = triangularise_bt(c))) return e;
+            Ap = c->Q;
+            Bp = c->Q + m * m;
+        }
+        const RefineParams prm{c->warm_ready, 1e-2 * acc};
+        if ((e = zeig_refined_large(s, (int)m, Ap, Bp, c->alpha, c->beta, c->Yv, c->warm_work, prm, &c->last_warm,
+                                    &c->st->timeout, &c->st->qz_sweeps, &c->gt, orth_oz(c))))
             return e;
-        if (!c->last_warm.accepted) FEAST_CUDA_TRY(cudaMemsetAsync(&c->st->qz_fail, 0, sizeof(int), s));
-    }
-    if (!c->last_warm.accepted && !rr && c->warm_work && acc >= kColdFp32AccMin) {
-        // cold, but the pairs are needed only to acc: the Schur form of the
-        // whole matrix by the FP32 QR (its rotation chains are shorter),
-        // made exact by the FP64 Newton step -- whose error, the square of
-        // the FP32 remainder over an eigenvalue gap, is far below acc
-        // (its products on the digit-sliced tensor-core GEMM where the
-        // context has the scratch: ~48-bit per row and column, far beyond acc)
-        const WarmParams prm{kWarmMinM, kWarmMinTail, kWarmTauMin, acc, 0.0, 1};
-        FEAST_CUDA_TRY(cudaMemcpyAsync(c->Q, c->P, sizeof(zd) * 2 * m * m, cudaMemcpyDeviceToDevice, s));
-        if ((e = zeig_warm(s, (int)m, c->Q, c->Q + m * m, c->alpha, c->beta, c->Yv, c->warm_work, c->qz_work, prm,
-                           &c->last_warm, &c->st->qz_fail, &c->st->timeout, &c->st->qz_sweeps, &c->gt, orth_oz(c))))
-            return e;
-        c->cold_fp32 = c->last_warm.accepted ? 1 : -1;
-        if (!c->last_warm.accepted) FEAST_CUDA_TRY(cudaMemsetAsync(&c->st->qz_fail, 0, sizeof(int), s));
+        if (!c->last_warm.accepted) c->cold_fp32 = -1;
+        else if (c->last_warm.tail == (int)m) c->cold_fp32 = 1;
     }
     if (!c->last_warm.accepted) {
         // before any pair has been accepted the stop cannot fire at this

@@ -1,185 +1,375 @@
-// Warm-started solve of the projected eigenproblem (GFEAST line 6).
+// Projected eigensolve of more than 64 rows (GFEAST line 6): an FP32 Schur
+// form made exact by a Newton iteration whose residual alone is FP64.
 //
-// When the filter of line 16 is applied to the Ritz vectors of the previous
-// pass, ordered by their expected residual after filtering (r_i /
-// |rho(lambda_i)|, rho the filter function of eq. 4.1, so the most
-// converged pairs come first), the QR factorisation of line 17
-// keeps the order, and every leading group of converged Ritz vectors spans
-// an (almost) invariant subspace.  The projected matrix C = B~^{-1} A~ is
-// then block upper triangular up to a small remainder:
+// The pencil (A, B), B upper triangular, is reduced in FP32: C = B^{-1} A,
+// C = Q T Q^H (k_zeig32.cu), T Y = Y Lambda, V = Q Y, L^H = (B V)^{-1} =
+// Y^{-1} Q^H B^{-1}.  Then, until what a step leaves is below the caller's
+// target,
+//
+//     R = A V - B V Lambda  (FP64),  W = L^H R,  lambda_j += W_jj,
+//     G_ij = W_ij / (lambda_j - lambda_i),  V += V G,  L^H -= G L^H,
+//
+// as in k_eig_refined (k_zqz.cu), whose file comment has the reasoning: only R
+// carries FP64 products, everything else multiplies something small.  Two
+// eigenvalues closer than FP32 resolves are separated by the eigenvectors of
+// their own 2 x 2 block of Lambda + W.  R's two products are FP64 GEMMs, or
+// digit-sliced tensor-core GEMMs (48-bit per row and column) while the
+// iteration is still above their resolution.  It replaces a double-single QR
+// of the whole matrix (226 ms at 300 rows) and, in the precision form, an
+// FP32 QR whose polish took seven digit-sliced products, two FP64 triangular
+// inverses and an FP64 back-substitution.
+//
+// Warm start.  When the filter of line 16 is applied to the Ritz vectors of
+// the previous pass, ordered by their expected residual after filtering (r_i /
+// |rho(lambda_i)|, rho the filter function of eq. 4.1, so the most converged
+// pairs come first), the QR factorisation of line 17 keeps the order, and
+// every leading group of converged Ritz vectors spans an (almost) invariant
+// subspace: C is block upper triangular up to a small remainder,
 //
 //     C = [ T11 + E11   C12 ]      T11 upper triangular (k x k),
 //         [ E21         C22 ]      E11 strictly lower, E11 and E21 small.
 //
-// The solve below takes k from the column norms of C's strictly lower
-// part, computes the Schur form of the trailing block only (C22 = Z T22
-// Z^H, the double-single multishift QR of k_zeig.cu on m - k instead of m
-// rows), and treats what is left as a perturbation: with Zh = diag(I, Z)
-// and C' = Zh^H C Zh = T^ + D (T^ upper triangular, D small), one Newton
-// step for the eigen-decomposition of C' starting from the eigenvectors V^
-// of T^ gives
-//
-//     F = V^{-1} C' V^,   lambda_i = F_ii,   G_ij = F_ij / (lambda_j - lambda_i),
-//     Y' = V^ (I + G),    Y = Zh Y'          (error O(|D|^2 / gap)).
-//
-// The products that define C and C' (B~^{-1} A~, the similarity with Z)
-// are FP64 GEMMs; the triangular solves are products with explicit
-// triangular inverses.  The Newton step itself runs in defect form: with
-// T^ V^ = V^ Lh (Lh = diag T^), W' = C' V^ - V^ Lh = D V^ is small, F =
-// Lh + V^{-1} W', and the residual C' Y' - Y' L = V^ S1 + W' (I + G) with
-// S1 small too.  Every one of these products has a small operand, so they
-// run on the digit-sliced tensor-core GEMM (48-bit fixed point per row and
-// column of its operands) at FP64 accuracy; computed as plain products of
-// O(1) matrices on it, the step's residual stalled near 3e-12 at m0 = 1280
-// instead of 1e-13.  (Without the digit-sliced scratch every product is an
-// FP64 GEMM.)  The eigenpairs are accepted only if each
-// ||C' y'_i - lambda_i y'_i|| / ((max|C_ij| + |lambda_i|) ||y'_i||) is at
-// most accept_tol; otherwise the caller runs the cold solve (Hessenberg
-// reduction and QR of the whole matrix).  The subspace of every pass is the
-// paper's (span of the filtered Ritz vectors = span of the filtered U1);
-// only the way the projected problem is solved changes.
+// k comes from the norms of the strictly lower parts of C's columns; the
+// Schur form is that of the trailing block alone (C22 = Z T22 Z^H, Q =
+// diag(I, Z), T = [T11 C12 Z; 0 T22]), and the iteration removes the
+// remainder along with FP32's error.  The subspace of every pass is the
+// paper's (span of the filtered Ritz vectors = span of the filtered U1); only
+// the way the projected problem is solved changes.
 #include "common.cuh"
 
 namespace feast {
 namespace {
 
-// Per column j: ||C[j+1:m, j]||_2 and max_i |C_ij|.  Warp per column.
-__global__ void k_col_stats(int m, const zd *__restrict__ C, double *__restrict__ lower, double *__restrict__ cmax)
+constexpr float RF_PAIR = 1.f / 16;   // largest G_ij of a step (beyond: the pair's own block)
+constexpr int RF_STEPS = 10;          // most steps
+constexpr float RF_TAU = 3e-6f;       // converged column: strictly lower part <= RF_TAU max|C|
+constexpr int RF_PART = 64;           // partial sums of the defect norm
+
+struct RefineStat {
+    unsigned gm;                      // bits of max |G|^2 (non-negative floats order like their bits)
+    int bad, paired, pad;
+};
+
+// X = [C | I], both m x m: C = A and the identity in FP32; B32 = the upper
+// triangle of Bt, Bu the same in FP64.  amax: bits of the largest |component|
+// of A and of B.
+__global__ void k_rf_cast(int m, const zd *__restrict__ A, const zd *__restrict__ Bt, cf *__restrict__ X,
+                          cf *__restrict__ B32, zd *__restrict__ Bu, unsigned *__restrict__ amax)
+{
+    const int64_t total = (int64_t)m * m;
+    float ma = 0.f, mb = 0.f;
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        const int i = (int)(e % m), j = (int)(e / m);
+        const zd a = A[e], b = (i <= j) ? Bt[e] : zmake(0.0, 0.0);
+        const cf af = cmakef((float)a.x, (float)a.y);
+        const cf bf = cmakef((float)b.x, (float)b.y);
+        X[e] = af;
+        X[total + e] = cmakef(i == j ? 1.f : 0.f, 0.f);
+        B32[e] = bf;
+        Bu[e] = b;
+        // (a NaN compares false below and must not be dropped: it counts as Inf)
+        const float sa = fabsf(af.x) + fabsf(af.y), sb = fabsf(bf.x) + fabsf(bf.y);
+        ma = (sa <= ma) ? ma : (sa == sa ? sa : __int_as_float(0x7f800000));
+        mb = (sb <= mb) ? mb : (sb == sb ? sb : __int_as_float(0x7f800000));
+    }
+    atomicMax(amax, __float_as_uint(ma));
+    atomicMax(amax + 1, __float_as_uint(mb));
+}
+
+// Per column j of C: ||C[j+1:m, j]||_2 and max_i |C_ij| (Inf for a NaN).  Warp per column.
+__global__ void k_col_stats32(int m, const cf *__restrict__ C, float *__restrict__ lower, float *__restrict__ cmax)
 {
     const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (j >= m) return;
-    const zd *c = C + (int64_t)j * m;
-    double s = 0.0, mx = 0.0;
+    const cf *c = C + (int64_t)j * m;
+    float s = 0.f, mx = 0.f;
     for (int i = lane; i < m; i += 32) {
-        const double a2 = zabs2(c[i]);
+        const float a2 = cabs2(c[i]);
         if (i > j) s += a2;
-        mx = fmax(mx, a2);
+        mx = (a2 <= mx) ? mx : (a2 == a2 ? a2 : __int_as_float(0x7f800000));
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
         s += __shfl_xor_sync(0xffffffffu, s, off);
-        mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
     }
     if (lane == 0) {
-        lower[j] = sqrt(s);
-        cmax[j] = sqrt(mx);
+        lower[j] = sqrtf(s);
+        cmax[j] = sqrtf(mx);
     }
 }
 
-__global__ void k_diag_lambda(int m, const zd *__restrict__ F, zd *__restrict__ alpha, zd *__restrict__ beta)
+// Out = In^T, complex64 m x m.
+__global__ void k_transpose32(int m, const cf *__restrict__ In, cf *__restrict__ Out)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= m) return;
-    alpha[i] = F[i + (int64_t)i * m];
-    beta[i] = zmake(1.0, 0.0);
+    __shared__ cf tile[32][33];
+    const int bx = blockIdx.x * 32, by = blockIdx.y * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    for (int r = ty; r < 32; r += 8)
+        if (bx + tx < m && by + r < m) tile[r][tx] = In[bx + tx + (int64_t)(by + r) * m];
+    __syncthreads();
+    for (int r = ty; r < 32; r += 8)
+        if (by + tx < m && bx + r < m) Out[by + tx + (int64_t)(bx + r) * m] = tile[tx][r];
 }
 
-// G_ij = F_ij / (lambda_j - lambda_i) off the diagonal, G_ii = 0 (in place).
-// A correction entry above 1/4 means the first-order step is not valid for
-// this pair: *bad is set and the solve is not accepted.
-__global__ void k_newton_g(int m, zd *__restrict__ F, const zd *__restrict__ lam, int *__restrict__ bad)
+// The eigenvectors of the upper triangle of T, one warp each: warps 0 .. m-1
+// the right ones (columns of Y, unit upper triangular, by back-substitution
+// along rows of T: Tt is T^T), warps m .. 2m-1 the left ones (rows of U =
+// Y^{-1}, by forward substitution along columns of T; U's conjugate transpose
+// is stored).  An entry whose eigenvalue is within small of the vector's own is
+// left at zero (the pair's block settles it in the iteration).  Bound by the
+// chain of m dot products; the warps of a CTA take vectors a grid apart, so
+// that long and short chains mix.
+__global__ void k_tri_vectors32(int m, const cf *__restrict__ T, const cf *__restrict__ Tt, cf *__restrict__ Y,
+                                cf *__restrict__ Uh, float small)
+{
+    extern __shared__ cf vec[];
+    const int lane = threadIdx.x & 31;
+    const int id = blockIdx.x + (int)gridDim.x * (threadIdx.x >> 5);
+    if (id >= 2 * m) return;
+    cf *y = vec + (size_t)(threadIdx.x >> 5) * m;
+    const bool right = id < m;
+    const int k = right ? id : id - m;
+    const cf lam = T[k + (int64_t)k * m];
+    const int cnt = right ? k : m - 1 - k;                 // entries to solve for
+    if (lane == 0) y[k] = cmakef(1.f, 0.f);
+    __syncwarp();
+    for (int st = 0; st < cnt; ++st) {
+        const int i = right ? k - 1 - st : k + 1 + st;
+        const cf *line = (right ? Tt : T) + (int64_t)i * m; // T[i, :] or T[:, i]
+        const int p0 = right ? i + 1 : k, p1 = right ? k : i - 1;
+        cf acc = cmakef(0.f, 0.f), ac2 = acc;
+        int p = p0 + lane;
+        for (; p + 32 <= p1; p += 64) {
+            cfma(acc, line[p], y[p]);
+            cfma(ac2, line[p + 32], y[p + 32]);
+        }
+        if (p <= p1) cfma(acc, line[p], y[p]);
+        acc = cadd(acc, ac2);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
+            acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
+        }
+        if (lane == 0) {
+            cf d = line[i];
+            d = cmakef(lam.x - d.x, lam.y - d.y);
+            y[i] = cabs2(d) < small * small ? cmakef(0.f, 0.f) : cdiv(acc, d);
+        }
+        __syncwarp();
+    }
+    cf *out = (right ? Y : Uh) + (int64_t)k * m;
+    for (int i = lane; i < m; i += 32) {
+        const bool on = right ? i <= k : i >= k;
+        const cf v = on ? y[i] : cmakef(0.f, 0.f);
+        out[i] = right ? v : cconj(v);
+    }
+}
+
+// Unit columns: V32 scaled, V its FP64 copy, nv the norms.  Warp per column.
+__global__ void k_rf_scale(int m, cf *__restrict__ V32, zd *__restrict__ V, float *__restrict__ nv)
+{
+    const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (j >= m) return;
+    cf *v = V32 + (int64_t)j * m;
+    float s = 0.f;
+    for (int i = lane; i < m; i += 32) s += cabs2(v[i]);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    const float nrm = sqrtf(s), inv = 1.f / nrm;
+    if (lane == 0) nv[j] = nrm;
+    for (int i = lane; i < m; i += 32) {
+        const cf x = cmakef(v[i].x * inv, v[i].y * inv);
+        v[i] = x;
+        V[i + (int64_t)j * m] = zmake((double)x.x, (double)x.y);
+    }
+}
+
+__global__ void k_rf_scale_rows(int m, cf *__restrict__ L, const float *__restrict__ nv)
 {
     const int64_t total = (int64_t)m * m;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
          e += (int64_t)gridDim.x * blockDim.x) {
-        const int i = (int)(e % m), j = (int)(e / m);
-        if (i == j) {
-            F[e] = zmake(0.0, 0.0);
-            continue;
-        }
-        const zd d = zsub(lam[j], lam[i]);
-        const zd f = F[e];
-        const double d2 = zabs2(d), f2 = zabs2(f);
-        if (!(f2 <= 0.0625 * d2)) {
-            if (f2 > 0.0) *bad = 1;
-            F[e] = zmake(0.0, 0.0);
-            continue;
-        }
-        F[e] = zdiv(f, d);
+        const float f = nv[e % m];
+        L[e] = cmakef(L[e].x * f, L[e].y * f);
     }
 }
 
-// max_i ||W_i - lambda_i Y_i|| / ((cnorm + |lambda_i|) ||Y_i||) into *out
-// (non-negative doubles order like their bit patterns); is_resid: W holds
-// the residual block itself.  Warp per column.
-__global__ void k_eig_resid(int m, const zd *__restrict__ W, const zd *__restrict__ Y, const zd *__restrict__ lam,
-                            double cnorm, unsigned long long *__restrict__ out, int is_resid = 0)
+// part[b] = block b's share of || E - I ||_F^2 (RF_PART blocks of 256).
+__global__ void k_rf_defect(int m, const cf *__restrict__ E, float *__restrict__ part)
 {
-    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (i >= m) return;
-    const zd l = lam[i];
-    const zd *w = W + (int64_t)i * m;
-    const zd *y = Y + (int64_t)i * m;
-    double r = 0.0, yy = 0.0;
-    for (int p = lane; p < m; p += 32) {
-        const zd yv = y[p];
-        const zd d = is_resid ? w[p] : zsub(w[p], zmul(l, yv));
-        r += zabs2(d);
-        yy += zabs2(yv);
+    __shared__ float red[8];
+    const int64_t total = (int64_t)m * m;
+    float s = 0.f;
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        cf v = E[e];
+        if (e % m == e / m) v.x -= 1.f;
+        s += cabs2(v);
     }
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        r += __shfl_xor_sync(0xffffffffu, r, off);
-        yy += __shfl_xor_sync(0xffffffffu, yy, off);
-    }
-    if (lane == 0) {
-        double rel = (yy > 0.0) ? sqrt(r / yy) / (cnorm + zabs(l)) : 1e300;
-        if (!(rel == rel)) rel = 1e300;
-        atomicMax(out, (unsigned long long)__double_as_longlong(rel));
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float r = 0.f;
+        for (int w = 0; w < 8; ++w) r += red[w];
+        part[blockIdx.x] = r;
     }
 }
 
-// D = C' - T^ (m x m; T^ upper triangular) and lamh = diag(T^).
-__global__ void k_defect_split(int m, const zd *__restrict__ Cq, const zd *__restrict__ Th, zd *__restrict__ D,
-                               zd *__restrict__ lamh)
+__global__ void k_rf_lam(int m, const cf *__restrict__ T, zd *__restrict__ lam)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < m) lam[i] = zmake((double)T[i + (int64_t)i * m].x, (double)T[i + (int64_t)i * m].y);
+}
+
+// R32 = A V - (B V) Lambda, rounded to FP32; part[j] = -1.
+__global__ void k_rf_resid(int m, const zd *__restrict__ AV, const zd *__restrict__ BV, const zd *__restrict__ lam,
+                           cf *__restrict__ R32, int *__restrict__ part)
 {
     const int64_t total = (int64_t)m * m;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
          e += (int64_t)gridDim.x * blockDim.x) {
-        const int i = (int)(e % m), j = (int)(e / m);
-        const zd t = Th[e];
-        D[e] = (i <= j) ? zsub(Cq[e], t) : Cq[e];
-        if (i == j) lamh[i] = t;
+        const int j = (int)(e / m);
+        const zd r = zsub(AV[e], zmul(lam[j], BV[e]));
+        R32[e] = cmakef((float)r.x, (float)r.y);
+        if (e % m == 0) part[j] = -1;
     }
 }
 
-// F_ii += lamh_i, then lambda_i = F_ii (alpha), beta_i = 1.
-__global__ void k_add_diag_lambda(int m, zd *__restrict__ F, const zd *__restrict__ lamh, zd *__restrict__ alpha,
-                                  zd *__restrict__ beta)
+// G from W (off the diagonal): see the file comment.  tiny: couplings at
+// rounding level are converged (only a small G is applied for them: V G in
+// FP32 would put FP32 errors back into V for a close pair).
+__global__ void k_rf_g(int m, const cf *__restrict__ W, const zd *__restrict__ lam, float tiny, cf *__restrict__ G,
+                       int *__restrict__ part, RefineStat *__restrict__ st)
+{
+    const int64_t total = (int64_t)m * m;
+    float gm = 0.f;
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        const int i = (int)(e % m), j = (int)(e / m);
+        cf g = cmakef(0.f, 0.f);
+        if (i != j) {
+            const cf w = W[e];
+            const zd dd = zsub(lam[j], lam[i]);
+            const cf d = cmakef((float)dd.x, (float)dd.y);
+            const float w2 = cabs2(w), d2 = cabs2(d);
+            if (sqrtf(w2) <= tiny) {
+                if (w2 <= 1e-16f * d2 && d2 > 1e-30f) g = cdiv(w, d);
+            } else if (w2 <= RF_PAIR * RF_PAIR * d2 && d2 > 1e-30f) {
+                g = cdiv(w, d);
+                gm = fmaxf(gm, cabs2(g));
+            } else {
+                const int pi = atomicCAS(part + i, -1, j), pj = atomicCAS(part + j, -1, i);
+                if ((pi != -1 && pi != j) || (pj != -1 && pj != i)) st->bad = 1;   // three or more that close
+                st->paired = 1;
+            }
+        }
+        G[e] = g;
+    }
+    if (gm > 0.f) atomicMax(&st->gm, __float_as_uint(gm));
+}
+
+__device__ __forceinline__ zd rf_sqrt(zd z)
+{
+    const double r = hypot(z.x, z.y);
+    if (r == 0.0) return zmake(0.0, 0.0);
+    if (z.x >= 0.0) {
+        const double t = sqrt(0.5 * (r + z.x));
+        return zmake(t, z.y / (2.0 * t));
+    }
+    const double t = sqrt(0.5 * (r - z.x));
+    return zmake(fabs(z.y) / (2.0 * t), copysign(t, z.y));
+}
+
+// lambda += diag(W); for a pair (i, j) the eigenvalues of its 2 x 2 block of
+// Lambda + W and the eigenvectors U = [1 pu_i; pu_j 1] (pd = det U), its
+// entries of G cleared.  lam_out is another array than lam.
+__global__ void k_rf_lambda(int m, const cf *__restrict__ W, const zd *__restrict__ lam, zd *__restrict__ lam_out,
+                            const int *__restrict__ part, cf *__restrict__ G, zd *__restrict__ pu,
+                            zd *__restrict__ pd, RefineStat *__restrict__ st)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m) return;
-    const zd f = zadd(F[i + (int64_t)i * m], lamh[i]);
-    F[i + (int64_t)i * m] = f;
-    alpha[i] = f;
+    const cf w = W[i + (int64_t)i * m];
+    const zd li = zmake(lam[i].x + (double)w.x, lam[i].y + (double)w.y);
+    const int j = part[i];
+    if (j < 0) lam_out[i] = li;
+    if (j <= i) return;
+    // block [a b; c d]: eigenvectors (1, c / g) and (-b / g, 1), g = h + s,
+    // h = (a - d) / 2, s = sqrt(h^2 + b c) on the side of h
+    const cf wj = W[j + (int64_t)j * m], wb = W[i + (int64_t)j * m], wc = W[j + (int64_t)i * m];
+    const zd lj = zmake(lam[j].x + (double)wj.x, lam[j].y + (double)wj.y);
+    const zd b = zmake((double)wb.x, (double)wb.y), c = zmake((double)wc.x, (double)wc.y);
+    const zd h = zscale(zsub(li, lj), 0.5);
+    zd s = rf_sqrt(zadd(zmul(h, h), zmul(b, c)));
+    if (s.x * h.x + s.y * h.y < 0.0) s = zscale(s, -1.0);
+    const zd g = zadd(h, s), mid = zscale(zadd(li, lj), 0.5);
+    zd u = zmake(0.0, 0.0), v = u;
+    if (g.x != 0.0 || g.y != 0.0) {
+        u = zscale(zdiv(b, g), -1.0);
+        v = zdiv(c, g);
+    } else {
+        st->bad = 1;
+    }
+    const zd det = zsub(zmake(1.0, 0.0), zmul(u, v));
+    if (!(zabs2(det) > 2.5e-3)) st->bad = 1;   // nearly parallel: not for this iteration
+    pu[i] = u;
+    pu[j] = v;
+    pd[i] = pd[j] = det;
+    lam_out[i] = zadd(mid, s);
+    lam_out[j] = zsub(mid, s);
+    G[i + (int64_t)j * m] = G[j + (int64_t)i * m] = cmakef(0.f, 0.f);
+}
+
+// V += VG; then, with pairs, V[:, (i j)] <- V[:, (i j)] U; V32 its FP32 copy.
+__global__ void k_rf_update(int m, const cf *__restrict__ VG, const int *__restrict__ part,
+                            const zd *__restrict__ pu, int paired, zd *__restrict__ V, cf *__restrict__ V32)
+{
+    const int64_t total = (int64_t)m * m;
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        const int r = (int)(e % m), i = (int)(e / m), j = paired ? part[i] : -1;
+        if (j >= 0 && j < i) continue;               // (its partner's thread writes both)
+        zd v = zmake(V[e].x + (double)VG[e].x, V[e].y + (double)VG[e].y);
+        if (j > i) {
+            const int64_t f = r + (int64_t)j * m;
+            const zd x = zmake(V[f].x + (double)VG[f].x, V[f].y + (double)VG[f].y);
+            const zd y = zadd(x, zmul(v, pu[i]));
+            v = zadd(v, zmul(x, pu[j]));
+            V[f] = y;
+            V32[f] = cmakef((float)y.x, (float)y.y);
+        }
+        V[e] = v;
+        V32[e] = cmakef((float)v.x, (float)v.y);
+    }
+}
+
+// Rows (i j) of L <- U^{-1} L for every pair.
+__global__ void k_rf_rows(int m, const int *__restrict__ part, const zd *__restrict__ pu, const zd *__restrict__ pd,
+                          cf *__restrict__ L)
+{
+    const int64_t total = (int64_t)m * m;
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        const int i = (int)(e % m), j = part[i];
+        if (j <= i) continue;
+        const int64_t f = e - i + j;
+        const zd di = zdiv(zmake(1.0, 0.0), pd[i]);
+        const zd xi = zmake((double)L[e].x, (double)L[e].y), xj = zmake((double)L[f].x, (double)L[f].y);
+        const zd yi = zmul(di, zsub(xi, zmul(pu[i], xj))), yj = zmul(di, zsub(xj, zmul(pu[j], xi)));
+        L[e] = cmakef((float)yi.x, (float)yi.y);
+        L[f] = cmakef((float)yj.x, (float)yj.y);
+    }
+}
+
+__global__ void k_rf_out(int m, const zd *__restrict__ lam, zd *__restrict__ alpha, zd *__restrict__ beta)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= m) return;
+    alpha[i] = lam[i];
     beta[i] = zmake(1.0, 0.0);
-}
-
-// S1 = (Lh - L) + Lh G - G L (Lh = diag(lamh), L = diag(lam)):
-// S1_ij = G_ij (lamh_i - lam_j) off the diagonal, lamh_i - lam_i on it
-// (G_ii = 0).
-__global__ void k_newton_s1(int m, const zd *__restrict__ G, const zd *__restrict__ lamh, const zd *__restrict__ lam,
-                            zd *__restrict__ S1)
-{
-    const int64_t total = (int64_t)m * m;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int i = (int)(e % m), j = (int)(e / m);
-        S1[e] = (i == j) ? zsub(lamh[i], lam[i]) : zmul(G[e], zsub(lamh[i], lam[j]));
-    }
-}
-
-// E <- (E - I) / 2 in place (m x m): the first-order term of (I + E)^{-1/2}.
-__global__ void k_sub_identity_half(int m, zd *__restrict__ E)
-{
-    const int64_t total = (int64_t)m * m;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int i = (int)(e % m), j = (int)(e / m);
-        zd v = E[e];
-        if (i == j) v.x -= 1.0;
-        E[e] = zmake(0.5 * v.x, 0.5 * v.y);
-    }
 }
 
 // Column gather: Vout[:, i] = Vin[:, perm[i]] (rows x m, leading dim rows).
@@ -195,28 +385,47 @@ __global__ void k_permute_cols(int64_t rows, int m, const int *__restrict__ perm
     }
 }
 
-struct WarmCarve {
-    zd *Cp, *W, *Yp, *S, *Z, *Ts;
-    double *lower, *cmax;
-    unsigned long long *res;
-    int *bad;
+struct RefineCarve {
+    cf *X, *T, *Q, *B32, *Y, *Uh, *V32, *L, *W, *G;   // X: [C | B^{-1}], 2 m^2 entries
+    zd *AV, *BV, *Bu, *lam, *lam2, *pu, *pd;
+    float *lower, *cmax, *nv, *part;
+    int *pair, *fail;
+    unsigned *amax;
+    RefineStat *st;
+    void *schur;
+    size_t bytes;
 };
 
-WarmCarve warm_carve(void *work, int m)
+RefineCarve refine_carve(void *work, int m)
 {
-    WarmCarve w;
+    RefineCarve w;
     const size_t mm = (size_t)m * m;
-    zd *p = (zd *)work;
-    w.Cp = p;
-    w.W = p + mm;
-    w.Yp = p + 2 * mm;
-    w.S = p + 3 * mm;
-    w.Z = p + 4 * mm;
-    w.Ts = p + 5 * mm;
-    w.lower = (double *)(w.Ts + tri_inverse_scratch_elems(m));
+    char *p = (char *)work;
+    size_t off = 0;
+    auto take = [&](size_t b) {
+        off = (off + 255) & ~(size_t)255;
+        char *q = p + off;
+        off += b;
+        return q;
+    };
+    w.X = (cf *)take(2 * mm * sizeof(cf));
+    cf **c32[] = {&w.T, &w.Q, &w.B32, &w.Y, &w.Uh, &w.V32, &w.L, &w.W, &w.G};
+    for (cf **c : c32) *c = (cf *)take(mm * sizeof(cf));
+    w.AV = (zd *)take(mm * sizeof(zd));
+    w.BV = (zd *)take(mm * sizeof(zd));
+    w.Bu = (zd *)take(mm * sizeof(zd));
+    zd **c64[] = {&w.lam, &w.lam2, &w.pu, &w.pd};
+    for (zd **c : c64) *c = (zd *)take((size_t)m * sizeof(zd));
+    w.lower = (float *)take(2 * (size_t)m * sizeof(float));
     w.cmax = w.lower + m;
-    w.res = (unsigned long long *)(w.cmax + m);
-    w.bad = (int *)(w.res + 1);
+    w.nv = (float *)take((size_t)m * sizeof(float));
+    w.part = (float *)take(RF_PART * sizeof(float));
+    w.pair = (int *)take((size_t)m * sizeof(int));
+    w.fail = (int *)take(sizeof(int));
+    w.amax = (unsigned *)take(8);
+    w.st = (RefineStat *)take(sizeof(RefineStat));
+    w.schur = take(schur32_work_bytes(m));
+    w.bytes = off;
     return w;
 }
 
@@ -228,10 +437,7 @@ unsigned grid_for(size_t count)
 
 }  // namespace
 
-size_t zeig_warm_work_bytes(int m)
-{
-    return sizeof(zd) * (5 * (size_t)m * m + tri_inverse_scratch_elems(m)) + sizeof(double) * 2 * (size_t)m + 64;
-}
+size_t zeig_refined_large_work_bytes(int m) { return refine_carve(nullptr, m).bytes + 256; }
 
 int permute_cols(cudaStream_t s, int64_t rows, int m, const int *perm, const zd *Vin, zd *Vout)
 {
@@ -240,184 +446,184 @@ int permute_cols(cudaStream_t s, int64_t rows, int m, const int *perm, const zd 
     return FEAST_OK;
 }
 
-int zeig_warm(cudaStream_t s, int m, zd *A, zd *Bt, zd *alpha, zd *beta, zd *V, void *warm_work, void *qz_work,
-              const WarmParams &prm, WarmResult *res, int *fail, int *timeout, int *stats, GemmTimer *gt,
-              const OzScratch *oz)
+
+int zeig_refined_large(cudaStream_t s, int m, const zd *A, const zd *Bt, zd *alpha, zd *beta, zd *V, void *work,
+                       const RefineParams &prm, RefineResult *res, int *timeout, int *stats, GemmTimer *gt,
+                       const OzScratch *oz)
 {
-    *res = WarmResult{};
-    if (m < prm.min_m) return FEAST_OK;
-    const WarmCarve w = warm_carve(warm_work, m);
+    *res = RefineResult{};
+    if (m < 3) return FEAST_OK;
+    const RefineCarve w = refine_carve((void *)(((uintptr_t)work + 255) & ~(uintptr_t)255), m);
     const size_t mm = (size_t)m * m;
     const zd one = zmake(1.0, 0.0), zero = zmake(0.0, 0.0);
-    const double m3 = (double)m * m * m, tri_inv = 8.0 * m3 / 6.0;   // m^3/6 MACs
-    // segment marks: begin, then end with the segment's algorithmic flops
-    auto mark = [&](double flops) -> int {
-        if (!gt || gt->used >= GemmTimer::kMax) return FEAST_OK;
-        FEAST_CUDA_TRY(cudaEventRecord(gt->ev[gt->used++], s));
-        gt->flops += flops;
-        return FEAST_OK;
-    };
+    const cf fone = cmakef(1.f, 0.f), fzero = cmakef(0.f, 0.f), fmone = cmakef(-1.f, 0.f);
     int e;
-    // C = beta C + alpha op(A) B: the FP64 GEMM (tri: the triangular zeros it
-    // may skip), or -- with oz, for a pass whose pairs are needed only well
-    // above FP64 rounding -- the FP64-accurate digit-sliced tensor-core GEMM
-    auto mul = [&](int conj_a, int64_t M, int64_t N, int64_t K, zd alpha, const zd *Am, int64_t lda, const zd *Bm,
-                   int64_t ldb, zd beta, zd *Cm, int64_t ldc, int tri) -> int {
-        if (!oz) return zgemm_batched(s, conj_a, M, N, K, alpha, Am, lda, 0, Bm, ldb, 0, beta, Cm, ldc, 0, 1, tri);
-        int r;
-        if ((r = oz_prepare_rows(s, M, K, Am, lda, oz->rows, conj_a))) return r;
-        if ((r = oz_prepare_cols(s, K, N, Bm, ldb, oz->cols))) return r;
-        return oz_gemm(s, M, N, K, oz->rows, oz->cols, alpha, nullptr, 0, beta, Cm, ldc, oz->err);
+    auto mul32 = [&](int conj_a, int64_t M, int64_t N, int64_t K, cf al, const cf *Am, int64_t lda, const cf *Bm,
+                     int64_t ldb, cf be, cf *Cm, int64_t ldc) {
+        return gemm_batched<cf>(s, conj_a, M, N, K, al, Am, lda, 0, Bm, ldb, 0, be, Cm, ldc, 0, 1);
     };
-    // the products that define C and C' themselves: FP64 unless the pass's
-    // pairs are needed only well above the digit-sliced GEMM's resolution
-    auto mulc = [&](int conj_a, int64_t M, int64_t N, int64_t K, zd alpha, const zd *Am, int64_t lda, const zd *Bm,
-                    int64_t ldb, zd beta, zd *Cm, int64_t ldc, int tri) -> int {
-        if (!prm.cold_fp32) return zgemm_batched(s, conj_a, M, N, K, alpha, Am, lda, 0, Bm, ldb, 0, beta, Cm, ldc, 0, 1, tri);
-        return mul(conj_a, M, N, K, alpha, Am, lda, Bm, ldb, beta, Cm, ldc, tri);
-    };
-    // C = B~^{-1} A~ (B~ = R2 is upper triangular), into Cp
-    if ((e = mark(0.0))) return e;
-    if ((e = tri_inverse(s, m, Bt, m, w.W, w.Ts))) return e;
-    if ((e = mulc(0, m, m, m, one, w.W, m, A, m, zero, w.Cp, m, 1))) return e;
-    if ((e = mark(tri_inv + 4.0 * m3))) return e;
-    const zd *C = w.Cp;
-    k_col_stats<<<cdiv((size_t)m * 32, 256), 256, 0, s>>>(m, C, w.lower, w.cmax);
+    // C = B^{-1} A and B^{-1}, FP32
+    FEAST_CUDA_TRY(cudaMemsetAsync(w.amax, 0, 8, s));
+    k_rf_cast<<<grid_for(mm), 256, 0, s>>>(m, A, Bt, w.X, w.B32, w.Bu, w.amax);
     FEAST_LAUNCH_CHECK();
-    double *h = (double *)malloc(sizeof(double) * 2 * (size_t)m);
-    if (!h) return FEAST_EINVAL;
-    if (cudaMemcpyAsync(h, w.lower, sizeof(double) * 2 * (size_t)m, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+    if ((e = trsm_upper_batched<cf>(s, m, 2 * m, 1, w.B32, m, 0, w.X, m, 0))) return e;
+    cf *C = w.X, *Bi = w.X + mm;
+    k_col_stats32<<<cdiv((size_t)m * 32, 256), 256, 0, s>>>(m, C, w.lower, w.cmax);
+    FEAST_LAUNCH_CHECK();
+    float *h = (float *)malloc(sizeof(float) * (2 * (size_t)m + RF_PART));
+    if (!h) return FEAST_ENOMEM;
+    float am[2] = {0.f, 0.f};
+    if (cudaMemcpyAsync(h, w.lower, sizeof(float) * 2 * (size_t)m, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaMemcpyAsync(am, w.amax, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess) {
         free(h);
         return FEAST_ECUDA;
     }
-    double hn = 0.0;
-    for (int j = 0; j < m; ++j) hn = fmax(hn, h[m + j]);
+    float cn = 0.f;
+    for (int j = 0; j < m; ++j) cn = h[m + j] > cn ? h[m + j] : cn;
     int k = 0;
-    if (!prm.cold_fp32)
-        while (k < m && h[k] <= prm.tau * hn) ++k;
-    free(h);
+    while (k < m && h[k] <= RF_TAU * cn) ++k;
     res->k = k;
-    if (prm.cold_fp32) {
-        k = 0;           // the whole matrix is the "tail"
-    } else if (k < m - prm.min_tail) {
-        if (k < m / 4) return FEAST_OK;  // too little has converged: cold solve
-    } else {
-        k = m - prm.min_tail;
-    }
+    free(h);
+    // (sizes whose squares FP32 holds; B singular shows as a non-finite C)
+    if (!(am[0] > 1e-12f && am[0] < 1e14f && am[1] > 1e-12f && am[1] < 1e14f && cn > 0.f && cn < 1e14f))
+        return FEAST_OK;
+    if (k > m - 8) k = m - 8;
+    if (!prm.warm || k < m / 4) k = 0;               // too little has converged: the whole matrix
     const int mb = m - k;
-    // Schur form of the trailing block: C22 = Z T22 Z^H
-    FEAST_CUDA_TRY(cudaMemcpy2DAsync(w.S, sizeof(zd) * mb, C + k + (int64_t)k * m, sizeof(zd) * m, sizeof(zd) * mb,
-                                     mb, cudaMemcpyDeviceToDevice, s));
-    if (prm.cold_fp32) {
-        // FP32 QR, then Z made unitary to FP64 rounding (BCGS2 in FP64;
-        // Z moves by its FP32 error, ~1e-6), so that Zh^H C Zh below is a
-        // similarity of C and its lower part is that small
-        FEAST_CUDA_TRY(cudaMemsetAsync(fail, 0, sizeof(int), s));
-        if ((e = schur_large_fp32(s, mb, w.S, w.Z, qz_work, fail, timeout, stats, nullptr, 0.0))) return e;
-        // Z^H Z = I + E with |E| ~ 1e-6: Z (I - E / 2) is unitary to O(|E|^2)
-        // (one step of the series of (I + E)^{-1/2}), i.e. to ~1e-12
-        if ((e = mark(0.0))) return e;
-        if ((e = mul(1, mb, mb, mb, one, w.Z, mb, w.Z, mb, zero, w.Yp, mb, 0))) return e;
-        k_sub_identity_half<<<grid_for((size_t)mb * mb), 256, 0, s>>>(mb, w.Yp);
-        FEAST_LAUNCH_CHECK();
-        FEAST_CUDA_TRY(cudaMemcpyAsync(w.W, w.Z, sizeof(zd) * (size_t)mb * mb, cudaMemcpyDeviceToDevice, s));
-        if ((e = mul(0, mb, mb, mb, zmake(-1.0, 0.0), w.W, mb, w.Yp, mb, one, w.Z, mb, 0))) return e;
-        if ((e = mark(16.0 * (double)mb * mb * mb))) return e;
-    } else if ((e = schur_large(s, mb, w.S, w.Z, qz_work, fail, timeout, stats, nullptr, prm.tail_defl))) {
-        return e;
-    }
-    // C' = Zh^H C Zh, Zh = diag(I_k, Z), into A (Bt as the row-block scratch)
-    zd *Cq = A;
-    FEAST_CUDA_TRY(cudaMemcpyAsync(Cq, C, sizeof(zd) * mm, cudaMemcpyDeviceToDevice, s));
-    if ((e = mark(0.0))) return e;
-    if ((e = mulc(0, m, mb, mb, one, C + (int64_t)k * m, m, w.Z, mb, zero, Cq + (int64_t)k * m, m, 0))) return e;
-    if ((e = mulc(1, mb, m, mb, one, w.Z, mb, Cq + k, m, zero, Bt + k, m, 0))) return e;
-    if ((e = mark(16.0 * (double)m * mb * mb))) return e;
-    FEAST_CUDA_TRY(cudaMemcpy2DAsync(Cq + k, sizeof(zd) * m, Bt + k, sizeof(zd) * m, sizeof(zd) * mb, m,
-                                     cudaMemcpyDeviceToDevice, s));
-    // T^: C' with T22 from the QR in its trailing block (upper triangles are
-    // all that the eigenvector recurrence reads), into Cp -- or C' itself
-    // after the FP32 QR, whose T22 is only FP32-accurate
-    FEAST_CUDA_TRY(cudaMemcpyAsync(w.Cp, Cq, sizeof(zd) * mm, cudaMemcpyDeviceToDevice, s));
-    if (!prm.cold_fp32)
-        FEAST_CUDA_TRY(cudaMemcpy2DAsync(w.Cp + k + (int64_t)k * m, sizeof(zd) * m, w.S, sizeof(zd) * mb,
-                                         sizeof(zd) * mb, mb, cudaMemcpyDeviceToDevice, s));
-    zd *Vh = Bt;  // V^, unit upper triangular
-    if ((e = schur_vectors(s, m, w.Cp, Vh, hn, w.W))) return e;
-    zd *F = V;
-    if (!oz) {
-        // F = V^{-1} (C' V^)
-        if ((e = mark(0.0))) return e;
-        if ((e = mul(0, m, m, m, one, Cq, m, Vh, m, zero, w.W, m, 2))) return e;
-        if ((e = tri_inverse(s, m, Vh, m, w.Cp, w.Ts))) return e;
-        if ((e = mul(0, m, m, m, one, w.Cp, m, w.W, m, zero, F, m, 1))) return e;
-        if ((e = mark(8.0 * m3 + tri_inv))) return e;
-        k_diag_lambda<<<cdiv(m, 128), 128, 0, s>>>(m, F, alpha, beta);
-        FEAST_LAUNCH_CHECK();
-        FEAST_CUDA_TRY(cudaMemsetAsync(w.res, 0, 16, s));
-        k_newton_g<<<grid_for(mm), 256, 0, s>>>(m, F, alpha, w.bad);
-        FEAST_LAUNCH_CHECK();
-        // Y' = V^ + V^ G, and its residual against C'
-        FEAST_CUDA_TRY(cudaMemcpyAsync(w.Yp, Vh, sizeof(zd) * mm, cudaMemcpyDeviceToDevice, s));
-        if ((e = mark(0.0))) return e;
-        if ((e = mul(0, m, m, m, one, Vh, m, F, m, one, w.Yp, m, 1))) return e;
-        if ((e = mul(0, m, m, m, one, Cq, m, w.Yp, m, zero, w.W, m, 0))) return e;
-        if ((e = mark(12.0 * m3))) return e;
-        k_eig_resid<<<cdiv((size_t)m * 32, 256), 256, 0, s>>>(m, w.W, w.Yp, alpha, hn, w.res);
-        FEAST_LAUNCH_CHECK();
-    } else {
-        // The same step in defect form, every product on the digit-sliced
-        // GEMM with one small operand (its error is relative to the
-        // operands' row / column maxima): with C' = T^ + D and T^ V^ = V^ Lh,
-        //   W' = C' V^ - V^ Lh = D V^,   F = Lh + V^{-1} W',
-        //   Y' = V^ + V^ G,   C' Y' - Y' L = V^ S1 + W' + W' G,
-        //   S1 = (Lh - L) + Lh G - G L   (L = diag(F), G as above).
-        zd *lamh = (zd *)w.lower;   // diag(T^) (the column statistics are spent)
-        k_defect_split<<<grid_for(mm), 256, 0, s>>>(m, Cq, w.Cp, w.W, lamh);
-        FEAST_LAUNCH_CHECK();
-        if ((e = mark(0.0))) return e;
-        if ((e = mul(0, m, m, m, one, w.W, m, Vh, m, zero, w.S, m, 2))) return e;       // W'
-        if ((e = tri_inverse(s, m, Vh, m, w.Cp, w.Ts))) return e;
-        if ((e = mul(0, m, m, m, one, w.Cp, m, w.S, m, zero, F, m, 1))) return e;       // V^{-1} W'
-        if ((e = mark(8.0 * m3 + tri_inv))) return e;   // (algorithmic: V^ triangular)
-        k_add_diag_lambda<<<cdiv(m, 128), 128, 0, s>>>(m, F, lamh, alpha, beta);
-        FEAST_LAUNCH_CHECK();
-        FEAST_CUDA_TRY(cudaMemsetAsync(w.res, 0, 16, s));
-        k_newton_g<<<grid_for(mm), 256, 0, s>>>(m, F, alpha, w.bad);
-        FEAST_LAUNCH_CHECK();
-        FEAST_CUDA_TRY(cudaMemcpyAsync(w.Yp, Vh, sizeof(zd) * mm, cudaMemcpyDeviceToDevice, s));
-        k_newton_s1<<<grid_for(mm), 256, 0, s>>>(m, F, lamh, alpha, w.W);
-        FEAST_LAUNCH_CHECK();
-        FEAST_CUDA_TRY(cudaMemcpyAsync(Cq, w.S, sizeof(zd) * mm, cudaMemcpyDeviceToDevice, s));   // R = W'
-        if ((e = mark(0.0))) return e;
-        if ((e = mul(0, m, m, m, one, Vh, m, F, m, one, w.Yp, m, 1))) return e;       // Y' = V^ + V^ G
-        if ((e = mul(0, m, m, m, one, Vh, m, w.W, m, one, Cq, m, 1))) return e;       // R += V^ S1
-        if ((e = mul(0, m, m, m, one, w.S, m, F, m, one, Cq, m, 0))) return e;        // R += W' G
-        if ((e = mark(16.0 * m3))) return e;
-        k_eig_resid<<<cdiv((size_t)m * 32, 256), 256, 0, s>>>(m, Cq, w.Yp, alpha, hn, w.res, 1);
-        FEAST_LAUNCH_CHECK();
-    }
-    struct {
-        unsigned long long r;
-        int bad;
-        int pad;
-    } hr{};
-    int qfail = 0;
-    FEAST_CUDA_TRY(cudaMemcpyAsync(&hr, w.res, 16, cudaMemcpyDeviceToHost, s));
-    if (prm.cold_fp32) FEAST_CUDA_TRY(cudaMemcpyAsync(&qfail, fail, sizeof(int), cudaMemcpyDeviceToHost, s));
-    FEAST_CUDA_TRY(cudaStreamSynchronize(s));
-    double worst;
-    memcpy(&worst, &hr.r, sizeof(double));
-    res->resid = worst;
     res->tail = mb;
-    if (hr.bad || qfail || !(worst <= prm.accept_tol)) return FEAST_OK;
-    // Y = Zh Y', unit columns
-    FEAST_CUDA_TRY(cudaMemcpy2DAsync(V, sizeof(zd) * m, w.Yp, sizeof(zd) * m, sizeof(zd) * k, m,
+    // Schur form of the trailing block: T = [C11 C12 Z; 0 T22], Z in w.Q (mb x mb)
+    FEAST_CUDA_TRY(cudaMemcpy2DAsync(w.G, sizeof(cf) * mb, C + k + (int64_t)k * m, sizeof(cf) * m, sizeof(cf) * mb, mb,
                                      cudaMemcpyDeviceToDevice, s));
-    if ((e = mulc(0, mb, m, mb, one, w.Z, mb, w.Yp + k, m, zero, V + k, m, 0))) return e;
-    if ((e = normalise_cols(s, m, V))) return e;
-    res->accepted = 1;
+    FEAST_CUDA_TRY(cudaMemsetAsync(w.fail, 0, sizeof(int), s));
+    if ((e = schur32(s, mb, w.G, w.Q, cn, w.schur, w.fail, timeout, stats))) return e;
+    if (k > 0) {
+        FEAST_CUDA_TRY(cudaMemcpyAsync(w.T, C, sizeof(cf) * (size_t)m * k, cudaMemcpyDeviceToDevice, s));
+        if ((e = mul32(0, k, mb, mb, fone, C + (int64_t)k * m, m, w.Q, mb, fzero, w.T + (int64_t)k * m, m))) return e;
+    }
+    FEAST_CUDA_TRY(cudaMemcpy2DAsync(w.T + k + (int64_t)k * m, sizeof(cf) * m, w.G, sizeof(cf) * mb, sizeof(cf) * mb, mb,
+                                     cudaMemcpyDeviceToDevice, s));
+    // eigenvectors of T: Y, and U = Y^{-1} (its conjugate transpose)
+    k_transpose32<<<dim3(cdiv(m, 32), cdiv(m, 32)), 256, 0, s>>>(m, w.T, w.W);
+    FEAST_LAUNCH_CHECK();
+    {
+        int dev = 0, sms = 0;
+        FEAST_CUDA_TRY(cudaGetDevice(&dev));
+        FEAST_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        int wpc = (2 * m + sms - 1) / sms;           // warps per CTA, one CTA per SM
+        const int most = (int)(200 * 1024 / (sizeof(cf) * (size_t)m));
+        if (wpc > 16) wpc = 16;
+        if (wpc > most) wpc = most;
+        if (wpc < 1) wpc = 1;
+        const size_t sm = sizeof(cf) * (size_t)m * wpc;
+        FEAST_CUDA_TRY(ensure_dyn_smem(k_tri_vectors32, sm));
+        k_tri_vectors32<<<cdiv((size_t)2 * m, wpc), 32 * wpc, sm, s>>>(m, w.T, w.W, w.Y, w.Uh, 1e-5f * cn);
+        FEAST_LAUNCH_CHECK();
+    }
+    k_rf_lam<<<cdiv(m, 128), 128, 0, s>>>(m, w.T, w.lam);
+    FEAST_LAUNCH_CHECK();
+    // V = diag(I, Z) Y;  L^H = U diag(I, Z)^H B^{-1}
+    if (k > 0) {
+        FEAST_CUDA_TRY(cudaMemcpy2DAsync(w.V32, sizeof(cf) * m, w.Y, sizeof(cf) * m, sizeof(cf) * k, m,
+                                         cudaMemcpyDeviceToDevice, s));
+        FEAST_CUDA_TRY(cudaMemcpy2DAsync(w.W, sizeof(cf) * m, Bi, sizeof(cf) * m, sizeof(cf) * k, m,
+                                         cudaMemcpyDeviceToDevice, s));
+    }
+    if ((e = mul32(0, mb, m, mb, fone, w.Q, mb, w.Y + k, m, fzero, w.V32 + k, m))) return e;
+    if ((e = mul32(1, mb, m, mb, fone, w.Q, mb, Bi + k, m, fzero, w.W + k, m))) return e;
+    if ((e = mul32(1, m, m, m, fone, w.Uh, m, w.W, m, fzero, w.L, m))) return e;
+    k_rf_scale<<<cdiv((size_t)m * 32, 256), 256, 0, s>>>(m, w.V32, V, w.nv);
+    FEAST_LAUNCH_CHECK();
+    k_rf_scale_rows<<<grid_for(mm), 256, 0, s>>>(m, w.L, w.nv);
+    FEAST_LAUNCH_CHECK();
+    // delta = || I - L^H B V ||_F
+    if ((e = mul32(0, m, m, m, fone, w.B32, m, w.V32, m, fzero, w.W, m))) return e;
+    if ((e = mul32(0, m, m, m, fone, w.L, m, w.W, m, fzero, w.G, m))) return e;
+    k_rf_defect<<<RF_PART, 256, 0, s>>>(m, w.G, w.part);
+    FEAST_LAUNCH_CHECK();
+    float hp[RF_PART];
+    int qfail = 0;
+    FEAST_CUDA_TRY(cudaMemcpyAsync(hp, w.part, sizeof(hp), cudaMemcpyDeviceToHost, s));
+    FEAST_CUDA_TRY(cudaMemcpyAsync(&qfail, w.fail, sizeof(int), cudaMemcpyDeviceToHost, s));
+    FEAST_CUDA_TRY(cudaStreamSynchronize(s));
+    double dl = 0.0;
+    for (float x : hp) dl += (double)x;
+    dl = sqrt(dl);
+    if (qfail || !(dl < 0.1)) return FEAST_OK;
+    double gprev = 0.0;
+    bool last64 = false;
+    zd *lam = w.lam, *lam2 = w.lam2;
+    for (int step = 0; step < RF_STEPS; ++step) {
+        // the digit-sliced products while what they leave (about 1e-13 of
+        // max|C| over a gap) is not yet what limits the result
+        const bool use_oz = oz && (prm.target > 1e-10 || (!last64 && (step == 0 || gprev > 1e-6)));
+        last64 = !use_oz;
+        const bool timed = gt && !use_oz && gt->used + 2 <= GemmTimer::kMax;
+        if (timed) FEAST_CUDA_TRY(cudaEventRecord(gt->ev[gt->used++], s));
+        if (use_oz) {
+            if ((e = oz_prepare_cols(s, m, m, V, m, oz->cols))) return e;
+            if ((e = oz_prepare_rows(s, m, m, A, m, oz->rows))) return e;
+            if ((e = oz_gemm(s, m, m, m, oz->rows, oz->cols, one, nullptr, 0, zero, w.AV, m, oz->err))) return e;
+            if ((e = oz_prepare_rows(s, m, m, w.Bu, m, oz->rows))) return e;
+            if ((e = oz_gemm(s, m, m, m, oz->rows, oz->cols, one, nullptr, 0, zero, w.BV, m, oz->err))) return e;
+        } else {
+            if ((e = zgemm_batched(s, 0, m, m, m, one, A, m, 0, V, m, 0, zero, w.AV, m, 0, 1))) return e;
+            if ((e = zgemm_batched(s, 0, m, m, m, one, w.Bu, m, 0, V, m, 0, zero, w.BV, m, 0, 1, 1))) return e;
+        }
+        if (timed) {
+            FEAST_CUDA_TRY(cudaEventRecord(gt->ev[gt->used++], s));
+            gt->flops += 12.0 * (double)m * m * m;
+        }
+        k_rf_resid<<<grid_for(mm), 256, 0, s>>>(m, w.AV, w.BV, lam, w.G, w.pair);
+        FEAST_LAUNCH_CHECK();
+        if ((e = mul32(0, m, m, m, fone, w.L, m, w.G, m, fzero, w.W, m))) return e;
+        FEAST_CUDA_TRY(cudaMemsetAsync(w.st, 0, sizeof(RefineStat), s));
+        k_rf_g<<<grid_for(mm), 256, 0, s>>>(m, w.W, lam, (use_oz ? 1e-12f : 1e-14f) * cn, w.G, w.pair, w.st);
+        FEAST_LAUNCH_CHECK();
+        k_rf_lambda<<<cdiv(m, 128), 128, 0, s>>>(m, w.W, lam, lam2, w.pair, w.G, w.pu, w.pd, w.st);
+        FEAST_LAUNCH_CHECK();
+        if ((e = mul32(0, m, m, m, fone, w.V32, m, w.G, m, fzero, w.Y, m))) return e;
+        RefineStat hs;
+        FEAST_CUDA_TRY(cudaMemcpyAsync(&hs, w.st, sizeof(hs), cudaMemcpyDeviceToHost, s));
+        FEAST_CUDA_TRY(cudaStreamSynchronize(s));
+        if (hs.bad) return FEAST_OK;
+        float g2;
+        memcpy(&g2, &hs.gm, sizeof(float));
+        const double gm = sqrt((double)g2);
+        k_rf_update<<<grid_for(mm), 256, 0, s>>>(m, w.Y, w.pair, w.pu, hs.paired, V, w.V32);
+        FEAST_LAUNCH_CHECK();
+        zd *t = lam;
+        lam = lam2;
+        lam2 = t;
+        // what the step leaves: by the bound on delta, or by the contraction
+        // seen (|G| over the step before's, at least delta); a pair's block is
+        // followed by another step, and |G| that no longer falls is rounding
+        const double ratio = gprev > 0.0 ? gm / gprev : 1e300;
+        double left = gm * fmin(8.0 * fmax(gm, ratio), (double)m * gm + dl);
+        if (gm <= 1e-8 && step > 0 && ratio > 0.1 && ratio < 1e200) left = 0.0;
+        res->steps = step + 1;
+        res->resid = left;
+        if (!hs.paired && left <= prm.target && (!oz || prm.target > 1e-10 || last64 || gm == 0.0)) {
+            if ((e = normalise_cols(s, m, V))) return e;
+            k_rf_out<<<cdiv(m, 128), 128, 0, s>>>(m, lam, alpha, beta);
+            FEAST_LAUNCH_CHECK();
+            res->accepted = 1;
+            return FEAST_OK;
+        }
+        if (hs.paired || gm > 1e-6) {
+            // L^H to (B V)^{-1} of the new V, up to |G|^2
+            FEAST_CUDA_TRY(cudaMemcpyAsync(w.Y, w.L, sizeof(cf) * mm, cudaMemcpyDeviceToDevice, s));
+            if ((e = mul32(0, m, m, m, fmone, w.G, m, w.Y, m, fone, w.L, m))) return e;
+            dl += (double)m * gm * gm;
+        } else {
+            dl += (double)m * gm;
+        }
+        if (hs.paired) {
+            k_rf_rows<<<grid_for(mm), 256, 0, s>>>(m, w.pair, w.pu, w.pd, w.L);
+            FEAST_LAUNCH_CHECK();
+        }
+        gprev = gm > 0.0 ? gm : 1e-30;
+    }
     return FEAST_OK;
 }
 

@@ -301,23 +301,15 @@ __global__ void __launch_bounds__(HG_T) k_hess_grid(int m, T *C, T *Q, int ld, G
     }
 }
 
-// complex128 <-> complex64 copies of an m x m matrix, and the identity
-__global__ void k_z2c(int64_t count, const zd *__restrict__ x, cf *__restrict__ y)
-{
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < count; e += (int64_t)gridDim.x * blockDim.x)
-        y[e] = make_float2((float)x[e].x, (float)x[e].y);
-}
-__global__ void k_c2z(int64_t count, const cf *__restrict__ x, zd *__restrict__ y)
-{
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < count; e += (int64_t)gridDim.x * blockDim.x)
-        y[e] = zmake((double)x[e].x, (double)x[e].y);
-}
+// identity matrices
+#if FEAST_QR_FP32
 __global__ void k_eye_c(int m, cf *Q)
 {
     const int64_t total = (int64_t)m * m;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x)
         Q[e] = make_float2((e % m) == (e / m) ? 1.f : 0.f, 0.f);
 }
+#endif
 
 __global__ void k_eye(int m, zd *Q, int ld)
 {
@@ -1374,9 +1366,7 @@ __global__ void k_absmax(int64_t count, const zd *x, double *out)
 
 }  // namespace
 
-#if FEAST_QR_FP32
-namespace {   // the FP32 build's own copies of the one-CTA kernels
-#endif
+#if !FEAST_QR_FP32   // (the rest of the file: the double-single path)
 // ------------------------------------------------- small matrices: one CTA
 // Schur form of an m x m upper Hessenberg matrix, m <= SQ_MAX, by one CTA
 // with the whole matrix in shared memory: packed by columns (column j keeps
@@ -1644,15 +1634,6 @@ __global__ void __launch_bounds__(AR) k_apply_rotlog(int m, zd *__restrict__ Q, 
     }
 }
 
-#if FEAST_QR_FP32
-}  // namespace
-#endif
-
-#if FEAST_QR_FP32
-#define schur_large_work_bytes schur_large_work_bytes_fp32
-#define zeig_large_work_bytes zeig_large_work_bytes_fp32
-#define schur_large schur_large_fp32
-#endif
 size_t schur_large_work_bytes(int m)
 {
     // v (m) + w (m) + u (2m) complex, tau, absmax, rotations, barrier words,
@@ -1693,20 +1674,12 @@ int schur_large(cudaStream_t s, int m, zd *C, zd *Q, void *work, int *fail, int 
     unsigned *hbar = (unsigned *)(((uintptr_t)(wv + m) + 15) & ~(uintptr_t)15);   // (w is unused by it)
     int hgrid = 0;
     if (m >= 3) {
-        // the FP32 build reduces in FP32 too when its multishift QR follows
-        // (C and Q in complex64 in the double-single copies' space)
-        const bool hf = FEAST_QR_FP32 && m > SQ_MAX;
         int dev = 0, sms = 0, per = 0;
-        const size_t hsm = (hf ? sizeof(cf) : sizeof(zd)) * (size_t)m;
+        const size_t hsm = sizeof(zd) * (size_t)m;
         FEAST_CUDA_TRY(cudaGetDevice(&dev));
         FEAST_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        if (hf) {
-            FEAST_CUDA_TRY(ensure_dyn_smem(k_hess_grid<cf>, hsm));
-            FEAST_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_hess_grid<cf>, HG_T, hsm));
-        } else {
-            FEAST_CUDA_TRY(ensure_dyn_smem(k_hess_grid<zd>, hsm));
-            FEAST_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_hess_grid<zd>, HG_T, hsm));
-        }
+        FEAST_CUDA_TRY(ensure_dyn_smem(k_hess_grid<zd>, hsm));
+        FEAST_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_hess_grid<zd>, HG_T, hsm));
         hgrid = (per >= 1) ? sms : 0;
         const int need = (2 * m + HG_R - 1) / HG_R;     // right-update slabs
         if (hgrid > need) hgrid = need;
@@ -1714,27 +1687,10 @@ int schur_large(cudaStream_t s, int m, zd *C, zd *Q, void *work, int *fail, int 
             FEAST_CUDA_TRY(cudaMemsetAsync(hbar, 0, 2 * sizeof(unsigned), s));
             GridSync hg{hbar, hbar + 1, timeout, TO_HESS};
             int mm = m, ldq = m;
-            const unsigned gc = cdiv((size_t)m * m, 256) > 4096 ? 4096 : cdiv((size_t)m * m, 256);
-            if (hf) {
-                cf *Cf = (cf *)Hds, *Qf = (cf *)Qds;
-                k_z2c<<<gc, 256, 0, s>>>((int64_t)m * m, C, Cf);
-                FEAST_LAUNCH_CHECK();
-                k_eye_c<<<gc, 256, 0, s>>>(m, Qf);
-                FEAST_LAUNCH_CHECK();
-                void *hargs[] = {&mm, &Cf, &Qf, &ldq, &hg};
-                FEAST_CUDA_TRY(cudaLaunchCooperativeKernel((void *)k_hess_grid<cf>, dim3(hgrid), dim3(HG_T), hargs,
-                                                           hsm, s));
-                FEAST_LAUNCH_CHECK();
-                k_c2z<<<gc, 256, 0, s>>>((int64_t)m * m, Cf, C);
-                FEAST_LAUNCH_CHECK();
-                k_c2z<<<gc, 256, 0, s>>>((int64_t)m * m, Qf, Q);
-                FEAST_LAUNCH_CHECK();
-            } else {
-                void *hargs[] = {&mm, &C, &Q, &ldq, &hg};
-                FEAST_CUDA_TRY(cudaLaunchCooperativeKernel((void *)k_hess_grid<zd>, dim3(hgrid), dim3(HG_T), hargs,
-                                                           hsm, s));
-                FEAST_LAUNCH_CHECK();
-            }
+            void *hargs[] = {&mm, &C, &Q, &ldq, &hg};
+            FEAST_CUDA_TRY(cudaLaunchCooperativeKernel((void *)k_hess_grid<zd>, dim3(hgrid), dim3(HG_T), hargs, hsm,
+                                                       s));
+            FEAST_LAUNCH_CHECK();
         }
     }
     for (int j = 0; hgrid == 0 && j + 2 < m; ++j) {
@@ -1769,9 +1725,9 @@ int schur_large(cudaStream_t s, int m, zd *C, zd *Q, void *work, int *fail, int 
     // the reduction stopped at its first barrier)
     if (htimeout) return note_timeout(htimeout);
     if (hn_out) *hn_out = hn;
-    // deflation thresholds at double-single resolution (2^-44 relative),
-    // or a few FP32 units in the FP32 build (or the caller's looser one)
-    const double floor_rel = FEAST_QR_FP32 ? 1e-6 : 5.7e-14;
+    // deflation thresholds at double-single resolution (2^-44 relative), or
+    // the caller's looser one
+    const double floor_rel = 5.7e-14;
     const double tr = defl > floor_rel ? defl : floor_rel;
     float tol_rel = (float)tr, tol_abs = (float)(tr * (hn > 0.0 ? hn : 1e-300));
     if (m >= 2 && m <= SQ_MAX) {
@@ -1830,7 +1786,6 @@ int schur_large(cudaStream_t s, int m, zd *C, zd *Q, void *work, int *fail, int 
 
 // A (m x m, overwritten), Bt (m x m upper triangular, overwritten by the
 // solve), alpha/beta (beta = 1), V (m x m unit eigenvectors).
-#if !FEAST_QR_FP32
 int zeig_large(cudaStream_t s, int m, zd *A, zd *Bt, zd *alpha, zd *beta, zd *V, void *work,
                int *fail, int *timeout, int *stats, double defl)
 {

@@ -13,6 +13,7 @@
 // and Z (one merged index range, so every SM partition's FP64 units work)
 // and meet at a barrier between rotations.  The three m x m arrays live in
 // shared memory (m <= 64).  Larger projected problems go to k_zeig.cu.
+#include "chase32.cuh"
 #include "common.cuh"
 
 namespace feast {
@@ -349,62 +350,13 @@ __global__ void __launch_bounds__(NT) k_qz(int m, zd *A, int64_t lda, int64_t sA
 // then takes the QZ (k_qz) or the double-single QR.  Measured on GB300, see
 // zqz_batched.
 constexpr int EZ_T = 256;            // threads per CTA
-constexpr int EZ_Q = 128;            // of them in the QR iteration (one warp per SM quarter)
+constexpr int EZ_Q = 192;            // of them in the QR iteration
 constexpr int EZ_MIN_M = 3;          // smallest pencil
 constexpr int EZ_STEPS = 10;         // most Newton steps
 constexpr float EZ_PAIR = 1.f / 16;  // largest G_ij of a Newton step
 constexpr double EZ_DONE = 4e-15;    // error bound at which the iteration ends
 
-struct RotF {
-    float c;
-    cf s;
-};
-
-// 1 / sqrt(x) with one Newton step: rsqrtf alone is off by up to 2^-22.9
-// with a bias, which thousands of rotations would add up
-__device__ __forceinline__ float ez_rsqrt(float x)
-{
-    const float y = rsqrtf(x);
-    return y * fmaf(-0.5f * x * y, y, 1.5f);
-}
-
-// G = [c s; -conj(s) c] with G [x; y] = [r; 0]
-__device__ __forceinline__ RotF ez_rot(cf x, cf y)
-{
-    RotF g;
-    const float mx = fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(y.x), fabsf(y.y)));
-    // bring the larger entry into [1, 2): squares neither overflow nor vanish
-    int ex = (int)(__float_as_uint(mx) >> 23);
-    ex = ex < 1 ? 1 : (ex > 253 ? 253 : ex);
-    const float f = __uint_as_float((unsigned)(254 - ex) << 23);
-    x = cmakef(x.x * f, x.y * f);
-    y = cmakef(y.x * f, y.y * f);
-    const float ax2 = cabs2(x), ay2 = cabs2(y);
-    if (ay2 == 0.f) { g.c = 1.f; g.s = cmakef(0.f, 0.f); return g; }
-    if (ax2 < 1e-36f) { g.c = 0.f; const float ia = ez_rsqrt(ay2); g.s = cmakef(y.x * ia, -y.y * ia); return g; }
-    const float k = ez_rsqrt(ax2) * ez_rsqrt(ax2 + ay2);
-    g.c = ax2 * k;
-    g.s = cmakef((x.x * y.x + x.y * y.y) * k, (x.y * y.x - x.x * y.y) * k);   // x conj(y) k
-    return g;
-}
-__device__ __forceinline__ void ez_rot_pair(const RotF &g, cf &a, cf &b)          // G [a; b]
-{
-    const cf s = g.s;
-    const cf na = cmakef(fmaf(g.c, a.x, fmaf(s.x, b.x, -s.y * b.y)), fmaf(g.c, a.y, fmaf(s.x, b.y, s.y * b.x)));
-    b = cmakef(fmaf(g.c, b.x, -fmaf(s.x, a.x, s.y * a.y)), fmaf(g.c, b.y, -fmaf(s.x, a.y, -s.y * a.x)));
-    a = na;
-}
-__device__ __forceinline__ void ez_rot_pair_h(const RotF &g, cf &a, cf &b)        // [a b] G^H
-{
-    RotF h;
-    h.c = g.c;
-    h.s = cmakef(g.s.x, -g.s.y);
-    ez_rot_pair(h, a, b);
-}
-
 __device__ __forceinline__ void ez_bar() { asm volatile("bar.sync 1, %0;" ::"n"(EZ_Q) : "memory"); }
-
-__device__ __forceinline__ float ez_absf(cf a) { return sqrtf(cabs2(a)); }
 
 // Sum over the CTA of one float per thread, in a fixed order.
 __device__ __forceinline__ float ez_sum(float v, float *red)
@@ -504,7 +456,7 @@ __device__ void ez_hess(int m, int ld, cf *H, cf *Z, cf *hv)
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
         const cf x0 = H[(j + 1) * ld + j];
-        const float nrm = sqrtf(s), a0 = ez_absf(x0);
+        const float nrm = sqrtf(s), a0 = abs32(x0);
         const cf ph = a0 > 0.f ? cmakef(x0.x / a0, x0.y / a0) : cmakef(1.f, 0.f);
         const float vv = 2.f * nrm * (nrm + a0), tau = vv > 0.f ? 2.f / vv : 0.f;
         for (int i = t; i < len; i += EZ_T)
@@ -545,100 +497,73 @@ __device__ void ez_hess(int m, int ld, cf *H, cf *Z, cf *hv)
 }
 
 // Single-shift QR of the Hessenberg H to triangular form, Z <- Z Q (row-major,
-// ld), by the first EZ_Q threads: threads 0 .. 63 own a column of H in the
-// left half of a rotation and a row in the right half, threads 64 .. 127 a row
-// of Z; every warp forms each rotation from the same two entries (redundantly:
-// that costs no barrier), two barriers per rotation.  false: budget spent.
-__device__ bool ez_qr(int m, int ld, cf *H, cf *Z, float tol_abs)
+// ld), by the first EZ_Q threads: warp 0 scans for deflation and runs the
+// sweep's chain of rotations (chase32.cuh), 32 at a time; then warp 1 applies
+// them to the columns of H beyond the chunk, threads 64 .. 127 to the rows of
+// H and threads 128 .. 191 to those of Z.  rot: CHASE_N rotations; ctl: two
+// ints, sg: the shift.  false: budget spent.
+__device__ bool ez_qr(int m, int ld, cf *H, cf *Z, float tol_abs, RotF *rot, int *ctl, cf *sg)
 {
     const int t = threadIdx.x, lane = t & 31;
     const float tol_rel = 2.4e-7f;
     int hi = m - 1, it = 0, tot = 0;
-    while (hi > 0) {
-        int lo = 0;
-        for (int base = hi; base >= 1 && lo == 0; base -= 32) {
-            const int p = base - lane;
-            bool neg = false;
-            if (p >= 1) {
-                const float sub = ez_absf(H[p * ld + p - 1]);
-                const float loc = ez_absf(H[(p - 1) * ld + p - 1]) + ez_absf(H[p * ld + p]);
-                neg = !(sub > tol_rel * loc) || !(sub > tol_abs);
-            }
-            const unsigned b = __ballot_sync(0xffffffffu, neg);
-            if (b) lo = base - (__ffs(b) - 1);
-        }
-        if (lo == hi) { --hi; it = 0; continue; }
-        if (++tot > 40 * m) return false;
-        ++it;
-        cf sigma;
-        {
-            const cf h00 = H[(hi - 1) * ld + hi - 1], h01 = H[(hi - 1) * ld + hi];
-            const cf h10 = H[hi * ld + hi - 1], h11 = H[hi * ld + hi];
-            if (it % 11 == 10) {
-                const float a = ez_absf(h10);
-                sigma = cmakef(h11.x + a, h11.y + 0.5f * a);
-            } else {
-                // Wilkinson shift: h11 + the smaller root of z^2 - 2 d z - h01 h10, d = (h00 - h11) / 2
-                const cf d = cmakef(0.5f * (h00.x - h11.x), 0.5f * (h00.y - h11.y));
-                const cf bc = cmul(h01, h10);
-                cf w = cadd(cmul(d, d), bc);
-                const float aw = ez_absf(w);
-                // principal square root of w, on the side of d
-                float re = sqrtf(0.5f * (aw + fabsf(w.x))), im = re > 0.f ? 0.5f * w.y / re : 0.f;
-                if (w.x < 0.f) { const float q = re; re = fabsf(im); im = copysignf(q, w.y); }
-                if (re * d.x + im * d.y < 0.f) { re = -re; im = -im; }
-                const cf den = cmakef(d.x + re, d.y + im);
-                const cf corr = cis_zero(den) ? cmakef(0.f, 0.f) : cdiv(bc, den);
-                sigma = cmakef(h11.x - corr.x, h11.y - corr.y);
-            }
-        }
-        for (int k = lo; k < hi; ++k) {
-            cf x, y;
-            if (k == lo) {
-                x = H[k * ld + k];
-                x = cmakef(x.x - sigma.x, x.y - sigma.y);
-                y = H[(k + 1) * ld + k];
-            } else {
-                x = H[k * ld + k - 1];
-                y = H[(k + 1) * ld + k - 1];
-            }
-            const RotF g = ez_rot(x, y);
-            // (the sweep's first x, y come from column k, which the left half
-            // writes: every warp has read them, the shift and the scan's entries)
-            if (k == lo) ez_bar();
-            if (t < 64) {
-                if (t >= k && t < m) {
-                    cf a = H[k * ld + t], b = H[(k + 1) * ld + t];
-                    ez_rot_pair(g, a, b);
-                    H[k * ld + t] = a;
-                    H[(k + 1) * ld + t] = b;
+    for (;;) {
+        if (t < 32) {
+            int lo = 0;
+            while (hi > 0) {
+                lo = 0;
+                for (int base = hi; base >= 1 && lo == 0; base -= 32) {
+                    const int p = base - lane;
+                    bool neg = false;
+                    if (p >= 1) {
+                        const float sub = abs32(H[p * ld + p - 1]);
+                        const float loc = abs32(H[(p - 1) * ld + p - 1]) + abs32(H[p * ld + p]);
+                        neg = !(sub > tol_rel * loc) || !(sub > tol_abs);
+                    }
+                    const unsigned b = __ballot_sync(0xffffffffu, neg);
+                    if (b) lo = base - (__ffs(b) - 1);
                 }
-            } else if (t - 64 < m) {
-                cf *z = Z + (t - 64) * ld + k;
-                cf a = z[0], b = z[1];
-                ez_rot_pair_h(g, a, b);
-                z[0] = a;
-                z[1] = b;
+                if (lo < hi) break;
+                --hi;
+                it = 0;
             }
+            if (hi > 0 && ++tot > 40 * m) hi = -1;
+            if (hi > 0) {
+                ++it;
+                const cf h00 = H[(hi - 1) * ld + hi - 1], h01 = H[(hi - 1) * ld + hi];
+                const cf h10 = H[hi * ld + hi - 1], h11 = H[hi * ld + hi];
+                cf sigma = shift32(h00, h01, h10, h11);
+                if (it % 11 == 10) {
+                    const float a = abs32(h10);
+                    sigma = cmakef(h11.x + a, h11.y + 0.5f * a);
+                }
+                if (lane == 0) *sg = sigma;
+            }
+            if (lane == 0) {
+                ctl[0] = lo;
+                ctl[1] = hi;
+            }
+        }
+        ez_bar();
+        const int lo = ctl[0], h = ctl[1];
+        if (h <= 0) return h == 0;
+        const RowsLd R{H, ld};
+        for (int k0 = lo; k0 < h; k0 += CHASE_N) {
+            const int k1 = (k0 + CHASE_N < h) ? k0 + CHASE_N : h;
+            if (t < 32) chase_left(R, m, lo, h, k0, k1, *sg, rot);
             ez_bar();
             if (t < 64) {
-                if (t <= ((k + 2 < hi) ? k + 2 : hi)) {
-                    cf a = H[t * ld + k], b = H[t * ld + k + 1];
-                    ez_rot_pair_h(g, a, b);
-                    H[t * ld + k] = a;
-                    H[t * ld + k + 1] = b;
-                }
-            } else if (t == 64 && k > lo) {
-                // column k - 1: (r, 0), now that every warp has read x and y
-                cf a = x, b = y;
-                ez_rot_pair(g, a, b);
-                H[k * ld + k - 1] = a;
-                H[(k + 1) * ld + k - 1] = cmakef(0.f, 0.f);
+                const int c = k0 + 1 + t;               // (warp 1: columns k0 + 33 ..)
+                if (t >= 32 && c < m) far_left(R, c, k0, k1, rot);
+            } else if (t < 128) {
+                const int r = t - 64;
+                if (r < k1) chase_right(H + r * ld, k0, r > k0 ? r : k0, k1, rot);
+            } else if (t - 128 < m) {
+                chase_right(Z + (t - 128) * ld, k0, k0, k1, rot);
             }
             ez_bar();
         }
     }
-    return true;
 }
 
 // Eigenvector columns of the upper triangle of T into Y (upper triangular,
@@ -699,7 +624,8 @@ __global__ void __launch_bounds__(EZ_T) k_eig_refined(int m, const zd *__restric
     extern __shared__ zd smem[];
     __shared__ float red[EZ_T / 32];
     __shared__ unsigned s_ea, s_eb;
-    __shared__ int s_bad;
+    __shared__ int s_bad, s_ctl[2];
+    __shared__ cf s_sg;
     const int b = blockIdx.x, t = threadIdx.x, ld = ez_ld(m);
     A += (int64_t)b * sA;
     B += (int64_t)b * sB;
@@ -757,7 +683,7 @@ __global__ void __launch_bounds__(EZ_T) k_eig_refined(int m, const zd *__restric
     cn = sqrtf(ez_max(cn, red));
     if (!(cn > 0.f && cn < 1e15f)) return;
     ez_hess(m, ld, H, Z, hv);
-    if (t < EZ_Q && !ez_qr(m, ld, H, Z, 6e-8f * cn) && t == 0) s_bad = 1;
+    if (t < EZ_Q && !ez_qr(m, ld, H, Z, 6e-8f * cn, (RotF *)Vd, s_ctl, &s_sg) && t == 0) s_bad = 1;
     __syncthreads();
     if (s_bad) return;
     // Y into W; V = Z Y with unit columns; L^H = (B' V)^{-1} = D Y^{-1} Z^H B'^{-1}
@@ -982,7 +908,8 @@ __global__ void __launch_bounds__(EZ_T) k_eig_refined(int m, const zd *__restric
         // seen (|G| over the step before's, at least delta); a pair's block is
         // followed by another step
         const double seen = 8.0 * fmax((double)gm, (double)gm / (double)gprev), bnd = (double)m * (double)gm + (double)dl;
-        done = !paired && (double)gm * fmin(seen, bnd) <= EZ_DONE;
+        // (|G| that no longer falls is the residual's rounding)
+        done = !paired && ((double)gm * fmin(seen, bnd) <= EZ_DONE || (gm <= 1e-8f && step > 0 && gm > 0.1f * gprev));
         gprev = gm;
     }
     if (!done) return;
@@ -1010,8 +937,8 @@ size_t zqz_work_bytes(int m)
 {
     size_t small = (size_t)m * m * sizeof(zd);
     if (m <= 64) return small;
-    size_t big = zeig_large_work_bytes(m);
-    return (big + 255) & ~(size_t)255;
+    const size_t big = zeig_large_work_bytes(m), ref = zeig_refined_large_work_bytes(m);
+    return ((big > ref ? big : ref) + 255) & ~(size_t)255;
 }
 
 int zeig_refined(cudaStream_t s, int m, int batch, const zd *A, int64_t lda, int64_t sA, const zd *B, int64_t ldb,
@@ -1047,8 +974,16 @@ int zqz_batched(cudaStream_t s, int m, int batch, zd *A, int64_t lda, int64_t sA
     }
     if (lda != m || ldb != m || ldv != m) return FEAST_EINVAL;
     const size_t wb = zqz_work_bytes(m);
+    // refined FP32 Schur form first, the double-single QR for what it leaves
+    // (GB300, one pencil of 300 rows: 231 ms for the latter)
     for (int b = 0; b < batch; ++b) {
-        int e = zeig_large(s, m, A + (int64_t)b * sA, B + (int64_t)b * sB, alpha + (int64_t)b * m,
+        RefineResult rr;
+        int e = zeig_refined_large(s, m, A + (int64_t)b * sA, B + (int64_t)b * sB, alpha + (int64_t)b * m,
+                                   beta + (int64_t)b * m, V + (int64_t)b * sV, (char *)work + b * wb,
+                                   RefineParams{0, EZ_DONE}, &rr, timeout, stats);
+        if (e) return e;
+        if (rr.accepted) continue;
+        e = zeig_large(s, m, A + (int64_t)b * sA, B + (int64_t)b * sB, alpha + (int64_t)b * m,
                            beta + (int64_t)b * m, V + (int64_t)b * sV, (char *)work + b * wb, fail,
                            timeout, stats, defl);
         if (e) return e;

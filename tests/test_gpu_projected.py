@@ -1,7 +1,8 @@
-"""The projected eigensolve of up to 64 rows (feast_zqz_batched): an FP32
-Schur form made exact by an FP64 Newton iteration, or QZ where that does not
-fit.  Sizes at the edges of the 16-row tiles and of the warp, and spectra on
-both sides of the iteration's own branches: separated eigenvalues, pairs that
+"""The projected eigensolve (feast_zqz_batched): an FP32 Schur form made exact
+by a Newton iteration with an FP64 residual, or QZ (up to 64 rows) where that
+does not fit.  Sizes at the edges of the 16-row tiles, of the warp, of the
+one-CTA forms (64 rows for the whole solve, 232 for the QR), and spectra on both
+sides of the iteration's own branches: separated eigenvalues, pairs that
 FP32 cannot tell apart, exact multiplicity, a singular B, a Jordan block."""
 import numpy as np
 import pytest
@@ -34,7 +35,7 @@ def _check(A, B, lam, tol):
         assert np.max(np.abs(np.linalg.norm(V[b], axis=0) - 1)) <= 4 * m * 2.0 ** -53
 
 
-@pytest.mark.parametrize("m", [3, 4, 15, 16, 17, 31, 32, 33, 63, 64])
+@pytest.mark.parametrize("m", [3, 4, 15, 16, 17, 31, 32, 33, 63, 64, 65, 97, 232, 233])
 def test_separated(m):
     rng = np.random.default_rng(m)
     lam = 2 * np.sqrt(rng.random(m)) * np.exp(2j * np.pi * rng.random(m))
@@ -42,7 +43,7 @@ def test_separated(m):
     _check(A, B, lam, 32 * m * 2.0 ** -53)   # (eigenvalue condition <= 2, B's <= 2)
 
 
-@pytest.mark.parametrize("m", [5, 18, 33, 64])
+@pytest.mark.parametrize("m", [5, 18, 33, 64, 66, 234])
 @pytest.mark.parametrize("gap", [1e-4, 1e-6, 1e-8, 1e-10, 0.0])
 def test_close_pairs(m, gap):
     rng = np.random.default_rng(100 + m)
