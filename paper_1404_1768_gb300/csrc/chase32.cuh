@@ -153,8 +153,9 @@ __device__ __forceinline__ void chase_left(Rows H, int w, int lo, int hi, int k0
         const bool more = k + 2 <= hi;
         const cf nn = (more && in) ? r2[c] : zero;
         const cf vn = more ? r2[k + 2] : zero;
-        cf *r3 = (k + 3 <= hi) ? H.row(k + 3) : r2;
-        const cf en = (k + 3 <= hi) ? r3[k + 2] : zero;
+        const bool third = k + 3 <= hi && k + 1 < k1;      // (a block may end at row k1 + 1)
+        cf *r3 = third ? H.row(k + 3) : r2;
+        const cf en = third ? r3[k + 2] : zero;
         const RotF g = rot32(x, y);
         const RotF gh = rot32_h(g);
         if (lane == 0) {

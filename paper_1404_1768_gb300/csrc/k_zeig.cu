@@ -27,6 +27,9 @@
 #ifndef FEAST_QR_FP32
 #define FEAST_QR_FP32 0
 #endif
+#if FEAST_QR_FP32
+#include "schur_cta.cuh"
+#endif
 
 namespace feast {
 
@@ -34,7 +37,7 @@ namespace {
 
 constexpr int CH = 32;           // rotations per chunk
 constexpr int BLK = CH + 3;      // local block edge
-constexpr int QT = 256;          // threads per CTA of the QR kernel
+constexpr int QT = FEAST_QR_FP32 ? 512 : 256;   // threads per CTA of the QR kernel
 constexpr int NSH = 16;          // most shifts (bulges) of a multishift sweep
 constexpr int DSEP = 2;          // phases between the entries of consecutive bulges
 constexpr int MS_MIN = 192;      // smallest active window that takes multishift sweeps
@@ -404,7 +407,20 @@ __device__ __forceinline__ ds cds_abs2(cds a) { return ds_add(ds_mul(a.re, a.re)
 __device__ __forceinline__ float cds_absf(cds a) { return hypotf(a.re.h, a.im.h); }
 __device__ __forceinline__ cds cds_zero() { cds r; r.re = ds_make(0.f, 0.f); r.im = r.re; return r; }
 
-// storage: float4 (re.h, re.l, im.h, im.l)
+// storage (dsv): float4 (re.h, re.l, im.h, im.l), or complex64 in the FP32 build
+#if FEAST_QR_FP32
+typedef float2 dsv;
+__device__ __forceinline__ cds ld_cds(const float2 *p)
+{
+    const float2 v = __ldcg(p);
+    cds r;
+    r.re = ds_make(v.x, 0.f);
+    r.im = ds_make(v.y, 0.f);
+    return r;
+}
+__device__ __forceinline__ void st_cds(float2 *p, cds v) { __stcg(p, make_float2(v.re.h, v.im.h)); }
+#else
+typedef float4 dsv;
 __device__ __forceinline__ cds ld_cds(const float4 *p)
 {
     float4 v = __ldcg(p);
@@ -414,6 +430,7 @@ __device__ __forceinline__ cds ld_cds(const float4 *p)
     return r;
 }
 __device__ __forceinline__ void st_cds(float4 *p, cds v) { __stcg(p, make_float4(v.re.h, v.re.l, v.im.h, v.im.l)); }
+#endif
 
 struct RotDS {
     ds c;   // real
@@ -531,7 +548,49 @@ __device__ __forceinline__ Bulge bulge_at(int t, int b, int l, int ihi, int m)
 // formed by every thread from the same shared values and applied by the
 // whole CTA.  A bulge enters at k == l with the first column of H - sigma I.
 // The rotations go to rots_g (global) for the far-part pass.
-__device__ __forceinline__ void chase_chunk(int m, float4 *H, int ld, int l, int ihi, const Bulge &bg, cds sigma,
+#if FEAST_QR_FP32
+// (FP32 build: the chain in one warp's registers, chase32.cuh; then warp 1
+// takes the rows passed and warp 2 the block's last column.)
+__device__ __forceinline__ void chase_chunk(int m, dsv *H, int ld, int l, int ihi, const Bulge &bg, cds sigma,
+                            cf (*blk)[BLK + 1], RotF *lrot, RotDS *rots_g)
+{
+    const int b0 = bg.b0, nb = bg.b1 - bg.b0 + 1, k0 = bg.k0 - b0, k1 = k0 + bg.nrot;
+    for (int e = threadIdx.x; e < nb * nb; e += QT) {
+        const int r = e % nb, c = e / nb;
+        blk[r][c] = __ldcg(H + (b0 + r) + (int64_t)(b0 + c) * ld);
+    }
+    __syncthreads();
+    const RowsLd R{&blk[0][0], BLK + 1};
+    const int t = threadIdx.x;
+    if (t < 32) chase_left(R, nb, l - b0, ihi - b0, k0, k1, cmakef(sigma.re.h, sigma.im.h), lrot);
+    __syncthreads();
+    if (t >= 32 && t < 64) {
+        for (int r = t - 32; r < k1; r += 32) chase_right(R.row(r), k0, r > k0 ? r : k0, k1, lrot);
+    } else if (t >= 64 && t < 96) {
+        const int c = k0 + CHASE_N + 1 + (t - 64);
+        if (c < nb) far_left(R, c, k0, k1, lrot);
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < nb * nb; e += QT) {
+        const int r = e % nb, c = e / nb;
+        __stcg(H + (b0 + r) + (int64_t)(b0 + c) * ld, blk[r][c]);
+    }
+    for (int e = t; e < bg.nrot; e += QT) {
+        RotDS g;
+        g.c = ds_make(lrot[e].c, 0.f);
+        g.s.re = ds_make(lrot[e].s.x, 0.f);
+        g.s.im = ds_make(lrot[e].s.y, 0.f);
+        float *o = (float *)(rots_g + e);
+        __stcg(o, g.c.h);
+        __stcg(o + 1, 0.f);
+        __stcg(o + 2, g.s.re.h);
+        __stcg(o + 3, 0.f);
+        __stcg(o + 4, g.s.im.h);
+        __stcg(o + 5, 0.f);
+    }
+}
+#else
+__device__ __forceinline__ void chase_chunk(int m, dsv *H, int ld, int l, int ihi, const Bulge &bg, cds sigma,
                             cds (*blk)[BLK + 1], RotDS *lrot, RotDS *rots_g)
 {
     const int b0 = bg.b0, nb = bg.b1 - bg.b0 + 1, k0 = bg.k0, k1 = bg.k0 + bg.nrot;
@@ -573,12 +632,13 @@ __device__ __forceinline__ void chase_chunk(int m, float4 *H, int ld, int l, int
     for (int e = threadIdx.x; e < bg.nrot * (int)(sizeof(RotDS) / sizeof(float)); e += QT)
         __stcg(((float *)rots_g) + e, ((const float *)lrot)[e]);
 }
+#endif
 
 // Left rotations of one chunk on the column segment col[0 .. nrot]: rotation
 // i mixes entries i and i+1, so entry i is final once rotation i is done and
 // only one entry is carried forward; loads go out FG entries at a time.
 constexpr int FG = 8;
-__device__ __forceinline__ void far_left(float4 *col, int nrot, const RotDS *rot)
+__device__ __forceinline__ void far_left(dsv *col, int nrot, const RotDS *rot)
 {
     cds carry = ld_cds(col);
     for (int g0 = 0; g0 < nrot; g0 += FG) {
@@ -598,7 +658,7 @@ __device__ __forceinline__ void far_left(float4 *col, int nrot, const RotDS *rot
     st_cds(col + nrot, carry);
 }
 // Right rotations of one chunk on the row segment row[0], row[ld], ...
-__device__ __forceinline__ void far_right(float4 *row, int ld, int nrot, const RotDS *rot)
+__device__ __forceinline__ void far_right(dsv *row, int ld, int nrot, const RotDS *rot)
 {
     cds carry = ld_cds(row);
     for (int g0 = 0; g0 < nrot; g0 += FG) {
@@ -715,70 +775,61 @@ __device__ bool win_schur(int w, cds (*T)[NWP], cds (*V)[NWP], float tol_rel, fl
 }
 
 #if FEAST_QR_FP32
-// FP32 build: the same single-shift QR by one warp.  The window's rows and
-// columns (at most NW) take one or two lanes each, and in FP32 a
-// rotation is a few operations per lane -- less than the CTA barriers the
-// whole-CTA form spends on each one; lanes order their shared-memory
-// updates with __syncwarp.  The other warps of the CTA wait at the caller's
-// barrier.
-__device__ bool win_schur_warp(int w, cds (*T)[NWP], cds (*V)[NWP], float tol_rel, float tol_abs)
+// FP32 build: the same single-shift QR on complex64 copies of T and V
+// (row-major, ld NWP): warp 0 scans, shifts, chases (chase32.cuh; the window's
+// NW columns are one chunk) and takes T's rows, while warp 1 applies the sweep
+// before to V.  rot: two sweeps of NW rotations; ctl: two ints.  The first 64
+// threads only; the result counts in warp 0.
+__device__ bool win_schur32(int w, cf *T, cf *V, float tol_rel, float tol_abs, RotF *rot, int *ctl)
 {
-    const int lane = threadIdx.x & 31;
+    const int t = threadIdx.x, lane = t & 31;
     int hi = w - 1, it = 0, tot = 0;
-    while (hi > 0) {
-        // lo: the largest p in [1, hi] with a negligible subdiagonal entry, else 0
+    for (int sweep = 0;; ++sweep) {
+        RotF *rs = rot + (sweep & 1) * NW;
         int lo = 0;
-        for (int base = hi; base >= 1 && lo == 0; base -= 32) {
-            const int p = base - lane;
-            bool neg = false;
-            if (p >= 1) {
-                const float sub = cds_absf(T[p][p - 1]);
-                const float loc = cds_absf(T[p - 1][p - 1]) + cds_absf(T[p][p]);
-                neg = (sub <= tol_rel * loc || sub <= tol_abs);
+        if (t < 32) {
+            while (hi > 0) {
+                // lo: the largest p in [1, hi] with a negligible subdiagonal entry, else 0
+                const int p = hi - lane;
+                bool neg = false;
+                if (p >= 1) {
+                    const float sub = abs32(T[p * NWP + p - 1]);
+                    const float loc = abs32(T[(p - 1) * NWP + p - 1]) + abs32(T[p * NWP + p]);
+                    neg = !(sub > tol_rel * loc) || !(sub > tol_abs);
+                }
+                const unsigned b = __ballot_sync(0xffffffffu, neg);
+                lo = b ? hi - (__ffs(b) - 1) : 0;
+                if (lo < hi) break;
+                --hi;
+                it = 0;
             }
-            const unsigned b = __ballot_sync(0xffffffffu, neg);
-            if (b) lo = base - (__ffs(b) - 1);
-        }
-        __syncwarp();
-        if (lo > 0 && lane == 0) T[lo][lo - 1] = cds_zero();
-        __syncwarp();
-        if (lo == hi) { --hi; it = 0; continue; }
-        if (++tot > 40 * w) return false;
-        ++it;
-        cds sigma;
-        {
-            const cds h00 = T[hi - 1][hi - 1], h01 = T[hi - 1][hi], h10 = T[hi][hi - 1], h11 = T[hi][hi];
-            if (it % 11 == 10) {
-                const float a = cds_absf(h10);
-                sigma = h11;
-                sigma.re = ds_add(sigma.re, ds_make(a, 0.f));
-                sigma.im = ds_add(sigma.im, ds_make(0.5f * a, 0.f));
-            } else {
-                cds half = cds_scale(cds_add(h00, h11), ds_make(0.5f, 0.f));
-                cds det = cds_sub(cds_mul(h00, h11), cds_mul(h01, h10));
-                cds disc = csqrt_ds_approx(cds_sub(cds_mul(half, half), det));
-                cds r1 = cds_add(half, disc), r2 = cds_sub(half, disc);
-                sigma = (cds_absf(cds_sub(r1, h11)) < cds_absf(cds_sub(r2, h11))) ? r1 : r2;
+            if (hi > 0 && ++tot > 40 * w) hi = -1;
+            if (hi > 0) {
+                ++it;
+                const cf h11 = T[hi * NWP + hi], h10 = T[hi * NWP + hi - 1];
+                cf sigma = shift32(T[(hi - 1) * NWP + hi - 1], T[(hi - 1) * NWP + hi], h10, h11);
+                if (it % 11 == 10) {
+                    const float a = abs32(h10);
+                    sigma = cmakef(h11.x + a, h11.y + 0.5f * a);
+                }
+                __syncwarp();
+                chase_left(RowsLd{T, NWP}, w, lo, hi, lo, hi, sigma, rs);
+            }
+            if (lane == 0) {
+                ctl[2 * (sweep & 1)] = lo;
+                ctl[2 * (sweep & 1) + 1] = hi;
             }
         }
-        __syncwarp();
-        for (int k = lo; k < hi; ++k) {
-            cds x, y;
-            if (k == lo) { x = cds_sub(T[k][k], sigma); y = T[k + 1][k]; }
-            else { x = T[k][k - 1]; y = T[k + 1][k - 1]; }
-            const RotDS gr = make_rot_ds(x, y);
+        asm volatile("bar.sync 1, 64;" ::: "memory");
+        const int l = ctl[2 * (sweep & 1)], h = ctl[2 * (sweep & 1) + 1];
+        if (h <= 0) return h == 0;
+        if (t < 32) {
+            if (lane < h) chase_right(T + lane * NWP, l, lane > l ? lane : l, h, rs);
             __syncwarp();
-            const int c0 = (k == lo) ? k : k - 1;
-            for (int j = c0 + lane; j < w; j += 32) rot_left_ds(gr, T[k][j], T[k + 1][j]);
-            if (k > lo && lane == 0) T[k + 1][k - 1] = cds_zero();   // (lane 0 rotated that column)
-            __syncwarp();
-            const int r1 = (k + 2 < hi) ? k + 2 : hi;
-            for (int i = lane; i <= r1; i += 32) rot_right_ds(gr, T[i][k], T[i][k + 1]);
-            for (int i = lane; i < w; i += 32) rot_right_ds(gr, V[i][k], V[i][k + 1]);
-            __syncwarp();
+        } else if (lane < w) {
+            chase_right(V + lane * NWP, l, l, h, rs);
         }
     }
-    return true;
 }
 #endif
 
@@ -879,6 +930,11 @@ struct AedShared {
     ds tau;
     cds alpha;
     int nd, ok;
+#if FEAST_QR_FP32
+    cf T32[NW * NWP], V32[NW * NWP];
+    RotF rot[2 * NW];
+    int ctl[4];
+#endif
 };
 
 // AED on the window [kw, kw + w - 1] (kw = ihi - w + 1) of the active block
@@ -886,8 +942,8 @@ struct AedShared {
 // spike column, the total window transform to vg (w x w), shifts of the
 // undeflated part (up to ns, the bottom-most) to shifts, and returns nd
 // (deflated count) in sh->nd; nd = 0 leaves H untouched.
-__device__ void aed_window(int m, float4 *H, int ld, int l, int kw, int w, int ns, float tol_rel, float tol_abs,
-                           AedShared *sh, float4 *vg, float2 *shifts)
+__device__ void aed_window(int m, dsv *H, int ld, int l, int kw, int w, int ns, float tol_rel, float tol_abs,
+                           AedShared *sh, dsv *vg, float2 *shifts)
 {
     const int t = threadIdx.x;
     for (int e = t; e < w * w; e += QT) {
@@ -900,9 +956,27 @@ __device__ void aed_window(int m, float4 *H, int ld, int l, int kw, int w, int n
     if (t == 0) { sh->nd = 0; sh->ok = 1; }
     __syncthreads();
 #if FEAST_QR_FP32
-    if (t < 32) {
-        const bool r = win_schur_warp(w, sh->T, sh->V, tol_rel, tol_abs);
+    for (int e = t; e < w * w; e += QT) {
+        const int r = e % w, c = e / w;
+        sh->T32[r * NWP + c] = cmakef(sh->T[r][c].re.h, sh->T[r][c].im.h);
+        sh->V32[r * NWP + c] = cmakef(sh->V[r][c].re.h, sh->V[r][c].im.h);
+    }
+    __syncthreads();
+    if (t < 64) {
+        const bool r = win_schur32(w, sh->T32, sh->V32, tol_rel, tol_abs, sh->rot, sh->ctl);
         if (t == 0) sh->ok = r ? 1 : 0;
+    }
+    __syncthreads();
+    for (int e = t; e < w * w; e += QT) {
+        const int r = e % w, c = e / w;
+        const cf x = sh->T32[r * NWP + c], y = sh->V32[r * NWP + c];
+        cds v;
+        v.re = ds_make(r <= c ? x.x : 0.f, 0.f);
+        v.im = ds_make(r <= c ? x.y : 0.f, 0.f);
+        sh->T[r][c] = v;
+        v.re = ds_make(y.x, 0.f);
+        v.im = ds_make(y.y, 0.f);
+        sh->V[r][c] = v;
     }
     __syncthreads();
     const bool ok = sh->ok != 0;
@@ -984,14 +1058,14 @@ __device__ void aed_window(int m, float4 *H, int ld, int l, int kw, int w, int n
 // Apply the window transform W (w x w, in shared memory) to the rest of H
 // and to Z: H[0:kw, win] <- H[0:kw, win] W, H[win, c] <- W^H H[win, c] for
 // c > kw + w - 1, Z[:, win] <- Z[:, win] W.  One warp per line.
-__device__ void aed_apply(int m, float4 *H, float4 *Z, int ld, int kw, int w, const cds (*W)[NWP])
+__device__ void aed_apply(int m, dsv *H, dsv *Z, int ld, int kw, int w, const cds (*W)[NWP])
 {
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * QT + threadIdx.x) >> 5, nwarps = (gridDim.x * QT) >> 5;
     const int right = m - (kw + w);
     const int lines = kw + m + right;
     for (int x = gw; x < lines; x += nwarps) {
-        float4 *base;
+        dsv *base;
         int64_t stride;
         bool colline;
         if (x < kw) { base = H + x + (int64_t)kw * ld; stride = ld; colline = false; }
@@ -1023,7 +1097,7 @@ __device__ void aed_apply(int m, float4 *H, float4 *Z, int ld, int kw, int w, co
 // The CTA tests QT candidates at a time from the bottom (the first hit of a
 // scan from ihi downwards).  Whole CTA, ihi uniform; every CTA finds the
 // same p from the same H.
-__device__ int scan_deflation(const float4 *H, int ld, int ihi, float tol_rel, float tol_abs)
+__device__ int scan_deflation(const dsv *H, int ld, int ihi, float tol_rel, float tol_abs)
 {
     __shared__ int s_l;
     for (int top = ihi; top >= 1; top -= QT) {
@@ -1055,16 +1129,21 @@ __device__ int scan_deflation(const float4 *H, int ld, int ihi, float tol_rel, f
 // (column segments above its block, and Z), so no two writers meet.  Blocks
 // of at most NW rows are brought to Schur form at once by the window
 // routine; those in between take single-shift sweeps (Wilkinson shift,
-// exceptional shift every 11th sweep).  H, Z: m x m double-single (float4),
+// exceptional shift every 11th sweep).  H, Z: m x m double-single (dsv),
 // leading dim ld; rots: NSH * CH rotations; shifts: NSH entries; vwin: the
 // NW x NW window transform; ctl: the window's deflation count.
-__global__ void __launch_bounds__(QT, 1) k_hqr(int m, float4 *H, float4 *Z, int ld, RotDS *rots, float2 *shifts,
-                                               float4 *vwin, int *ctl, GridSync g, int *fail, float tol_rel,
-                                               float tol_abs, int *stats)
+__global__ void __launch_bounds__(QT, 1) k_hqr(int m, dsv *H, dsv *Z, int ld, RotDS *rots, float2 *shifts,
+                                               dsv *vwin, int *ctl, GridSync g, int *fail, float tol_rel,
+                                               float tol_abs, int *stats, float4 *rlog, int max_log)
 {
     extern __shared__ __align__(16) unsigned char hqr_dyn[];
     AedShared *sh = (AedShared *)hqr_dyn;
+#if FEAST_QR_FP32
+    __shared__ cf blk[BLK][BLK + 1];
+    __shared__ RotF crot[CH];
+#else
     __shared__ cds blk[BLK][BLK + 1];
+#endif
     __shared__ RotDS srot[NSH][CH];
     const int gtid = blockIdx.x * QT + threadIdx.x, gthreads = gridDim.x * QT;
     int ihi = m - 1, iter = 0, total = 0;
@@ -1082,6 +1161,39 @@ __global__ void __launch_bounds__(QT, 1) k_hqr(int m, float4 *H, float4 *Z, int 
         total += ns;
         if (total > 30 * m) { if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(fail, 1); return; }
         ++iter;
+#if FEAST_QR_FP32
+        if (L < MS_MIN) {
+            // the whole active block fits the shared memory of a CTA: its
+            // triangular form at once (a sweep here costs two barriers of one
+            // CTA per 32 rotations, not three of the grid), then the logged
+            // rotations on the rest of H and on Z
+            cf *sp = (cf *)hqr_dyn;
+            const RowsPacked R{sp, L};
+            if (blockIdx.x == 0) {
+                for (int c = threadIdx.x >> 5; c < L; c += QT / 32)
+                    for (int r = threadIdx.x & 31; r < L && r <= c + 2; r += 32)
+                        R.row(r)[c] = (r <= c + 1) ? __ldcg(H + (l + r) + (int64_t)(l + c) * ld) : cmakef(0.f, 0.f);
+                __syncthreads();
+                int nr = 0, tot = 0;
+                const int st = schur_cta_core<QT>(R, L, tol_rel, tol_abs, rlog, max_log, &nr, &tot);
+                for (int c = threadIdx.x >> 5; c < L; c += QT / 32)
+                    for (int r = threadIdx.x & 31; r < L; r += 32)
+                        __stcg(H + (l + r) + (int64_t)(l + c) * ld, (r <= c) ? R.row(r)[c] : cmakef(0.f, 0.f));
+                if (threadIdx.x == 0) {
+                    __stcg(ctl + 1, st);
+                    __stcg(ctl + 2, nr);
+                    if (stats) stats[0] += tot;
+                }
+            }
+            if (!grid_barrier(g)) return;
+            if (__ldcg(ctl + 1)) { if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(fail, 1); return; }
+            apply_log_lines(m, H, Z, ld, l, L, rlog, __ldcg(ctl + 2), sp);
+            if (!grid_barrier(g)) return;
+            ihi = l - 1;
+            iter = 0;
+            continue;
+        }
+#endif
         if (L <= NW) {
             // the whole active block fits a window: its Schur form at once
             if (blockIdx.x == 0) {
@@ -1113,9 +1225,9 @@ __global__ void __launch_bounds__(QT, 1) k_hqr(int m, float4 *H, float4 *Z, int 
                     const int nd = sh->nd;
                     for (int b = threadIdx.x; b < ns; b += QT) {
                         const int i = ihi - nd - b;
-                        float4 d = __ldcg(H + i + (int64_t)i * ld), e = __ldcg(H + i + (int64_t)(i - 1) * ld);
-                        const float s = hypotf(e.x, e.z);
-                        shifts[b] = make_float2(d.x + 0.75f * s, d.z + 0.4f * s);
+                        const cds d = ld_cds(H + i + (int64_t)i * ld), e = ld_cds(H + i + (int64_t)(i - 1) * ld);
+                        const float s = cds_absf(e);
+                        shifts[b] = make_float2(d.re.h + 0.75f * s, d.im.h + 0.4f * s);
                     }
                 }
             }
@@ -1148,7 +1260,11 @@ __global__ void __launch_bounds__(QT, 1) k_hqr(int m, float4 *H, float4 *Z, int 
                         cds sigma = cds_zero();
                         sigma.re = ds_make(sf.x, 0.f);
                         sigma.im = ds_make(sf.y, 0.f);
+#if FEAST_QR_FP32
+                        chase_chunk(m, H, ld, l, ihi, bg, sigma, blk, crot, rots + (size_t)b * CH);
+#else
                         chase_chunk(m, H, ld, l, ihi, bg, sigma, blk, srot[0], rots + (size_t)b * CH);
+#endif
                     }
                 }
                 if (!grid_barrier(g)) return;
@@ -1191,7 +1307,7 @@ __global__ void __launch_bounds__(QT, 1) k_hqr(int m, float4 *H, float4 *Z, int 
                             if (rem < cnt) break;
                             rem -= cnt;
                         }
-                        float4 *row = (rem < bg.b0) ? H + rem + (int64_t)bg.k0 * ld
+                        dsv *row = (rem < bg.b0) ? H + rem + (int64_t)bg.k0 * ld
                                                     : Z + (rem - bg.b0) + (int64_t)bg.k0 * ld;
                         far_right(row, ld, bg.nrot, srot[b]);
                     }
@@ -1200,6 +1316,7 @@ __global__ void __launch_bounds__(QT, 1) k_hqr(int m, float4 *H, float4 *Z, int 
             }
             continue;
         }
+#if !FEAST_QR_FP32
         // ---------------------------------------------------- single-shift sweep
         cds sigma;
         {
@@ -1250,12 +1367,13 @@ __global__ void __launch_bounds__(QT, 1) k_hqr(int m, float4 *H, float4 *Z, int 
                     far_left(H + (int64_t)(bg.b1 + 1 + x) * ld + k0, bg.nrot, srot[0]);
                 } else {
                     const int r = (x < ncol + nrowH) ? x - ncol : x - ncol - nrowH;
-                    float4 *row = ((x < ncol + nrowH) ? H : Z) + r + (int64_t)k0 * ld;
+                    dsv *row = ((x < ncol + nrowH) ? H : Z) + r + (int64_t)k0 * ld;
                     far_right(row, ld, bg.nrot, srot[0]);
                 }
             }
             if (!grid_barrier(g)) return;
         }
+#endif
     }
 }
 
@@ -1774,7 +1892,10 @@ int schur_large(cudaStream_t s, int m, zd *C, zd *Q, void *work, int *fail, int 
     FEAST_LAUNCH_CHECK();
     k_to_ds<<<gcv, 256, 0, s>>>((int64_t)m * m, Q, Qds);
     FEAST_LAUNCH_CHECK();
-    void *args[] = {&mm, &Hds, &Qds, &ldh, &rots, &shifts, &vwin, &ctl, &gs, &fail, &tol_rel, &tol_abs, &stats};
+    float4 *rlog = nullptr;   // (FP32 build only)
+    int max_log = 0;
+    void *args[] = {&mm,   &Hds, &Qds,     &ldh,     &rots,  &shifts, &vwin,    &ctl,
+                    &gs,   &fail, &tol_rel, &tol_abs, &stats, &rlog,   &max_log};
     FEAST_CUDA_TRY(cudaLaunchCooperativeKernel((void *)k_hqr, dim3(grid), dim3(QT), args, dyn, s));
     FEAST_LAUNCH_CHECK();
     k_from_ds<<<gcv, 256, 0, s>>>((int64_t)m * m, Hds, C);
