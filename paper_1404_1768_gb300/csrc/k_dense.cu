@@ -15,7 +15,7 @@ namespace feast {
 
 // ------------------------------------------------------------------ GEMM
 namespace {
-constexpr int GB_M = 64, GB_N = 64, GB_K = 8, GB_T = 256;
+constexpr int GB_K = 8, GB_T = 256;
 
 constexpr int GB_SMAX = 8;     // most K-slices of a tile summed in one (portable) cluster
 
@@ -65,7 +65,9 @@ __device__ __forceinline__ double2 gb_dsmem_load(const double2 *p, unsigned rank
 // not depend on which slice finishes first; beyond that (long, skinny
 // products) the slices add alpha * partial into C atomically, C pre-scaled
 // by beta on the host side of the launch.
-template <typename T>
+// A CTA of 16 x 16 threads computes a 16 TM x 16 TM tile, TM x TM entries per
+// thread.
+template <typename T, int TM>
 __global__ void __launch_bounds__(GB_T) k_gemm(int conj_a, int64_t m, int64_t n, int64_t k,
                                                T alpha, const T *__restrict__ A, int64_t lda,
                                                int64_t sA, const T *__restrict__ B,
@@ -73,6 +75,7 @@ __global__ void __launch_bounds__(GB_T) k_gemm(int conj_a, int64_t m, int64_t n,
                                                T *__restrict__ C, int64_t ldc, int64_t sC,
                                                int splits, int64_t kchunk, int tri)
 {
+    constexpr int GB_M = 16 * TM, GB_N = 16 * TM;
     __shared__ T As[GB_K][GB_M + 1];
     __shared__ T Bs[GB_K][GB_N + 1];
     extern __shared__ __align__(16) unsigned char gb_red_raw[];   // splits > 1: this slice's tile
@@ -87,11 +90,11 @@ __global__ void __launch_bounds__(GB_T) k_gemm(int conj_a, int64_t m, int64_t n,
     B += (int64_t)b * sB;
     C += (int64_t)b * sC;
     const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    T acc[4][4];
+    T acc[TM][TM];
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < TM; ++a)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[a][c] = cx<T>(0, 0);
+        for (int c = 0; c < TM; ++c) acc[a][c] = cx<T>(0, 0);
 
     for (int64_t k0 = kbeg; k0 < kend; k0 += GB_K) {
         // A tile: op(A)(i0 + r, k0 + kk)
@@ -112,23 +115,23 @@ __global__ void __launch_bounds__(GB_T) k_gemm(int conj_a, int64_t m, int64_t n,
         __syncthreads();
 #pragma unroll
         for (int kk = 0; kk < GB_K; ++kk) {
-            T av[4], bv[4];
+            T av[TM], bv[TM];
 #pragma unroll
-            for (int a = 0; a < 4; ++a) av[a] = As[kk][ty + 16 * a];
+            for (int a = 0; a < TM; ++a) av[a] = As[kk][ty + 16 * a];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) bv[c] = Bs[kk][tx + 16 * c];
+            for (int c = 0; c < TM; ++c) bv[c] = Bs[kk][tx + 16 * c];
 #pragma unroll
-            for (int a = 0; a < 4; ++a)
+            for (int a = 0; a < TM; ++a)
 #pragma unroll
-                for (int c = 0; c < 4; ++c) cfma(acc[a][c], av[a], bv[c]);
+                for (int c = 0; c < TM; ++c) cfma(acc[a][c], av[a], bv[c]);
         }
         __syncthreads();
     }
     if (splits > GB_SMAX) {
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
+        for (int a = 0; a < TM; ++a)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
+            for (int c = 0; c < TM; ++c) {
                 int64_t gi = i0 + ty + 16 * a, gj = j0 + tx + 16 * c;
                 if (gi < m && gj < n) atomic_cadd(&C[gi + gj * ldc], cmul(alpha, acc[a][c]));
             }
@@ -141,25 +144,25 @@ __global__ void __launch_bounds__(GB_T) k_gemm(int conj_a, int64_t m, int64_t n,
         T *red = reinterpret_cast<T *>(gb_red_raw);
         const unsigned rank = gb_cluster_rank();
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
+        for (int a = 0; a < TM; ++a)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) red[(a * 4 + c) * GB_T + threadIdx.x] = acc[a][c];
+            for (int c = 0; c < TM; ++c) red[(a * TM + c) * GB_T + threadIdx.x] = acc[a][c];
         gb_cluster_sync();
         if (rank == 0)
             for (int r = 1; r < splits; ++r)
 #pragma unroll
-                for (int a = 0; a < 4; ++a)
+                for (int a = 0; a < TM; ++a)
 #pragma unroll
-                    for (int c = 0; c < 4; ++c)
-                        acc[a][c] = cadd(acc[a][c], gb_dsmem_load(red + (a * 4 + c) * GB_T + threadIdx.x, r));
+                    for (int c = 0; c < TM; ++c)
+                        acc[a][c] = cadd(acc[a][c], gb_dsmem_load(red + (a * TM + c) * GB_T + threadIdx.x, r));
         gb_cluster_sync();
         if (rank != 0) return;
     }
     const bool beta0 = cis_zero(beta);
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < TM; ++a)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < TM; ++c) {
             int64_t gi = i0 + ty + 16 * a, gj = j0 + tx + 16 * c;
             if (gi < m && gj < n) {
                 T v = cmul(alpha, acc[a][c]);
@@ -183,21 +186,18 @@ __global__ void k_scale(int64_t m, int64_t n, T beta, T *C, int64_t ldc, int64_t
 }
 }  // namespace
 
-template <typename T>
-int gemm_batched(cudaStream_t s, int conj_a, int64_t m, int64_t n, int64_t k, T alpha,
-                 const T *A, int64_t lda, int64_t sA, const T *B, int64_t ldb, int64_t sB,
-                 T beta, T *C, int64_t ldc, int64_t sC, int batch, int tri)
+// gemm_batched with a given tile.
+template <typename T, int TM>
+static int gemm_tiled(cudaStream_t s, int conj_a, int64_t m, int64_t n, int64_t k, T alpha, const T *A, int64_t lda,
+                      int64_t sA, const T *B, int64_t ldb, int64_t sB, T beta, T *C, int64_t ldc, int64_t sC, int batch,
+                      int tri)
 {
-    if (m <= 0 || n <= 0 || batch <= 0) return FEAST_OK;
-    if (batch > 65535) return FEAST_EINVAL;
-    if (tri < 0 || tri > 3 || (conj_a && (tri == 1 || tri == 2))) return FEAST_EINVAL;
+    constexpr int GB_M = 16 * TM, GB_N = 16 * TM;
     const unsigned tiles = cdiv(m, GB_M) * cdiv(n, GB_N) * (unsigned)batch;
-    // split K when the output tiles cannot fill the GPU twice over (the
-    // FP64 pipe is the bound, so every SM counts: a 64 x 64 tile with
-    // K = 256 is ~1 ms of one SM's FP64 pipe), in slices of at least 32
-    // (complex64: 128); up to GB_SMAX slices are summed in a fixed order
-    // (one cluster per tile), more of them atomically (products with a
-    // long K and only a tile or two of output)
+    // split K when the output tiles cannot fill the GPU twice over, in slices
+    // of at least 32 (complex64: 128); up to GB_SMAX slices are summed in a
+    // fixed order (one cluster per tile), more of them atomically (products
+    // with a long K and only a tile or two of output)
     const bool fp64 = sizeof(T) == sizeof(zd);
     const int64_t kmin = fp64 ? 32 : 128;
     int splits = 1;
@@ -215,8 +215,8 @@ int gemm_batched(cudaStream_t s, int conj_a, int64_t m, int64_t n, int64_t k, T 
     dim3 grid(cdiv(m, GB_M), cdiv(n, GB_N), batch * splits);
     if (grid.y > 65535) return FEAST_EINVAL;
     if (splits == 1) {
-        k_gemm<T><<<grid, GB_T, 0, s>>>(conj_a, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, 1, kchunk,
-                                        tri);
+        k_gemm<T, TM><<<grid, GB_T, 0, s>>>(conj_a, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, 1, kchunk,
+                                            tri);
         FEAST_LAUNCH_CHECK();
         return FEAST_OK;
     }
@@ -227,13 +227,13 @@ int gemm_batched(cudaStream_t s, int conj_a, int64_t m, int64_t n, int64_t k, T 
             k_scale<T><<<dim3(gx > 4096 ? 4096 : gx, batch), 256, 0, s>>>(m, n, beta, C, ldc, sC);
             FEAST_LAUNCH_CHECK();
         }
-        k_gemm<T><<<grid, GB_T, 0, s>>>(conj_a, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, splits,
-                                        kchunk, tri);
+        k_gemm<T, TM><<<grid, GB_T, 0, s>>>(conj_a, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, splits,
+                                            kchunk, tri);
         FEAST_LAUNCH_CHECK();
         return FEAST_OK;
     }
-    const size_t red = sizeof(T) * 16 * GB_T;
-    FEAST_CUDA_TRY(ensure_dyn_smem(k_gemm<T>, red));
+    const size_t red = sizeof(T) * TM * TM * GB_T;
+    FEAST_CUDA_TRY(ensure_dyn_smem(k_gemm<T, TM>, red));
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -246,10 +246,32 @@ int gemm_batched(cudaStream_t s, int conj_a, int64_t m, int64_t n, int64_t k, T 
     cfg.stream = s;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    FEAST_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_gemm<T>, conj_a, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc,
+    FEAST_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_gemm<T, TM>, conj_a, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc,
                                       sC, splits, kchunk, tri));
     FEAST_LAUNCH_CHECK();
     return FEAST_OK;
+}
+
+template <typename T>
+int gemm_batched(cudaStream_t s, int conj_a, int64_t m, int64_t n, int64_t k, T alpha,
+                 const T *A, int64_t lda, int64_t sA, const T *B, int64_t ldb, int64_t sB,
+                 T beta, T *C, int64_t ldc, int64_t sC, int batch, int tri)
+{
+    if (m <= 0 || n <= 0 || batch <= 0) return FEAST_OK;
+    if (batch > 65535) return FEAST_EINVAL;
+    if (tri < 0 || tri > 3 || (conj_a && (tri == 1 || tri == 2))) return FEAST_EINVAL;
+    // Tile: a 64 x 64 x 32 product keeps one SM's FP64 pipe busy for 137 us
+    // (2 DFMA a clock), so a few large tiles leave the other SMs idle, and a
+    // smaller tile costs that pipe nothing: 64 x 64 only from eight waves of
+    // them on (a last wave then costs at most an eighth), 32 x 32 down to two
+    // waves, 16 x 16 below (a rank-32 update of 16 nodes of 200 x 64: 150 ->
+    // 30 us).  In FP32 the large tile's reuse pays as soon as it fills the GPU.
+    const bool fp64 = sizeof(T) == sizeof(zd);
+    auto tiles_of = [&](int tm) { return (long long)cdiv(m, 16 * tm) * cdiv(n, 16 * tm) * batch; };
+    const int tm = tiles_of(4) >= (fp64 ? 8 * 152 : 152) ? 4 : (tiles_of(2) >= 2 * 152 || !fp64) ? 2 : 1;
+    if (tm == 4) return gemm_tiled<T, 4>(s, conj_a, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, batch, tri);
+    if (tm == 2) return gemm_tiled<T, 2>(s, conj_a, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, batch, tri);
+    return gemm_tiled<T, 1>(s, conj_a, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, batch, tri);
 }
 template int gemm_batched<double2>(cudaStream_t, int, int64_t, int64_t, int64_t, double2, const double2 *,
                                    int64_t, int64_t, const double2 *, int64_t, int64_t, double2, double2 *,
@@ -292,6 +314,127 @@ int zform_shifted(cudaStream_t s, int64_t n, int q, const zd *A, const zd *B, in
     FEAST_LAUNCH_CHECK();
     return FEAST_OK;
 }
+
+// ------------------------------------------------------------------ diagonal solves
+namespace {
+constexpr int SV_NB = 32;
+
+// X rows [k0, k0+nb) <- T^{-1} X rows [k0, k0+nb) for the diagonal block T of
+// the factor (lower = unit lower L, else upper U).  One thread per column.
+template <typename C>
+__global__ void k_trsv_diag(int64_t nrhs, int64_t k0, int nb, int lower,
+                            const C *F, int64_t ldf, int64_t sF, C *X, int64_t ldx, int64_t sX)
+{
+    const int b = blockIdx.y;
+    const C *Am = F + (int64_t)b * sF;
+    C *Xb = X + (int64_t)b * sX;
+    __shared__ C T[SV_NB][SV_NB + 1];
+    for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
+        int r = e % nb, c = e / nb;
+        T[r][c] = Am[(k0 + r) + (k0 + c) * ldf];
+    }
+    __syncthreads();
+    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= nrhs) return;
+    C x[SV_NB];
+#pragma unroll
+    for (int r = 0; r < SV_NB; ++r)
+        if (r < nb) x[r] = Xb[(k0 + r) + c * ldx];
+    if (lower) {
+#pragma unroll
+        for (int i = 0; i < SV_NB; ++i) {
+            if (i >= nb) break;
+#pragma unroll
+            for (int r = i + 1; r < SV_NB; ++r)
+                if (r < nb) cfma(x[r], cneg(T[r][i]), x[i]);
+        }
+    } else {
+#pragma unroll
+        for (int i = SV_NB - 1; i >= 0; --i) {
+            if (i >= nb) continue;
+            x[i] = cdiv(x[i], T[i][i]);
+#pragma unroll
+            for (int r = 0; r < SV_NB; ++r)
+                if (r < i) cfma(x[r], cneg(T[r][i]), x[i]);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < SV_NB; ++r)
+        if (r < nb) Xb[(k0 + r) + c * ldx] = x[r];
+}
+
+
+// The same with a warp per column, lane r holding row r: the rows of T and of
+// X are divided by the diagonal once (upper), and each step passes one solved
+// entry by shuffles.  32 dependent steps instead of 496 multiply-adds per
+// thread.
+constexpr int SW_W = 8;    // columns (warps) per CTA
+template <typename C>
+__global__ void __launch_bounds__(32 * SW_W) k_trsv_warp(int64_t nrhs, int64_t k0, int nb, int lower, const C *F,
+                                                         int64_t ldf, int64_t sF, C *X, int64_t ldx, int64_t sX)
+{
+    const int b = blockIdx.y;
+    const C *Am = F + (int64_t)b * sF;
+    C *Xb = X + (int64_t)b * sX;
+    __shared__ C T[SV_NB][SV_NB + 1];
+    __shared__ C dinv[SV_NB];
+    const int lane = threadIdx.x & 31;
+    for (int e = threadIdx.x; e < nb * nb; e += 32 * SW_W) {
+        const int r = e % nb, c = e / nb;
+        T[r][c] = Am[(k0 + r) + (k0 + c) * ldf];
+    }
+    __syncthreads();
+    if (!lower) {
+        if (threadIdx.x < nb) dinv[threadIdx.x] = cdiv(cx<C>(1, 0), T[threadIdx.x][threadIdx.x]);
+        __syncthreads();
+        for (int e = threadIdx.x; e < nb * nb; e += 32 * SW_W) {
+            const int r = e % nb, c = e / nb;
+            if (c > r) T[r][c] = cmul(T[r][c], dinv[r]);
+        }
+        __syncthreads();
+    }
+    const int64_t c = (int64_t)blockIdx.x * SW_W + (threadIdx.x >> 5);
+    if (c >= nrhs) return;
+    const bool on = lane < nb;
+    C x = on ? Xb[(k0 + lane) + c * ldx] : cx<C>(0, 0);
+    if (lower) {
+        for (int i = 0; i + 1 < nb; ++i) {
+            C xi;
+            xi.x = __shfl_sync(0xffffffffu, x.x, i);
+            xi.y = __shfl_sync(0xffffffffu, x.y, i);
+            if (lane > i && on) cfma(x, cneg(T[lane][i]), xi);
+        }
+    } else {
+        if (on) x = cmul(x, dinv[lane]);
+        for (int i = nb - 1; i > 0; --i) {
+            C xi;
+            xi.x = __shfl_sync(0xffffffffu, x.x, i);
+            xi.y = __shfl_sync(0xffffffffu, x.y, i);
+            if (lane < i) cfma(x, cneg(T[lane][i]), xi);
+        }
+    }
+    if (on) Xb[(k0 + lane) + c * ldx] = x;
+}
+
+// X rows [k0, k0 + nb) <- T^{-1} X rows (see the kernels).  A warp per column
+// takes 32 dependent steps, a thread per column 496; in FP64 a warp-wide
+// instruction holds its SM quarter's pipe for 64 clocks whatever the lanes, so
+// the warp form costs ~8 k clocks per column and quarter (608 quarters)
+// against ~127 k per 32 columns: it wins up to 16 columns a quarter (8 nodes x
+// 150 columns: 98 -> ~20 us).  In FP32 the warp form always wins (32 nodes x
+// 640 columns: 27 -> ~8 us).
+template <typename C>
+int trsv_diag(cudaStream_t s, int64_t nrhs, int batch, int64_t k0, int nb, int lower, const C *F, int64_t ldf,
+              int64_t sF, C *X, int64_t ldx, int64_t sX)
+{
+    if (sizeof(C) == sizeof(cf) || nrhs * batch <= 16 * 608)
+        k_trsv_warp<C><<<dim3(cdiv(nrhs, SW_W), batch), 32 * SW_W, 0, s>>>(nrhs, k0, nb, lower, F, ldf, sF, X, ldx, sX);
+    else
+        k_trsv_diag<C><<<dim3(cdiv(nrhs, 64), batch), 64, 0, s>>>(nrhs, k0, nb, lower, F, ldf, sF, X, ldx, sX);
+    FEAST_LAUNCH_CHECK();
+    return FEAST_OK;
+}
+}  // namespace
 
 // ------------------------------------------------------------------ LU
 namespace {
@@ -394,36 +537,6 @@ __global__ void k_laswp_outside(int64_t n, int64_t k0, int nb, T *F, int64_t ldf
     }
 }
 
-// U12 = L11^{-1} A12 for the nb rows of the panel (L11 unit lower), one
-// thread per column in [cbeg, cend).
-template <typename T>
-__global__ void k_trsm_u12(int64_t cbeg, int64_t cend, int64_t k0, int nb, T *F, int64_t ldf, int64_t sF)
-{
-    const int b = blockIdx.y;
-    T *Am = F + (int64_t)b * sF;
-    __shared__ T L[LU_NB][LU_NB + 1];
-    for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-        int r = e % nb, c = e / nb;
-        L[r][c] = Am[(k0 + r) + (k0 + c) * ldf];
-    }
-    __syncthreads();
-    const int64_t c = cbeg + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= cend) return;
-    T x[LU_NB];
-#pragma unroll
-    for (int r = 0; r < LU_NB; ++r)
-        if (r < nb) x[r] = Am[(k0 + r) + c * ldf];
-#pragma unroll
-    for (int i = 0; i < LU_NB; ++i) {
-        if (i >= nb) break;
-#pragma unroll
-        for (int r = i + 1; r < LU_NB; ++r)
-            if (r < nb) cfma(x[r], cneg(L[r][i]), x[i]);
-    }
-#pragma unroll
-    for (int r = 0; r < LU_NB; ++r)
-        if (r < nb) Am[(k0 + r) + c * ldf] = x[r];
-}
 }  // namespace
 
 template <typename T>
@@ -440,9 +553,9 @@ int getrf_batched(cudaStream_t s, int64_t n, int batch, T *F, int64_t ldf, int64
         FEAST_LAUNCH_CHECK();
         int64_t rest = n - k0 - nb;
         if (rest > 0) {
-            k_trsm_u12<T><<<dim3(cdiv(rest, 128), batch), 128, 0, s>>>(k0 + nb, n, k0, nb, F, ldf, sF);
-            FEAST_LAUNCH_CHECK();
-            int e = gemm_batched<T>(s, 0, rest, rest, nb, cx<T>(-1, 0), F + k0 + nb + k0 * ldf,
+            int e = trsv_diag<T>(s, rest, batch, k0, nb, 1, F, ldf, sF, F + (k0 + nb) * ldf, ldf, sF);
+            if (e) return e;
+            e = gemm_batched<T>(s, 0, rest, rest, nb, cx<T>(-1, 0), F + k0 + nb + k0 * ldf,
                                     ldf, sF, F + k0 + (k0 + nb) * ldf, ldf, sF, cx<T>(1, 0),
                                     F + (k0 + nb) + (k0 + nb) * ldf, ldf, sF, batch);
             if (e) return e;
@@ -483,8 +596,7 @@ int getrf_batched_tc(cudaStream_t s, int64_t n, int batch, cf *F, int64_t ldf, i
             if (kend > c1) {
                 // inside the outer block only: columns beyond it keep their
                 // original values (row swaps included) until the block is done
-                k_trsm_u12<cf><<<dim3(cdiv(kend - c1, 128), batch), 128, 0, s>>>(c1, kend, kk, nb, F, ldf, sF);
-                FEAST_LAUNCH_CHECK();
+                if ((e = trsv_diag<cf>(s, kend - c1, batch, kk, nb, 1, F, ldf, sF, F + c1 * ldf, ldf, sF))) return e;
                 if ((e = gemm_batched<cf>(s, 0, n - c1, kend - c1, nb, mone, F + c1 + kk * ldf, ldf, sF,
                                           F + kk + c1 * ldf, ldf, sF, one, F + c1 + c1 * ldf, ldf, sF, batch)))
                     return e;
@@ -495,8 +607,7 @@ int getrf_batched_tc(cudaStream_t s, int64_t n, int batch, cf *F, int64_t ldf, i
         // U12 = L11^{-1} A12 for the columns beyond the block, LU_NB rows at a time
         for (int64_t kk = k0; kk < kend; kk += LU_NB) {
             const int nb = (int)((kend - kk) < LU_NB ? (kend - kk) : LU_NB);
-            k_trsm_u12<cf><<<dim3(cdiv(rest, 128), batch), 128, 0, s>>>(kend, n, kk, nb, F, ldf, sF);
-            FEAST_LAUNCH_CHECK();
+            if ((e = trsv_diag<cf>(s, rest, batch, kk, nb, 1, F, ldf, sF, F + kend * ldf, ldf, sF))) return e;
             const int64_t r1 = kk + nb;
             if (r1 < kend) {
                 if ((e = gemm_batched<cf>(s, 0, kend - r1, rest, nb, mone, F + r1 + kk * ldf, ldf, sF,
@@ -538,52 +649,6 @@ int zgetrf_batched(cudaStream_t s, int64_t n, int batch, zd *F, int64_t ldf, int
 
 // ------------------------------------------------------------------ solves
 namespace {
-constexpr int SV_NB = 32;
-
-// X rows [k0, k0+nb) <- T^{-1} X rows [k0, k0+nb) for the diagonal block T of
-// the factor (lower = unit lower L, else upper U).  One thread per column.
-template <typename C>
-__global__ void k_trsv_diag(int64_t n, int64_t nrhs, int64_t k0, int nb, int lower,
-                            const C *F, int64_t ldf, int64_t sF, C *X, int64_t ldx, int64_t sX)
-{
-    const int b = blockIdx.y;
-    const C *Am = F + (int64_t)b * sF;
-    C *Xb = X + (int64_t)b * sX;
-    __shared__ C T[SV_NB][SV_NB + 1];
-    for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-        int r = e % nb, c = e / nb;
-        T[r][c] = Am[(k0 + r) + (k0 + c) * ldf];
-    }
-    __syncthreads();
-    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= nrhs) return;
-    C x[SV_NB];
-#pragma unroll
-    for (int r = 0; r < SV_NB; ++r)
-        if (r < nb) x[r] = Xb[(k0 + r) + c * ldx];
-    if (lower) {
-#pragma unroll
-        for (int i = 0; i < SV_NB; ++i) {
-            if (i >= nb) break;
-#pragma unroll
-            for (int r = i + 1; r < SV_NB; ++r)
-                if (r < nb) cfma(x[r], cneg(T[r][i]), x[i]);
-        }
-    } else {
-#pragma unroll
-        for (int i = SV_NB - 1; i >= 0; --i) {
-            if (i >= nb) continue;
-            x[i] = cdiv(x[i], T[i][i]);
-#pragma unroll
-            for (int r = 0; r < SV_NB; ++r)
-                if (r < i) cfma(x[r], cneg(T[r][i]), x[i]);
-        }
-    }
-#pragma unroll
-    for (int r = 0; r < SV_NB; ++r)
-        if (r < nb) Xb[(k0 + r) + c * ldx] = x[r];
-}
-
 // Apply the interchanges piv[0..n) to each column of X in sequence.
 template <typename T>
 __global__ void k_laswp_rhs(int64_t n, int64_t nrhs, const int *piv, T *X, int64_t ldx,
@@ -685,15 +750,13 @@ int trsm_lu_tc(cudaStream_t s, int64_t n, int64_t nrhs, int batch, const cf *F, 
     if (n <= 0 || nrhs <= 0 || batch <= 0) return FEAST_OK;
     size_t coff = 0;
     const cf mone = cx<cf>(-1, 0), one = cx<cf>(1, 0);
-    dim3 g(cdiv(nrhs, 64), batch);
     int e;
     // forward: unit lower L
     for (int64_t k0 = 0; k0 < n; k0 += LU_NBO) {
         const int64_t kend = (k0 + LU_NBO < n) ? k0 + LU_NBO : n;
         for (int64_t kk = k0; kk < kend; kk += SV_NB) {
             const int nb = (int)((kend - kk) < SV_NB ? (kend - kk) : SV_NB);
-            k_trsv_diag<cf><<<g, 64, 0, s>>>(n, nrhs, kk, nb, 1, F, ldf, sF, X, ldx, sX);
-            FEAST_LAUNCH_CHECK();
+            if ((e = trsv_diag<cf>(s, nrhs, batch, kk, nb, 1, F, ldf, sF, X, ldx, sX))) return e;
             const int64_t r1 = kk + nb;
             if (r1 < kend &&
                 (e = gemm_batched<cf>(s, 0, kend - r1, nrhs, nb, mone, F + r1 + kk * ldf, ldf, sF, X + kk, ldx, sX,
@@ -719,8 +782,7 @@ int trsm_lu_tc(cudaStream_t s, int64_t n, int64_t nrhs, int batch, const cf *F, 
         const int64_t ilast = k0 + ((kend - k0 - 1) / SV_NB) * SV_NB;
         for (int64_t kk = ilast; kk >= k0; kk -= SV_NB) {
             const int nb = (int)((kend - kk) < SV_NB ? (kend - kk) : SV_NB);
-            k_trsv_diag<cf><<<g, 64, 0, s>>>(n, nrhs, kk, nb, 0, F, ldf, sF, X, ldx, sX);
-            FEAST_LAUNCH_CHECK();
+            if ((e = trsv_diag<cf>(s, nrhs, batch, kk, nb, 0, F, ldf, sF, X, ldx, sX))) return e;
             if (kk > k0 &&
                 (e = gemm_batched<cf>(s, 0, kk - k0, nrhs, nb, mone, F + k0 + kk * ldf, ldf, sF, X + kk, ldx, sX,
                                       one, X + k0, ldx, sX, batch)))
@@ -775,14 +837,13 @@ int trsm_lower_batched(cudaStream_t s, int64_t n, int64_t nrhs, int batch, const
                        int64_t sF, T *X, int64_t ldx, int64_t sX)
 {
     if (n <= 0 || nrhs <= 0 || batch <= 0) return FEAST_OK;
-    dim3 g(cdiv(nrhs, 64), batch);
     for (int64_t k0 = 0; k0 < n; k0 += SV_NB) {
         int nb = (int)((n - k0) < SV_NB ? (n - k0) : SV_NB);
-        k_trsv_diag<T><<<g, 64, 0, s>>>(n, nrhs, k0, nb, 1, F, ldf, sF, X, ldx, sX);
-        FEAST_LAUNCH_CHECK();
+        int e = trsv_diag<T>(s, nrhs, batch, k0, nb, 1, F, ldf, sF, X, ldx, sX);
+        if (e) return e;
         int64_t rest = n - k0 - nb;
         if (rest > 0) {
-            int e = gemm_batched<T>(s, 0, rest, nrhs, nb, cx<T>(-1, 0), F + (k0 + nb) + k0 * ldf,
+            e = gemm_batched<T>(s, 0, rest, nrhs, nb, cx<T>(-1, 0), F + (k0 + nb) + k0 * ldf,
                                     ldf, sF, X + k0, ldx, sX, cx<T>(1, 0), X + k0 + nb, ldx, sX,
                                     batch);
             if (e) return e;
@@ -797,14 +858,13 @@ int trsm_upper_batched(cudaStream_t s, int64_t n, int64_t nrhs, int batch, const
                        int64_t sF, T *X, int64_t ldx, int64_t sX)
 {
     if (n <= 0 || nrhs <= 0 || batch <= 0) return FEAST_OK;
-    dim3 g(cdiv(nrhs, 64), batch);
     int64_t last = ((n - 1) / SV_NB) * SV_NB;
     for (int64_t k0 = last; k0 >= 0; k0 -= SV_NB) {
         int nb = (int)((n - k0) < SV_NB ? (n - k0) : SV_NB);
-        k_trsv_diag<T><<<g, 64, 0, s>>>(n, nrhs, k0, nb, 0, F, ldf, sF, X, ldx, sX);
-        FEAST_LAUNCH_CHECK();
+        int e = trsv_diag<T>(s, nrhs, batch, k0, nb, 0, F, ldf, sF, X, ldx, sX);
+        if (e) return e;
         if (k0 > 0) {
-            int e = gemm_batched<T>(s, 0, k0, nrhs, nb, cx<T>(-1, 0), F + k0 * ldf, ldf, sF,
+            e = gemm_batched<T>(s, 0, k0, nrhs, nb, cx<T>(-1, 0), F + k0 * ldf, ldf, sF,
                                     X + k0, ldx, sX, cx<T>(1, 0), X, ldx, sX, batch);
             if (e) return e;
         }
