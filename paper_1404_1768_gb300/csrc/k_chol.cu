@@ -7,7 +7,7 @@
 // The Gram matrices and the products V R^{-1} are FP64-accurate GEMMs on the
 // tensor cores (k_oz.cu); the triangular inverses are FP64 (recursive
 // doubling), the Cholesky factorisations one cooperative launch each: FP64,
-// or -- the first one, on the digit-sliced path from m = 256 -- FP32 on the
+// or -- the first one, on the digit-sliced path from m = 33 -- FP32 on the
 // unit-diagonal Gram matrix, since the second pass corrects whatever the
 // first leaves.  The first pass leaves Q_1 orthonormal to ~eps cond(V)^2
 // (FP64) or ~2^-24 cond of the scaled Gram matrix (FP32), the second to
@@ -22,7 +22,11 @@ namespace feast {
 namespace {
 
 constexpr int CB = 32;  // Cholesky block
-constexpr int kChol32MinM = 256;      // the FP32 first factorisation from this block width up
+// the FP32 first factorisation from this block width up: a 32-column diagonal
+// block is a chain of FP64 square roots, divisions and a 496-term inverse per
+// thread (~180 us a block; 1.38 ms at m = 192 against 0.24 ms in FP32), and one
+// block alone does not pay for the scaling and the copy of V
+constexpr int kChol32MinM = 33;
 constexpr double kChol32Tol = 1e-4;   // its pivots against the unit diagonal
 constexpr double kSeriesMax = 1e-2;   // largest Gram defect repeated series rounds take on (no R)
 
