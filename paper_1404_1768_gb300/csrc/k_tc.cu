@@ -305,46 +305,62 @@ __global__ void __launch_bounds__(K2_THREADS, 1)
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
 }
 
-// A (m x k complex, column-major, ld) -> head / tail of A' (2m x 2k real,
-// row-major with leading dim ldr), batched.
-__global__ void k_realify_split(int m, int k, const float2 *A, int64_t lda, int64_t sA, float *head,
-                                float *tail, int64_t ldr, int64_t sR)
+__device__ __forceinline__ float tf32_head(float v)
 {
-    const int b = blockIdx.y;
+    return __uint_as_float(__float_as_uint(v) & 0xFFFFE000u);   // truncated: the tail is exact
+}
+
+// A (m x k complex, column-major, ld) -> head / tail of A' (2m x 2k real,
+// row-major with leading dim ldr), batched.  A CTA transposes 32 x 32 complex
+// entries through shared memory, read along A's columns and written along the
+// rows of A' (256 bytes a warp).  HBM-bound: 8 bytes read and 32 written per
+// entry (the form that wrote row by row from a column walk took 169 us for 8 x
+// 1792 x 256, against 22 us of traffic).
+__global__ void __launch_bounds__(256) k_realify_split(int m, int k, const float2 *__restrict__ A, int64_t lda,
+                                                       int64_t sA, float *__restrict__ head, float *__restrict__ tail,
+                                                       int64_t ldr, int64_t sR)
+{
+    __shared__ float2 tile[32][33];
+    const int b = blockIdx.z, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int i0 = blockIdx.x * 32, p0 = blockIdx.y * 32;
     const float2 *Ab = A + (int64_t)b * sA;
-    float *H = head + (int64_t)b * sR, *Tt = tail + (int64_t)b * sR;
-    const int64_t total = (int64_t)m * k;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int i = (int)(e % m), p = (int)(e / m);
-        const float2 a = Ab[i + (int64_t)p * lda];
-        const float v[4] = {a.x, -a.y, a.y, a.x};   // (2i,2p) (2i,2p+1) (2i+1,2p) (2i+1,2p+1)
-        const int64_t o[4] = {(int64_t)(2 * i) * ldr + 2 * p, (int64_t)(2 * i) * ldr + 2 * p + 1,
-                              (int64_t)(2 * i + 1) * ldr + 2 * p, (int64_t)(2 * i + 1) * ldr + 2 * p + 1};
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const float h = __uint_as_float(__float_as_uint(v[t]) & 0xFFFFE000u);  // TF32 head (truncated)
-            H[o[t]] = h;
-            Tt[o[t]] = v[t] - h;
-        }
+    for (int p = w; p < 32; p += 8)
+        if (i0 + lane < m && p0 + p < k) tile[lane][p] = Ab[i0 + lane + (int64_t)(p0 + p) * lda];
+    __syncthreads();
+    if (p0 + lane >= k) return;
+    for (int i = w; i < 32; i += 8) {
+        if (i0 + i >= m) break;
+        const float2 a = tile[i][lane];
+        const float2 h = make_float2(tf32_head(a.x), tf32_head(a.y));
+        const float2 t = make_float2(a.x - h.x, a.y - h.y);
+        const int64_t o = (int64_t)b * sR + (int64_t)(2 * (i0 + i)) * ldr + 2 * (p0 + lane);
+        *(float2 *)(head + o) = make_float2(h.x, -h.y);          // (2i, 2p), (2i, 2p + 1)
+        *(float2 *)(tail + o) = make_float2(t.x, -t.y);
+        *(float2 *)(head + o + ldr) = make_float2(h.y, h.x);     // (2i + 1, ..)
+        *(float2 *)(tail + o + ldr) = make_float2(t.y, t.x);
     }
 }
 
-// X (k x n complex, column-major, ld) -> head / tail (same layout, as reals)
-__global__ void k_split_tf32(int64_t rows2, int n, const float *X, int64_t ldx2, int64_t sX, float *head,
-                             float *tail, int64_t ldh2, int64_t sH)
+// X (k x n complex, column-major, ld) -> head / tail (same layout, as reals): a
+// warp per column, 256 rows of it per CTA row.
+__global__ void __launch_bounds__(256) k_split_tf32(int64_t k, int n, const float2 *__restrict__ X, int64_t ldx,
+                                                    int64_t sX, float *__restrict__ head, float *__restrict__ tail,
+                                                    int64_t ldh2, int64_t sH)
 {
-    const int b = blockIdx.y;
-    const float *Xb = X + (int64_t)b * sX;
-    float *H = head + (int64_t)b * sH, *Tt = tail + (int64_t)b * sH;
-    const int64_t total = rows2 * n;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = e % rows2, c = e / rows2;
-        const float v = Xb[r + c * ldx2];
-        const float h = __uint_as_float(__float_as_uint(v) & 0xFFFFE000u);
-        H[r + c * ldh2] = h;
-        Tt[r + c * ldh2] = v - h;
+    const int b = blockIdx.z, lane = threadIdx.x & 31;
+    const int64_t c = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (c >= n) return;
+    const float2 *x = X + (int64_t)b * sX + c * ldx;
+    float2 *h = (float2 *)(head + (int64_t)b * sH + c * ldh2), *t = (float2 *)(tail + (int64_t)b * sH + c * ldh2);
+    const int64_t r0 = (int64_t)blockIdx.y * 256;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const int64_t r = r0 + 32 * u + lane;
+        if (r >= k) continue;
+        const float2 v = x[r];
+        const float2 hv = make_float2(tf32_head(v.x), tf32_head(v.y));
+        h[r] = hv;
+        t[r] = make_float2(v.x - hv.x, v.y - hv.y);
     }
 }
 
@@ -452,9 +468,8 @@ int tc_prepare_A(cudaStream_t s, int64_t m, int64_t k, const cf *A, int64_t lda,
     const int64_t mr = 2 * m;
     float *Ah = Aprep, *At = Ah + (size_t)batch * mr * kr;
     if (kr != 2 * k) FEAST_CUDA_TRY(cudaMemsetAsync(Ah, 0, sizeof(float) * 2 * (size_t)batch * mr * kr, s));
-    unsigned g = cdiv((size_t)m * k, 256);
-    k_realify_split<<<dim3(g > 4096 ? 4096 : g, batch), 256, 0, s>>>((int)m, (int)k, A, lda, sA, Ah, At, kr,
-                                                                     mr * kr);
+    if (cdiv(k, 32) > 65535 || batch > 65535) return FEAST_EINVAL;
+    k_realify_split<<<dim3(cdiv(m, 32), cdiv(k, 32), batch), 256, 0, s>>>((int)m, (int)k, A, lda, sA, Ah, At, kr, mr * kr);
     FEAST_LAUNCH_CHECK();
     return FEAST_OK;
 }
@@ -471,9 +486,8 @@ int tc_cgemm_prepA(cudaStream_t s, int64_t m, int64_t n, int64_t k, cf alpha, co
     const float *Ah = Aprep, *At = Ah + (size_t)batch * mr * kr;
     float *Xh = scratch, *Xt = Xh + (size_t)batch * kr * n;
     if (kr != 2 * k) FEAST_CUDA_TRY(cudaMemsetAsync(Xh, 0, sizeof(float) * 2 * (size_t)batch * kr * n, s));
-    unsigned g2 = cdiv((size_t)2 * k * n, 256);
-    k_split_tf32<<<dim3(g2 > 4096 ? 4096 : g2, batch), 256, 0, s>>>(2 * k, (int)n, (const float *)X, 2 * ldx,
-                                                                    2 * sX, Xh, Xt, kr, kr * n);
+    if (cdiv(k, 256) > 65535 || batch > 65535) return FEAST_EINVAL;
+    k_split_tf32<<<dim3(cdiv(n, 8), cdiv(k, 256), batch), 256, 0, s>>>(k, (int)n, X, ldx, sX, Xh, Xt, kr, kr * n);
     FEAST_LAUNCH_CHECK();
     CUtensorMap mAh, mAt, mXh, mXt;
     int e;
