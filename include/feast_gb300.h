@@ -433,10 +433,10 @@ int feast_grad_abs2(feast_ctx *right, feast_ctx *left, void *gA, void *gB, int64
  * lda, ldb, ldc).  This is the product of the refinement residual
  * R_j = B V - (z_j B - A) X_j of the precision form (the refinement of the
  * shifted solves of eq. 4.2).  Each row of the real form of A and each
- * column of B is scaled by a power of two and written as 8 base-64 digits;
- * digit products and their sums over K-chunks of 2048 are exact in the
- * tensor cores' FP32 accumulators, and the chunk sums are combined in FP64.
- * Error: about 2^-47 times max_k|A_ik| * max_k|B_kj| * k per entry (not
+ * column of B is scaled by a power of two and written as 7 base-128 digits;
+ * digit products and their sums over K-chunks of 512 are exact in the tensor
+ * cores' FP32 accumulators, and the chunk sums are combined as 64-bit integers.
+ * Error: about 2^-48 times max_k|A_ik| * max_k|B_kj| * k per entry (not
  * relative to |C|).  work: device, >= feast_zgemm_oz_work_bytes bytes, 256-
  * byte aligned (digit planes).  err: device int32, set non-zero (0x400) if
  * a bounded pipeline wait (4 s of device time) gave up (C is then

@@ -521,7 +521,7 @@ int tc_prepare_A(cudaStream_t s, int64_t m, int64_t k, const cf *A, int64_t lda,
 int tc_cgemm_prepA(cudaStream_t s, int64_t m, int64_t n, int64_t k, cf alpha, const float *Aprep, const cf *X,
                    int64_t ldx, int64_t sX, cf beta, cf *C, int64_t ldc, int64_t sC, int batch, float *scratch,
                    int *err, TcTimer *tt = nullptr);
-// FP64-accurate complex GEMM on the bf16 tensor cores by exact base-64
+// FP64-accurate complex GEMM on the bf16 tensor cores by exact base-128
 // digit slicing (k_oz.cu): prepare digit planes of the left operand (rows)
 // and the right operand (columns), then C = beta C + alpha_c A B with
 // alpha_c = alpha * zcol[c / cblk] when zcol is given.

@@ -95,7 +95,7 @@ struct feast_ctx {
     float *tcs;         // tensor-core LU operand scratch (complex64 dense)
     float *tcA;         // the factors' off-block panels as tensor-core operands (made once)
     float4 *Ads, *Xds;  // band A and the solutions as double-single pairs (banded precision form, B = I)
-    void *ozA, *ozB;    // base-64 digit planes of A and B (refinement residual)
+    void *ozA, *ozB;    // base-128 digit planes of A and B (refinement residual)
     void *ozX;          // digit planes of the q solution blocks, n x (q m0); right-operand scratch
     void *ozR;          // left-operand digit planes: U2^H, U1, A U1, B U1 (m0 x n or n x m0)
     OzScratch oz_orth;  // the same scratch, handed to the orthonormalisation

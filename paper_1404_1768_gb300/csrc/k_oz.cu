@@ -7,29 +7,39 @@
 // Complex as real: A' (2M x 2K) has rows 2i = [Re a_ik, -Im a_ik]_k and
 // 2i+1 = [Im a_ik, Re a_ik]_k; B' (2K x N) is B's columns read as
 // interleaved reals.  Every row of A' is scaled by a power of two 2^-e_i so
-// its entries lie in (-1, 1) and written in base 64 with OZ_S signed digits
-// (digit 1 in [-64, 64], later digits in [-32, 32]):
-//     A' = diag(2^e) sum_s 64^-s A_s ,   likewise B' = (sum_t 64^-t B_t) diag(2^f).
+// its entries lie in (-1, 1) and written in base 128 with OZ_S signed digits
+// (digit 1 in [-128, 128], later digits in [-64, 64]):
+//     A' = diag(2^e) sum_s 128^-s A_s ,   likewise B' = (sum_t 128^-t B_t) diag(2^f).
 // Digits are small integers, exact in bf16, and a digit product is exact in
 // the FP32 accumulator; so is any sum of products of one weight class
-// g = s + t over a K-chunk of OZ_KC terms while it stays below 2^24 (the
-// leading classes always do; a late class can pass it only by a factor
-// ~1.3 at worst, and rounds then at a weight below 2^-60).  The kernel keeps
-// one tensor-memory accumulator per class g = 2..9 (all products with
-// s + t <= OZ_S + 1; the rest weigh < 2^-60), reads the classes out after
-// each K-chunk, combines them on the integer pipe into two exact int64
-// partials and adds acc += sum_g 64^-(g-2) S_g in FP64 with two roundings;
-// finally C gets alpha_c 2^(e_i + f_j - 12) acc.
-// Representation and truncation error: ~2^-48 relative to
+// g = s + t over a K-chunk of OZ_KC terms while it stays below 2^24 (all but
+// the last class always do; it can pass it only by a factor 1.13 at worst, and
+// rounds then at a weight below 2^-60).  The kernel keeps one tensor-memory
+// accumulator per class g = 2..8 (all products with s + t <= OZ_S + 1; the
+// rest weigh < 2^-50), reads the classes out after each K-chunk and adds them
+// on the integer pipe into two exact int64 sums per entry,
+//     hi = sum_(g<=5) 128^(5-g) S_g ,   lo = sum_(g>=6) 128^(8-g) S_g ;
+// FP64 enters once per entry, at the end: C gets alpha_c 2^(e_i + f_j - 14)
+// 2^-21 (hi + 2^-21 lo).  Integer sums do not depend on their order, so K is
+// split over the CTAs of a cluster where the tiles do not fill the GPU evenly,
+// with the same result.
+// Representation and truncation error: ~2^-49 relative to
 // max_k |A'_ik| * max_k |B'_kj| per entry, K-fold at most.
 //
-// Per CTA: one 128 x 64 tile of A'B'.  Warp 4 (one lane) streams K-stages of
-// 32 bf16 (64-byte swizzle rows) of all OZ_S slices of both operands with
-// TMA into a two-deep ring; warp 5 (one lane) issues the 36 slice products
-// per K-step of 16 into the eight accumulators (8 x 64 = all 512 TMEM
-// columns) and commits each stage and each K-chunk; warps 0-3 own TMEM
-// lanes 0-127 and run the chunk read-outs and the final write.  All waits
-// are bounded; on expiry the CTA raises *err and finishes.
+// Seven base-128 digits are 28 slice products and 49 bits; the eight base-64
+// digits before them were 36 products and 48 bits, with an FP64 sum per chunk
+// that the shorter chunks (512 instead of 2048 terms) would have made a third
+// of the time: an FP64 instruction takes 64 clocks of an SM quarter here.
+//
+// Per CTA: one 128 x 64 tile of A'B' over its share of K.  Warp 8 (one lane)
+// streams K-stages of 32 bf16 (64-byte swizzle rows) of all OZ_S slices of both
+// operands with TMA into a two-deep ring; warp 9 (one lane) issues the 28 slice
+// products per K-step of 16 into the seven accumulators (7 x 64 TMEM columns)
+// and commits each stage and each K-chunk; warps 0-7 read the chunks out (TMEM
+// lane quarter = warp % 4, columns 0-31 or 32-63) and write the result.  What
+// bounds it: shared-memory reads of the A slices (4 KB per 128 x 64 x 16
+// product, 48 clocks for 32 of MMA).  All waits are bounded; on expiry the CTA
+// raises *err and finishes.
 #include "tcgen05.cuh"
 
 namespace feast {
@@ -37,31 +47,28 @@ namespace feast {
 namespace {
 using namespace tc;
 
-constexpr int OZ_S = 8;                      // digits per operand entry
+constexpr int OZ_S = 7;                      // digits per operand entry
+constexpr int OZ_BITS = 7;                   // base 128
 constexpr int OZ_NG = OZ_S;                  // weight classes g = 2 .. OZ_S + 1
 constexpr int OZ_BM = 128;                   // rows of A' per tile
 constexpr int OZ_BN = 64;                    // columns per tile
 constexpr int OZ_BK = 32;                    // bf16 per stage row (64 bytes)
 constexpr int OZ_STAGES = 2;
-constexpr int OZ_KC = 2048;                  // K per exact chunk (real K)
+constexpr int OZ_KC = 512;                   // K per exact chunk (real K)
 constexpr int OZ_GM = 8;                     // row tiles per raster group
-constexpr int OZ_THREADS = 192;
+constexpr int OZ_READ = 256;                 // read-out threads
+constexpr int OZ_THREADS = OZ_READ + 64;
+constexpr int OZ_SMAX = 8;                   // most CTAs that share a tile's K
 constexpr int OZ_A_TILE = OZ_BM * OZ_BK * 2; // 8 KiB per slice
 constexpr int OZ_B_TILE = OZ_BN * OZ_BK * 2; // 4 KiB per slice
 constexpr int OZ_STAGE = OZ_S * (OZ_A_TILE + OZ_B_TILE);
+static_assert(OZ_STAGES * OZ_STAGE >= OZ_BM * OZ_BN * 16, "the int64 sums of a tile reuse the ring");
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
 {
-    // exact: |digit| <= 64
+    // exact: |digit| <= 128
     const uint32_t a = __float_as_uint(lo) >> 16, b = __float_as_uint(hi) >> 16;
     return a | (b << 16);
-}
-
-// x as a double, exactly, for |x| < 2^51: 1.5 2^52 + x has x in its low
-// significand bits
-__device__ __forceinline__ double exact_double(long long x)
-{
-    return __longlong_as_double(x + 0x4338000000000000LL) - 6755399441055744.0;
 }
 
 // A row or column with an Inf or NaN entry: its products are NaN (its
@@ -79,6 +86,14 @@ __device__ __forceinline__ void fold_mag(zd v, unsigned long long &mx, bool &bad
     mx = m > mx ? m : mx;
 }
 
+// The exponent e with |x| < 2^e for the magnitude bits of x (0 for zero).
+__device__ __forceinline__ int exponent_of(unsigned long long mx)
+{
+    if (mx == 0) return 0;
+    const int bexp = (int)(mx >> 52);
+    return bexp ? bexp - 1022 : 64 - __clzll((long long)mx) - 1074;   // (subnormal)
+}
+
 // Warp-wide: the exponent e with max < 2^e (frexp's; 0 for zero), or
 // OZ_NONFINITE, in every lane.
 __device__ __forceinline__ int warp_exponent(unsigned long long mx, bool bad)
@@ -89,28 +104,36 @@ __device__ __forceinline__ int warp_exponent(unsigned long long mx, bool bad)
         mx = o > mx ? o : mx;
     }
     if (__any_sync(0xffffffffu, bad)) return OZ_NONFINITE;
-    if (mx == 0) return 0;
-    const int bexp = (int)(mx >> 52);
-    return bexp ? bexp - 1022 : 64 - __clzll((long long)mx) - 1074;   // (subnormal max)
+    return exponent_of(mx);
 }
 
-// e_i with max_k max(|Re a_ik|, |Im a_ik|) < 2^e_i (0 for a zero row); one
-// warp per row.  ct: the operand is the conjugate transpose of the stored
-// matrix, a_ik = conj(A[k + i lda]).
-__global__ void k_oz_rowexp(int64_t M, int64_t K, const zd *__restrict__ A, int64_t lda, int ct,
-                            int *__restrict__ e)
+// e_i with max_k max(|Re a_ik|, |Im a_ik|) < 2^e_i (0 for a zero row).  32 rows
+// per CTA, lane = row, the warps share K: reads run along the stored columns.
+constexpr int RE_W = 16;
+__global__ void __launch_bounds__(32 * RE_W) k_oz_rowexp(int64_t M, int64_t K, const zd *__restrict__ A, int64_t lda,
+                                                         int *__restrict__ e)
 {
-    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (i >= M) return;
+    __shared__ unsigned long long smx[RE_W][32];
+    __shared__ int sbad[RE_W][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t i = (int64_t)blockIdx.x * 32 + lane;
     unsigned long long mx = 0;
     bool bad = false;
-    for (int64_t k = lane; k < K; k += 32) fold_mag(ct ? A[k + i * lda] : A[i + k * lda], mx, bad);
-    const int ex = warp_exponent(mx, bad);
-    if (lane == 0) e[i] = ex;
+    if (i < M)
+        for (int64_t k = w; k < K; k += RE_W) fold_mag(A[i + k * lda], mx, bad);
+    smx[w][lane] = mx;
+    sbad[w][lane] = bad;
+    __syncthreads();
+    if (w != 0 || i >= M) return;
+    for (int x = 1; x < RE_W; ++x) {
+        mx = smx[x][lane] > mx ? smx[x][lane] : mx;
+        bad = bad || sbad[x][lane];
+    }
+    e[i] = bad ? OZ_NONFINITE : exponent_of(mx);
 }
 
-// f_j for column j of B (one warp per column).
+// f_j for column j of B (one warp per column); also e_j of a conjugate-
+// transposed left operand, whose rows are stored columns.
 __global__ void k_oz_colexp(int64_t K, int64_t N, const zd *__restrict__ B, int64_t ldb, int *__restrict__ f)
 {
     const int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -124,9 +147,9 @@ __global__ void k_oz_colexp(int64_t K, int64_t N, const zd *__restrict__ B, int6
 }
 
 // Digits of one real value v (IEEE bits b) scaled by 2^-e into (-1, 1):
-// with N_s = rint(64^s v 2^-e) (round half to even), digit s is
-// N_s - 64 N_(s-1) -- the same digits as the recursion t = 64 r, d = rint(t),
-// r = t - d, whose steps are all exact (a subtracted multiple of 64 is even,
+// with N_s = rint(128^s v 2^-e) (round half to even), digit s is
+// N_s - 128 N_(s-1) -- the same digits as the recursion t = 128 r, d = rint(t),
+// r = t - d, whose steps are all exact (a subtracted multiple of 128 is even,
 // so it commutes with the rounding).  Each N_s comes from the 53-bit
 // significand by an integer shift with round-half-even, so the slicing runs
 // on the integer pipe, not the FP64 one (1/64 of the FP32 rate on this part),
@@ -141,7 +164,7 @@ __device__ __forceinline__ void digits(unsigned long long b, int e, float (&d)[O
     long long prev = 0;
 #pragma unroll
     for (int s = 1; s <= OZ_S; ++s) {
-        const int rs = -(base + 6 * s);
+        const int rs = -(base + OZ_BITS * s);
         unsigned long long q;
         if (rs <= 0) {
             q = mant << (-rs);                       // (a subnormal row: no bits below the point)
@@ -153,55 +176,72 @@ __device__ __forceinline__ void digits(unsigned long long b, int e, float (&d)[O
             q += (rem > half || (rem == half && (q & 1))) ? 1ull : 0ull;
         }
         const long long N = neg ? -(long long)q : (long long)q;
-        d[s - 1] = (float)(int)(N - 64 * prev);      // |digit| <= 64: exact
+        d[s - 1] = (float)(int)(N - (prev << OZ_BITS));   // |digit| <= 128: exact
         prev = N;
     }
 }
 
-// A' digit planes: plane s is (2M x kp) bf16, row-major; thread per
-// (real row, complex column).  Columns K .. kp/2 - 1 are zero padding.
-__global__ void k_oz_slice_rows(int64_t M, int64_t K, const zd *__restrict__ A, int64_t lda, int ct,
-                                const int *__restrict__ e, uint32_t *__restrict__ planes, int64_t kp)
+// A' digit planes: plane s is (2M x kp) bf16, row-major, columns K .. kp/2 - 1
+// zero padding.  A CTA takes 32 rows x 32 complex columns of A through shared
+// memory, read along the stored columns and written along the rows; an entry's
+// digits serve both of its rows (those of -x are the negatives).  HBM-bound:
+// 16 bytes read and 56 written per entry (at 2048 x 2048 the thread-per-row
+// form, whose reads strode through A, took 184 us).
+__global__ void __launch_bounds__(256) k_oz_slice_rows(int64_t M, int64_t K, const zd *__restrict__ A, int64_t lda,
+                                                       int ct, const int *__restrict__ e,
+                                                       uint32_t *__restrict__ planes, int64_t kp)
 {
-    const int64_t half = kp / 2;
-    const int64_t total = 2 * M * half;
-    const int64_t plane = 2 * M * kp / 2;   // in 32-bit words
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < total;
-         x += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t rr = x / half, kc = x % half;
-        const int64_t i = rr >> 1;
-        float d0[OZ_S], d1[OZ_S];
+    __shared__ zd tile[32][33];
+    const int64_t half = kp / 2, plane = M * kp;   // in 32-bit words
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t i0 = (int64_t)blockIdx.x * 32, k0 = (int64_t)blockIdx.y * 32;
+    for (int r = w; r < 32; r += 8) {
+        const int64_t a = ct ? k0 + lane : i0 + lane, b = ct ? i0 + r : k0 + r;   // stored row, column
+        const bool in = ct ? (a < K && b < M) : (a < M && b < K);
+        zd v = in ? A[a + b * lda] : zmake(0.0, 0.0);
+        if (ct) tile[r][lane] = zconj(v);
+        else tile[lane][r] = v;
+    }
+    __syncthreads();
+    const int64_t kc = k0 + lane;
+    if (kc >= half) return;
+    for (int r = w; r < 32; r += 8) {
+        const int64_t i = i0 + r;
+        if (i >= M) break;
         const int ei = e[i];
+        float dr[OZ_S], di[OZ_S];
         if (kc < K && ei != OZ_NONFINITE) {
-            const zd v = ct ? A[kc + i * lda] : A[i + kc * lda];
-            const unsigned long long sgn = 1ull << 63;
-            const unsigned long long a = (unsigned long long)__double_as_longlong(v.x);
-            const unsigned long long b = (unsigned long long)__double_as_longlong(v.y) ^ (ct ? sgn : 0ull);
-            if ((rr & 1) == 0) { digits(a, ei, d0); digits(b ^ sgn, ei, d1); }
-            else { digits(b, ei, d0); digits(a, ei, d1); }
+            const zd v = tile[r][lane];
+            digits((unsigned long long)__double_as_longlong(v.x), ei, dr);
+            digits((unsigned long long)__double_as_longlong(v.y), ei, di);
         } else {
 #pragma unroll
-            for (int s = 0; s < OZ_S; ++s) { d0[s] = 0.f; d1[s] = 0.f; }
+            for (int s = 0; s < OZ_S; ++s) { dr[s] = 0.f; di[s] = 0.f; }
         }
-        const int64_t o = rr * half + kc;
+        const int64_t o = 2 * i * half + kc;
 #pragma unroll
-        for (int s = 0; s < OZ_S; ++s) planes[(int64_t)s * plane + o] = pack_bf16x2(d0[s], d1[s]);
+        for (int s = 0; s < OZ_S; ++s) {
+            planes[(int64_t)s * plane + o] = pack_bf16x2(dr[s], -di[s]);
+            planes[(int64_t)s * plane + o + half] = pack_bf16x2(di[s], dr[s]);
+        }
     }
 }
 
 // B' digit planes: plane s is (N x kp) bf16, row j = column j of B as
-// interleaved reals; thread per (column, complex row).
-__global__ void k_oz_slice_cols(int64_t K, int64_t N, const zd *__restrict__ B, int64_t ldb,
-                                const int *__restrict__ f, uint32_t *__restrict__ planes, int64_t kp)
+// interleaved reals; a warp per column.
+__global__ void __launch_bounds__(256) k_oz_slice_cols(int64_t K, int64_t N, const zd *__restrict__ B, int64_t ldb,
+                                                       const int *__restrict__ f, uint32_t *__restrict__ planes,
+                                                       int64_t kp)
 {
     const int64_t half = kp / 2;
-    const int64_t total = N * half;
     const int64_t plane = N * half;
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < total;
-         x += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = x / half, kc = x % half;
+    const int lane = threadIdx.x & 31;
+    const int64_t j = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (j >= N) return;
+    const int fj = f[j];
+    const int64_t k1 = ((int64_t)blockIdx.y + 1) * 256 < half ? ((int64_t)blockIdx.y + 1) * 256 : half;
+    for (int64_t kc = (int64_t)blockIdx.y * 256 + lane; kc < k1; kc += 32) {
         float d0[OZ_S], d1[OZ_S];
-        const int fj = f[j];
         if (kc < K && fj != OZ_NONFINITE) {
             const zd v = B[kc + j * ldb];
             digits((unsigned long long)__double_as_longlong(v.x), fj, d0);
@@ -211,7 +251,7 @@ __global__ void k_oz_slice_cols(int64_t K, int64_t N, const zd *__restrict__ B, 
             for (int s = 0; s < OZ_S; ++s) { d0[s] = 0.f; d1[s] = 0.f; }
         }
 #pragma unroll
-        for (int s = 0; s < OZ_S; ++s) planes[(int64_t)s * plane + x] = pack_bf16x2(d0[s], d1[s]);
+        for (int s = 0; s < OZ_S; ++s) planes[(int64_t)s * plane + j * half + kc] = pack_bf16x2(d0[s], d1[s]);
     }
 }
 
@@ -224,9 +264,27 @@ struct OzOut {
     zd beta;
 };
 
+__device__ __forceinline__ void oz_cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// 64-bit word at p's place in the shared memory of CTA rank of the cluster.
+__device__ __forceinline__ long long oz_peer(const long long *p, int rank)
+{
+    uint32_t a;
+    long long v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+    asm volatile("ld.shared::cluster.s64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
+    return v;
+}
+
+// splits CTAs (a cluster, 1 to OZ_SMAX) share a tile: CTA r takes K-blocks
+// [r kbs, (r + 1) kbs), then finishes 64 / splits of the tile's columns from
+// all of their sums.
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     k_oz_gemm(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tB, int mr, int n,
-              int kr, const int *__restrict__ ea, const int *__restrict__ fb, OzOut out, int *err)
+              int kr, int splits, int kbs, const int *__restrict__ ea, const int *__restrict__ fb, OzOut out,
+              int *err)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *base = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -235,16 +293,19 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     __shared__ int s_fail;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = splits > 1 ? (int)(blockIdx.x % splits) : 0;
     // raster: OZ_GM row tiles side by side share each column tile's operands in L2
     const int Mt = (mr + OZ_BM - 1) / OZ_BM, Nt = (n + OZ_BN - 1) / OZ_BN;
-    const int L = blockIdx.x;
+    const int L = blockIdx.x / splits;
     const int grp = L / (OZ_GM * Nt);
     const int gbase = grp * OZ_GM;
     const int gsz = (Mt - gbase) < OZ_GM ? (Mt - gbase) : OZ_GM;
     const int rem = L - grp * OZ_GM * Nt;
     const int rt = gbase + rem % gsz, ct = rem / gsz;
     const int row0 = rt * OZ_BM, col0 = ct * OZ_BN;
-    const int kb_n = (kr + OZ_BK - 1) / OZ_BK;
+    const int kb_all = (kr + OZ_BK - 1) / OZ_BK, kb0 = rank * kbs;
+    int kb_n = kb_all - kb0 < kbs ? kb_all - kb0 : kbs;    // this CTA's K-blocks (maybe none)
+    if (kb_n < 0) kb_n = 0;
     constexpr int KB_CHUNK = OZ_KC / OZ_BK;
     const int nchunk = (kb_n + KB_CHUNK - 1) / KB_CHUNK;
 
@@ -254,7 +315,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             mbar_init(&empty[s], 1);
         }
         mbar_init(&chunk_full, 1);
-        mbar_init(&tmem_empty, 128);
+        mbar_init(&tmem_empty, OZ_READ);
         s_fail = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -268,8 +329,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = tmem_base;
+    // the read-out threads' exact sums: 32 columns each
+    long long hi[32], lo[32];
 
-    if (warp == 4) {
+    if (warp == OZ_READ / 32) {
         if (lane == 0) {
             // producer
             int issued = 0;
@@ -279,7 +342,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                 if (!mbar_wait(&empty[s], ph ^ 1u) || *(volatile int *)&s_fail) { s_fail = 1; break; }
                 unsigned char *st = base + s * OZ_STAGE;
                 mbar_expect_tx(&full[s], OZ_STAGE);
-                const int kx = kb * OZ_BK;
+                const int kx = (kb0 + kb) * OZ_BK;
 #pragma unroll 1
                 for (int sl = 0; sl < OZ_S; ++sl) {
                     tma_load_3d(st + sl * OZ_A_TILE, &tA, &full[s], kx, row0, sl);
@@ -292,7 +355,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                 for (int kb = (issued > OZ_STAGES ? issued - OZ_STAGES : 0); kb < issued; ++kb)
                     mbar_wait(&full[kb % OZ_STAGES], (uint32_t)((kb / OZ_STAGES) & 1));
         }
-    } else if (warp == 5) {
+    } else if (warp == OZ_READ / 32 + 1) {
         if (lane == 0) {
             constexpr uint32_t idesc = idesc_f32acc(1u, OZ_BM, OZ_BN);
             bool ok = true;
@@ -309,10 +372,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                 if (!mbar_wait(&full[s], ph) || *(volatile int *)&s_fail) { ok = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;");
                 unsigned char *st = base + s * OZ_STAGE;
-                const uint32_t a0 = smem_u32(st), b0 = smem_u32(st + OZ_S * OZ_A_TILE);
                 const uint64_t adesc = sdesc<64>(st), bdesc = sdesc<64>(st + OZ_S * OZ_A_TILE);
-                (void)a0;
-                (void)b0;
 #pragma unroll
                 for (int kk = 0; kk < OZ_BK / 16; ++kk) {
 #pragma unroll
@@ -333,103 +393,119 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             if (!ok) s_fail = 1;
         }
     } else {
-        // read-out warps 0-3: TMEM lanes 32 * warp ..
-        double acc[OZ_BN];
+        // read-out: TMEM lanes 32 (warp % 4) .., columns 32 (warp / 4) ..
 #pragma unroll
-        for (int j = 0; j < OZ_BN; ++j) acc[j] = 0.0;
-        bool good = true;
+        for (int j = 0; j < 32; ++j) hi[j] = lo[j] = 0;
+        const uint32_t tw = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * 32);
+        static_assert(OZ_NG == 7, "the read-out takes seven weight classes");
         for (int c = 0; c < nchunk; ++c) {
-            if (!mbar_wait(&chunk_full, (uint32_t)(c & 1)) || *(volatile int *)&s_fail) { good = false; break; }
+            if (!mbar_wait(&chunk_full, (uint32_t)(c & 1)) || *(volatile int *)&s_fail) {
+                if (lane == 0) s_fail = 1;
+                break;
+            }
             asm volatile("tcgen05.fence::after_thread_sync;");
-            // acc += sum_g 64^-g S_g = 2^-18 (hi + 2^-24 lo) with the exact
-            // integers hi = sum_(g<4) 64^(3-g) S_g, lo = sum_(g>=4) 64^(7-g) S_g
-            // (|hi|, |lo| < 2^45): two roundings per chunk instead of eight,
-            // and the class sums combined on the integer pipe
-            static_assert(OZ_NG == 8, "the read-out pairs eight weight classes");
-            const uint32_t tw = tmem + ((uint32_t)(warp * 32) << 16);
 #pragma unroll
-            for (int cg = 0; cg < OZ_BN / 8; ++cg) {
-                int p[4][8];   // p_q = 64 S_2q + S_(2q+1) (|p_q| < 2^31)
+            for (int cg = 0; cg < 4; ++cg) {
+                uint32_t va[8], vb[8];
+                int p01[8], p23[8], p45[8];
+                // p = 128 S_g + S_(g+1) fits 32 bits for the first four classes
+                // (|S| <= 1.5 2^23, and 1.25 2^23 for the one scaled up)
+                tmem_ld8x2(tw + (uint32_t)(0 * OZ_BN + cg * 8), tw + (uint32_t)(1 * OZ_BN + cg * 8), va, vb);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    uint32_t va[8], vb[8];
-                    tmem_ld8x2(tw + (uint32_t)(2 * q * OZ_BN + cg * 8), tw + (uint32_t)((2 * q + 1) * OZ_BN + cg * 8),
-                               va, vb);
-#pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        p[q][j] = __float2int_rn(__uint_as_float(va[j])) * 64 + __float2int_rn(__uint_as_float(vb[j]));
-                }
+                for (int j = 0; j < 8; ++j)
+                    p01[j] = __float2int_rn(__uint_as_float(va[j])) * 128 + __float2int_rn(__uint_as_float(vb[j]));
+                tmem_ld8x2(tw + (uint32_t)(2 * OZ_BN + cg * 8), tw + (uint32_t)(3 * OZ_BN + cg * 8), va, vb);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    const long long hi = (long long)p[0][j] * 4096 + p[1][j];
-                    const long long lo = (long long)p[2][j] * 4096 + p[3][j];
-                    const double t = fma(exact_double(lo), 0x1p-24, exact_double(hi));
-                    acc[cg * 8 + j] = fma(t, 0x1p-18, acc[cg * 8 + j]);
+                    p23[j] = __float2int_rn(__uint_as_float(va[j])) * 128 + __float2int_rn(__uint_as_float(vb[j]));
+                    hi[cg * 8 + j] += (long long)p01[j] * 16384 + p23[j];
                 }
+                tmem_ld8x2(tw + (uint32_t)(4 * OZ_BN + cg * 8), tw + (uint32_t)(5 * OZ_BN + cg * 8), va, vb);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    lo[cg * 8 + j] += (long long)__float2int_rn(__uint_as_float(va[j])) * 16384;
+                    p45[j] = __float2int_rn(__uint_as_float(vb[j]));
+                }
+                tmem_ld8x2(tw + (uint32_t)(6 * OZ_BN + cg * 8), tw + (uint32_t)(6 * OZ_BN + cg * 8), va, vb);
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    lo[cg * 8 + j] += (long long)p45[j] * 128 + __float2int_rn(__uint_as_float(va[j]));
             }
             asm volatile("tcgen05.fence::before_thread_sync;");
             mbar_arrive(&tmem_empty);
         }
-        if (!good) {
-            if (lane == 0) s_fail = 1;
-        } else {
-            const int r = row0 + warp * 32 + lane;           // real row
-            const bool im_row = (r & 1) != 0;
-            const int64_t ci = r >> 1;
-            const int er = (r < mr) ? ea[ci] : 0;
-            // pair the Re / Im rows (neighbouring lanes); the even lane writes
-            // columns 0..31 of the tile, the odd lane 32..63, eight at a time
-            // with the old values loaded first
-            const int hsel = im_row ? 1 : 0;
-            const bool rd = (out.beta.x != 0.0 || out.beta.y != 0.0);
-            // (a real alpha and a unit beta, the common cases, skip the complex products)
-            const bool real_alpha = out.zcol == nullptr && out.alpha.y == 0.0;
-            const bool unit_beta = out.beta.x == 1.0 && out.beta.y == 0.0;
-#pragma unroll
-            for (int g8 = 0; g8 < OZ_BN / 2; g8 += 8) {
-                zd d[8], o[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const double m0v = acc[g8 + i], m1v = acc[32 + g8 + i];
-                    const double o0 = __shfl_xor_sync(0xffffffffu, m0v, 1);
-                    const double o1 = __shfl_xor_sync(0xffffffffu, m1v, 1);
-                    const double mine = hsel ? m1v : m0v, other = hsel ? o1 : o0;
-                    d[i] = zmake(im_row ? other : mine, im_row ? mine : other);
-                }
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int col = col0 + hsel * 32 + g8 + i;
-                    o[i] = (rd && r < mr && col < n) ? out.C[ci + (int64_t)col * out.ldc] : zmake(0.0, 0.0);
-                }
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int col = col0 + hsel * 32 + g8 + i;
-                    if (r < mr && col < n && (er == OZ_NONFINITE || fb[col] == OZ_NONFINITE)) {
-                        out.C[ci + (int64_t)col * out.ldc] = zmake(__longlong_as_double(0x7ff8000000000000LL),
-                                                                   __longlong_as_double(0x7ff8000000000000LL));
-                    } else if (r < mr && col < n) {
-                        // d 2^(e_i + f_j - 12): a power of two built from its bits, or
-                        // (a result near the ends of the range) ldexp, one rounding
-                        const int ex = er + fb[col] - 12;
-                        zd res = (ex >= -1022 && ex <= 1023)
-                                     ? zscale(d[i], __longlong_as_double((long long)(ex + 1023) << 52))
-                                     : zmake(ldexp(d[i].x, ex), ldexp(d[i].y, ex));
-                        if (real_alpha) {
-                            if (out.alpha.x != 1.0) res = zscale(res, out.alpha.x);
-                        } else {
-                            zd al = out.alpha;
-                            if (out.zcol) al = zmul(al, out.zcol[col / out.cblk]);
-                            res = zmul(al, res);
-                        }
-                        if (rd) res = zadd(res, unit_beta ? o[i] : zmul(out.beta, o[i]));
-                        out.C[ci + (int64_t)col * out.ldc] = res;
-                    }
-                }
-            }
-        }
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();   // every copy has landed and every MMA is done: the ring is free
+    // sums[(2 column + {hi, lo}) * 128 + row]
+    long long *sums = (long long *)base;
+    const int quarter = warp & 3, half = warp >> 2;
+    if (threadIdx.x < OZ_READ) {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+            long long *q = sums + (size_t)(2 * (half * 32 + j)) * OZ_BM + quarter * 32 + lane;
+            q[0] = hi[j];
+            q[OZ_BM] = lo[j];
+        }
+    }
+    if (splits > 1) oz_cluster_sync();
+    else __syncthreads();
+    if (threadIdx.x < OZ_READ && !s_fail) {
+        const int r = row0 + quarter * 32 + lane;            // real row
+        const bool im_row = (r & 1) != 0;
+        const int64_t ci = r >> 1;
+        const int er = (r < mr) ? ea[ci] : 0;
+        const int cw = OZ_BN / splits;                       // columns of this CTA
+        const bool rd = (out.beta.x != 0.0 || out.beta.y != 0.0);
+        // (a real alpha and a unit beta, the common cases, skip the complex products)
+        const bool real_alpha = out.zcol == nullptr && out.alpha.y == 0.0;
+        const bool unit_beta = out.beta.x == 1.0 && out.beta.y == 0.0;
+        // two columns at a time: neighbouring lanes hold the Re and Im rows of
+        // one complex row; the even lane finishes the first column, the odd the
+        // second
+        for (int c2 = rank * cw + half * (cw / 2); c2 < rank * cw + half * (cw / 2) + cw / 2; c2 += 2) {
+            double v[2];
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                const long long *q = sums + (size_t)(2 * (c2 + t)) * OZ_BM + quarter * 32 + lane;
+                long long h = q[0], l = q[OZ_BM];
+                for (int x = 1; x < splits; ++x) {
+                    const int pr = (rank + x) % splits;
+                    h += oz_peer(q, pr);
+                    l += oz_peer(q + OZ_BM, pr);
+                }
+                v[t] = fma((double)l, 0x1p-21, (double)h);
+            }
+            const double o0 = __shfl_xor_sync(0xffffffffu, v[0], 1);
+            const double o1 = __shfl_xor_sync(0xffffffffu, v[1], 1);
+            const zd d = im_row ? zmake(o1, v[1]) : zmake(v[0], o0);
+            const int col = col0 + c2 + (im_row ? 1 : 0);
+            if (r >= mr || col >= n) continue;
+            zd &C = out.C[ci + (int64_t)col * out.ldc];
+            const int fc = fb[col];
+            if (er == OZ_NONFINITE || fc == OZ_NONFINITE) {
+                C = zmake(__longlong_as_double(0x7ff8000000000000LL), __longlong_as_double(0x7ff8000000000000LL));
+                continue;
+            }
+            // d 2^(e_i + f_j - 35): a power of two built from its bits, or (a
+            // result near the ends of the range) ldexp, one rounding
+            const int ex = er + fc - 35;
+            zd res = (ex >= -1022 && ex <= 1023)
+                         ? zscale(d, __longlong_as_double((long long)(ex + 1023) << 52))
+                         : zmake(ldexp(d.x, ex), ldexp(d.y, ex));
+            if (real_alpha) {
+                if (out.alpha.x != 1.0) res = zscale(res, out.alpha.x);
+            } else {
+                zd al = out.alpha;
+                if (out.zcol) al = zmul(al, out.zcol[col / out.cblk]);
+                res = zmul(al, res);
+            }
+            if (rd) res = zadd(res, unit_beta ? C : zmul(out.beta, C));
+            C = res;
+        }
+    }
     __syncthreads();
+    if (splits > 1) oz_cluster_sync();   // no CTA leaves while a peer reads its sums
     if (threadIdx.x == 0 && s_fail) atomicOr(err, TO_OZ);
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
 }
@@ -449,11 +525,11 @@ int oz_prepare_rows(cudaStream_t s, int64_t M, int64_t K, const zd *A, int64_t l
     const int64_t kp = oz_kp(K);
     uint32_t *planes = (uint32_t *)work;
     int *e = (int *)((char *)work + (size_t)OZ_S * 2 * M * kp * 2 + 256);
-    k_oz_rowexp<<<cdiv((size_t)M * 32, 256), 256, 0, s>>>(M, K, A, lda, ct, e);
+    if (ct) k_oz_colexp<<<cdiv((size_t)M * 32, 256), 256, 0, s>>>(K, M, A, lda, e);
+    else k_oz_rowexp<<<cdiv((size_t)M, 32), 32 * RE_W, 0, s>>>(M, K, A, lda, e);
     FEAST_LAUNCH_CHECK();
-    const int64_t total = 2 * M * (kp / 2);
-    k_oz_slice_rows<<<cdiv(total, 256) > 16384 ? 16384 : cdiv(total, 256), 256, 0, s>>>(M, K, A, lda, ct, e, planes,
-                                                                                         kp);
+    if (cdiv((size_t)kp / 2, 32) > 65535) return FEAST_EINVAL;
+    k_oz_slice_rows<<<dim3(cdiv((size_t)M, 32), cdiv((size_t)kp / 2, 32)), 256, 0, s>>>(M, K, A, lda, ct, e, planes, kp);
     FEAST_LAUNCH_CHECK();
     return FEAST_OK;
 }
@@ -467,8 +543,8 @@ int oz_prepare_cols(cudaStream_t s, int64_t K, int64_t N, const zd *B, int64_t l
     int *f = (int *)((char *)work + (size_t)OZ_S * N * kp * 2 + 256);
     k_oz_colexp<<<cdiv((size_t)N * 32, 256), 256, 0, s>>>(K, N, B, ldb, f);
     FEAST_LAUNCH_CHECK();
-    const int64_t total = N * (kp / 2);
-    k_oz_slice_cols<<<cdiv(total, 256) > 16384 ? 16384 : cdiv(total, 256), 256, 0, s>>>(K, N, B, ldb, f, planes, kp);
+    if (cdiv((size_t)kp / 2, 256) > 65535) return FEAST_EINVAL;
+    k_oz_slice_cols<<<dim3(cdiv((size_t)N, 8), cdiv((size_t)kp / 2, 256)), 256, 0, s>>>(K, N, B, ldb, f, planes, kp);
     FEAST_LAUNCH_CHECK();
     return FEAST_OK;
 }
@@ -495,8 +571,37 @@ int oz_gemm(cudaStream_t s, int64_t M, int64_t N, int64_t K, const void *Arows, 
     FEAST_CUDA_TRY(allow_dyn_smem(k_oz_gemm));
     const int64_t tiles = ((mr + OZ_BM - 1) / OZ_BM) * ((N + OZ_BN - 1) / OZ_BN);
     if (tiles > 0x7fffffff) return FEAST_EINVAL;
+    // K split over a cluster: the split with the least waves x (its K-blocks at
+    // 2 x 28 x 48 clocks + the fixed cost of a CTA: pipeline fill, read-out,
+    // result, and the exchange when it shares its tile)
+    const int kb = (int)((2 * K + OZ_BK - 1) / OZ_BK);
+    int splits = 1;
+    double best = 0.0;
+    for (int x = 1; x <= OZ_SMAX; x *= 2) {
+        if (x > 1 && kb / x < 4) break;
+        const double waves = (double)((tiles * x + 151) / 152);
+        const double cost = waves * (((kb + x - 1) / x) * 2688.0 + (x > 1 ? 14000.0 : 10000.0));
+        if (x == 1 || cost < best) {
+            best = cost;
+            splits = x;
+        }
+    }
+    if (tiles * splits > 0x7fffffff) return FEAST_EINVAL;
     OzOut o{C, ldc, alpha, zcol, cblk > 0 ? cblk : 1, beta};
-    k_oz_gemm<<<(unsigned)tiles, OZ_THREADS, smem, s>>>(mA, mB, (int)mr, (int)N, (int)(2 * K), ea, fb, o, err);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)splits;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)(tiles * splits));
+    cfg.blockDim = dim3(OZ_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    FEAST_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_oz_gemm, mA, mB, (int)mr, (int)N, (int)(2 * K), splits,
+                                      (kb + splits - 1) / splits, ea, fb, o, err));
     FEAST_LAUNCH_CHECK();
     return FEAST_OK;
 }

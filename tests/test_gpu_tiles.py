@@ -29,3 +29,36 @@ def test_lu_solve_edges(n, batch, nrhs):
         assert np.linalg.norm(L @ U - P) <= 2 * n * 2.0 ** -53 * np.linalg.norm(L) * np.linalg.norm(U)
         res = np.linalg.norm(M[b] @ X[b] - R[b]) / (np.linalg.norm(M[b]) * np.linalg.norm(X[b]))
         assert res <= 4 * n * 2.0 ** -53
+
+
+@pytest.mark.parametrize("m,n,k", [(1, 1, 1), (63, 64, 16), (64, 65, 255), (65, 63, 257), (31, 33, 31), (130, 70, 1025),
+                                   (700, 600, 128), (33, 257, 3000)])
+@pytest.mark.parametrize("update", [False, True])
+def test_digit_sliced_gemm_edges(m, n, k, update):
+    """Tiles of 64 x 64, K-blocks of 16, chunks of 256 and the K splits of 1 to
+    8 CTAs a tile: 2^-48 k max|A_i.| max|B_.j| an entry (the entry point's
+    bound), the alpha A B + beta C rounding on top."""
+    import paper_1404_1768_gb300 as fg
+    rng = np.random.default_rng(m + n + k)
+    A, B = inputs.complex_normal(rng, (m, k)), inputs.complex_normal(rng, (k, n))
+    C0 = inputs.complex_normal(rng, (m, n))
+    out = fg.zgemm_oz(A, B, C0, alpha=-1.0, beta=1.0) if update else fg.zgemm_oz(A, B)
+    ref = C0 - A @ B if update else A @ B
+    ra = np.max(np.maximum(np.abs(A.real), np.abs(A.imag)), axis=1)
+    cb = np.max(np.maximum(np.abs(B.real), np.abs(B.imag)), axis=0)
+    bound = 2 * (2.0 ** -48 * k * np.outer(ra, cb) + 4 * 2.0 ** -53 * (np.abs(C0) + np.abs(ref)))
+    assert np.all(np.abs(out - ref) <= bound)
+
+
+@pytest.mark.parametrize("m,n,k,batch", [(1, 1, 1, 1), (31, 33, 17, 2), (32, 256, 16, 3), (129, 257, 255, 1),
+                                         (200, 8, 300, 2)])
+def test_tf32_split_gemm_edges(m, n, k, batch):
+    """The operand transposes of the complex64 GEMM at the edges of their 32 x
+    32 tiles and 256-row columns: FP32-like error, 2^-20 sqrt(k) of the norms."""
+    import paper_1404_1768_gb300 as fg
+    rng = np.random.default_rng(m * n + k)
+    A = [inputs.complex_normal(rng, (m, k)).astype(np.complex64) for _ in range(batch)]
+    X = [inputs.complex_normal(rng, (k, n)).astype(np.complex64) for _ in range(batch)]
+    for a, x, c in zip(A, X, fg.cgemm_tc(A, X)):
+        ref = a.astype(np.complex128) @ x.astype(np.complex128)
+        assert np.linalg.norm(c - ref) <= 2.0 ** -20 * np.sqrt(k) * max(np.linalg.norm(ref), 1e-30)
