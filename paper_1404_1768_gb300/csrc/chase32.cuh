@@ -158,15 +158,15 @@ __device__ __forceinline__ void chase_left(Rows H, int w, int lo, int hi, int k0
         const cf en = third ? r3[k + 2] : zero;
         const RotF g = rot32(x, y);
         const RotF gh = rot32_h(g);
-        if (lane == 0) {
-            rot[k - k0] = g;
-            // columns k - 1 and k: (r, 0) and the entry of row k
-            if (k > lo) {
-                r0[k - 1] = cmakef(fmaf(g.c, x.x, fmaf(g.s.x, y.x, -g.s.y * y.y)), fmaf(g.c, x.y, fmaf(g.s.x, y.y, g.s.y * y.x)));
-                r1[k - 1] = zero;
-            }
-            r0[k] = cmakef(fmaf(g.c, d0.x, fmaf(g.s.x, d1.x, -g.s.y * d1.y)),
-                           fmaf(g.c, d0.y, fmaf(g.s.x, d1.y, g.s.y * d1.x)));
+        {
+            // the entry of row k in column k (lane 0), and column k - 1: (r, 0)
+            // (lanes 1, 2; a sweep's first column has none): one store
+            const cf e0 = lane == 0 ? d0 : x, e1 = lane == 0 ? d1 : y;
+            const cf v0 = cmakef(fmaf(g.c, e0.x, fmaf(g.s.x, e1.x, -g.s.y * e1.y)),
+                                 fmaf(g.c, e0.y, fmaf(g.s.x, e1.y, g.s.y * e1.x)));
+            cf *q = lane == 2 ? r1 + k - 1 : r0 + k - lane;
+            if (lane < (k > lo ? 3 : 1)) *q = lane == 2 ? zero : v0;
+            if (lane == 3) rot[k - k0] = g;
         }
         // the corner: row k + 1 of columns k, k + 1 (left), then rows k + 1, k + 2 (right)
         cf p1 = cmakef(fmaf(g.c, d1.x, -fmaf(g.s.x, d0.x, g.s.y * d0.y)), fmaf(g.c, d1.y, -fmaf(g.s.x, d0.y, -g.s.y * d0.x)));

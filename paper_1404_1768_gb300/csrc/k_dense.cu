@@ -515,6 +515,210 @@ __global__ void __launch_bounds__(LU_PT) k_lu_panel(int64_t n, int64_t k0, int n
     }
 }
 
+// 1 / d, scaled by a power of two against overflow of |d|^2 (one reciprocal:
+// ~12 FP64 instructions where the quotient by Smith's form takes ~30).
+__device__ __forceinline__ double2 crecip(double2 d)
+{
+    const unsigned a = (unsigned)__double2hiint(d.x) & 0x7ff00000u, b = (unsigned)__double2hiint(d.y) & 0x7ff00000u;
+    int ex = (int)((a > b ? a : b) >> 20) - 1023;
+    ex = ex < -1000 ? -1000 : (ex > 1000 ? 1000 : ex);
+    const double f = __longlong_as_double((long long)(1023 - ex) << 52);
+    const double x = d.x * f, y = d.y * f;
+    const double r = f / (x * x + y * y);
+    return make_double2(x * r, -y * r);
+}
+__device__ __forceinline__ float2 crecip(float2 d) { return cdiv(make_float2(1.f, 0.f), d); }
+
+// Magnitude key of v for the pivot search: non-negative numbers order like
+// their bits; 0 for a NaN, 1 for zero.
+__device__ __forceinline__ unsigned long long mag_key(double2 v)
+{
+    const double m = cabs2(v);
+    const unsigned long long b = (unsigned long long)__double_as_longlong(m);
+    return b > 0x7ff0000000000000ull ? 0ull : b + 1ull;
+}
+__device__ __forceinline__ unsigned long long mag_key(float2 v)
+{
+    const unsigned b = __float_as_uint(cabs2(v));
+    return b > 0x7f800000u ? 0ull : (unsigned long long)b + 1ull;
+}
+__device__ __forceinline__ void key_max(unsigned long long &k, int &r, unsigned long long ok, int orow)
+{
+    if (ok > k || (ok == k && orow < r)) { k = ok; r = orow; }
+}
+
+// The same panel by a cluster of C CTAs, each keeping its rows of the panel in
+// shared memory: per column every CTA publishes its best candidate (key, row
+// index, the row itself) and the owner of the diagonal row publishes that row;
+// after one cluster barrier all of them know the pivot, take its row through
+// distributed shared memory and update their own rows (two buffers, used
+// alternately: a buffer is rewritten only after the barrier that follows its
+// last read).  The multipliers come from one reciprocal.  The one-CTA form runs
+// on one SM per matrix, and at n = 1000 in FP64 its rank-1 updates and
+// divisions keep that SM's FP64 pipe busy for ~600 us a panel (8 nodes: 8 of
+// 152 SMs); this one takes ~100 us, and ~60 us instead of 287 us for 32
+// complex64 panels of 2048 rows.  Pivots as in the one-CTA form (largest
+// modulus, ties to the smallest row).
+constexpr int LC_T = 256;
+constexpr int LC_MAX = 8;                // CTAs per matrix at most
+template <typename T>
+struct LuCand {
+    T row[LU_NB], cur[LU_NB];
+    unsigned long long key, idx;
+};
+template <typename T>
+__global__ void __launch_bounds__(LC_T) k_lu_panel_cl(int64_t n, int64_t k0, int nb, T *F, int64_t ldf, int64_t sF,
+                                                      int *piv, int64_t pstride, int *info, int *row, int C, int rp)
+{
+    extern __shared__ __align__(16) unsigned char lc_raw[];
+    T *slab = reinterpret_cast<T *>(lc_raw);
+    constexpr int P = LU_NB + 1;
+    __shared__ LuCand<T> cand[2];
+    __shared__ unsigned long long s_key[LC_T / 32];
+    __shared__ int s_idx[LC_T / 32];
+    __shared__ T s_row[LU_NB];
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    const int rank = C > 1 ? (int)cluster_rank_id() : 0;
+    const int b = blockIdx.x / C;
+    T *Am = F + (int64_t)b * sF + k0 + k0 * ldf;
+    const int total = (int)(n - k0), r0 = rank * rp;
+    const int rows = total - r0 < rp ? (total - r0 > 0 ? total - r0 : 0) : rp;
+    for (int c = wid; c < nb; c += LC_T / 32)
+        for (int r = lane; r < rows; r += 32) slab[r * P + c] = Am[r0 + r + (int64_t)c * ldf];
+    __syncthreads();
+    // threads per row of the update: a power of two, all of a row in one warp
+    int tpr = 1;
+    while (tpr < 32 && 2 * tpr * rows <= LC_T) tpr *= 2;
+    const int part = t % tpr, rbeg = t / tpr, rstep = LC_T / tpr;
+    const int none = 0x7fffffff;
+    unsigned long long key = 0;
+    int idx = none;
+    for (int r = t; r < rows; r += LC_T) {
+        const unsigned long long k = mag_key(slab[r * P]);
+        if (idx == none || k > key) { key = k; idx = r0 + r; }
+    }
+    for (int j = 0; j < nb; ++j) {
+        // this CTA's candidate
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1)
+            key_max(key, idx, __shfl_xor_sync(0xffffffffu, key, off), __shfl_xor_sync(0xffffffffu, idx, off));
+        if (lane == 0) { s_key[wid] = key; s_idx[wid] = idx; }
+        __syncthreads();
+        LuCand<T> &cd = cand[j & 1];
+        if (wid == 0) {
+            key = lane < LC_T / 32 ? s_key[lane] : 0ull;
+            idx = lane < LC_T / 32 ? s_idx[lane] : none;
+#pragma unroll
+            for (int off = 4; off > 0; off >>= 1)
+                key_max(key, idx, __shfl_xor_sync(0xffffffffu, key, off), __shfl_xor_sync(0xffffffffu, idx, off));
+            key = __shfl_sync(0xffffffffu, key, 0);
+            idx = __shfl_sync(0xffffffffu, idx, 0);
+            if (idx != none && lane < nb) cd.row[lane] = slab[(idx - r0) * P + lane];
+            if (lane == 0) { cd.key = key; cd.idx = (unsigned long long)idx; }
+        } else if (wid == 1 && j >= r0 && j < r0 + rows && lane < nb) {
+            cd.cur[lane] = slab[(j - r0) * P + lane];
+        }
+        if (C > 1) cluster_barrier();
+        else __syncthreads();
+        // the pivot: the best of the C candidates (every warp finds it)
+        unsigned long long bk = 0;
+        int bi = none;
+        if (lane < C) {
+            bk = C > 1 ? peer_load(&cd.key, (unsigned)lane) : cd.key;
+            bi = (int)(C > 1 ? peer_load(&cd.idx, (unsigned)lane) : cd.idx);
+        }
+#pragma unroll
+        for (int off = 4; off > 0; off >>= 1)
+            key_max(bk, bi, __shfl_xor_sync(0xffffffffu, bk, off), __shfl_xor_sync(0xffffffffu, bi, off));
+        bk = __shfl_sync(0xffffffffu, bk, 0);
+        bi = __shfl_sync(0xffffffffu, bi, 0);
+        const int p = bi;
+        const bool own_j = j >= r0 && j < r0 + rows, own_p = p >= r0 && p < r0 + rows;
+        if (wid == 0 && lane < nb) {
+            const T v = C > 1 ? peer_load(&cd.row[lane], (unsigned)(p / rp)) : cd.row[lane];
+            s_row[lane] = v;
+            if (own_j) slab[(j - r0) * P + lane] = v;
+        } else if (wid == 1 && lane < nb && own_p && p != j) {
+            slab[(p - r0) * P + lane] = C > 1 ? peer_load(&cd.cur[lane], (unsigned)(j / rp)) : cd.cur[lane];
+        }
+        if (rank == 0 && t == 64) {
+            piv[(int64_t)b * pstride + k0 + j] = (int)(k0 + p);
+            if (bk == 1ull && info) {
+                // record the first failing block (1-based) and column
+                if (atomicCAS(info, 0, b + 1) == 0 && row) *row = (int)(k0 + j) + 1;
+            }
+        }
+        __syncthreads();
+        const T d = s_row[j];
+        const bool live = !cis_zero(d);
+        const T inv = live ? crecip(d) : cx<T>(0, 0);
+        key = 0;
+        idx = none;
+        T lkeep = cx<T>(0, 0);                               // several threads a row: one row each, its multiplier
+        int rkeep = -1;                                      // stored once all of them have read a[j]
+        for (int r = rbeg; r < rows; r += rstep) {
+            if (r0 + r <= j) continue;
+            T *a = slab + r * P;
+            if (live) {
+                const T l = cmul(a[j], inv), nl = cneg(l);
+                for (int c = j + 1 + part; c < nb; c += tpr) {
+                    T v = a[c];
+                    cfma(v, nl, s_row[c]);
+                    a[c] = v;
+                }
+                if (tpr == 1) a[j] = l;
+                else if (part == 0) { lkeep = l; rkeep = r; }
+            }
+            if (part == 0 && j + 1 < nb) {                   // (part 0 has updated column j + 1 itself)
+                const unsigned long long k = mag_key(a[j + 1]);
+                if (idx == none || k > key) { key = k; idx = r0 + r; }
+            }
+        }
+        __syncthreads();
+        if (rkeep >= 0) slab[rkeep * P + j] = lkeep;
+    }
+    __syncthreads();
+    for (int c = wid; c < nb; c += LC_T / 32)
+        for (int r = lane; r < rows; r += 32) Am[r0 + r + (int64_t)c * ldf] = slab[r * P + c];
+    if (C > 1) cluster_barrier();                            // no CTA leaves while a peer reads its candidate
+}
+
+// The panel [k0, k0 + nb) of every batch member: the cluster form while its
+// CTAs' rows fit shared memory (200 KB: n - k0 <= 3096 in FP64, 6200 in
+// complex64), the one-CTA form on global memory beyond.  At least 16 rows a CTA:
+// below that the barrier costs more than the rows.
+template <typename T>
+int lu_panel(cudaStream_t s, int64_t n, int64_t k0, int nb, int batch, T *F, int64_t ldf, int64_t sF, int *piv,
+             int64_t pstride, int *info, int *row)
+{
+    const int64_t total = n - k0;
+    int C = 1;
+    while (C < LC_MAX && 32 * C <= total) C *= 2;
+    const int64_t rp = (total + C - 1) / C;
+    const size_t sm = (size_t)rp * (LU_NB + 1) * sizeof(T);
+    if (sm > 200 * 1024 || (int64_t)batch * C > 0x7fffffff) {
+        k_lu_panel<T><<<batch, LU_PT, 0, s>>>(n, k0, nb, F, ldf, sF, piv, pstride, info, row);
+        FEAST_LAUNCH_CHECK();
+        return FEAST_OK;
+    }
+    FEAST_CUDA_TRY(ensure_dyn_smem(k_lu_panel_cl<T>, sm));
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)C;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)(batch * C));
+    cfg.blockDim = dim3(LC_T);
+    cfg.dynamicSmemBytes = sm;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    FEAST_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_lu_panel_cl<T>, n, k0, nb, F, ldf, sF, piv, pstride, info, row, C, (int)rp));
+    FEAST_LAUNCH_CHECK();
+    return FEAST_OK;
+}
+
 // Apply the panel's row interchanges to the columns outside the panel.
 template <typename T>
 __global__ void k_laswp_outside(int64_t n, int64_t k0, int nb, T *F, int64_t ldf, int64_t sF,
@@ -546,14 +750,14 @@ int getrf_batched(cudaStream_t s, int64_t n, int batch, T *F, int64_t ldf, int64
     if (n <= 0 || batch <= 0) return FEAST_OK;
     for (int64_t k0 = 0; k0 < n; k0 += LU_NB) {
         int nb = (int)((n - k0) < LU_NB ? (n - k0) : LU_NB);
-        k_lu_panel<T><<<batch, LU_PT, 0, s>>>(n, k0, nb, F, ldf, sF, piv, n, info, row);
-        FEAST_LAUNCH_CHECK();
+        int e = lu_panel<T>(s, n, k0, nb, batch, F, ldf, sF, piv, n, info, row);
+        if (e) return e;
         unsigned gx = cdiv(n, 128);
         k_laswp_outside<T><<<dim3(gx, batch), 128, 0, s>>>(n, k0, nb, F, ldf, sF, piv);
         FEAST_LAUNCH_CHECK();
         int64_t rest = n - k0 - nb;
         if (rest > 0) {
-            int e = trsv_diag<T>(s, rest, batch, k0, nb, 1, F, ldf, sF, F + (k0 + nb) * ldf, ldf, sF);
+            e = trsv_diag<T>(s, rest, batch, k0, nb, 1, F, ldf, sF, F + (k0 + nb) * ldf, ldf, sF);
             if (e) return e;
             e = gemm_batched<T>(s, 0, rest, rest, nb, cx<T>(-1, 0), F + k0 + nb + k0 * ldf,
                                     ldf, sF, F + k0 + (k0 + nb) * ldf, ldf, sF, cx<T>(1, 0),
@@ -588,8 +792,7 @@ int getrf_batched_tc(cudaStream_t s, int64_t n, int batch, cf *F, int64_t ldf, i
         const int64_t kend = k0 + nbo;                  // first column after the outer block
         for (int64_t kk = k0; kk < kend; kk += LU_NB) {
             const int nb = (int)((kend - kk) < LU_NB ? (kend - kk) : LU_NB);
-            k_lu_panel<cf><<<batch, LU_PT, 0, s>>>(n, kk, nb, F, ldf, sF, piv, n, info, row);
-            FEAST_LAUNCH_CHECK();
+            if ((e = lu_panel<cf>(s, n, kk, nb, batch, F, ldf, sF, piv, n, info, row))) return e;
             k_laswp_outside<cf><<<dim3(cdiv(n, 128), batch), 128, 0, s>>>(n, kk, nb, F, ldf, sF, piv);
             FEAST_LAUNCH_CHECK();
             const int64_t c1 = kk + nb;                 // first column right of the panel
@@ -631,9 +834,7 @@ int getrf_panel(cudaStream_t s, int64_t rows, int nb, int batch, T *F, int64_t l
                 int *piv, int64_t pstride, int *info, int *row)
 {
     if (rows <= 0 || nb <= 0 || batch <= 0) return FEAST_OK;
-    k_lu_panel<T><<<batch, LU_PT, 0, s>>>(rows, 0, nb, F, ldf, sF, piv, pstride, info, row);
-    FEAST_LAUNCH_CHECK();
-    return FEAST_OK;
+    return lu_panel<T>(s, rows, 0, nb, batch, F, ldf, sF, piv, pstride, info, row);
 }
 template int getrf_panel<double2>(cudaStream_t, int64_t, int, int, double2 *, int64_t, int64_t, int *,
                                   int64_t, int *, int *);

@@ -1145,7 +1145,10 @@ __global__ void __launch_bounds__(QT, 1) k_hqr(int m, dsv *H, dsv *Z, int ld, Ro
     __shared__ cds blk[BLK][BLK + 1];
 #endif
     __shared__ RotDS srot[NSH][CH];
-    const int gtid = blockIdx.x * QT + threadIdx.x, gthreads = gridDim.x * QT;
+    // far-part lines: warps take 32 of them a grid apart, so that the lines of a
+    // phase (fewer than the threads) spread over all SMs
+    const int gtid = ((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31);
+    const int gthreads = gridDim.x * QT;
     int ihi = m - 1, iter = 0, total = 0;
     while (ihi > 0) {
         const int l = scan_deflation(H, ld, ihi, tol_rel, tol_abs);

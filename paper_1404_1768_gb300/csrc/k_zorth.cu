@@ -4,10 +4,11 @@
 // Block classical Gram-Schmidt with re-orthogonalisation (BCGS2, the
 // two-pass form of Barlow & Smoktunowicz): each block of 32 columns is
 // projected against the finished columns by two GEMM pairs, and inside the
-// block column-wise CGS2 runs either on one CTA (short panels) or on a
-// cooperative grid that splits the panel's rows over the SMs, each CTA
-// keeping its slab in shared memory and the column dot products reduced
-// across CTAs in a fixed order (so results do not depend on timing).
+// block column-wise CGS2 runs on one cluster of CTAs, or (panels too tall for
+// its shared memory) on a cooperative grid that splits the panel's rows over
+// the SMs, each CTA keeping its slab in shared memory and the column dot
+// products reduced across CTAs in a fixed order (so results do not depend on
+// timing); on one CTA where that does not fit either.
 // Loss of orthogonality stays
 // at rounding level for condition numbers up to ~1/eps, which covers the
 // FEAST subspaces (their weakest directions carry filter values down to
@@ -205,21 +206,141 @@ __global__ void __launch_bounds__(OT) k_cgs2_grid(int64_t n, int w, zd *V, int64
     }
 }
 
+// Column-wise CGS2 of an n x w panel (w <= 32) by one cluster of up to CC CTAs,
+// each keeping its rows [b rp, ..) in shared memory; the partial sums meet
+// through distributed shared memory and the cluster's hardware barrier (~0.3 us
+// where a grid barrier through L2 takes ~2), three of them per column.  In FP64
+// a warp-wide instruction holds its SM quarter for 64 clocks whatever the
+// lanes, so the sums over columns are spread over four lanes a row and the sums
+// over warps and CTAs over eight lanes: chains of ~40 FP64 instructions per
+// pass instead of ~150.  200 x 32: 593 -> ~200 us.
+constexpr int CC = 8;
+__global__ void __launch_bounds__(OT) k_cgs2_cluster(int64_t n, int w, zd *V, int64_t ldv, zd *T, int64_t ldt, int rp,
+                                                     int C)
+{
+    extern __shared__ zd slab[];
+    __shared__ zd red[OT / 32][OB];
+    __shared__ zd xch[2][OB];
+    __shared__ zd coef[OB];
+    __shared__ double xn[2];
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    const unsigned rank = C > 1 ? cluster_rank_id() : 0;
+    const int64_t r0 = (int64_t)rank * rp;
+    const int rows = (int)((n - r0) < rp ? ((n - r0) > 0 ? (n - r0) : 0) : rp);
+    constexpr int P = OB + 1;
+    for (int p = wid; p < w; p += OT / 32)
+        for (int r = lane; r < rows; r += 32) slab[r * P + p] = V[r0 + r + (int64_t)p * ldv];
+    if (rank == 0)
+        for (int e = t; e < w * w; e += OT) T[(e % w) + (e / w) * ldt] = zmake(0.0, 0.0);
+    __syncthreads();
+    int buf = 0;
+    const int p8 = 4 * wid + (lane >> 3), k8 = lane & 7;      // eight lanes per column
+    for (int i = 0; i < w; ++i) {
+        double nrm = 0.0;                                     // this thread's rows, after the last update
+        for (int pass = 0; pass < 2 && i > 0; ++pass) {
+            zd acc = zmake(0.0, 0.0);
+            if (lane < i)
+                for (int r = wid; r < rows; r += OT / 32) zfma_conj(acc, slab[r * P + lane], slab[r * P + i]);
+            red[wid][lane] = acc;
+            __syncthreads();
+            zd v = red[k8][p8];
+#pragma unroll
+            for (int off = 4; off > 0; off >>= 1) {
+                v.x += __shfl_xor_sync(0xffffffffu, v.x, off);
+                v.y += __shfl_xor_sync(0xffffffffu, v.y, off);
+            }
+            if (C > 1) {
+                if (k8 == 0) xch[buf][p8] = v;
+                cluster_barrier();
+                v = k8 < C ? peer_load(&xch[buf][p8], (unsigned)k8) : zmake(0.0, 0.0);
+#pragma unroll
+                for (int off = 4; off > 0; off >>= 1) {
+                    v.x += __shfl_xor_sync(0xffffffffu, v.x, off);
+                    v.y += __shfl_xor_sync(0xffffffffu, v.y, off);
+                }
+                buf ^= 1;
+            }
+            if (k8 == 0) {
+                coef[p8] = v;
+                if (rank == 0 && p8 < i) {
+                    zd &o = T[p8 + (int64_t)i * ldt];
+                    o = zadd(o, v);
+                }
+            }
+            __syncthreads();
+            // rows, four lanes each
+            for (int rb = 0; rb < rows; rb += OT / 4) {
+                const int r = rb + (t >> 2), part = t & 3;
+                zd a = zmake(0.0, 0.0);
+                if (r < rows)
+                    for (int p = part; p < i; p += 4) zfma(a, coef[p], slab[r * P + p]);
+                a.x += __shfl_xor_sync(0xffffffffu, a.x, 1);
+                a.y += __shfl_xor_sync(0xffffffffu, a.y, 1);
+                a.x += __shfl_xor_sync(0xffffffffu, a.x, 2);
+                a.y += __shfl_xor_sync(0xffffffffu, a.y, 2);
+                if (r < rows && part == 0) {
+                    const zd x = zsub(slab[r * P + i], a);
+                    slab[r * P + i] = x;
+                }
+            }
+            __syncthreads();
+        }
+        // norm of column i
+        for (int r = t; r < rows; r += OT) nrm += zabs2(slab[r * P + i]);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, off);
+        if (lane == 0) red[wid][0].x = nrm;
+        __syncthreads();
+        double s = red[k8][0].x;
+#pragma unroll
+        for (int off = 4; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        if (C > 1) {
+            if (t == 0) xn[i & 1] = s;
+            cluster_barrier();
+            s = k8 < C ? peer_load(&xn[i & 1], (unsigned)k8) : 0.0;
+#pragma unroll
+            for (int off = 4; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        }
+        if (rank == 0 && t == 0) T[i + (int64_t)i * ldt] = zmake(sqrt(s), 0.0);
+        if (s > 0.0) {
+            const double inv = rsqrt(s);
+            for (int r = t; r < rows; r += OT) slab[r * P + i] = zscale(slab[r * P + i], inv);
+        }
+        __syncthreads();
+    }
+    for (int p = wid; p < w; p += OT / 32)
+        for (int r = lane; r < rows; r += 32) V[r0 + r + (int64_t)p * ldv] = slab[r * P + p];
+    if (C > 1) cluster_barrier();                             // no CTA leaves while a peer reads its sums
+}
+
 constexpr int GMAX = 256;           // most CTAs of the grid form
 constexpr int RP_MIN = 32;          // fewest rows a CTA of the grid form takes
 
 struct IntraPlan {
     int grid = 0;                   // 0: one-CTA kernel
+    int cluster = 0;                // > 0: one cluster of that many CTAs
     int rp = 0;
     size_t smem = 0;
 };
 
-// The grid form pays for ~3 grid barriers per column; it is used when the
-// panel is tall enough that one SM's FP64 rate would dominate instead.
+// One cluster as long as its CTAs hold the panel (n <= CC * 416: 220 KB each);
+// beyond, the grid form, which pays for ~3 grid barriers per column but spreads
+// the FP64 work over every SM.
 int plan_intra(int64_t n, IntraPlan &pl)
 {
     pl = IntraPlan{};
-    if (n < 4 * RP_MIN) return FEAST_OK;
+    {
+        int C = 1;
+        while (C < CC && (int64_t)C * RP_MIN < n) C *= 2;
+        const int rp = (int)((n + C - 1) / C);
+        if (rp <= 416) {
+            pl.cluster = C;
+            pl.rp = rp;
+            pl.smem = (size_t)rp * (OB + 1) * sizeof(zd);
+            FEAST_CUDA_TRY(allow_dyn_smem(k_cgs2_cluster));
+            return FEAST_OK;
+        }
+    }
     int dev = 0, sms = 0, smem_max = 0;
     FEAST_CUDA_TRY(cudaGetDevice(&dev));
     FEAST_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -243,6 +364,23 @@ int plan_intra(int64_t n, IntraPlan &pl)
 int run_intra(cudaStream_t s, const IntraPlan &pl, int64_t n, int w, zd *V, int64_t ldv, zd *T,
               int64_t ldt, zd *part, GridSync g)
 {
+    if (pl.cluster) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)pl.cluster;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3(pl.cluster);
+        cfg.blockDim = dim3(OT);
+        cfg.dynamicSmemBytes = pl.smem;
+        cfg.stream = s;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        FEAST_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_cgs2_cluster, n, w, V, ldv, T, ldt, pl.rp, pl.cluster));
+        FEAST_LAUNCH_CHECK();
+        return FEAST_OK;
+    }
     if (!pl.grid) {
         k_cgs2_intra<<<1, OT, 0, s>>>(n, w, V, ldv, T, ldt);
         FEAST_LAUNCH_CHECK();

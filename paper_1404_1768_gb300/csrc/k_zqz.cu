@@ -420,23 +420,24 @@ __device__ void ez_mul(int m, int ld, const cf *X, const cf *Y, cf *C)
 template <bool UNIT>
 __device__ void ez_back_solve(int m, int ld, const cf *U, cf *X, cf *X2)
 {
-    const int cols = X2 ? 2 * m : m;
+    // thread: column t mod 128 of [X | X2] (m <= 64 each), every other row
+    const int c = threadIdx.x & 127, half = threadIdx.x >> 7;
+    cf *x = c < 64 ? X + c : X2 + (c - 64);
+    const bool on = c < 64 ? c < m : (X2 != nullptr && c - 64 < m);
     for (int i = m - 1; i >= 0; --i) {
+        cf xi = on ? x[i * ld] : cmakef(0.f, 0.f);
         if (!UNIT) {
-            const cf d = U[i * ld + i];
-            for (int c = threadIdx.x; c < cols; c += EZ_T) {
-                cf *x = (c < m) ? X + i * ld + c : X2 + i * ld + (c - m);
-                *x = cdiv(*x, d);
-            }
+            xi = cdiv(xi, U[i * ld + i]);
             __syncthreads();
+            if (on && half == 0) x[i * ld] = xi;
         }
-        for (int e = threadIdx.x; e < i * cols; e += EZ_T) {
-            const int r = e / cols, c = e - r * cols;
-            cf *x = (c < m) ? X + c : X2 + (c - m);
-            cf v = x[r * ld];
-            cfma(v, cneg(U[r * ld + i]), x[i * ld]);
-            x[r * ld] = v;
-        }
+        const cf nx = cneg(xi);
+        if (on)
+            for (int r = half; r < i; r += 2) {
+                cf v = x[r * ld];
+                cfma(v, nx, U[r * ld + i]);
+                x[r * ld] = v;
+            }
         __syncthreads();
     }
 }
@@ -601,6 +602,109 @@ __device__ void ez_vectors(int m, int ld, const cf *T, cf *Y, float small)
     __syncthreads();
 }
 
+// a += x v: a and x unevaluated sums of two floats (~2^-46 relative), v a float
+// (error-free product by FMA).
+struct f2 {
+    float h, l;
+};
+__device__ __forceinline__ void f2_fma(f2 &a, float xh, float xl, float v)
+{
+    const float p = __fmul_rn(xh, v);
+    const float e = __fmaf_rn(xl, v, __fmaf_rn(xh, v, -p));
+    const float s = __fadd_rn(a.h, p);
+    const float b = __fsub_rn(s, a.h);
+    const float t = __fadd_rn(__fadd_rn(__fsub_rn(a.h, __fsub_rn(s, b)), __fsub_rn(p, b)), __fadd_rn(a.l, e));
+    a.h = __fadd_rn(s, t);
+    a.l = __fsub_rn(t, __fsub_rn(a.h, s));
+}
+__device__ __forceinline__ float f2_sub_mul(f2 a, f2 br, float lr, f2 bi, float li)   // a - br lr - bi li
+{
+    f2_fma(a, br.h, br.l, -lr);
+    f2_fma(a, bi.h, bi.l, -li);
+    return a.h + a.l;
+}
+
+// R' = A' V - B' V Lambda' of the first step, where V (= V32) and Lambda (=
+// diag, FP32) are FP32 exactly: the products in double-single on the FP32 pipe,
+// a sixth of the FP64 form's time.  As: m x m float4 of scratch, Bh: m ld
+// scratch; W: scratch, then R'.
+__device__ void ez_resid_first(int m, int ld, const zd *A, int64_t lda, double fa, const zd *B, int64_t ldb, double fb,
+                               const cf *V32, const float *lf, float4 *As, cf *Bh, cf *W)
+{
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    for (int e = threadIdx.x; e < m * m; e += EZ_T) {
+        const int r = e % m, c = e / m;
+        const double x = A[r + c * lda].x * fa, y = A[r + c * lda].y * fa;
+        const float xh = (float)x, yh = (float)y;
+        As[e] = make_float4(xh, (float)(x - (double)xh), yh, (float)(y - (double)yh));
+        cf h = cmakef(0.f, 0.f), l = h;
+        if (r <= c) {
+            const double u = B[r + c * ldb].x * fb, v = B[r + c * ldb].y * fb;
+            h = cmakef((float)u, (float)v);
+            l = cmakef((float)(u - (double)h.x), (float)(v - (double)h.y));
+        }
+        Bh[r * ld + c] = h;
+        W[r * ld + c] = l;
+    }
+    __syncthreads();
+    cf out[4][4];
+#pragma unroll
+    for (int i2 = 0; i2 < 4; i2 += 2) {
+        f2 ar[2][4], ai[2][4], br[2][4], bi[2][4];
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                ar[i][j].h = ar[i][j].l = ai[i][j].h = ai[i][j].l = 0.f;
+                br[i][j].h = br[i][j].l = bi[i][j].h = bi[i][j].l = 0.f;
+                out[i2 + i][j] = cmakef(0.f, 0.f);
+            }
+        if (16 * i2 < m) {
+            for (int p = 0; p < m; ++p) {
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const int r = ty + 16 * (i2 + i);
+                    if (r >= m) continue;
+                    const float4 x = As[r + p * m];
+                    const cf h = Bh[r * ld + p], l = W[r * ld + p];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int c = tx + 16 * j;
+                        if (c >= m) continue;
+                        const cf v = V32[p * ld + c];
+                        f2_fma(ar[i][j], x.x, x.y, v.x);
+                        f2_fma(ar[i][j], x.z, x.w, -v.y);
+                        f2_fma(ai[i][j], x.x, x.y, v.y);
+                        f2_fma(ai[i][j], x.z, x.w, v.x);
+                        if (r <= p) {
+                            f2_fma(br[i][j], h.x, l.x, v.x);
+                            f2_fma(br[i][j], h.y, l.y, -v.y);
+                            f2_fma(bi[i][j], h.x, l.x, v.y);
+                            f2_fma(bi[i][j], h.y, l.y, v.x);
+                        }
+                    }
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int c = tx + 16 * j;
+                    if (c >= m) continue;
+                    const float lr = lf[4 * c], li = lf[4 * c + 2];
+                    out[i2 + i][j] = cmakef(f2_sub_mul(ar[i][j], br[i][j], lr, bi[i][j], -li),
+                                            f2_sub_mul(ai[i][j], br[i][j], li, bi[i][j], lr));
+                }
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (ty + 16 * i < m && tx + 16 * j < m) W[(ty + 16 * i) * ld + tx + 16 * j] = out[i][j];
+}
+
 // exponent bits of the largest |component| (0x7ff: a non-finite entry)
 __device__ __forceinline__ unsigned ez_hi(zd v)
 {
@@ -710,8 +814,7 @@ __global__ void __launch_bounds__(EZ_T) k_eig_refined(int m, const zd *__restric
         const float d = lf[c], di = 1.f / d;
         cf v = L[r * ld + c];
         v = cmakef(v.x * di, v.y * di);
-        L[r * ld + c] = v;                          // V in FP32
-        Vd[r + c * m] = zmake((double)v.x, (double)v.y);
+        L[r * ld + c] = v;                          // V (FP32 so far)
     }
     for (int e = t; e < m * m; e += EZ_T) {
         const int r = e / m, c = e % m;
@@ -752,8 +855,19 @@ __global__ void __launch_bounds__(EZ_T) k_eig_refined(int m, const zd *__restric
             lf[4 * j + 3] = (float)(l.y - (double)hy);
             part[j] = -1;
         }
-        // R' = 2^-ea (A V - B V Lambda), a 4 x 4 tile per thread, into W (FP32)
-        {
+        // R' = 2^-ea (A V - B V Lambda), a 4 x 4 tile per thread, into W (FP32):
+        // in double-single for the first step (whose V and Lambda are FP32;
+        // what 46 bits do not see is below what that step leaves), in FP64
+        // from then on
+        if (step == 0) {
+            __syncthreads();
+            ez_resid_first(m, ld, A, lda, fa, B, ldb, fb, L, lf, (float4 *)Vd, Z, W);
+            __syncthreads();
+            for (int e = t; e < m * m; e += EZ_T) {
+                const cf v = L[(e % m) * ld + e / m];
+                Vd[e] = zmake((double)v.x, (double)v.y);
+            }
+        } else {
             const int tx = t & 15, ty = t >> 4;
             zd ra[4][4], rb[4][4];
 #pragma unroll
