@@ -35,32 +35,47 @@ __device__ __forceinline__ float rsqrt_nr(float x)
     return y * fmaf(-0.5f * x * y, y, 1.5f);
 }
 
-// G = [c s; -conj(s) c] with G [x; y] = [r; 0]
-__device__ __forceinline__ RotF rot32(cf x, cf y)
+// G = [c s; -conj(s) c] with G [x; y] = [r; 0], whatever the sizes of x and y:
+// the larger entry is brought into [1, 2) first, so that squares neither
+// overflow nor vanish.
+static __device__ __noinline__ RotF rot32_scaled(cf x, cf y)
 {
     RotF g;
-    float ax2 = cabs2(x), ay2 = cabs2(y);
-    if (!(ax2 + ay2 > 1e-24f && ax2 + ay2 < 1e30f) || ax2 < 1e-30f) {
-        // bring the larger entry into [1, 2): squares neither overflow nor vanish
-        const float mx = fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(y.x), fabsf(y.y)));
-        int ex = (int)(__float_as_uint(mx) >> 23);
-        ex = ex < 1 ? 1 : (ex > 253 ? 253 : ex);
-        const float f = __uint_as_float((unsigned)(254 - ex) << 23);
-        x = cmakef(x.x * f, x.y * f);
-        y = cmakef(y.x * f, y.y * f);
-        ax2 = cabs2(x);
-        ay2 = cabs2(y);
-        if (ay2 == 0.f) { g.c = 1.f; g.s = cmakef(0.f, 0.f); return g; }
-        if (ax2 < 1e-36f) {
-            g.c = 0.f;
-            const float ia = rsqrt_nr(ay2);
-            g.s = cmakef(y.x * ia, -y.y * ia);
-            return g;
-        }
+    const float mx = fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(y.x), fabsf(y.y)));
+    int ex = (int)(__float_as_uint(mx) >> 23);
+    ex = ex < 1 ? 1 : (ex > 253 ? 253 : ex);
+    const float f = __uint_as_float((unsigned)(254 - ex) << 23);
+    x = cmakef(x.x * f, x.y * f);
+    y = cmakef(y.x * f, y.y * f);
+    const float ax2 = cabs2(x), ay2 = cabs2(y);
+    if (ay2 == 0.f) { g.c = 1.f; g.s = cmakef(0.f, 0.f); return g; }
+    if (ax2 < 1e-36f) {
+        g.c = 0.f;
+        const float ia = rsqrt_nr(ay2);
+        g.s = cmakef(y.x * ia, -y.y * ia);
+        return g;
     }
     const float k = rsqrt_nr(ax2) * rsqrt_nr(ax2 + ay2);
     g.c = ax2 * k;
     g.s = cmakef((x.x * y.x + x.y * y.y) * k, (x.y * y.x - x.x * y.y) * k);   // x conj(y) k
+    return g;
+}
+// The same; the reciprocal roots are under way before the sizes are looked at
+// (the test ahead of them cost 50 of 134 clocks).
+__device__ __forceinline__ RotF rot32(cf x, cf y)
+{
+    RotF g;
+    const float ax2 = cabs2(x), s2 = ax2 + cabs2(y);
+    float ia, ir;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(ia) : "f"(ax2));
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(ir) : "f"(s2));
+    const float px = fmaf(x.x, y.x, x.y * y.y), py = fmaf(x.y, y.x, -x.x * y.y);
+    if (__builtin_expect(!(ax2 > 1e-30f && s2 > 1e-24f && s2 < 1e30f), 0)) return rot32_scaled(x, y);
+    ia *= fmaf(-0.5f * ax2 * ia, ia, 1.5f);
+    ir *= fmaf(-0.5f * s2 * ir, ir, 1.5f);
+    const float k = ia * ir;
+    g.c = ax2 * k;
+    g.s = cmakef(px * k, py * k);
     return g;
 }
 __device__ __forceinline__ void rot32_pair(const RotF &g, cf &a, cf &b)          // G [a; b]
@@ -104,6 +119,9 @@ struct RowsLd {
     cf *p;
     int ld;
     __device__ __forceinline__ cf *row(int k) const { return p + k * ld; }
+    // shared-memory byte address of row k, and of row k + 1 from it
+    __device__ __forceinline__ uint32_t addr(int k) const { return (uint32_t)__cvta_generic_to_shared(p) + 8u * (uint32_t)(k * ld); }
+    __device__ __forceinline__ uint32_t next(uint32_t a, int) const { return a + 8u * (uint32_t)ld; }
 };
 __host__ __device__ __forceinline__ int packed_base(int m, int k)
 {
@@ -114,7 +132,22 @@ struct RowsPacked {
     cf *p;
     int m;
     __device__ __forceinline__ cf *row(int k) const { return p + packed_base(m, k); }
+    __device__ __forceinline__ uint32_t addr(int k) const
+    {
+        return (uint32_t)__cvta_generic_to_shared(p) + 8u * (uint32_t)packed_base(m, k);
+    }
+    __device__ __forceinline__ uint32_t next(uint32_t a, int k) const { return a + 8u * (uint32_t)(k < 2 ? m : m + 1 - k); }
 };
+__device__ __forceinline__ cf lds32(uint32_t a)
+{
+    cf v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void sts32(uint32_t a, cf v)
+{
+    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
+}
 
 // Most rotations of one chase_left() call.
 constexpr int CHASE_N = 32;
@@ -126,6 +159,11 @@ constexpr int CHASE_N = 32;
 // k0 + 32 are updated (left rotations); those beyond wait for far_left(), the
 // rows above k1 for chase_right().  On return the bulge stands at
 // H[k1 + 1][k1 - 1] (k1 < hi).  Ends with __syncwarp().
+//
+// Nothing but the column's own store is written inside the chain: lane k - k0
+// keeps what rotation k was made of and of column k, and finishes column k - 1
+// and the diagonal entry after the chunk (a store by single lanes inside the
+// loop cost 100 clocks per rotation and more).  ~240 clocks per rotation on 64 rows (366 before).
 template <typename Rows>
 __device__ __forceinline__ void chase_left(Rows H, int w, int lo, int hi, int k0, int k1, cf sigma, RotF *rot)
 {
@@ -133,42 +171,44 @@ __device__ __forceinline__ void chase_left(Rows H, int w, int lo, int hi, int k0
     const cf zero = cmakef(0.f, 0.f);
     const int c = k0 + 1 + lane;
     const bool in = c < w;
-    cf *r0 = H.row(k0), *r1 = H.row(k0 + 1);
-    cf d0 = r0[k0], d1 = r1[k0], x, y;
+    const uint32_t oc = 8u * (uint32_t)(in ? c : w - 1);       // (a lane without a column reads the last one)
+    uint32_t r0 = H.addr(k0), r1 = H.next(r0, k0);
+    cf d0 = lds32(r0 + 8 * k0), d1 = lds32(r1 + 8 * k0), x, y;
     if (k0 == lo) {
         x = cmakef(d0.x - sigma.x, d0.y - sigma.y);
         y = d1;
     } else {
-        x = r0[k0 - 1];
-        y = r1[k0 - 1];
+        x = lds32(r0 + 8 * (k0 - 1));
+        y = lds32(r1 + 8 * (k0 - 1));
     }
     // this lane's column: the carried entry of row k, and row k + 1's
-    cf a = in ? r0[c] : zero, n = in ? r1[c] : zero;
-    cf v = r1[k0 + 1];
-    cf *r2 = (k0 + 2 <= hi) ? H.row(k0 + 2) : r1;
-    cf e = (k0 + 2 <= hi) ? r2[k0 + 1] : zero;
+    cf a = lds32(r0 + oc), n = lds32(r1 + oc);
+    cf v = lds32(r1 + 8 * (k0 + 1));
+    uint32_t r2 = (k0 + 2 <= hi) ? H.next(r1, k0 + 1) : r1;
+    cf e = (k0 + 2 <= hi) ? lds32(r2 + 8 * (k0 + 1)) : zero;
+    cf kx = zero, ky = zero, kd0 = zero, kd1 = zero;           // lane k - k0: rotation k's
+    RotF kg;
+    kg.c = 1.f;
+    kg.s = zero;
     for (int k = k0; k < k1; ++k) {
         // the next column's entry of row k, and the next step's entries
         const cf u = cmakef(__shfl_sync(0xffffffffu, a.x, k - k0), __shfl_sync(0xffffffffu, a.y, k - k0));
-        const bool more = k + 2 <= hi;
-        const cf nn = (more && in) ? r2[c] : zero;
-        const cf vn = more ? r2[k + 2] : zero;
-        const bool third = k + 3 <= hi && k + 1 < k1;      // (a block may end at row k1 + 1)
-        cf *r3 = third ? H.row(k + 3) : r2;
-        const cf en = third ? r3[k + 2] : zero;
+        const cf nn = lds32(r2 + oc);                           // (row k + 2; past the end: row hi again, unused)
+        const cf vn = lds32(r2 + 8 * (k + 2 <= hi ? k + 2 : hi));
+        const bool third = k + 3 <= hi && k + 1 < k1;          // (a block may end at row k1 + 1)
+        const uint32_t r3 = third ? H.next(r2, k + 2) : r2;
+        const cf el = lds32(r3 + 8 * (third ? k + 2 : k));
+        const cf en = third ? el : zero;
         const RotF g = rot32(x, y);
-        const RotF gh = rot32_h(g);
-        {
-            // the entry of row k in column k (lane 0), and column k - 1: (r, 0)
-            // (lanes 1, 2; a sweep's first column has none): one store
-            const cf e0 = lane == 0 ? d0 : x, e1 = lane == 0 ? d1 : y;
-            const cf v0 = cmakef(fmaf(g.c, e0.x, fmaf(g.s.x, e1.x, -g.s.y * e1.y)),
-                                 fmaf(g.c, e0.y, fmaf(g.s.x, e1.y, g.s.y * e1.x)));
-            cf *q = lane == 2 ? r1 + k - 1 : r0 + k - lane;
-            if (lane < (k > lo ? 3 : 1)) *q = lane == 2 ? zero : v0;
-            if (lane == 3) rot[k - k0] = g;
-        }
+        const bool mine = lane == k - k0;
+        kx = mine ? x : kx;
+        ky = mine ? y : ky;
+        kd0 = mine ? d0 : kd0;
+        kd1 = mine ? d1 : kd1;
+        kg.c = mine ? g.c : kg.c;
+        kg.s = mine ? g.s : kg.s;
         // the corner: row k + 1 of columns k, k + 1 (left), then rows k + 1, k + 2 (right)
+        const RotF gh = rot32_h(g);
         cf p1 = cmakef(fmaf(g.c, d1.x, -fmaf(g.s.x, d0.x, g.s.y * d0.y)), fmaf(g.c, d1.y, -fmaf(g.s.x, d0.y, -g.s.y * d0.x)));
         cf q1 = cmakef(fmaf(g.c, v.x, -fmaf(g.s.x, u.x, g.s.y * u.y)), fmaf(g.c, v.y, -fmaf(g.s.x, u.y, -g.s.y * u.x)));
         rot32_pair(gh, p1, q1);
@@ -178,7 +218,7 @@ __device__ __forceinline__ void chase_left(Rows H, int w, int lo, int hi, int k0
         d1 = cmakef(g.c * e.x, g.c * e.y);
         // this lane's column (from k + 1 on)
         rot32_pair(g, a, n);
-        if (c > k && in) r0[c] = a;
+        if (c > k && in) sts32(r0 + oc, a);
         a = n;
         n = nn;
         v = vn;
@@ -188,14 +228,27 @@ __device__ __forceinline__ void chase_left(Rows H, int w, int lo, int hi, int k0
         r2 = r3;
     }
     // row k1 and the bulge (r0 = row k1, r1 = row k1 + 1 when k1 < hi)
-    if (c > k1 && in) r0[c] = a;
+    if (c > k1 && in) sts32(r0 + oc, a);
     if (lane == 0) {
-        r0[k1] = d0;
-        r0[k1 - 1] = x;
+        sts32(r0 + 8 * k1, d0);
+        sts32(r0 + 8 * (k1 - 1), x);
         if (k1 < hi) {
-            r1[k1] = d1;
-            r1[k1 - 1] = y;
+            sts32(r1 + 8 * k1, d1);
+            sts32(r1 + 8 * (k1 - 1), y);
         }
+    }
+    // rotation k = k0 + lane: columns k - 1, (r, 0), and k, the entry of row k
+    const int k = k0 + lane;
+    if (k < k1) {
+        const uint32_t rk = H.addr(k);
+        rot32_pair(kg, kd0, kd1);
+        sts32(rk + 8 * k, kd0);
+        if (k > lo) {
+            rot32_pair(kg, kx, ky);
+            sts32(rk + 8 * (k - 1), kx);
+            sts32(H.next(rk, k) + 8 * (k - 1), zero);
+        }
+        rot[lane] = kg;
     }
     __syncwarp();
 }

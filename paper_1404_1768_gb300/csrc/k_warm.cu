@@ -52,7 +52,9 @@ constexpr int RF_PART = 64;           // partial sums of the defect norm
 
 struct RefineStat {
     unsigned gm;                      // bits of max |G|^2 (non-negative floats order like their bits)
-    int bad, paired, pad;
+    int bad, paired;
+    unsigned wm;                      // the same of max |W_ij|^2, i != j
+    int tiny, pad[3];                 // a close pair's coupling at rounding level was seen
 };
 
 // X = [C | I], both m x m: C = A and the identity in FP32; B32 = the upper
@@ -229,7 +231,7 @@ __global__ void k_rf_lam(int m, const cf *__restrict__ T, zd *__restrict__ lam)
     if (i < m) lam[i] = zmake((double)T[i + (int64_t)i * m].x, (double)T[i + (int64_t)i * m].y);
 }
 
-// R32 = A V - (B V) Lambda, rounded to FP32; part[j] = -1.
+// R32 = A V - (B V) Lambda, rounded to FP32; part and near (the m after it) = -1.
 __global__ void k_rf_resid(int m, const zd *__restrict__ AV, const zd *__restrict__ BV, const zd *__restrict__ lam,
                            cf *__restrict__ R32, int *__restrict__ part)
 {
@@ -239,18 +241,19 @@ __global__ void k_rf_resid(int m, const zd *__restrict__ AV, const zd *__restric
         const int j = (int)(e / m);
         const zd r = zsub(AV[e], zmul(lam[j], BV[e]));
         R32[e] = cmakef((float)r.x, (float)r.y);
-        if (e % m == 0) part[j] = -1;
+        if (e % m == 0) part[j] = part[m + j] = -1;
     }
 }
 
 // G from W (off the diagonal): see the file comment.  tiny: couplings at
 // rounding level are converged (only a small G is applied for them: V G in
-// FP32 would put FP32 errors back into V for a close pair).
+// FP32 would put FP32 errors back into V for a close pair; near[] names such
+// pairs, whose blocks are then settled in FP64).
 __global__ void k_rf_g(int m, const cf *__restrict__ W, const zd *__restrict__ lam, float tiny, cf *__restrict__ G,
-                       int *__restrict__ part, RefineStat *__restrict__ st)
+                       int *__restrict__ part, int *__restrict__ near, RefineStat *__restrict__ st)
 {
     const int64_t total = (int64_t)m * m;
-    float gm = 0.f;
+    float gm = 0.f, wm = 0.f;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
          e += (int64_t)gridDim.x * blockDim.x) {
         const int i = (int)(e % m), j = (int)(e / m);
@@ -260,8 +263,15 @@ __global__ void k_rf_g(int m, const cf *__restrict__ W, const zd *__restrict__ l
             const zd dd = zsub(lam[j], lam[i]);
             const cf d = cmakef((float)dd.x, (float)dd.y);
             const float w2 = cabs2(w), d2 = cabs2(d);
+            wm = fmaxf(wm, w2);
             if (sqrtf(w2) <= tiny) {
-                if (w2 <= 1e-16f * d2 && d2 > 1e-30f) g = cdiv(w, d);
+                if (w2 <= 1e-16f * d2 && d2 > 1e-30f) {
+                    g = cdiv(w, d);
+                } else if (w2 <= RF_PAIR * RF_PAIR * d2 && d2 > 1e-30f) {
+                    atomicMax(near + i, j);
+                    atomicMax(near + j, i);
+                    st->tiny = 1;
+                }
             } else if (w2 <= RF_PAIR * RF_PAIR * d2 && d2 > 1e-30f) {
                 g = cdiv(w, d);
                 gm = fmaxf(gm, cabs2(g));
@@ -274,6 +284,7 @@ __global__ void k_rf_g(int m, const cf *__restrict__ W, const zd *__restrict__ l
         G[e] = g;
     }
     if (gm > 0.f) atomicMax(&st->gm, __float_as_uint(gm));
+    if (wm > 0.f) atomicMax(&st->wm, __float_as_uint(wm));
 }
 
 __device__ __forceinline__ zd rf_sqrt(zd z)
@@ -292,14 +303,19 @@ __device__ __forceinline__ zd rf_sqrt(zd z)
 // Lambda + W and the eigenvectors U = [1 pu_i; pu_j 1] (pd = det U), its
 // entries of G cleared.  lam_out is another array than lam.
 __global__ void k_rf_lambda(int m, const cf *__restrict__ W, const zd *__restrict__ lam, zd *__restrict__ lam_out,
-                            const int *__restrict__ part, cf *__restrict__ G, zd *__restrict__ pu,
-                            zd *__restrict__ pd, RefineStat *__restrict__ st)
+                            const int *__restrict__ part, const int *__restrict__ near, int *__restrict__ eff,
+                            cf *__restrict__ G, zd *__restrict__ pu, zd *__restrict__ pd, RefineStat *__restrict__ st)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m) return;
     const cf w = W[i + (int64_t)i * m];
     const zd li = zmake(lam[i].x + (double)w.x, lam[i].y + (double)w.y);
-    const int j = part[i];
+    int j = part[i];
+    if (j < 0) {
+        const int k = near[i];
+        if (k >= 0 && near[k] == i && part[k] < 0) j = k;
+    }
+    eff[i] = j;
     if (j < 0) lam_out[i] = li;
     if (j <= i) return;
     // block [a b; c d]: eigenvectors (1, c / g) and (-b / g, 1), g = h + s,
@@ -394,7 +410,7 @@ struct RefineCarve {
     cf *X, *T, *Q, *B32, *Y, *Uh, *V32, *L, *W, *G;   // X: [C | B^{-1}], 2 m^2 entries
     zd *AV, *BV, *Bu, *lam, *lam2, *pu, *pd;
     float *lower, *cmax, *nv, *part;
-    int *pair, *fail;
+    int *pair, *near, *eff, *fail;
     unsigned *amax;
     RefineStat *st;
     void *schur;
@@ -425,7 +441,9 @@ RefineCarve refine_carve(void *work, int m)
     w.cmax = w.lower + m;
     w.nv = (float *)take((size_t)m * sizeof(float));
     w.part = (float *)take(RF_PART * sizeof(float));
-    w.pair = (int *)take((size_t)m * sizeof(int));
+    w.pair = (int *)take(3 * (size_t)m * sizeof(int));
+    w.near = w.pair + m;
+    w.eff = w.near + m;
     w.fail = (int *)take(sizeof(int));
     w.amax = (unsigned *)take(8);
     w.st = (RefineStat *)take(sizeof(RefineStat));
@@ -555,13 +573,13 @@ static int refined_attempt(cudaStream_t s, int m, const zd *A, const zd *Bt, zd 
     for (float x : hp) dl += (double)x;
     dl = sqrt(dl);
     if (qfail || !(dl < 0.1)) return FEAST_OK;
-    double gprev = 0.0;
-    bool last64 = false;
+    double gprev = 0.0, wprev = 0.0;
+    bool last64 = false, ever = false;
     zd *lam = w.lam, *lam2 = w.lam2;
     for (int step = 0; step < RF_STEPS; ++step) {
         // the digit-sliced products while what they leave (about 1e-13 of
         // max|C| over a gap) is not yet what limits the result
-        const bool use_oz = oz && (prm.target > 1e-10 || (!last64 && (step == 0 || gprev > 1e-6)));
+        const bool use_oz = oz && (prm.target > 1e-10 || (!last64 && (step == 0 || gprev == 0.0 || gprev > 1e-6)));
         last64 = !use_oz;
         const bool timed = gt && !use_oz && gt->used + 2 <= GemmTimer::kMax;
         if (timed) FEAST_CUDA_TRY(cudaEventRecord(gt->ev[gt->used++], s));
@@ -583,19 +601,20 @@ static int refined_attempt(cudaStream_t s, int m, const zd *A, const zd *Bt, zd 
         FEAST_LAUNCH_CHECK();
         if ((e = mul32(0, m, m, m, fone, w.L, m, w.G, m, fzero, w.W, m))) return e;
         FEAST_CUDA_TRY(cudaMemsetAsync(w.st, 0, sizeof(RefineStat), s));
-        k_rf_g<<<grid_for(mm), 256, 0, s>>>(m, w.W, lam, (use_oz ? 1e-12f : 1e-14f) * cn, w.G, w.pair, w.st);
+        k_rf_g<<<grid_for(mm), 256, 0, s>>>(m, w.W, lam, (use_oz ? 1e-12f : 1e-14f) * cn, w.G, w.pair, w.near, w.st);
         FEAST_LAUNCH_CHECK();
-        k_rf_lambda<<<cdiv(m, 128), 128, 0, s>>>(m, w.W, lam, lam2, w.pair, w.G, w.pu, w.pd, w.st);
+        k_rf_lambda<<<cdiv(m, 128), 128, 0, s>>>(m, w.W, lam, lam2, w.pair, w.near, w.eff, w.G, w.pu, w.pd, w.st);
         FEAST_LAUNCH_CHECK();
         if ((e = mul32(0, m, m, m, fone, w.V32, m, w.G, m, fzero, w.Y, m))) return e;
         RefineStat hs;
         FEAST_CUDA_TRY(cudaMemcpyAsync(&hs, w.st, sizeof(hs), cudaMemcpyDeviceToHost, s));
         FEAST_CUDA_TRY(cudaStreamSynchronize(s));
         if (hs.bad) return FEAST_OK;
-        float g2;
+        float g2, w2;
         memcpy(&g2, &hs.gm, sizeof(float));
-        const double gm = sqrt((double)g2);
-        k_rf_update<<<grid_for(mm), 256, 0, s>>>(m, w.Y, w.pair, w.pu, hs.paired, V, w.V32);
+        memcpy(&w2, &hs.wm, sizeof(float));
+        const double gm = sqrt((double)g2), wm = sqrt((double)w2);
+        k_rf_update<<<grid_for(mm), 256, 0, s>>>(m, w.Y, w.eff, w.pu, hs.paired || hs.tiny, V, w.V32);
         FEAST_LAUNCH_CHECK();
         zd *t = lam;
         lam = lam2;
@@ -603,12 +622,14 @@ static int refined_attempt(cudaStream_t s, int m, const zd *A, const zd *Bt, zd 
         // what the step leaves: by the bound on delta, or by the contraction
         // seen (|G| over the step before's, at least delta); a pair's block is
         // followed by another step, and |G| that no longer falls is rounding
+        // (when |W| does not either: a close pair's G can stand still while
+        // the others still converge)
         const double ratio = gprev > 0.0 ? gm / gprev : 1e300;
         double left = gm * fmin(8.0 * fmax(gm, ratio), (double)m * gm + dl);
-        if (gm <= 1e-8 && step > 0 && ratio > 0.1 && ratio < 1e200) left = 0.0;
+        if (gm <= 1e-8 && step > 0 && ratio > 0.1 && ratio < 1e200 && wm > 0.1 * wprev) left = 0.0;
         res->steps = step + 1;
         res->resid = left;
-        if (!hs.paired && left <= prm.target && (!oz || prm.target > 1e-10 || last64)) {
+        if (!hs.paired && left <= (ever ? 0.25 : 1.0) * prm.target && (!oz || prm.target > 1e-10 || last64)) {
             if ((e = normalise_cols(s, m, V))) return e;
             k_rf_out<<<cdiv(m, 128), 128, 0, s>>>(m, lam, alpha, beta);
             FEAST_LAUNCH_CHECK();
@@ -623,11 +644,14 @@ static int refined_attempt(cudaStream_t s, int m, const zd *A, const zd *Bt, zd 
         } else {
             dl += (double)m * gm;
         }
-        if (hs.paired) {
-            k_rf_rows<<<grid_for(mm), 256, 0, s>>>(m, w.pair, w.pu, w.pd, w.L);
+        if (hs.paired || hs.tiny) {
+            k_rf_rows<<<grid_for(mm), 256, 0, s>>>(m, w.eff, w.pu, w.pd, w.L);
             FEAST_LAUNCH_CHECK();
         }
-        gprev = gm > 0.0 ? gm : 1e-30;
+        // (after a pair's block neither size says how the iteration contracts)
+        gprev = hs.paired ? 0.0 : gm > 0.0 ? gm : 1e-30;
+        wprev = wm;
+        ever = ever || hs.paired;
     }
     return FEAST_OK;
 }

@@ -717,7 +717,7 @@ __host__ __device__ inline int ez_ld(int m) { return m | 1; }   // odd: rows fal
 __host__ inline size_t ez_smem_bytes(int m)
 {
     return sizeof(zd) * (size_t)m * m + 4 * sizeof(cf) * (size_t)m * ez_ld(m) + sizeof(cf) * (size_t)m +
-           sizeof(zd) * (size_t)m + 4 * sizeof(float) * (size_t)m + 2 * sizeof(zd) * (size_t)m + sizeof(int) * (size_t)m;
+           sizeof(zd) * (size_t)m + 4 * sizeof(float) * (size_t)m + 2 * sizeof(zd) * (size_t)m + 2 * sizeof(int) * (size_t)m;
 }
 
 __global__ void __launch_bounds__(EZ_T) k_eig_refined(int m, const zd *__restrict__ A, int64_t lda, int64_t sA,
@@ -744,6 +744,7 @@ __global__ void __launch_bounds__(EZ_T) k_eig_refined(int m, const zd *__restric
     cf *H = (cf *)(pd + m), *Z = H + m * ld, *W = Z + m * ld, *L = W + m * ld, *hv = L + m * ld;
     float *lf = (float *)(hv + m);                  // lambda as double-single pairs: 4 floats each
     int *part = (int *)(lf + 4 * m);                // the index this one is too close to, or -1
+    int *near = part + m;                           // the same where the coupling is at rounding level
     const cf zero = cmakef(0.f, 0.f);
     if (t == 0) { s_ea = 0; s_eb = 0; s_bad = 0; *redo = 1; }
     __syncthreads();
@@ -843,8 +844,8 @@ __global__ void __launch_bounds__(EZ_T) k_eig_refined(int m, const zd *__restric
     }
     dl = sqrtf(ez_sum(dl, red));
     if (!(dl < 0.05f)) return;
-    bool done = false;
-    float gprev = 0.f;
+    bool done = false, ever = false;
+    float gprev = 0.f, wprev = 0.f;
     for (int step = 0; step < EZ_STEPS && !done; ++step) {
         for (int j = t; j < m; j += EZ_T) {
             const zd l = lam[j];
@@ -853,7 +854,7 @@ __global__ void __launch_bounds__(EZ_T) k_eig_refined(int m, const zd *__restric
             lf[4 * j + 1] = (float)(l.x - (double)hx);
             lf[4 * j + 2] = hy;
             lf[4 * j + 3] = (float)(l.y - (double)hy);
-            part[j] = -1;
+            part[j] = near[j] = -1;
         }
         // R' = 2^-ea (A V - B V Lambda), a 4 x 4 tile per thread, into W (FP32):
         // in double-single for the first step (whose V and Lambda are FP32;
@@ -915,7 +916,7 @@ __global__ void __launch_bounds__(EZ_T) k_eig_refined(int m, const zd *__restric
         }
         __syncthreads();
         ez_mul<false>(m, ld, H, W, Z);              // Z = L^H R'
-        float gm = 0.f;
+        float gm = 0.f, wm = 0.f;
         bool paired = false;
         for (int e = t; e < m * m; e += EZ_T) {
             const int i = e / m, j = e % m;
@@ -924,13 +925,19 @@ __global__ void __launch_bounds__(EZ_T) k_eig_refined(int m, const zd *__restric
             const cf d = cmakef((lf[4 * j] - lf[4 * i]) + (lf[4 * j + 1] - lf[4 * i + 1]),
                                 (lf[4 * j + 2] - lf[4 * i + 2]) + (lf[4 * j + 3] - lf[4 * i + 3]));
             const float w2 = cabs2(w), d2 = cabs2(d);
+            wm = fmaxf(wm, w2);
             cf gg = zero;
             if (sqrtf(w2) <= 1e-14f * cn) {
                 // coupling at rounding level: converged.  (For a close pair G
                 // may still be large, and V G in FP32 would put FP32 errors
-                // back into V: only a small one is applied.)
-                if (w2 <= 1e-16f * d2 && d2 > 1e-30f) W[i * ld + j] = cdiv(w, d);
-                else W[i * ld + j] = zero;
+                // back into V: only a small one is applied that way, a larger one
+                // as the pair's block, in FP64.)
+                const bool small = w2 <= 1e-16f * d2 && d2 > 1e-30f;
+                W[i * ld + j] = small ? cdiv(w, d) : zero;
+                if (!small && w2 <= EZ_PAIR * EZ_PAIR * d2 && d2 > 1e-30f) {
+                    atomicMax(near + i, j);
+                    atomicMax(near + j, i);
+                }
                 continue;
             } else if (w2 <= EZ_PAIR * EZ_PAIR * d2 && d2 > 1e-30f) {
                 gg = cdiv(w, d);
@@ -943,10 +950,19 @@ __global__ void __launch_bounds__(EZ_T) k_eig_refined(int m, const zd *__restric
             W[i * ld + j] = gg;
         }
         gm = sqrtf(ez_max(gm, red));                // (a barrier: s_bad, the pairs and G are out)
+        wm = sqrtf(ez_max(wm, red));
         paired = __syncthreads_or(paired);
         if (s_bad) return;
+        int mate = -1;
         if (t < m) {
-            const int i = t, j = part[t];
+            mate = part[t];
+            const int k = near[t];
+            if (mate < 0 && k >= 0 && near[k] == t && part[k] < 0) mate = k;
+        }
+        __syncthreads();
+        if (t < m) {
+            const int i = t, j = mate;
+            part[i] = j;
             const cf w = Z[i * ld + i];
             const zd li = zmake(lam[i].x + (double)w.x, lam[i].y + (double)w.y);
             if (j > i) {
@@ -1022,9 +1038,13 @@ __global__ void __launch_bounds__(EZ_T) k_eig_refined(int m, const zd *__restric
         // seen (|G| over the step before's, at least delta); a pair's block is
         // followed by another step
         const double seen = 8.0 * fmax((double)gm, (double)gm / (double)gprev), bnd = (double)m * (double)gm + (double)dl;
-        // (|G| that no longer falls is the residual's rounding)
-        done = !paired && ((double)gm * fmin(seen, bnd) <= EZ_DONE || (gm <= 1e-8f && step > 0 && gm > 0.1f * gprev));
-        gprev = gm;
+        // (|G| that no longer falls is the residual's rounding, when |W| does not
+        // either: a close pair's G can stand still while the others still converge)
+        done = !paired && ((double)gm * fmin(seen, bnd) <= (ever ? 0.25 : 1.0) * EZ_DONE || (gm <= 1e-8f && gprev > 0.f && gm > 0.1f * gprev && wm > 0.1f * wprev));
+        // (after a pair's block neither size says how the iteration contracts)
+        gprev = paired ? 0.f : gm;
+        wprev = wm;
+        ever = ever || paired;
     }
     if (!done) return;
     // unit columns, the eigenvalues on their own scale
