@@ -47,35 +47,62 @@ __global__ void k_zero_lower(int m, zd *__restrict__ R, int64_t ld)
     }
 }
 
-// Inverse of each CB x CB diagonal block of the upper triangular R (ld
-// ldr) into Ri (ld m): block b by CTA b, thread k builds column k of the
-// block's inverse by back-substitution.
-__global__ void __launch_bounds__(CB) k_trinv_diag(int m, const zd *__restrict__ R, int64_t ldr, zd *__restrict__ Ri)
+// X <- T^{-1}, T upper triangular CB x CB in shared memory, dinv its inverted
+// diagonal, by NT threads (from 16 CB / 2 up): adjacent inverted blocks
+// [A^{-1} B; 0 C^{-1}] get -A^{-1} B C^{-1}, from 1 x 1 blocks up.  Bound by
+// the FP64 units of one SM (a warp's instruction takes 64 clocks whatever its
+// lanes do): a back-substitution by one thread per column keeps one of the
+// four busy for 496 terms, the doubling spreads 256 dot products of at most
+// 16 terms over all of them.
+template <typename T, int NT>
+__device__ __forceinline__ void tri_inv_block(const T (*Tb)[CB + 1], T (*X)[CB + 1], const T *dinv)
 {
-    __shared__ zd T[CB][CB + 1];
+    static_assert(NT >= CB * CB / 4, "one entry per thread");
+    const int tid = threadIdx.x;
+    for (int e = tid; e < CB * CB; e += NT) X[e / CB][e % CB] = (e / CB == e % CB) ? dinv[e % CB] : cx<T>(0, 0);
+    __syncthreads();
+#pragma unroll
+    for (int L = 1; L < CB; L *= 2) {
+        const int p = tid / (L * L), r = tid % (L * L);
+        const bool on = tid < CB / 2 * L;
+        const int a0 = 2 * L * p, c0 = a0 + L;
+        if (on) {                                   // B C^{-1}: a column's lanes share the length of the sum
+            const int i = r % L, j = r / L;
+            T acc = cx<T>(0, 0);
+            for (int q = 0; q <= j; ++q) cfma(acc, Tb[a0 + i][c0 + q], X[c0 + q][c0 + j]);
+            X[a0 + i][c0 + j] = acc;
+        }
+        __syncthreads();
+        const int i = r / L, j = r % L;
+        T acc = cx<T>(0, 0);
+        if (on)                                     // -A^{-1} of that: a row's lanes share it
+            for (int q = i; q < L; ++q) cfma(acc, X[a0 + i][a0 + q], X[a0 + q][c0 + j]);
+        __syncthreads();
+        if (on) X[a0 + i][c0 + j] = cx<T>(-acc.x, -acc.y);
+        __syncthreads();
+    }
+}
+
+// Inverse of each CB x CB diagonal block of the upper triangular R (ld
+// ldr) into Ri (ld m): block b by CTA b.
+constexpr int TI = 256;
+__global__ void __launch_bounds__(TI) k_trinv_diag(int m, const zd *__restrict__ R, int64_t ldr, zd *__restrict__ Ri)
+{
+    __shared__ zd T[CB][CB + 1], X[CB][CB + 1], dinv[CB];
     const int b0 = blockIdx.x * CB;
     const int nb = (m - b0) < CB ? (m - b0) : CB;
-    const int k = threadIdx.x;
-    for (int i = 0; i < nb; ++i)
-        if (k < nb) T[i][k] = R[(b0 + i) + (int64_t)(b0 + k) * ldr];
-    __syncthreads();
-    if (k >= nb) return;
-    zd x[CB];
-#pragma unroll
-    for (int i = 0; i < CB; ++i) x[i] = zmake(0.0, 0.0);
-    x[k] = zdiv(zmake(1.0, 0.0), T[k][k]);
-#pragma unroll
-    for (int i = CB - 1; i >= 0; --i) {
-        if (i >= k) continue;
-        zd acc = zmake(0.0, 0.0);
-#pragma unroll
-        for (int p = 0; p < CB; ++p)
-            if (p > i && p <= k) zfma(acc, T[i][p], x[p]);
-        x[i] = zdiv(zmake(-acc.x, -acc.y), T[i][i]);
+    for (int e = threadIdx.x; e < CB * CB; e += TI) {
+        const int i = e % CB, k = e / CB;
+        const zd v = (i <= k && k < nb) ? R[(b0 + i) + (int64_t)(b0 + k) * ldr] : zmake(0.0, 0.0);
+        T[i][k] = v;
+        if (i == k) dinv[k] = k < nb ? zdiv(zmake(1.0, 0.0), v) : zmake(1.0, 0.0);
     }
-#pragma unroll
-    for (int i = 0; i < CB; ++i)
-        if (i < nb) Ri[(b0 + i) + (int64_t)(b0 + k) * m] = x[i];
+    __syncthreads();
+    tri_inv_block<zd, TI>(T, X, dinv);
+    for (int e = threadIdx.x; e < CB * CB; e += TI) {
+        const int i = e % CB, k = e / CB;
+        if (i < nb && k < nb) Ri[(b0 + i) + (int64_t)(b0 + k) * m] = X[i][k];
+    }
 }
 
 // The whole right-looking Cholesky in one cooperative launch (one CTA per
@@ -89,6 +116,18 @@ __global__ void __launch_bounds__(CB) k_trinv_diag(int m, const zd *__restrict__
 // pivot at or below tol times its reference (d0, or 1 without one) sets
 // *fail.
 constexpr int PT = 256;
+// *dp = the pivot d, or 1 (and *fail) where it is at or below tol times its
+// reference; its reciprocal.
+template <typename R, typename T>
+__device__ __forceinline__ void chol_pivot(R d, const double *ref, double tol, int *fail, R *dp, T *dinv)
+{
+    if (!((double)d > tol * *ref) || !(*ref > 0.0)) {
+        *fail = 1;
+        d = (R)1;
+    }
+    *dp = d;
+    *dinv = cx<T>((R)1 / d, 0);
+}
 template <typename T>
 __global__ void __launch_bounds__(PT, 1) k_chol_grid(int m, T *__restrict__ G, const double *__restrict__ d0,
                                                      double tol, int *__restrict__ fail, T *__restrict__ rinv,
@@ -97,7 +136,9 @@ __global__ void __launch_bounds__(PT, 1) k_chol_grid(int m, T *__restrict__ G, c
     using R = typename CxReal<T>::type;
     __shared__ T Tb[CB][CB + 1];
     __shared__ T P2[CB][CB + 1];
-    __shared__ R rsh;
+    __shared__ T dinv[CB];
+    __shared__ R dp[CB];
+    __shared__ double piv[CB];
     const int tid = threadIdx.x, lane = tid & 31;
     const int gwarp = blockIdx.x * (PT / 32) + (tid >> 5), nwarp = gridDim.x * (PT / 32);
     for (int k0 = 0; k0 < m; k0 += CB) {
@@ -109,56 +150,56 @@ __global__ void __launch_bounds__(PT, 1) k_chol_grid(int m, T *__restrict__ G, c
                 Tb[i][k] = (i < nb && k < nb) ? G[(k0 + i) + (int64_t)(k0 + k) * m] : cx<T>(0, 0);
             }
             __syncthreads();
+            // L D L^H with one barrier per column: warp 0 forms the next pivot
+            // and its reciprocal while the others update the rest of the
+            // triangle (row r and row n - 1 - r of it share a warp's lanes);
+            // the square roots come at the end, all at once
+            if (tid < CB) piv[tid] = (tid < nb && d0) ? d0[k0 + tid] : 1.0;
+            __syncthreads();
+            if (tid == 0) chol_pivot(Tb[0][0].x, piv, tol, fail, dp, dinv);
             for (int j = 0; j < nb; ++j) {
-                if (tid == 0) {
-                    const double d = (double)Tb[j][j].x, ref = d0 ? d0[k0 + j] : 1.0;
-                    R r;
-                    if (!(d > tol * ref) || !(ref > 0.0)) {
-                        *fail = 1;
-                        r = (R)1;
-                    } else {
-                        r = sqrt((R)d);
+                __syncthreads();
+                const R inv = dinv[j].x;
+                const int n = nb - 1 - j;
+                if (tid < 32) {
+                    if (tid == 0 && n > 0) {
+                        const T v = Tb[j][j + 1];
+                        const R d = Tb[j + 1][j + 1].x - (v.x * v.x + v.y * v.y) * inv;
+                        chol_pivot(d, piv + j + 1, tol, fail, dp + j + 1, dinv + j + 1);
                     }
-                    Tb[j][j] = cx<T>(r, 0);
-                    rsh = (R)1 / r;
+                    continue;
                 }
-                __syncthreads();
-                for (int k = j + 1 + tid; k < nb; k += PT) Tb[j][k] = cx<T>(Tb[j][k].x * rsh, Tb[j][k].y * rsh);
-                __syncthreads();
-                for (int e = tid; e < CB * CB; e += PT) {
-                    const int i = e % CB, k = e / CB;
-                    if (i > j && k >= i && k < nb) {
-                        const T rji = Tb[j][i], rjk = Tb[j][k];
-                        Tb[i][k] = cx<T>(Tb[i][k].x - (rji.x * rjk.x + rji.y * rjk.y),
-                                         Tb[i][k].y - (rji.x * rjk.y - rji.y * rjk.x));
-                    }
+                for (int f = (tid >> 5) - 1; f < (n + 1) / 2; f += PT / 32 - 1) {
+                    const bool second = lane >= n - f;
+                    const int row = second ? n - 1 - f : f, o = second ? lane - (n - f) : lane;
+                    if (second && (row == f || o > f)) continue;
+                    if (row == 0 && o == 0) continue;
+                    const int i = j + 1 + row, k = i + o;
+                    const T u = Tb[j][i], w = Tb[j][k], old = Tb[i][k];
+                    const R ux = u.x * inv, uy = u.y * inv;
+                    Tb[i][k] = cx<T>(old.x - (ux * w.x + uy * w.y), old.y - (ux * w.y - uy * w.x));
                 }
-                __syncthreads();
             }
+            __syncthreads();
+            if (tid < nb) {
+                const R r = sqrt(dp[tid]);
+                dp[tid] = r;
+                dinv[tid] = cx<T>((R)1 / r, 0);
+            }
+            if (tid >= nb && tid < CB) dinv[tid] = cx<T>(1, 0);
+            __syncthreads();
             for (int e = tid; e < CB * CB; e += PT) {
                 const int i = e % CB, k = e / CB;
-                if (i < nb && k < nb && k >= i) G[(k0 + i) + (int64_t)(k0 + k) * m] = Tb[i][k];
-            }
-            // R11^{-1} (upper), column k by thread k: back-substitution
-            if (tid < nb) {
-                const int k = tid;
-                T x[CB];
-#pragma unroll
-                for (int i = 0; i < CB; ++i) x[i] = cx<T>(0, 0);
-                x[k] = cx<T>((R)1 / Tb[k][k].x, 0);
-#pragma unroll
-                for (int i = CB - 1; i >= 0; --i) {
-                    if (i >= k) continue;
-                    T acc = cx<T>(0, 0);
-#pragma unroll
-                    for (int p = 0; p < CB; ++p)
-                        if (p > i && p <= k) cfma(acc, Tb[i][p], x[p]);
-                    const R di = (R)1 / Tb[i][i].x;
-                    x[i] = cx<T>(-acc.x * di, -acc.y * di);
+                T v = Tb[i][k];
+                if (i < nb && k < nb && k >= i) {
+                    v = (i == k) ? cx<T>(dp[i], 0) : cx<T>(v.x * dinv[i].x, v.y * dinv[i].x);
+                    Tb[i][k] = v;
+                    G[(k0 + i) + (int64_t)(k0 + k) * m] = v;
                 }
-#pragma unroll
-                for (int i = 0; i < CB; ++i) rinv[i + k * CB] = x[i];
             }
+            __syncthreads();
+            tri_inv_block<T, PT>(Tb, P2, dinv);
+            for (int e = tid; e < CB * CB; e += PT) rinv[e] = P2[e % CB][e / CB];
         }
         if (!grid_barrier(gs)) return;
         if (k1 >= m) break;
@@ -356,7 +397,7 @@ int tri_inverse(cudaStream_t s, int m, const zd *R, int64_t ldr, zd *Ri, zd *T)
 {
     if (m <= 0) return FEAST_OK;
     FEAST_CUDA_TRY(cudaMemsetAsync(Ri, 0, sizeof(zd) * (size_t)m * m, s));
-    k_trinv_diag<<<cdiv(m, CB), CB, 0, s>>>(m, R, ldr, Ri);
+    k_trinv_diag<<<cdiv(m, CB), TI, 0, s>>>(m, R, ldr, Ri);
     FEAST_LAUNCH_CHECK();
     const zd one = zmake(1.0, 0.0), mone = zmake(-1.0, 0.0), zero = zmake(0.0, 0.0);
     int e;

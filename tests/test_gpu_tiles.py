@@ -62,3 +62,24 @@ def test_tf32_split_gemm_edges(m, n, k, batch):
     for a, x, c in zip(A, X, fg.cgemm_tc(A, X)):
         ref = a.astype(np.complex128) @ x.astype(np.complex128)
         assert np.linalg.norm(c - ref) <= 2.0 ** -20 * np.sqrt(k) * max(np.linalg.norm(ref), 1e-30)
+
+
+@pytest.mark.parametrize("m0", [1, 2, 5, 31, 32, 33, 48, 63, 65, 97])
+def test_cholesky_blocks(m0):
+    """U2 R2 = B U1 at the edges of the 32-column Cholesky blocks and of the
+    halves their inverses are built from (FP64 up to 32 columns, the first
+    factorisation in FP32 from 33), U1 orthonormal: errors of m0 roundings of
+    B's norm, on top of 2^-48 n of the digit-sliced products."""
+    import paper_1404_1768_gb300 as fg
+    n = 128
+    rng = np.random.default_rng(m0)
+    B = np.eye(n) + 0.1 * inputs.complex_normal(rng, (n, n)) / np.sqrt(n)
+    U1 = np.linalg.qr(inputs.complex_normal(rng, (n, m0)))[0]
+    g = fg.Feast(B, B, U1.copy(), prec=fg.FEAST_C64_REFINE, q=8, center=0j, a=1.0)
+    g.set_subspace(U1)
+    U2, R2 = g.get("U2"), g.get("R2")
+    g.close()
+    tol = 4 * n * 2.0 ** -48 * np.linalg.norm(B, 2)
+    assert np.allclose(np.tril(R2, -1), 0) and np.all(np.diag(R2).real > 0)
+    assert np.abs(U2.conj().T @ U2 - np.eye(m0)).max() < tol
+    assert np.abs(U2 @ R2 - B @ U1).max() < tol
