@@ -230,6 +230,89 @@ __device__ __forceinline__ void cp_async(void *dst, const void *src, bool valid)
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
+// Division by b: the same bits as cdiv (Smith's form; each quotient is the
+// correctly rounded one, by Markstein's correction of n * (1 / d)), with the
+// divisor's part done once -- 32 divisions in turn are the solve's chain.
+// FP64: by the reciprocal.
+template <typename T>
+struct GbDiv;
+template <>
+struct GbDiv<cf> {
+    float r, d, y;
+    bool h;
+    __device__ __forceinline__ explicit GbDiv(cf b)
+    {
+        h = fabsf(b.x) >= fabsf(b.y);
+        const float p = h ? b.x : b.y, q = h ? b.y : b.x;
+        r = q / p;
+        d = fmaf(q, r, p);
+        y = 1.f / d;
+    }
+    __device__ __forceinline__ float quot(float n) const
+    {
+        const float q = n * y;
+        return fmaf(fmaf(-q, d, n), y, q);
+    }
+    __device__ __forceinline__ cf operator()(cf a) const
+    {
+        const float u = h ? a.x : a.y, v = h ? a.y : a.x;
+        const float im = fmaf(-u, r, v);
+        return cmakef(quot(fmaf(v, r, u)), quot(h ? im : -im));
+    }
+};
+template <>
+struct GbDiv<zd> {
+    zd inv;
+    __device__ __forceinline__ explicit GbDiv(zd b) : inv(crecip(b)) {}
+    __device__ __forceinline__ zd operator()(zd a) const { return zmul(a, inv); }
+};
+
+template <int N>
+struct GbInt {
+    static constexpr int value = N;
+};
+
+// C consecutive entries of a row of the window (shared memory), in 16-byte loads
+// where they divide it.
+template <int C, typename T>
+__device__ __forceinline__ void gb_row(T (&v)[C], const T *p)
+{
+    if constexpr (sizeof(T) < 16 && C * sizeof(T) % 16 == 0) {
+        union {
+            float4 f[C * sizeof(T) / 16];
+            T t[C];
+        } u;
+#pragma unroll
+        for (int i = 0; i < (int)(C * sizeof(T) / 16); ++i) u.f[i] = reinterpret_cast<const float4 *>(p)[i];
+#pragma unroll
+        for (int i = 0; i < C; ++i) v[i] = u.t[i];
+    } else {
+#pragma unroll
+        for (int i = 0; i < C; ++i) v[i] = p[i];
+    }
+}
+// acc[c] -= f_jj x_jj[c], jj = jj0 .. jc - 1: the factor's entries f[jj * fs], the
+// solved rows of the window from slot s on in steps of STEP (+-1, mod WL).
+template <int C, int STEP, int CW, typename T>
+__device__ __forceinline__ void gb_rank_update(T (&acc)[C], const T *f, int64_t fs, const T *W, int WL, int s, int jj0,
+                                               int jc)
+{
+    int sj = s + STEP * jj0;
+    if (sj >= WL) sj -= WL;
+    if (sj < 0) sj += WL;
+#pragma unroll 4
+    for (int jj = jj0; jj < jc; ++jj) {
+        const T u = cneg(f[jj * fs]);
+        T x[C];
+        gb_row<C>(x, W + (size_t)sj * CW);
+#pragma unroll
+        for (int c = 0; c < C; ++c) cfma(acc[c], u, x[c]);
+        sj += STEP;
+        if (STEP > 0 && sj == WL) sj = 0;
+        if (STEP < 0 && sj < 0) sj = WL - 1;
+    }
+}
+
 // Forward pass of the solve (unblocked convention: for j = 0..n-1, swap
 // rows j and piv[j], then rows j+1 .. j+kl -= l_j x_j), taken jc steps at a
 // time.  Within a chunk the interchanges commute to the front: the chunk is
@@ -240,18 +323,26 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // side, a lane per row, the solved value passed by shuffles), (3) one
 // rank-jc update of the kl rows below it.  CTA = (chunk of cw <= GB_CW
 // right-hand sides, node); the right-hand sides live in a circular window
-// of WL = kl + 1 + jcm rows in shared memory, the chunk's multipliers
-// (jcm + kl rows x jcm columns, column-major) and pivots beside it, in
-// nbuf = 2 buffers when they fit (the next chunk's copied in meanwhile).
+// of WL = kl + 1 + jcm rows of cw entries in shared memory, the chunk's
+// multipliers (jcm + kl rows x jcm columns, column-major) and pivots beside it,
+// in nbuf = 2 buffers when they fit (the next chunk's copied in meanwhile).
+//
+// Bound by the chain of chunks (512 of them at n = 16384): the solve's shuffles
+// and the update's FP32 rate on one SM.  The window keeps the right-hand sides
+// of a row together, so an update step reads its cw solved values in cw / 2
+// loads; the copies run a warp per column without a division; only the
+// interchanges that move a row are walked; up to kl = 128 the two halves of the
+// CTA share the right-hand sides of a row.  n = 16384, kl = ku = 128, 16 nodes
+// x 64 right-hand sides: before, forward 3.82 ms and backward 7.01 ms.
 template <typename T, int CW>
 __global__ void __launch_bounds__(GB_ST) k_gb_fwd(int64_t n, int64_t kl, int64_t ku, int64_t nrhs,
                                                   const T *F, int64_t ldab, int64_t sF, const int *piv, T *X,
                                                   int64_t ldx, int64_t sX, int jcm, int nbuf)
 {
-    constexpr int cw = CW;
+    constexpr int cw = CW, NW = GB_ST / 32;
     extern __shared__ __align__(16) unsigned char sm_raw[];
     const int WL = (int)(kl + 1 + jcm), LR = (int)(jcm + kl), kv = (int)(kl + ku);
-    T *W = reinterpret_cast<T *>(sm_raw);      // cw columns of WL slots: row r of column cc at W[cc * WL + r % WL]
+    T *W = reinterpret_cast<T *>(sm_raw);      // WL slots of cw entries: row r of column cc at W[(r % WL) * cw + cc]
     T *const Lb0 = W + (size_t)WL * cw;         // LR x jcm: Lb[jj * LR + rho] = L'(j0 + rho, j0 + jj)
     T *const Lb1 = Lb0 + (size_t)(nbuf - 1) * LR * jcm;
     int *const pb0 = reinterpret_cast<int *>(Lb0 + (size_t)nbuf * LR * jcm);   // the chunk's pivots (global rows)
@@ -265,20 +356,20 @@ __global__ void __launch_bounds__(GB_ST) k_gb_fwd(int64_t n, int64_t kl, int64_t
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     auto stage = [&](int64_t js, T *Lb, int *ps) {
         const int jcs = (int)((n - js) < jcm ? (n - js) : jcm);
-        for (int e = threadIdx.x; e < LR * jcs; e += GB_ST) {
-            const int jj = e / LR, rho = e % LR;
-            const int64_t r = js + rho, c = js + jj;
-            const bool in = rho > jj && rho <= jj + kl && r < n;
-            cp_async<sizeof(T)>(Lb + jj * LR + rho, in ? (const void *)(Fb + bidx(kv, ldab, r, c)) : (const void *)Fb,
-                                in);
+        for (int jj = wid; jj < jcs; jj += NW) {
+            const T *col = Fb + bidx(kv, ldab, js, js + jj);
+            for (int rho = lane; rho < LR; rho += 32) {
+                const bool in = rho > jj && rho <= jj + kl && js + rho < n;
+                cp_async<sizeof(T)>(Lb + jj * LR + rho, in ? (const void *)(col + rho) : (const void *)Fb, in);
+            }
         }
         if (threadIdx.x < jcs) cp_async<4>(ps + threadIdx.x, pv + js + threadIdx.x, true);
     };
-    for (int e = threadIdx.x; e < WL * cw; e += GB_ST) {
-        const int r = e % WL, cc = e / WL;
-        const bool in = r < n && cc < ncol;
-        cp_async<sizeof(T)>(W + cc * WL + r, in ? (const void *)(Xb + r + (c0 + cc) * ldx) : (const void *)Xb, in);
-    }
+    for (int cc = wid; cc < cw; cc += NW)
+        for (int r = lane; r < WL; r += 32) {
+            const bool in = r < n && cc < ncol;
+            cp_async<sizeof(T)>(W + r * cw + cc, in ? (const void *)(Xb + r + (c0 + cc) * ldx) : (const void *)Xb, in);
+        }
     stage(0, Lb0, pb0);
     cp_async_commit();
     int k = 0;
@@ -289,27 +380,24 @@ __global__ void __launch_bounds__(GB_ST) k_gb_fwd(int64_t n, int64_t kl, int64_t
         const int *ps = (k & 1) ? pb1 : pb0;
         cp_async_wait_all();
         __syncthreads();
-        if (threadIdx.x < cw) {
-            // (1) the chunk's interchanges, in order, on this right-hand side
-            const int cc = threadIdx.x;
-            for (int jj = 0; jj < jc; ++jj) {
-                const int p = (int)(ps[jj] - j0);
-                if (p != jj) {
-                    int sa = s0 + jj, sb = s0 + p;
+        if (wid < 2) {
+            const int pl = lane < jc ? (int)(ps[lane] - j0) : lane;
+            unsigned moves = __ballot_sync(0xffffffffu, pl != lane);
+            while (moves) {
+                const int jp = __ffs(moves) - 1, p = __shfl_sync(0xffffffffu, pl, jp);
+                moves &= moves - 1;
+                if (wid == 0 && lane < cw) {
+                    // (1) the chunk's interchanges, in order, on the right-hand sides
+                    int sa = s0 + jp, sb = s0 + p;
                     if (sa >= WL) sa -= WL;
                     if (sb >= WL) sb -= WL;
-                    const T t = W[cc * WL + sa];
-                    W[cc * WL + sa] = W[cc * WL + sb];
-                    W[cc * WL + sb] = t;
+                    const T t = W[sa * cw + lane];
+                    W[sa * cw + lane] = W[sb * cw + lane];
+                    W[sb * cw + lane] = t;
                 }
-            }
-        } else if (threadIdx.x >= 32 && threadIdx.x < 32 + jc) {
-            // L'_jj: the later interchanges of the chunk on column jj
-            const int jj = threadIdx.x - 32;
-            T *col = Lb + jj * LR;
-            for (int jp = jj + 1; jp < jc; ++jp) {
-                const int p = (int)(ps[jp] - j0);
-                if (p != jp) {
+                if (wid == 1 && lane < jp) {
+                    // L'_jj: the later interchanges of the chunk on column jj
+                    T *col = Lb + lane * LR;
                     const T t = col[jp];
                     col[jp] = col[p];
                     col[p] = t;
@@ -326,49 +414,51 @@ __global__ void __launch_bounds__(GB_ST) k_gb_fwd(int64_t n, int64_t kl, int64_t
         if (wid < cw) {
             int sl = s0 + lane;
             if (sl >= WL) sl -= WL;
-            T x = (lane < jc) ? W[wid * WL + sl] : cx<T>(0, 0);
-            for (int jj = 0; jj + 1 < jc; ++jj) {
+            T x = (lane < jc) ? W[sl * cw + wid] : cx<T>(0, 0);
+#pragma unroll 8
+            for (int jj = 0; jj < jc - 1; ++jj) {
+                const T l = cneg(Lb[jj * LR + (lane < jc ? lane : 0)]);
                 const T xj = shfl_cx(x, jj);
-                if (lane > jj && lane < jc) cfma(x, cneg(Lb[jj * LR + lane]), xj);
+                if (lane > jj && lane < jc) cfma(x, l, xj);
             }
             if (lane < jc) {
-                W[wid * WL + sl] = x;
+                W[sl * cw + wid] = x;
                 if (wid < ncol) Xb[j0 + lane + (c0 + wid) * ldx] = x;
             }
         }
         __syncthreads();
         // (3) rows j0 + jc .. j0 + jc + kl - 1 -= L'(those rows, chunk) x(chunk):
-        // a thread per row and all cw right-hand sides (one multiplier load
-        // per cw products; the x values are broadcast)
-        for (int t = threadIdx.x; t < kl; t += GB_ST) {
-            const int64_t r = j0 + jc + t;
-            if (r >= n) continue;
-            int sr = s0 + jc + t;
-            while (sr >= WL) sr -= WL;
-            T acc[CW];
+        // a thread per row and all cw right-hand sides, or half of them (one
+        // multiplier load per cw products; the x values are broadcast)
+        auto update = [&](auto cn, int t0, int step, int cc) {
+            constexpr int C = decltype(cn)::value;
+            for (int t = t0; t < kl; t += step) {
+                if (j0 + jc + t >= n) break;
+                int sr = s0 + jc + t;
+                while (sr >= WL) sr -= WL;
+                T acc[C];
+                gb_row<C>(acc, W + sr * cw + cc);
+                gb_rank_update<C, 1, CW>(acc, Lb + jc + t, LR, W + cc, WL, s0, 0, jc);
 #pragma unroll
-            for (int cc = 0; cc < CW; ++cc) acc[cc] = W[cc * WL + sr];
-            int sj = s0;
-            for (int jj = 0; jj < jc; ++jj) {
-                const T l = cneg(Lb[jj * LR + jc + t]);
-#pragma unroll
-                for (int cc = 0; cc < CW; ++cc) cfma(acc[cc], l, W[cc * WL + sj]);
-                if (++sj == WL) sj = 0;
+                for (int c = 0; c < C; ++c) W[sr * cw + cc + c] = acc[c];
             }
-#pragma unroll
-            for (int cc = 0; cc < CW; ++cc) W[cc * WL + sr] = acc[cc];
-        }
+        };
+        if (CW >= 4 && kl <= GB_ST / 2)
+            update(GbInt<(CW >= 4 ? CW / 2 : CW)>(), threadIdx.x % (GB_ST / 2), GB_ST / 2,
+                   (threadIdx.x / (GB_ST / 2)) * (CW / 2));
+        else
+            update(GbInt<CW>(), threadIdx.x, GB_ST, 0);
         __syncthreads();
         // rows j0 .. j0+jc-1 are final; their slots take rows j0+WL ..
-        for (int e = threadIdx.x; e < jc * cw; e += GB_ST) {
-            const int jj = e / cw, cc = e % cw;
-            const int64_t r = j0 + jj + WL;
-            int sl = s0 + jj;
-            if (sl >= WL) sl -= WL;
-            const bool in = r < n && cc < ncol;
-            cp_async<sizeof(T)>(W + cc * WL + sl, in ? (const void *)(Xb + r + (c0 + cc) * ldx) : (const void *)Xb,
-                                in);
-        }
+        for (int cc = wid; cc < cw; cc += NW)
+            if (lane < jc) {
+                const int64_t r = j0 + lane + WL;
+                int sl = s0 + lane;
+                if (sl >= WL) sl -= WL;
+                const bool in = r < n && cc < ncol;
+                cp_async<sizeof(T)>(W + sl * cw + cc, in ? (const void *)(Xb + r + (c0 + cc) * ldx) : (const void *)Xb,
+                                    in);
+            }
         if (nbuf == 1 && more) stage(j0 + jcm, Lb0, pb0);   // (its buffer is free only now)
         cp_async_commit();
     }
@@ -377,19 +467,20 @@ __global__ void __launch_bounds__(GB_ST) k_gb_fwd(int64_t n, int64_t kl, int64_t
 
 // Backward pass: for j = n-1..0: x_j /= U(j,j); rows j-kv .. j-1 -= U(:, j) x_j,
 // taken jc columns at a time: an upper triangular solve on the chunk's rows
-// (a warp per right-hand side), then one rank-jc update of the kv rows
-// above it.  Window of WL = kv + 1 + jcm rows; the chunk's columns of U
-// (diagonal included) staged column-major, Us[jj * (kv + 1) + t] =
-// U(j - t, j) with j = j1 - jj, in nbuf buffers as in the forward pass.
+// (a warp per right-hand side; the divisions prepared first, all at once),
+// then one rank-jc update of the kv rows above it.  Window of WL = kv + 1 + jcm
+// rows; the chunk's columns of U (diagonal included) staged column-major,
+// Us[jj * (kv + 1) + t] = U(j - t, j) with j = j1 - jj, in nbuf buffers as in the
+// forward pass.
 template <typename T, int CW>
 __global__ void __launch_bounds__(GB_ST) k_gb_bwd(int64_t n, int64_t kl, int64_t ku, int64_t nrhs,
                                                   const T *F, int64_t ldab, int64_t sF, T *X,
                                                   int64_t ldx, int64_t sX, int jcm, int nbuf)
 {
-    constexpr int cw = CW;
+    constexpr int cw = CW, NW = GB_ST / 32;
     extern __shared__ __align__(16) unsigned char sm_raw[];
     const int kv = (int)(kl + ku), WL = kv + 1 + jcm, UL = kv + 1;
-    T *W = reinterpret_cast<T *>(sm_raw);      // cw columns of WL slots: row r of column cc at W[cc * WL + r % WL]
+    T *W = reinterpret_cast<T *>(sm_raw);      // WL slots of cw entries: row r of column cc at W[(r % WL) * cw + cc]
     T *const Ub0 = W + (size_t)WL * cw;
     T *const Ub1 = Ub0 + (size_t)(nbuf - 1) * jcm * UL;
     const int b = blockIdx.y;
@@ -400,23 +491,23 @@ __global__ void __launch_bounds__(GB_ST) k_gb_bwd(int64_t n, int64_t kl, int64_t
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     auto stage = [&](int64_t js, T *Us) {
         const int jcs = (int)((js + 1) < jcm ? (js + 1) : jcm);
-        for (int e = threadIdx.x; e < jcs * UL; e += GB_ST) {
-            const int jj = e / UL, t = e % UL;
-            const int64_t c = js - jj, r = c - t;
-            const bool in = r >= 0;
-            cp_async<sizeof(T)>(Us + jj * UL + t, in ? (const void *)(Fb + bidx(kv, ldab, r, c)) : (const void *)Fb,
-                                in);
+        for (int jj = wid; jj < jcs; jj += NW) {
+            const int64_t c = js - jj;
+            const T *col = Fb + bidx(kv, ldab, c, c);
+            for (int t = lane; t < UL; t += 32) {
+                const bool in = c - t >= 0;
+                cp_async<sizeof(T)>(Us + jj * UL + t, in ? (const void *)(col - t) : (const void *)Fb, in);
+            }
         }
     };
-    for (int e = threadIdx.x; e < WL * cw; e += GB_ST) {
-        const int t = e % WL, cc = e / WL;
-        const int64_t r = n - 1 - t;
-        if (r >= 0) {
+    for (int cc = wid; cc < cw; cc += NW)
+        for (int t = lane; t < WL; t += 32) {
+            const int64_t r = n - 1 - t;
+            if (r < 0) break;
             const bool in = cc < ncol;
-            cp_async<sizeof(T)>(W + cc * WL + (int)(r % WL), in ? (const void *)(Xb + r + (c0 + cc) * ldx)
+            cp_async<sizeof(T)>(W + (int)(r % WL) * cw + cc, in ? (const void *)(Xb + r + (c0 + cc) * ldx)
                                                                 : (const void *)Xb, in);
         }
-    }
     stage(n - 1, Ub0);
     cp_async_commit();
     int k = 0;
@@ -435,55 +526,50 @@ __global__ void __launch_bounds__(GB_ST) k_gb_bwd(int64_t n, int64_t kl, int64_t
         if (wid < cw) {
             int sl = s1 - lane;
             if (sl < 0) sl += WL;
-            T x = (lane < jc) ? W[wid * WL + sl] : cx<T>(0, 0);
+            T x = (lane < jc) ? W[sl * cw + wid] : cx<T>(0, 0);
+            const GbDiv<T> div((lane < jc) ? Us[lane * UL] : cx<T>(1, 0));
+#pragma unroll 8
             for (int jj = 0; jj < jc; ++jj) {
-                if (lane == jj) x = cdiv(x, Us[jj * UL]);
-                const T xj = shfl_cx(x, jj);
                 const int t = lane - jj;
-                if (t > 0 && t <= kv && lane < jc) cfma(x, cneg(Us[jj * UL + t]), xj);
+                const bool on = t > 0 && t <= kv && lane < jc;
+                const T u = cneg(Us[jj * UL + (on ? t : 0)]);
+                const T y = div(x);
+                const T xj = shfl_cx(y, jj);
+                if (t == 0) x = y;
+                if (on) cfma(x, u, xj);
             }
             if (lane < jc) {
-                W[wid * WL + sl] = x;
+                W[sl * cw + wid] = x;
                 if (wid < ncol) Xb[j1 - lane + (c0 + wid) * ldx] = x;
             }
         }
         __syncthreads();
         // rows above the chunk: r = j1 - jc - tt, tt = 0 .. kv-1, a thread
-        // per row and all cw right-hand sides
+        // per row and all cw right-hand sides (column jj reaches it from
+        // jj = jc + tt - kv on)
         for (int tt = threadIdx.x; tt < kv; tt += GB_ST) {
-            const int64_t r = j1 - jc - tt;
-            if (r < 0) continue;
+            if (j1 - jc - tt < 0) break;
             int sr = s1 - jc - tt;
             while (sr < 0) sr += WL;
             T acc[CW];
+            gb_row<CW>(acc, W + sr * cw);
+            const int jj0 = jc + tt > kv ? jc + tt - kv : 0;
+            gb_rank_update<CW, -1, CW>(acc, Us + jc + tt, (int64_t)UL - 1, W, WL, s1, jj0, jc);
 #pragma unroll
-            for (int cc = 0; cc < CW; ++cc) acc[cc] = W[cc * WL + sr];
-            int sj = s1;
-            for (int jj = 0; jj < jc; ++jj) {
-                const int t = jc - jj + tt;       // (j1 - jj) - r
-                if (t <= kv) {
-                    const T u = cneg(Us[jj * UL + t]);
-#pragma unroll
-                    for (int cc = 0; cc < CW; ++cc) cfma(acc[cc], u, W[cc * WL + sj]);
-                }
-                if (--sj < 0) sj = WL - 1;
-            }
-#pragma unroll
-            for (int cc = 0; cc < CW; ++cc) W[cc * WL + sr] = acc[cc];
+            for (int c = 0; c < CW; ++c) W[sr * cw + c] = acc[c];
         }
         __syncthreads();
         // rows j1-jc+1 .. j1 are final; their slots take rows j - WL
-        for (int e = threadIdx.x; e < jc * cw; e += GB_ST) {
-            const int jj = e / cw, cc = e % cw;
-            const int64_t r = j1 - jj - WL;
-            int sl = s1 - jj;
-            if (sl < 0) sl += WL;
-            if (r >= 0) {
+        for (int cc = wid; cc < cw; cc += NW)
+            if (lane < jc) {
+                const int64_t r = j1 - lane - WL;
+                int sl = s1 - lane;
+                if (sl < 0) sl += WL;
                 const bool in = cc < ncol;
-                cp_async<sizeof(T)>(W + cc * WL + sl, in ? (const void *)(Xb + r + (c0 + cc) * ldx) : (const void *)Xb,
-                                    in);
+                if (r >= 0)
+                    cp_async<sizeof(T)>(W + sl * cw + cc, in ? (const void *)(Xb + r + (c0 + cc) * ldx)
+                                                             : (const void *)Xb, in);
             }
-        }
         if (nbuf == 1 && more) stage(j1 - jcm, Ub0);
         cp_async_commit();
     }
@@ -507,18 +593,24 @@ __global__ void k_gb_matmul(int64_t n, int64_t kl, int64_t ku, const zd *M, int6
 }
 
 // The whole band LU of one node in one cluster of GL_C CTAs (complex64;
-// one launch for all nodes): for each panel of nb columns, every CTA of the
-// cluster (1) copies the panel's nb + kl rows into its shared memory and
-// (2) factors it there with partial pivoting (pivot: largest |.|^2, the
-// first on ties) -- the same arithmetic in the same order in every CTA, so
-// their panels agree bit for bit and nothing is exchanged; then each CTA
-// takes its own slice of the kv columns right of the panel: (3) the
-// panel's interchanges, (4) U12 = L11^{-1} A12 (a warp per column, in
-// shared memory), (5) A22 -= L21 U12 on the band (a warp per 32 rows x 4
-// columns); (6) CTA 0 writes the panel back with its multipliers in the
-// unblocked convention.  A cluster barrier closes each panel.  The same
-// factors as the multi-launch form; the clusters (nodes) never wait for
-// one another.
+// one launch for all nodes), GL_NB columns at a time.  Every CTA of the cluster
+// factors the panel's nb + kl rows with partial pivoting (pivot: largest |.|^2,
+// the first on ties) -- the same arithmetic in the same order in every CTA, so
+// their panels agree bit for bit and nothing is exchanged -- and takes its own
+// slice of the kv columns right of the panel: U12 = L11^{-1} A12, then
+// A22 -= L21 U12.  A cluster barrier closes each panel; the clusters (nodes)
+// never wait for one another.
+//
+// Bound by the chain of pivots, 32 a panel: a thread keeps its row (RPT rows
+// from 256 up) in registers for the whole panel and only its position moves, so
+// an interchange costs nothing; each warp offers its best row in shared memory
+// and one barrier a column settles the pivot.  The multipliers go back in the
+// unblocked convention as they arise (column j by CTA j mod GL_C, at the
+// positions of step j).  The slice right of the panel is copied to shared memory
+// under the panel and read there through the final positions.  Before, each
+// column took four barriers and a pass over the panel in shared memory, and the
+// interchanges right of it were a chain of loads and stores in L2: 49.5 ms
+// for 16 nodes of n = 16384, kl = ku = 128.
 constexpr int GL_T = 256;
 constexpr int GL_C = 8;          // CTAs per node (a portable cluster)
 constexpr int GL_NB = 32;
@@ -532,193 +624,199 @@ __device__ __forceinline__ void gl_cluster_sync()
 {
     asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-template <typename T>
-__global__ void __launch_bounds__(GL_T) k_gb_lu_fused(int64_t n, int kl, int ku, T *F, int64_t ldab, int64_t sF,
-                                                     int *piv, int nbp, int *info, int *row)
+// Order of the pivot search: 0 no candidate, 1 a NaN on the diagonal (taken
+// when there is nothing else), 2 zero, then by magnitude.
+__device__ __forceinline__ unsigned gl_key(cf v, bool diag)
 {
-    typedef typename CxReal<T>::type R;
+    const unsigned b = __float_as_uint(cabs2(v));
+    return b > 0x7f800000u ? (diag ? 1u : 0u) : b + 2u;
+}
+template <int RPT>
+__global__ void __launch_bounds__(GL_T) k_gb_lu_fused(int64_t n, int kl, int ku, cf *F, int64_t ldab, int64_t sF,
+                                                     int *piv, int tc, int *info, int *row)
+{
+    constexpr int NB = GL_NB, NW = GL_T / 32;
     extern __shared__ __align__(16) unsigned char sm_raw[];
-    const int kv = kl + ku, ldd = nbp + kl;
+    __shared__ __align__(16) cf s_row[2][NW][NB];
+    __shared__ unsigned s_key[2][NW];
+    __shared__ int s_pos[2][NW];
+    __shared__ int s_piv[NB];
+    const int kv = kl + ku, ldd = NB + kl, ldu = tc + 2;
     const int rank = (int)gl_rank(), kvs = (kv + GL_C - 1) / GL_C;
-    const int cb = rank * kvs, ce = (cb + kvs < kv) ? cb + kvs : kv;   // this CTA's columns cc in [cb, ce)
-    const int nc = ce > cb ? ce - cb : 0, ldu = kvs + 1;
-    T *D = reinterpret_cast<T *>(sm_raw);      // ldd x nbp panel, column-major
-    T *U = D + (size_t)ldd * nbp;               // nbp x kvs slice of U12, row-major: U[k * ldu + cc - cb]
-    int *ps = reinterpret_cast<int *>(U + (size_t)nbp * ldu);  // local pivots of the panel
-    __shared__ R s_val[GL_T / 32];
-    __shared__ int s_idx[GL_T / 32];
-    __shared__ int s_p;
+    const int cb = rank * kvs, ce = (cb + kvs < kv) ? cb + kvs : kv;   // this CTA's columns [cb, ce) right of a panel
+    cf *D = reinterpret_cast<cf *>(sm_raw);          // the factored panel by final position, column-major
+    cf *U = D + (size_t)ldd * NB;                     // NB x tc slice of U12, row-major
+    cf *Tr = U + (size_t)NB * ldu;                    // the rows of tc columns right of the panel, column-major
+    int *prow = reinterpret_cast<int *>(Tr + (size_t)tc * ldd);   // row of the panel that ends at a position
     const int b = blockIdx.x / GL_C;
-    T *Fb = F + (int64_t)b * sF;
+    cf *Fb = F + (int64_t)b * sF;
     int *pvb = piv + (int64_t)b * n;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const T zero = cx<T>(0, 0);
-    for (int64_t k0 = 0; k0 < n; k0 += nbp) {
-        const int nb = (int)((n - k0) < nbp ? (n - k0) : nbp);
+    const cf zero = cmakef(0.f, 0.f);
+    for (int64_t k0 = 0; k0 < n; k0 += NB) {
+        const int nb = (int)((n - k0) < NB ? (n - k0) : NB);
         const int rows = (int)((n - k0) < ldd ? (n - k0) : ldd);
-        // (1) gather (asynchronous copies, all in flight at once)
-        for (int e = tid; e < ldd * nb; e += GL_T) {
-            const int r = e % ldd, cc = e / ldd;
-            const int64_t i = k0 + r, c = k0 + cc;
-            const bool in = r < rows && i - c <= kl && c - i <= kv;
-            cp_async<sizeof(T)>(D + cc * ldd + r, in ? (const void *)(Fb + bidx(kv, ldab, i, c)) : (const void *)Fb, in);
+        auto gather = [&](int x0) {
+            const int w = (ce - x0) < tc ? (ce - x0) : tc;
+            for (int cl = wid; cl < w; cl += NW) {
+                const int64_t c = k0 + nb + x0 + cl;
+                for (int r = lane; r < rows; r += 32) {
+                    const bool in = c < n && c - (k0 + r) <= kv;
+                    cp_async<sizeof(cf)>(Tr + cl * ldd + r, in ? (const void *)(Fb + bidx(kv, ldab, k0 + r, c)) : (const void *)Fb,
+                                         in);
+                }
+            }
+            cp_async_commit();
+        };
+        // the panel, a row per thread (a warp's loads run along the columns)
+        cf a[RPT][NB];
+        int pos[RPT];
+#pragma unroll
+        for (int q = 0; q < RPT; ++q) {
+            const int r = tid + q * GL_T;
+            pos[q] = r;
+#pragma unroll
+            for (int cc = 0; cc < NB; ++cc) {
+                const bool in = r < rows && cc < nb && r - cc <= kl && cc - r <= kv;
+                a[q][cc] = in ? Fb[bidx(kv, ldab, k0 + r, k0 + cc)] : zero;
+            }
         }
-        cp_async_commit();
-        cp_async_wait_all();
-        __syncthreads();
-        // every CTA holds the panel before CTA 0 can write it back (step 6)
+        if (cb < ce) gather(cb);
+        // every CTA holds the panel before any of it is written back
         gl_cluster_sync();
-        // (2) panel LU
-        for (int j = 0; j < nb; ++j) {
-            const T *dj = D + j * ldd;
-            R best = -1;
-            int bi = j;
-            for (int r = j + tid; r < rows; r += GL_T) {
-                const R v = cabs2(dj[r]);
-                if (v > best) { best = v; bi = r; }
-            }
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                const R ov = __shfl_down_sync(0xffffffffu, best, off);
-                const int oi = __shfl_down_sync(0xffffffffu, bi, off);
-                if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
+        for (int j = 0; j < NB; ++j) {
+            if (j >= nb) break;
+            const int pb = j & 1;
+            unsigned key[RPT], km = 0;
+#pragma unroll
+            for (int q = 0; q < RPT; ++q) {
+                key[q] = (pos[q] >= j && pos[q] < rows) ? gl_key(a[q][j], pos[q] == j) : 0u;
+                km = key[q] > km ? key[q] : km;
             }
-            if (lane == 0) { s_val[wid] = best; s_idx[wid] = bi; }
+            km = __reduce_max_sync(0xffffffffu, km);
+            int pm = 0x7fffffff;
+#pragma unroll
+            for (int q = 0; q < RPT; ++q)
+                if (key[q] == km && pos[q] < pm) pm = pos[q];
+            pm = __reduce_min_sync(0xffffffffu, pm);
+#pragma unroll
+            for (int q = 0; q < RPT; ++q)
+                if (pos[q] == pm && km > 0) {
+#pragma unroll
+                    for (int cc = 0; cc < NB; ++cc)
+                        if (cc >= j) s_row[pb][wid][cc] = a[q][cc];
+                }
+            if (lane == 0) {
+                s_key[pb][wid] = km;
+                s_pos[pb][wid] = pm;
+            }
             __syncthreads();
-            // every warp reduces the warp partials itself (a shuffle tree in
-            // the same order everywhere)
-            R bv = (lane < GL_T / 32) ? s_val[lane] : (R)-1;
-            int p = (lane < GL_T / 32) ? s_idx[lane] : j;
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                const R ov = __shfl_xor_sync(0xffffffffu, bv, off);
-                const int oi = __shfl_xor_sync(0xffffffffu, p, off);
-                if (ov > bv || (ov == bv && oi < p)) { bv = ov; p = oi; }
-            }
+            const unsigned kk = lane < NW ? s_key[pb][lane] : 0u;
+            const int pp = lane < NW ? s_pos[pb][lane] : 0x7fffffff;
+            const unsigned kbest = __reduce_max_sync(0xffffffffu, kk);
+            const int p = __reduce_min_sync(0xffffffffu, (lane < NW && kk == kbest) ? pp : 0x7fffffff);
+            const int src = __ffs(__ballot_sync(0xffffffffu, lane < NW && kk == kbest && pp == p)) - 1;
+            const cf *pr = s_row[pb][src];
             if (tid == 0) {
-                ps[j] = p;
-                if (bv == 0 && rank == 0 && info && atomicCAS(info, 0, b + 1) == 0 && row) *row = (int)(k0 + j) + 1;
+                s_piv[j] = p;
+                if (kbest == 2u && rank == 0 && info && atomicCAS(info, 0, b + 1) == 0 && row) *row = (int)(k0 + j) + 1;
             }
-            if (p != j && tid < nb) {
-                const T t = D[tid * ldd + j];
-                D[tid * ldd + j] = D[tid * ldd + p];
-                D[tid * ldd + p] = t;
-            }
-            __syncthreads();
-            const T d = D[j * ldd + j];
-            if (!cis_zero(d)) {
-                for (int r = j + 1 + tid; r < rows; r += GL_T) D[j * ldd + r] = cdiv(D[j * ldd + r], d);
-                __syncthreads();
-                // rows j+1 .. rows-1 by lane, columns j+1 .. nb-1 by warp
-                for (int r = j + 1 + lane; r < rows; r += 32) {
-                    const T l = cneg(D[j * ldd + r]);
-                    for (int cc = j + 1 + wid; cc < nb; cc += GL_T / 32) {
-                        T v = D[cc * ldd + r];
-                        cfma(v, l, D[cc * ldd + j]);
-                        D[cc * ldd + r] = v;
+            const cf d = pr[j];
+            const bool live = !cis_zero(d);
+            const GbDiv<cf> div(live ? d : cmakef(1.f, 0.f));
+            const bool store = rank == j % GL_C;
+#pragma unroll
+            for (int q = 0; q < RPT; ++q) {
+                const int o = pos[q];
+                if (o == p) pos[q] = j;
+                else if (o == j) pos[q] = p;
+                if (pos[q] <= j || pos[q] >= rows) continue;
+                if (live) {
+                    const cf l = div(a[q][j]), nl = cneg(l);
+                    a[q][j] = l;
+#pragma unroll
+                    for (int c2 = 0; c2 < NB; c2 += 2) {
+                        if (c2 + 1 <= j) continue;
+                        const float4 v = *reinterpret_cast<const float4 *>(pr + c2);
+                        if (c2 > j) cfma(a[q][c2], nl, cmakef(v.x, v.y));
+                        cfma(a[q][c2 + 1], nl, cmakef(v.z, v.w));
                     }
                 }
+                if (store && pos[q] - j <= kl) Fb[bidx(kv, ldab, k0 + pos[q], k0 + j)] = a[q][j];
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < RPT; ++q) {
+            const int o = pos[q];
+            if (o >= rows) continue;
+            prow[o] = tid + q * GL_T;
+#pragma unroll
+            for (int cc = 0; cc < NB; ++cc) {
+                D[cc * ldd + o] = a[q][cc];
+                if (cc % GL_C == rank && o <= cc && cc < nb && cc - o <= kv) Fb[bidx(kv, ldab, k0 + o, k0 + cc)] = a[q][cc];
+            }
+        }
+        __syncthreads();
+        if (rank == 0 && tid < nb) pvb[k0 + tid] = (int)(k0 + s_piv[tid]);
+        const int R2 = rows - nb, rt = (R2 + 31) / 32;
+        for (int x0 = cb; x0 < ce; x0 += tc) {
+            const int w = (ce - x0) < tc ? (ce - x0) : tc;
+            if (x0 > cb) gather(x0);
+            cp_async_wait_all();
+            __syncthreads();
+            // U12: four columns per warp, a lane per row, the solved values by shuffles
+            for (int g = wid * 4; g < w; g += NW * 4) {
+                cf x[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) x[u] = (lane < nb && g + u < w) ? Tr[(g + u) * ldd + prow[lane]] : zero;
+                for (int i = 0; i + 1 < nb; ++i) {
+                    const cf l = cneg(D[i * ldd + lane]);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const cf xi = shfl_cx(x[u], i);
+                        if (lane > i && lane < nb) cfma(x[u], l, xi);
+                    }
+                }
+                if (lane < nb)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int64_t c = k0 + nb + x0 + g + u;
+                        U[lane * ldu + g + u] = x[u];
+                        if (g + u < w && c < n && c - (k0 + lane) <= kv) Fb[bidx(kv, ldab, k0 + lane, c)] = x[u];
+                    }
             }
             __syncthreads();
-        }
-        if (rank == 0 && tid < nb) pvb[k0 + tid] = (int)(k0 + ps[tid]);
-        // (3) the interchanges on this CTA's columns right of the panel
-        for (int cc = cb + tid; cc < ce; cc += GL_T) {
-            const int64_t c = k0 + nb + cc;
-            if (c >= n) continue;
-            for (int j = 0; j < nb; ++j) {
-                const int64_t r = k0 + j, p = k0 + ps[j];
-                if (p != r && c - r <= kv) {
-                    T &x = Fb[bidx(kv, ldab, r, c)], &y = Fb[bidx(kv, ldab, p, c)];
-                    const T t = x;
-                    x = y;
-                    y = t;
-                }
-            }
-        }
-        __syncthreads();
-        // (4) U12 = L11^{-1} A12 on this CTA's columns, in shared memory
-        // (rows padded to kvs + 1)
-        for (int e = tid; e < nbp * nc; e += GL_T) {
-            const int r = e % nbp, cl = e / nbp;
-            const int64_t c = k0 + nb + cb + cl;
-            const bool in = r < nb && c < n && c - (k0 + r) <= kv;
-            cp_async<sizeof(T)>(U + r * ldu + cl, in ? (const void *)(Fb + bidx(kv, ldab, k0 + r, c)) : (const void *)Fb,
-                                in);
-        }
-        cp_async_commit();
-        cp_async_wait_all();
-        __syncthreads();
-        // a warp per column, a lane per row, the solved value by shuffles
-        for (int cl = wid; cl < nc; cl += GL_T / 32) {
-            T x = (lane < nb) ? U[lane * ldu + cl] : zero;
-            for (int i = 0; i + 1 < nb; ++i) {
-                const T xi = shfl_cx(x, i);
-                if (lane > i && lane < nb) cfma(x, cneg(D[i * ldd + lane]), xi);
-            }
-            if (lane < nb) U[lane * ldu + cl] = x;
-        }
-        __syncthreads();
-        for (int e = tid; e < nb * nc; e += GL_T) {
-            const int r = e % nb, cl = e / nb;
-            const int64_t c = k0 + nb + cb + cl;
-            if (c < n && c - (k0 + r) <= kv) Fb[bidx(kv, ldab, k0 + r, c)] = U[r * ldu + cl];
-        }
-        // (5) A22 -= L21 U12: rows k0+nb+t (t < rows-nb <= kl), this CTA's
-        // columns k0+nb+cc -- all inside the band; a warp per 32 rows x 4
-        // columns, a lane per row
-        {
-            const int R2 = rows - nb;
-            const int rt = (R2 + 31) / 32, ct = (nc + 3) / 4;
-            for (int task = wid; task < rt * ct; task += GL_T / 32) {
-                const int t = (task % rt) * 32 + lane, c4 = (task / rt) * 4;
+            // A22 -= L21 U12: rows k0 + nb + t (t < R2 <= kl), all inside the
+            // band; a warp per 32 rows x 8 columns
+            for (int task = wid; task < rt * ((w + 7) / 8); task += NW) {
+                const int t = (task % rt) * 32 + lane, c8 = (task / rt) * 8;
                 if (t >= R2) continue;
-                const int64_t i = k0 + nb + t;
-                // the destinations first: their loads run under the products
-                T old[4];
+                cf acc[8];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int64_t c = k0 + nb + cb + c4 + u;
-                    old[u] = (c4 + u < nc && c < n) ? Fb[bidx(kv, ldab, i, c)] : zero;
-                }
-                T acc[4] = {zero, zero, zero, zero};
+                for (int u = 0; u < 8; ++u) acc[u] = zero;
                 for (int k = 0; k < nb; ++k) {
-                    const T l = D[k * ldd + nb + t];
+                    const cf l = D[k * ldd + nb + t];
+                    const float4 *uk = reinterpret_cast<const float4 *>(U + k * ldu + c8);
 #pragma unroll
-                    for (int u = 0; u < 4; ++u)
-                        if (c4 + u < nc) cfma(acc[u], l, U[k * ldu + c4 + u]);
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int64_t c = k0 + nb + cb + c4 + u;
-                    if (c4 + u < nc && c < n) Fb[bidx(kv, ldab, i, c)] = cadd(old[u], cneg(acc[u]));
-                }
-            }
-        }
-        __syncthreads();   // (step 5 reads L21 from the panel that step 6 rewrites)
-        // (6) the panel back (CTA 0), multipliers in the unblocked convention
-        // (the panel's later interchanges undone on each column)
-        if (rank == 0) {
-            if (tid < nb) {
-                T *col = D + tid * ldd;
-                for (int t = nb - 1; t > tid; --t) {
-                    const int p = ps[t];
-                    if (p != t) {
-                        const T v = col[t];
-                        col[t] = col[p];
-                        col[p] = v;
+                    for (int u = 0; u < 4; ++u) {
+                        const float4 v = uk[u];
+                        cfma(acc[2 * u], l, cmakef(v.x, v.y));
+                        cfma(acc[2 * u + 1], l, cmakef(v.z, v.w));
                     }
                 }
+                const int pt = prow[nb + t];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int64_t c = k0 + nb + x0 + c8 + u;
+                    if (c8 + u < w && c < n)
+                        Fb[bidx(kv, ldab, k0 + nb + t, c)] = cadd(Tr[(c8 + u) * ldd + pt], cneg(acc[u]));
+                }
             }
-            __syncthreads();
-            for (int e = tid; e < rows * nb; e += GL_T) {
-                const int r = e % rows, cc = e / rows;
-                const int64_t i = k0 + r, c = k0 + cc;
-                if (i - c <= kl && c - i <= kv) Fb[bidx(kv, ldab, i, c)] = D[cc * ldd + r];
-            }
+            __syncthreads();   // (the next columns, or the next panel, come into the same buffers)
         }
         // every CTA's updates (and the panel) are in memory before any
-        // CTA gathers the next panel
+        // CTA reads the next panel
         gl_cluster_sync();
     }
 }
@@ -867,11 +965,12 @@ int gb_form(cudaStream_t s, int64_t n, int64_t kl, int64_t ku, const zd *A, cons
     return FEAST_OK;
 }
 
-// Shared memory of the one-launch band LU (per CTA) for a panel width nbp.
-static size_t gb_lu_fused_smem(int64_t kl, int64_t ku, int nbp, size_t es)
+// Shared memory of the one-launch band LU (per CTA) with tc columns right of the
+// panel at a time.
+static size_t gb_lu_fused_smem(int64_t kl, int tc)
 {
-    const int64_t kvs = (kl + ku + GL_C - 1) / GL_C;
-    return ((size_t)(nbp + kl) * nbp + (size_t)nbp * (kvs + 1)) * es + (size_t)nbp * sizeof(int);
+    const size_t ldd = (size_t)(GL_NB + kl);
+    return (ldd * GL_NB + (size_t)GL_NB * (tc + 2) + (size_t)tc * ldd) * sizeof(cf) + ldd * sizeof(int);
 }
 
 template <typename T>
@@ -880,16 +979,19 @@ int gb_getrf(cudaStream_t s, int64_t n, int64_t kl, int64_t ku, int q, T *F, int
 {
     const int64_t ldab = 2 * kl + ku + 1, kv = kl + ku, sF = ldab * n;
     if constexpr (sizeof(T) == sizeof(cf)) {
-        // complex64: the whole LU of each node in one cluster when its
-        // panel and its slice of U12 fit shared memory (the widest panel
-        // that does) and the band is narrow enough that the cluster's
-        // share of the trailing updates (kl x kv x nb per panel) stays
-        // near the panel's own latency; wider bands spread their updates
-        // over the whole GPU below
-        for (int nbp = GL_NB; nbp >= 8 && kv <= 512; nbp /= 2) {
-            const size_t sm = gb_lu_fused_smem(kl, ku, nbp, sizeof(T));
-            if (sm + 1024 > kSmemOptinMax) continue;
-            FEAST_CUDA_TRY(ensure_dyn_smem(k_gb_lu_fused<T>, sm));
+        // complex64: the whole LU of each node in one cluster when the band is
+        // narrow enough that the cluster's share of the trailing updates
+        // (kl x kv x nb per panel) stays near the panel's own latency; wider
+        // bands spread their updates over the whole GPU below.  The widest
+        // slice of trailing columns whose shared memory fits (8 always do).
+        if (kv <= 512) {
+            int tc = (int)((kv + GL_C - 1) / GL_C + 7) & ~7;
+            if (tc < 8) tc = 8;
+            while (tc > 8 && gb_lu_fused_smem(kl, tc) + 8192 > kSmemOptinMax) tc -= 8;
+            const int rpt = (int)((GL_NB + kl + GL_T - 1) / GL_T);
+            auto kern = rpt == 1 ? k_gb_lu_fused<1> : rpt == 2 ? k_gb_lu_fused<2> : k_gb_lu_fused<3>;
+            const size_t sm = gb_lu_fused_smem(kl, tc);
+            FEAST_CUDA_TRY(ensure_dyn_smem(kern, sm));
             cudaLaunchConfig_t cfg = {};
             cudaLaunchAttribute at[1];
             at[0].id = cudaLaunchAttributeClusterDimension;
@@ -902,8 +1004,7 @@ int gb_getrf(cudaStream_t s, int64_t n, int64_t kl, int64_t ku, int q, T *F, int
             cfg.stream = s;
             cfg.attrs = at;
             cfg.numAttrs = 1;
-            FEAST_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_gb_lu_fused<T>, n, (int)kl, (int)ku, F, ldab, sF, piv, nbp,
-                                              info, row));
+            FEAST_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, n, (int)kl, (int)ku, F, ldab, sF, piv, tc, info, row));
             FEAST_LAUNCH_CHECK();
             return FEAST_OK;
         }

@@ -66,6 +66,27 @@ def _fast_band(n, kl, ku, seed):
 
 
 @pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("n,kl,ku,m0", [(31, 0, 3, 1), (33, 5, 0, 8), (64, 31, 1, 9), (65, 33, 33, 7), (300, 130, 10, 17),
+                                        (290, 128, 128, 3), (600, 230, 20, 5), (620, 500, 8, 4), (700, 256, 256, 9)])
+def test_band_lu_solve_edges(prec, n, kl, ku, m0):
+    """The one-launch LU at the edges of its 32-column panels, of one, two and
+    three rows a thread (256 and 512 rows of a panel) and of a slice right of
+    the panel in one or several pieces; the solves with one or two halves a row
+    (kl = 128): against the oracle, the bounds of the filter above."""
+    fg = _fg()
+    A, B = _fast_band(n, kl, ku, n + 1), _fast_band(n, kl, ku, n + 2)
+    B[ku, :] += 6.0 + 2.0 * np.sqrt(kl + ku)
+    Y = inputs.complex_normal(np.random.default_rng(3), (n, m0))
+    kw = dict(contour_kind=1, rule=1, q=3, center=0.5 + 0.2j, a=1.5, b=0.8, kind=1, kl=kl, ku=ku)
+    g = fg.Feast(A, B, Y, prec=prec, refine_tol=1e-14, max_refine=6, **kw)
+    o = oracle.Feast(A, B, Y, **kw)
+    Ug, Uo = g.filter(Y), o.filter(Y)
+    err = np.abs(Ug - Uo).max() / np.abs(Uo).max()
+    g.close(); o.close()
+    assert err < (1e-11 if prec == 0 else 1e-10), err
+
+
+@pytest.mark.parametrize("prec", [0, 1])
 @pytest.mark.parametrize("n,kl,ku,q,b_identity", [(1900, 900, 900, 4, False), (2000, 1500, 1400, 3, True),
                                                   (3064, 3000, 2800, 2, True)])
 def test_wide_band_filter_matches_oracle(prec, n, kl, ku, q, b_identity):
