@@ -185,23 +185,24 @@ typedef struct {
     int qz_warm;      /* 1: the projected problem was solved warm (only its
                          unconverged trailing block went through the QR) */
     int qz_rows;      /* rows given to the QR this pass (m0 when cold) */
-    double qz_warm_resid; /* largest relative eigen-residual of the warm
-                         solve's Newton step (0 when not tried) */
+    double qz_warm_resid; /* what the last Newton step of the projected solve
+                         (m0 > 64) left of the eigenvectors, by its own
+                         bound (0 when not tried) */
     int qz_warm_k;    /* converged leading columns the warm solve found
                          (-1 when it was not tried) */
-    double ms_warm_gemm;   /* device time of the warm solve's FP64 product
-                              segments (GEMMs and triangular inverses) */
+    double ms_warm_gemm;   /* device time of the FP64 residual products of
+                              the projected solve's Newton steps (m0 > 64) */
     double warm_gemm_flop; /* their algorithmic flops (complex MAC = 8) */
     double ms_tc_gemm;     /* dense precision form: device time of the
                               tensor-core GEMM launches alone -- the LU's
                               trailing updates (feast_setup) or this pass's
                               shifted solves' off-block updates (feast_iterate) */
     double tc_gemm_flop;   /* their algorithmic flops (complex MAC = 8) */
-    int qz_cold_fp32;      /* the projected solve started cold: 1 = its Schur
-                              form came from the FP32 QR, polished by the
-                              FP64 Newton step and accepted; -1 = that was
+    int qz_cold_fp32;      /* the projected solve (m0 > 64): 1 = the Schur form
+                              of the whole matrix came from the FP32 QR and
+                              the Newton iteration was accepted; -1 = that was
                               tried and rejected (the double-single QR ran);
-                              0 = not tried */
+                              0 = solved warm, or not tried */
 } feast_iter_info;
 
 typedef struct feast_ctx feast_ctx;
@@ -231,8 +232,8 @@ int feast_setup(feast_ctx **out, const feast_pencil *pencil, const feast_contour
  * subspace as U1's) when m0 >= 96 (ordered by r_i / |rho(lambda_i)|, most
  * converged first) and always under FEAST_C64_REFINE; from the second pass
  * on, line 6 for m0 >= 96 reuses that order (QR of the unconverged
- * trailing block only, one FP64 Newton step for the rest, accepted against
- * a residual bound, else the full solve).  Synchronises the stream a few
+ * trailing block only, Newton steps with an FP64 residual for the rest,
+ * else the full solve).  Synchronises the stream a few
  * times (projected-solve decisions, c(k), e(k) and the flag).  Returns
  * FEAST_EDONE if the algorithm has stopped and no_stop is 0. */
 int feast_iterate(feast_ctx *ctx, feast_iter_info *info);
@@ -452,13 +453,18 @@ int feast_zgemm_oz(int64_t m, int64_t n, int64_t k, double alpha_re, double alph
  * as the projected B~ = U2^H B U1 = R2 is), both overwritten.  alpha, beta:
  * device m per pencil, eigenvalue alpha/beta; V: device m x m per pencil,
  * unit-norm right eigenvectors (beta A v = alpha B v).
- *   m <= 64: complex QZ (Hessenberg-triangular reduction, single-shift QZ),
- *            one warp per pencil in shared memory.
- *   m >  64: B must be nonsingular; C = B^{-1} A is reduced to Hessenberg
- *            form and QR-iterated by the whole GPU (beta = 1).
+ *   m <= 64: one CTA per pencil.  From m = 3: an FP32 Schur form of B^{-1} A
+ *            made exact by a Newton iteration with an FP64 residual (beta =
+ *            1); pencils that does not fit (B singular or beyond FP32's
+ *            reach, three or more eigenvalues closer than FP32 tells apart)
+ *            and m < 3: complex QZ (Hessenberg-triangular reduction,
+ *            single-shift QZ) in shared memory.
+ *   m >  64: B must be nonsingular; the same iteration by the whole GPU, or,
+ *            for what it leaves, a double-single QR of B^{-1} A (beta = 1).
+ *            Synchronises the stream.
  * work: device, feast_zqz_work_bytes(m, batch) bytes.  status: device
  * int32[2]: [0] pencils whose iteration cap was hit, [1] non-zero if a
- * bounded device barrier timed out.  Asynchronous. */
+ * bounded device barrier timed out.  Asynchronous up to m = 64. */
 size_t feast_zqz_work_bytes(int m, int batch);
 int feast_zqz_batched(int m, int batch, void *A, void *B, void *alpha, void *beta, void *V,
                       void *work, int *status, void *stream);

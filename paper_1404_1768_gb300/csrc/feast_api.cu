@@ -917,7 +917,7 @@ static int iterate_impl(feast_ctx *c, feast_iter_info *info)
         if (rr && (e = triangularise_bt(c))) return e;
         // B~ is upper triangular here (R2, or made so for Rayleigh-Ritz).
         // Up to 64 rows one CTA solves the pencil to FP64 accuracy (an FP32
-        // Schur form and an FP64 Newton iteration, k_zqz.cu: 3.6 ms at m0 =
+        // Schur form and an FP64 Newton iteration, k_zqz.cu: 2.5 ms at m0 =
         // 64).  What it leaves goes to the double-single standard-form QR
         // (~7 ms) from m = kZeigMinM up, or to the FP64 QZ (~70 ms) when eps
         // is within ~1000x of that QR's backward error (2^-44 of ||C||), so

@@ -1,4 +1,6 @@
-// Projected eigenproblem for large subspaces (m0 > 64), FP64, GFEAST line 6.
+// Projected eigenproblem (GFEAST line 6) by a QR iteration of the whole
+// matrix in double-single arithmetic: for what the FP32 Schur form and its
+// Newton iteration (k_zqz.cu up to 64 rows, k_warm.cu beyond) leave.
 //
 // B~ = U2^H B U1 equals R2 of the QR B U1 = U2 R2 (upper triangular; its
 // condition number is that of B on the search space), so the projected
@@ -18,8 +20,7 @@
 //      iteration limit and report a timeout instead of hanging;
 //   3. right eigenvectors of the triangular Schur form by back-substitution
 //      (one warp per eigenvector), mapped back by Q (a GEMM), unit norm.
-// The small-pencil path (m0 <= 64, one warp, shared memory) is the QZ
-// kernel in k_zqz.cu.
+// The same kernels are built in FP32 by k_zeig32.cu, for k_warm.cu.
 #include <cooperative_groups.h>
 
 #include "common.cuh"

@@ -1,9 +1,10 @@
-// Batched complex QZ for the projected pencil (A~, B~) of GFEAST line 6, in
-// FP64, one CTA per pencil.
+// Projected pencils (A~, B~) of GFEAST line 6 with up to 64 rows, one CTA per
+// pencil: an FP32 Schur form made exact by a Newton iteration with an FP64
+// residual (k_eig_refined, below), and, for what that leaves, complex QZ in FP64.
 //
 // B~ = U2^H B U1 is upper triangular by construction (U2 R2 = B U1, so
 // B~ = R2 up to rounding), so the usual initial QR of B is skipped and its
-// strictly lower part is treated as zero.  Then: Hessenberg-triangular
+// strictly lower part is treated as zero.  QZ: Hessenberg-triangular
 // reduction by Givens rotations, single-shift complex QZ sweeps with
 // deflation (Moler-Stewart), and right eigenvectors by back-substitution on
 // the generalized Schur form (beta S - alpha P) y = 0 mapped back by Z.
@@ -12,7 +13,7 @@
 // column pair; the CTA's four warps share each rotation's updates of H, T
 // and Z (one merged index range, so every SM partition's FP64 units work)
 // and meet at a barrier between rotations.  The three m x m arrays live in
-// shared memory (m <= 64).  Larger projected problems go to k_zeig.cu.
+// shared memory (m <= 64).  Larger projected problems go to k_warm.cu.
 #include "chase32.cuh"
 #include "common.cuh"
 
@@ -1092,8 +1093,8 @@ int zqz_batched(cudaStream_t s, int m, int batch, zd *A, int64_t lda, int64_t sA
     if (m <= 0 || batch <= 0) return FEAST_OK;
     if (m <= 64) {
         size_t sm = 3 * (size_t)m * m * sizeof(zd);
-        // refined FP32 Schur form first (GB300, one pencil per SM: 0.61 ms at
-        // m = 24 and 3.6 ms at m = 64, against 10.5 and 67 ms for k_qz, whose
+        // refined FP32 Schur form first (GB300, one pencil per SM: 0.41 ms at
+        // m = 24 and 2.5 ms at m = 64, against 10.5 and 67 ms for k_qz, whose
         // every rotation is a chain of FP64 instructions); k_qz then solves
         // the pencils that it left (its CTAs return at once on the others).
         // Up to two rows there is nothing to iterate: k_qz alone.
@@ -1109,7 +1110,7 @@ int zqz_batched(cudaStream_t s, int m, int batch, zd *A, int64_t lda, int64_t sA
     if (lda != m || ldb != m || ldv != m) return FEAST_EINVAL;
     const size_t wb = zqz_work_bytes(m);
     // refined FP32 Schur form first, the double-single QR for what it leaves
-    // (GB300, one pencil of 300 rows: 231 ms for the latter)
+    // (GB300, one pencil of 300 rows: 33 ms against 231 ms for the latter)
     for (int b = 0; b < batch; ++b) {
         RefineResult rr;
         int e = zeig_refined_large(s, m, A + (int64_t)b * sA, B + (int64_t)b * sB, alpha + (int64_t)b * m,
