@@ -588,11 +588,7 @@ def solve_step(fg, *a, step="", **kw):
         return solve_once(fg, *a, **kw)
 
 
-# DRAM bytes per launch of the kernels that lead two workloads' roofline
-# entries, from ncu captures of exactly those workloads (the summaries under
-# profiles/ give the commands); valid for those sizes only
-HQR_FP32_DRAM_BYTES = 40165376 + 52448512                      # k_hqr, cold pass, n = 4096, m0 = 1280
-BAND_SOLVE_DRAM_BYTES = (434.031616 + 110.770432 + 700.294144 + 119.855616) * 1e6   # k_gb_fwd + k_gb_bwd
+OZ_PRODUCTS = 28   # bf16 digit products of k_oz_gemm per real product (7 base-128 digits, s + t <= 8)
 
 
 def _bf16_peak():
@@ -618,73 +614,66 @@ def roofline_phases(prob, args, ph, infos):
     gms = sum(i.get("ms_warm_gemm", 0.0) for i in warm)
     gfl = sum(i.get("warm_gemm_flop", 0.0) for i in warm)
     if warm and t_warm >= t_cold and gms > 0.0 and gfl > 0.0:
-        # the library's own CUDA events around exactly the product launches
-        # of the warm Newton step: FP64 GEMMs and triangular inverses for C
-        # and C', the defect-form products on the digit-sliced tensor-core
-        # GEMM; reported against the FP64 peak (what the arithmetic needs)
+        # the library's own CUDA events around exactly the FP64 residual
+        # products of the Newton steps, against the FP64 peak
         ach = gfl / (gms / 1e3) / 1e12
         out["projected eigensolve"] = {
             "bound": "alu", "achieved": ach, "peak": FP64_MEASURED_TFLOPS, "unit": "TFLOP/s",
             "frac": ach / FP64_MEASURED_TFLOPS, "traffic": None,
-            "kernel": "warm Newton step: k_gemm<double2> + triangular inverses (C = B~^-1 A~, C' = Zh^H C Zh) "
-                      "and k_oz_gemm for the defect-form products (D V^, V^-1 W', V^ G, V^ S1, W' G), "
-                      "FP64-equivalent flops; CUDA events around exactly those launches",
+            "kernel": "Newton steps of the warm projected solve: k_gemm<double2> for the FP64 residual A~ V and "
+                      "B~ V; CUDA events around exactly those launches",
             "peak_source": FP64_SOURCE,
             "algorithmic_flops_per_pass": gfl / len(warm), "kernel_ms_per_pass": gms / len(warm),
             "warm_passes": len(warm), "cold_passes": len(cold),
             "tail_schur_rows": statistics.mean(i["qz_rows"] for i in warm)}
     elif warm and t_warm >= t_cold:
-        # warm solve without the library's segment events: FP64 products at
-        # m0 (4 with a triangular factor, half the MACs; 1 full), 2
-        # triangular inverses (~m0^3/3 MACs each), over the warm phase time
-        flops = 8.0 * (4 * 0.5 + 1 + 2.0 / 3.0) * m0 ** 3 * len(warm)
+        # warm solve without FP64 products of its own (all digit-sliced): one
+        # residual at m0 (a full product, one with a triangular factor), over
+        # the warm phase time
+        flops = 8.0 * 1.5 * m0 ** 3 * len(warm)
         ach = flops / (t_warm / 1e3) / 1e12
         out["projected eigensolve"] = {
             "bound": "alu", "achieved": ach, "peak": FP64_MEASURED_TFLOPS, "unit": "TFLOP/s",
             "frac": ach / FP64_MEASURED_TFLOPS, "traffic": None,
-            "kernel": "k_gemm<double2> (warm Newton step) on the FP64 pipe, with the tail Schur form inside "
-                      "the same phase time",
+            "kernel": "Newton residual A~ V - B~ V Lambda of the warm projected solve, with the FP32 Schur form of "
+                      "the tail inside the same phase time",
             "peak_source": FP64_SOURCE,
             "algorithmic_flops_per_pass": flops / len(warm), "warm_passes": len(warm), "cold_passes": len(cold)}
     elif cold:
         # cold projected solve: the multishift QR's rotations (phases x 32
         # rotations x 2 m0 element pairs x the FP32 operations of one
         # element-pair rotation: ~172 in double-single arithmetic, ~24 in the
-        # FP32 build that the cold passes with a loose acceptance take), over
-        # the whole cold projected-eigensolve phase time
+        # FP32 build), over the whole cold projected-eigensolve phase time
         fp32 = [i for i in cold if i.get("qz_cold_fp32") == 1]
         ops = sum(i["qz_phases"] * 32 * 2 * m0 * (24.0 if i.get("qz_cold_fp32") == 1 else 172.0) for i in cold)
-        # DRAM bytes of one cold-pass k_hqr launch from the ncu capture of
-        # this workload (profiles/k_hqr_fp32_dense_n4096_m1280_q32.md)
-        meas = HQR_FP32_DRAM_BYTES if (n, m0, q) == (4096, 1280, 32) and fp32 else None
         out["projected eigensolve"] = {
             "bound": "alu", "achieved": ops / (t_cold / 1e3) / 1e12, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
-            "frac": ops / (t_cold / 1e3) / 1e12 / FP32_PEAK_TFLOPS, "traffic": meas,
-            "kernel": ("k_hqr multishift QR with early deflation (FP32 build on %d of %d cold passes, then the FP64 "
-                       "Newton polish; double-single otherwise): a latency-bound rotation chain; phase time of the "
-                       "cold passes (Hessenberg reduction, Newton step and eigenvectors included)" % (len(fp32), len(cold))),
+            "frac": ops / (t_cold / 1e3) / 1e12 / FP32_PEAK_TFLOPS, "traffic": None,
+            "kernel": ("k_hqr multishift QR with early deflation (FP32 build on %d of %d cold passes, then the "
+                       "Newton iteration; double-single otherwise): a latency-bound rotation chain; phase time of the "
+                       "cold passes (Hessenberg reduction, Newton steps and eigenvectors included)" % (len(fp32), len(cold))),
             "peak_source": "derived: 152 SMs x 128 FFMA/clk x 2 flop x 2.07 GHz",
             "algorithmic_ops_per_pass": ops / len(cold), "warm_passes": len(warm), "cold_passes": len(cold)}
     if args.prec != "fp64":
         # orthonormalisation: two Cholesky-QR-twice (U and B U1) + B U1:
         # Gram m0^2 n and V R^-1 n m0^2 MACs per Cholesky-QR pass on the
-        # digit-sliced tensor-core GEMM (36 bf16 products of the realified
-        # operands per real product: 36 * 8 tensor flops per complex MAC)
+        # digit-sliced tensor-core GEMM (OZ_PRODUCTS bf16 products of the
+        # realified operands per real product, 8 tensor flops per complex MAC each)
         tc_macs = 2 * (2 * (2 * n * m0 * m0) + m0 ** 3) + (0 if prob.kw.get("b_identity") else n * n * m0)
-        tflops = 36 * 8.0 * tc_macs
+        tflops = OZ_PRODUCTS * 8.0 * tc_macs
         t_qr = ph["ms_qr"] / 1e3
         pk = _bf16_peak()
         out["orthonormalisation"] = {
             "bound": "tensor", "achieved": tflops / t_qr / 1e12, "peak": pk, "unit": "TFLOP/s",
             "frac": tflops / t_qr / 1e12 / pk, "traffic": None,
-            "kernel": "k_oz_gemm (Gram matrices, V R^-1, B U1; bf16 digit products) with the FP64 Cholesky and "
+            "kernel": "k_oz_gemm (Gram matrices, V R^-1, B U1; bf16 digit products) with the Cholesky and "
                       "triangular inverses inside the same phase time",
             "peak_source": "MEASURED_PEAKS.json bf16_tflops_sustained (timed inside a pass)",
             "fp64_equivalent_tflops": 8.0 * tc_macs / t_qr / 1e12,
             "algorithmic_flops_per_pass": tflops}
         # projection U2^H [A U1 | B U1] + A U1 (and the Ritz products of line 6)
         pm = n * n * m0 + 2 * m0 * n * m0 + 3 * n * m0 * m0
-        pf = 36 * 8.0 * pm
+        pf = OZ_PRODUCTS * 8.0 * pm
         t_p = ph["ms_proj"] / 1e3
         out["projection"] = {
             "bound": "tensor", "achieved": pf / t_p / 1e12, "peak": pk, "unit": "TFLOP/s",
@@ -726,12 +715,8 @@ def roofline(prob, args, ph):
         es = 16 if args.prec == "fp64" else 8
         traffic = q * (2 * kl + ku + 1) * n * es + 4 * q * n * m0 * es
         peak = FP64_PEAK_TFLOPS if args.prec == "fp64" else FP32_PEAK_TFLOPS
-        # DRAM bytes of one forward + backward solve from the ncu capture of
-        # this workload (profiles/k_gb_solve_band_n16384_m64_q16.md)
-        meas = (BAND_SOLVE_DRAM_BYTES if (args.prec != "fp64" and (n, kl, ku, q, m0) == (16384, 128, 128, 16, 64))
-                else None)
         return {"bound": "alu", "achieved": flops / t_solve / 1e12, "peak": peak, "unit": "TFLOP/s",
-                "frac": flops / t_solve / 1e12 / peak, "traffic": meas,
+                "frac": flops / t_solve / 1e12 / peak, "traffic": None,
                 "kernel": "band solves k_gb_fwd + k_gb_bwd (subspace-build phase), "
                           + ("FP64 pipe" if args.prec == "fp64" else "FP32 pipe"),
                 "peak_source": "derived: 152 SMs x " + ("2 DFMA" if args.prec == "fp64" else "128 FFMA")
@@ -742,14 +727,14 @@ def roofline(prob, args, ph):
     if args.prec == "fp64":
         return {"bound": "alu", "achieved": flops / t_solve / 1e12, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                 "frac": flops / t_solve / 1e12 / FP64_PEAK_TFLOPS, "traffic": None,
-                "kernel": "subspace-build solves (k_gemm<double2> + k_trsv_diag), FP64 pipe",
+                "kernel": "subspace-build solves (k_gemm<double2> + k_trsv_warp / k_trsv_diag), FP64 pipe",
                 "peak_source": "derived: 152 SMs x 2 DFMA/clk x 2 flop x 2.07 GHz",
                 "algorithmic_flops_per_pass": flops}
     pk = TF32_PEAK_TFLOPS / 3.0
     return {"bound": "tensor", "achieved": flops / t_solve / 1e12, "peak": pk, "unit": "TFLOP/s",
             "frac": flops / t_solve / 1e12 / pk, "traffic": None,
             "kernel": "subspace-build complex64 solves, whole phase (k_tc_cgemm2 tcgen05 kind::tf32 + "
-                      "k_trsv_diag + in-block k_gemm<float2> + right-hand-side splits); complex flops of the "
+                      "k_trsv_warp / k_trsv_diag + in-block k_gemm<float2> + right-hand-side splits); complex flops of the "
                       "solves",
             "peak_source": TF32_SOURCE + ", / 3 (three TF32 products per FP32-accurate product)",
             "algorithmic_flops_per_pass": flops}
@@ -987,12 +972,12 @@ def batch_arm(args, cfg):
     solves = {"bound": "tensor" if args.prec == "c64r" else "alu", "achieved": solve_flops / t_solve / 1e12,
               "peak": pk, "unit": "TFLOP/s", "frac": solve_flops / t_solve / 1e12 / pk, "traffic": None,
               "phase": "subspace-build solves of all pencils", "share_of_pass_time": t_solve / t_pass,
-              "kernel": "node-batched complex64 LU solves (k_tc_cgemm2 off-block updates, k_trsv_diag, in-block "
+              "kernel": "node-batched complex64 LU solves (k_tc_cgemm2 off-block updates, k_trsv_warp / k_trsv_diag, in-block "
                         "k_gemm<float2>) per pencil; summed per-pencil stream time (concurrent pencils overlap)",
               "peak_source": (TF32_SOURCE + ", / 3") if args.prec == "c64r" else FP64_SOURCE}
     qz = {"bound": "alu", "achieved": None, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": None,
           "traffic": None, "phase": "projected eigensolves of all pencils", "share_of_pass_time": t_qz / t_pass,
-          "kernel": "k_qz / k_small_schur / k_hqr (latency-bound rotation chains; no flop-rate reported)"}
+          "kernel": "k_eig_refined / k_schur_cta / k_hqr (latency-bound rotation chains; no flop-rate reported)"}
     roof = qz if t_qz >= t_solve else solves
     roof_others = [solves] if roof is qz else [qz]
     cb = None
