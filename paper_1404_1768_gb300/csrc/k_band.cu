@@ -230,22 +230,27 @@ __device__ __forceinline__ void cp_async(void *dst, const void *src, bool valid)
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
-// Division by b: the same bits as cdiv (Smith's form; each quotient is the
-// correctly rounded one, by Markstein's correction of n * (1 / d)), with the
-// divisor's part done once -- 32 divisions in turn are the solve's chain.
-// FP64: by the reciprocal.
-template <typename T>
+// Division by b in Smith's form (cdiv) with the divisor's part done once -- 32
+// divisions in turn are the solve's chain; each quotient n / d is the correctly
+// rounded one, by Markstein's correction of n * (1 / d).  FUSED false rounds the
+// products of d and of the numerators by themselves, as cdiv compiles: the LU's
+// multipliers are cdiv's bit for bit.  FP64: by the reciprocal.
+template <typename T, bool FUSED>
 struct GbDiv;
-template <>
-struct GbDiv<cf> {
+template <bool FUSED>
+struct GbDiv<cf, FUSED> {
     float r, d, y;
     bool h;
+    static __device__ __forceinline__ float mad(float a, float b, float c)
+    {
+        return FUSED ? fmaf(a, b, c) : __fadd_rn(c, __fmul_rn(a, b));
+    }
     __device__ __forceinline__ explicit GbDiv(cf b)
     {
         h = fabsf(b.x) >= fabsf(b.y);
         const float p = h ? b.x : b.y, q = h ? b.y : b.x;
         r = q / p;
-        d = fmaf(q, r, p);
+        d = mad(q, r, p);
         y = 1.f / d;
     }
     __device__ __forceinline__ float quot(float n) const
@@ -256,12 +261,12 @@ struct GbDiv<cf> {
     __device__ __forceinline__ cf operator()(cf a) const
     {
         const float u = h ? a.x : a.y, v = h ? a.y : a.x;
-        const float im = fmaf(-u, r, v);
-        return cmakef(quot(fmaf(v, r, u)), quot(h ? im : -im));
+        const float im = mad(-u, r, v);
+        return cmakef(quot(mad(v, r, u)), quot(h ? im : -im));
     }
 };
-template <>
-struct GbDiv<zd> {
+template <bool FUSED>
+struct GbDiv<zd, FUSED> {
     zd inv;
     __device__ __forceinline__ explicit GbDiv(zd b) : inv(crecip(b)) {}
     __device__ __forceinline__ zd operator()(zd a) const { return zmul(a, inv); }
@@ -527,7 +532,7 @@ __global__ void __launch_bounds__(GB_ST) k_gb_bwd(int64_t n, int64_t kl, int64_t
             int sl = s1 - lane;
             if (sl < 0) sl += WL;
             T x = (lane < jc) ? W[sl * cw + wid] : cx<T>(0, 0);
-            const GbDiv<T> div((lane < jc) ? Us[lane * UL] : cx<T>(1, 0));
+            const GbDiv<T, true> div((lane < jc) ? Us[lane * UL] : cx<T>(1, 0));
 #pragma unroll 8
             for (int jj = 0; jj < jc; ++jj) {
                 const int t = lane - jj;
@@ -724,7 +729,7 @@ __global__ void __launch_bounds__(GL_T) k_gb_lu_fused(int64_t n, int kl, int ku,
             }
             const cf d = pr[j];
             const bool live = !cis_zero(d);
-            const GbDiv<cf> div(live ? d : cmakef(1.f, 0.f));
+            const GbDiv<cf, false> div(live ? d : cmakef(1.f, 0.f));
             const bool store = rank == j % GL_C;
 #pragma unroll
             for (int q = 0; q < RPT; ++q) {
