@@ -59,6 +59,7 @@ constexpr int OZ_GM = 8;                     // row tiles per raster group
 constexpr int OZ_READ = 256;                 // read-out threads
 constexpr int OZ_THREADS = OZ_READ + 64;
 constexpr int OZ_SMAX = 8;                   // most CTAs that share a tile's K
+constexpr int OZ_COL1_MAX = 2048;            // longest column of a one-launch right operand
 constexpr int OZ_A_TILE = OZ_BM * OZ_BK * 2; // 8 KiB per slice
 constexpr int OZ_B_TILE = OZ_BN * OZ_BK * 2; // 4 KiB per slice
 constexpr int OZ_STAGE = OZ_S * (OZ_A_TILE + OZ_B_TILE);
@@ -229,21 +230,13 @@ __global__ void __launch_bounds__(256) k_oz_slice_rows(int64_t M, int64_t K, con
 
 // B' digit planes: plane s is (N x kp) bf16, row j = column j of B as
 // interleaved reals; a warp per column.
-__global__ void __launch_bounds__(256) k_oz_slice_cols(int64_t K, int64_t N, const zd *__restrict__ B, int64_t ldb,
-                                                       const int *__restrict__ f, uint32_t *__restrict__ planes,
-                                                       int64_t kp)
+__device__ __forceinline__ void slice_col(int64_t K, int64_t half, int64_t plane, int64_t j, const zd *__restrict__ col,
+                                          int fj, int64_t k0, int64_t k1, int step, uint32_t *__restrict__ planes)
 {
-    const int64_t half = kp / 2;
-    const int64_t plane = N * half;
-    const int lane = threadIdx.x & 31;
-    const int64_t j = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (j >= N) return;
-    const int fj = f[j];
-    const int64_t k1 = ((int64_t)blockIdx.y + 1) * 256 < half ? ((int64_t)blockIdx.y + 1) * 256 : half;
-    for (int64_t kc = (int64_t)blockIdx.y * 256 + lane; kc < k1; kc += 32) {
+    for (int64_t kc = k0; kc < k1; kc += step) {
         float d0[OZ_S], d1[OZ_S];
         if (kc < K && fj != OZ_NONFINITE) {
-            const zd v = B[kc + j * ldb];
+            const zd v = col[kc];
             digits((unsigned long long)__double_as_longlong(v.x), fj, d0);
             digits((unsigned long long)__double_as_longlong(v.y), fj, d1);
         } else {
@@ -253,6 +246,55 @@ __global__ void __launch_bounds__(256) k_oz_slice_cols(int64_t K, int64_t N, con
 #pragma unroll
         for (int s = 0; s < OZ_S; ++s) planes[(int64_t)s * plane + j * half + kc] = pack_bf16x2(d0[s], d1[s]);
     }
+}
+__global__ void __launch_bounds__(256) k_oz_slice_cols(int64_t K, int64_t N, const zd *__restrict__ B, int64_t ldb,
+                                                       const int *__restrict__ f, uint32_t *__restrict__ planes,
+                                                       int64_t kp)
+{
+    const int64_t half = kp / 2;
+    const int lane = threadIdx.x & 31;
+    const int64_t j = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (j >= N) return;
+    const int64_t k1 = ((int64_t)blockIdx.y + 1) * 256 < half ? ((int64_t)blockIdx.y + 1) * 256 : half;
+    slice_col(K, half, N * half, j, B + j * ldb, f[j], (int64_t)blockIdx.y * 256 + lane, k1, 32, planes);
+}
+
+// The columns' exponents and digits in one launch (K <= OZ_COL1_MAX): w warps
+// (1, 2, 4 or 8) per column, which is read a second time from L1.  A small product
+// is bound by its launches, and a column's digits waited for all columns' exponents.
+__global__ void __launch_bounds__(256) k_oz_cols(int64_t K, int64_t N, int w, const zd *__restrict__ B, int64_t ldb,
+                                                 int *__restrict__ f, uint32_t *__restrict__ planes, int64_t kp)
+{
+    __shared__ unsigned long long smx[8];
+    __shared__ int sbad[8];
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = wid % w, g0 = wid - sub;
+    const int64_t j = (int64_t)blockIdx.x * (8 / w) + wid / w;
+    const zd *col = B + j * ldb;
+    unsigned long long mx = 0;
+    bool bad = false;
+    if (j < N)
+        for (int64_t k = sub * 32 + lane; k < K; k += 32 * w) fold_mag(col[k], mx, bad);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        const unsigned long long o = __shfl_xor_sync(0xffffffffu, mx, off);
+        mx = o > mx ? o : mx;
+    }
+    const int any = __any_sync(0xffffffffu, bad);
+    if (lane == 0) {
+        smx[wid] = mx;
+        sbad[wid] = any;
+    }
+    __syncthreads();
+    if (j >= N) return;
+    bad = false;
+    for (int x = g0; x < g0 + w; ++x) {
+        mx = smx[x] > mx ? smx[x] : mx;
+        bad = bad || sbad[x];
+    }
+    const int fj = bad ? OZ_NONFINITE : exponent_of(mx);
+    if (sub == 0 && lane == 0) f[j] = fj;
+    const int64_t half = kp / 2;
+    slice_col(K, half, N * half, j, col, fj, sub * 32 + lane, half, 32 * w, planes);
 }
 
 struct OzOut {
@@ -541,9 +583,18 @@ int oz_prepare_cols(cudaStream_t s, int64_t K, int64_t N, const zd *B, int64_t l
     const int64_t kp = oz_kp(K);
     uint32_t *planes = (uint32_t *)work;
     int *f = (int *)((char *)work + (size_t)OZ_S * N * kp * 2 + 256);
+    if (cdiv((size_t)kp / 2, 256) > 65535) return FEAST_EINVAL;
+    // one launch while a column is a few loads a thread; longer columns spread
+    // their slicing over more CTAs than there are columns
+    if (K <= OZ_COL1_MAX) {
+        int w = 1;
+        while (w < 8 && w * 64 < K) w *= 2;
+        k_oz_cols<<<cdiv((size_t)N * w, 8), 256, 0, s>>>(K, N, w, B, ldb, f, planes, kp);
+        FEAST_LAUNCH_CHECK();
+        return FEAST_OK;
+    }
     k_oz_colexp<<<cdiv((size_t)N * 32, 256), 256, 0, s>>>(K, N, B, ldb, f);
     FEAST_LAUNCH_CHECK();
-    if (cdiv((size_t)kp / 2, 256) > 65535) return FEAST_EINVAL;
     k_oz_slice_cols<<<dim3(cdiv((size_t)N, 8), cdiv((size_t)kp / 2, 256)), 256, 0, s>>>(K, N, B, ldb, f, planes, kp);
     FEAST_LAUNCH_CHECK();
     return FEAST_OK;
