@@ -261,7 +261,8 @@ __global__ void __launch_bounds__(256) k_oz_slice_cols(int64_t K, int64_t N, con
 
 // The columns' exponents and digits in one launch (K <= OZ_COL1_MAX): w warps
 // (1, 2, 4 or 8) per column, which is read a second time from L1.  A small product
-// is bound by its launches, and a column's digits waited for all columns' exponents.
+// is bound by its launches, and a column's digits waited for all columns' exponents
+// (2048 x 640: two launches of 20 and 34 us; the whole product 831 -> 813 us).
 __global__ void __launch_bounds__(256) k_oz_cols(int64_t K, int64_t N, int w, const zd *__restrict__ B, int64_t ldb,
                                                  int *__restrict__ f, uint32_t *__restrict__ planes, int64_t kp)
 {
