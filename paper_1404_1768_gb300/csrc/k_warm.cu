@@ -57,31 +57,62 @@ struct RefineStat {
     int tiny, pad[3];                 // a close pair's coupling at rounding level was seen
 };
 
-// X = [C | I], both m x m: C = A and the identity in FP32; B32 = the upper
-// triangle of Bt, Bu the same in FP64.  amax: bits of the largest |component|
-// of A and of B.
-__global__ void k_rf_cast(int m, const zd *__restrict__ A, const zd *__restrict__ Bt, cf *__restrict__ X,
-                          cf *__restrict__ B32, zd *__restrict__ Bu, unsigned *__restrict__ amax)
+// Sizes: the iteration runs on A' = 2^-ea A and B' = 2^-eb B, whose largest
+// components lie in [1/2, 1), with lambda' = 2^(eb - ea) lambda, since its FP32
+// parts square what they compare (couplings of 1e-14 max|C|, gaps): all scales
+// are powers of two, so nothing is rounded.  ext[0], ext[1]: high words of
+// the largest |component| of A and of the upper triangle of B.
+__device__ __forceinline__ unsigned rf_high(zd v)
+{
+    const unsigned a = (unsigned)__double2hiint(v.x) & 0x7fffffffu, b = (unsigned)__double2hiint(v.y) & 0x7fffffffu;
+    return a > b ? a : b;
+}
+constexpr int RF_EXP = 500;           // largest |exponent| taken
+__host__ __device__ inline bool rf_exp_ok(unsigned ext)   // (0x7ff: an Inf or a NaN)
+{
+    const int x = (int)(ext >> 20) - 1023;
+    return x >= -RF_EXP && x <= RF_EXP;
+}
+__global__ void k_rf_extent(int m, const zd *__restrict__ A, const zd *__restrict__ Bt, unsigned *__restrict__ ext)
 {
     const int64_t total = (int64_t)m * m;
-    float ma = 0.f, mb = 0.f;
+    unsigned ma = 0, mb = 0;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
          e += (int64_t)gridDim.x * blockDim.x) {
         const int i = (int)(e % m), j = (int)(e / m);
-        const zd a = A[e], b = (i <= j) ? Bt[e] : zmake(0.0, 0.0);
-        const cf af = cmakef((float)a.x, (float)a.y);
-        const cf bf = cmakef((float)b.x, (float)b.y);
-        X[e] = af;
-        X[total + e] = cmakef(i == j ? 1.f : 0.f, 0.f);
-        B32[e] = bf;
-        Bu[e] = b;
-        // (a NaN compares false below and must not be dropped: it counts as Inf)
-        const float sa = fabsf(af.x) + fabsf(af.y), sb = fabsf(bf.x) + fabsf(bf.y);
-        ma = (sa <= ma) ? ma : (sa == sa ? sa : __int_as_float(0x7f800000));
-        mb = (sb <= mb) ? mb : (sb == sb ? sb : __int_as_float(0x7f800000));
+        const unsigned a = rf_high(A[e]), b = (i <= j) ? rf_high(Bt[e]) : 0u;
+        ma = a > ma ? a : ma;
+        mb = b > mb ? b : mb;
     }
-    atomicMax(amax, __float_as_uint(ma));
-    atomicMax(amax + 1, __float_as_uint(mb));
+    ma = __reduce_max_sync(0xffffffffu, ma);
+    mb = __reduce_max_sync(0xffffffffu, mb);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(ext, ma);
+        atomicMax(ext + 1, mb);
+    }
+}
+__device__ __forceinline__ double rf_scale(unsigned ext)   // 2^-e (1 where the size is out of range: the caller leaves)
+{
+    const int x = rf_exp_ok(ext) ? (int)(ext >> 20) : 1022;
+    return __longlong_as_double((long long)(2045 - x) << 52);
+}
+
+// X = [C | I], both m x m: C = A' and the identity in FP32; B32 = the upper
+// triangle of B', Bu the same in FP64.
+__global__ void k_rf_cast(int m, const zd *__restrict__ A, const zd *__restrict__ Bt, cf *__restrict__ X,
+                          cf *__restrict__ B32, zd *__restrict__ Bu, const unsigned *__restrict__ ext)
+{
+    const int64_t total = (int64_t)m * m;
+    const double fa = rf_scale(ext[0]), fb = rf_scale(ext[1]);
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        const int i = (int)(e % m), j = (int)(e / m);
+        const zd a = A[e], b = (i <= j) ? zscale(Bt[e], fb) : zmake(0.0, 0.0);
+        X[e] = cmakef((float)(a.x * fa), (float)(a.y * fa));
+        X[total + e] = cmakef(i == j ? 1.f : 0.f, 0.f);
+        B32[e] = cmakef((float)b.x, (float)b.y);
+        Bu[e] = b;
+    }
 }
 
 // Per column j of C: ||C[j+1:m, j]||_2 and max_i |C_ij| (Inf for a NaN).  Warp per column.
@@ -231,15 +262,16 @@ __global__ void k_rf_lam(int m, const cf *__restrict__ T, zd *__restrict__ lam)
     if (i < m) lam[i] = zmake((double)T[i + (int64_t)i * m].x, (double)T[i + (int64_t)i * m].y);
 }
 
-// R32 = A V - (B V) Lambda, rounded to FP32; part and near (the m after it) = -1.
-__global__ void k_rf_resid(int m, const zd *__restrict__ AV, const zd *__restrict__ BV, const zd *__restrict__ lam,
-                           cf *__restrict__ R32, int *__restrict__ part)
+// R32 = A' V - (B' V) Lambda', rounded to FP32 (fa: A' = fa A); part and near
+// (the m after it) = -1.
+__global__ void k_rf_resid(int m, const zd *__restrict__ AV, double fa, const zd *__restrict__ BV,
+                           const zd *__restrict__ lam, cf *__restrict__ R32, int *__restrict__ part)
 {
     const int64_t total = (int64_t)m * m;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
          e += (int64_t)gridDim.x * blockDim.x) {
         const int j = (int)(e / m);
-        const zd r = zsub(AV[e], zmul(lam[j], BV[e]));
+        const zd r = zsub(zscale(AV[e], fa), zmul(lam[j], BV[e]));
         R32[e] = cmakef((float)r.x, (float)r.y);
         if (e % m == 0) part[j] = part[m + j] = -1;
     }
@@ -385,11 +417,12 @@ __global__ void k_rf_rows(int m, const int *__restrict__ part, const zd *__restr
     }
 }
 
-__global__ void k_rf_out(int m, const zd *__restrict__ lam, zd *__restrict__ alpha, zd *__restrict__ beta)
+// alpha = lambda = fl lambda', beta = 1.
+__global__ void k_rf_out(int m, const zd *__restrict__ lam, double fl, zd *__restrict__ alpha, zd *__restrict__ beta)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m) return;
-    alpha[i] = lam[i];
+    alpha[i] = zscale(lam[i], fl);
     beta[i] = zmake(1.0, 0.0);
 }
 
@@ -411,7 +444,7 @@ struct RefineCarve {
     zd *AV, *BV, *Bu, *lam, *lam2, *pu, *pd;
     float *lower, *cmax, *nv, *part;
     int *pair, *near, *eff, *fail;
-    unsigned *amax;
+    unsigned *ext;
     RefineStat *st;
     void *schur;
     size_t bytes;
@@ -445,7 +478,7 @@ RefineCarve refine_carve(void *work, int m)
     w.near = w.pair + m;
     w.eff = w.near + m;
     w.fail = (int *)take(sizeof(int));
-    w.amax = (unsigned *)take(8);
+    w.ext = (unsigned *)take(8);
     w.st = (RefineStat *)take(sizeof(RefineStat));
     w.schur = take(schur32_work_bytes(m));
     w.bytes = off;
@@ -485,9 +518,11 @@ static int refined_attempt(cudaStream_t s, int m, const zd *A, const zd *Bt, zd 
                      int64_t ldb, cf be, cf *Cm, int64_t ldc) {
         return gemm_batched<cf>(s, conj_a, M, N, K, al, Am, lda, 0, Bm, ldb, 0, be, Cm, ldc, 0, 1);
     };
-    // C = B^{-1} A and B^{-1}, FP32
-    FEAST_CUDA_TRY(cudaMemsetAsync(w.amax, 0, 8, s));
-    k_rf_cast<<<grid_for(mm), 256, 0, s>>>(m, A, Bt, w.X, w.B32, w.Bu, w.amax);
+    // C = B'^{-1} A' and B'^{-1}, FP32
+    FEAST_CUDA_TRY(cudaMemsetAsync(w.ext, 0, 8, s));
+    k_rf_extent<<<grid_for(mm), 256, 0, s>>>(m, A, Bt, w.ext);
+    FEAST_LAUNCH_CHECK();
+    k_rf_cast<<<grid_for(mm), 256, 0, s>>>(m, A, Bt, w.X, w.B32, w.Bu, w.ext);
     FEAST_LAUNCH_CHECK();
     if ((e = trsm_upper_batched<cf>(s, m, 2 * m, 1, w.B32, m, 0, w.X, m, 0))) return e;
     cf *C = w.X, *Bi = w.X + mm;
@@ -495,9 +530,9 @@ static int refined_attempt(cudaStream_t s, int m, const zd *A, const zd *Bt, zd 
     FEAST_LAUNCH_CHECK();
     float *h = (float *)malloc(sizeof(float) * (2 * (size_t)m + RF_PART));
     if (!h) return FEAST_ENOMEM;
-    float am[2] = {0.f, 0.f};
+    unsigned ext[2] = {0, 0};
     if (cudaMemcpyAsync(h, w.lower, sizeof(float) * 2 * (size_t)m, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaMemcpyAsync(am, w.amax, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaMemcpyAsync(ext, w.ext, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess) {
         free(h);
         return FEAST_ECUDA;
@@ -508,9 +543,10 @@ static int refined_attempt(cudaStream_t s, int m, const zd *A, const zd *Bt, zd 
     while (k < m && h[k] <= RF_TAU * cn) ++k;
     res->k = k;
     free(h);
-    // (sizes whose squares FP32 holds; B singular shows as a non-finite C)
-    if (!(am[0] > 1e-12f && am[0] < 1e14f && am[1] > 1e-12f && am[1] < 1e14f && cn > 0.f && cn < 1e14f))
-        return FEAST_OK;
+    // (zero, non-finite or far out of range; B singular shows as a non-finite C)
+    if (!rf_exp_ok(ext[0]) || !rf_exp_ok(ext[1]) || !(cn > 0.f && cn < 1e14f)) return FEAST_OK;
+    const int xa = (int)(ext[0] >> 20) - 1022, xb = (int)(ext[1] >> 20) - 1022;
+    const double fa = ldexp(1.0, -xa), fl = ldexp(1.0, xa - xb);
     if (k > m - 8) k = m - 8;
     if (!prm.warm || k < m / 4) k = 0;               // too little has converged: the whole matrix
     const int mb = m - k;
@@ -597,7 +633,7 @@ static int refined_attempt(cudaStream_t s, int m, const zd *A, const zd *Bt, zd 
             FEAST_CUDA_TRY(cudaEventRecord(gt->ev[gt->used++], s));
             gt->flops += 12.0 * (double)m * m * m;
         }
-        k_rf_resid<<<grid_for(mm), 256, 0, s>>>(m, w.AV, w.BV, lam, w.G, w.pair);
+        k_rf_resid<<<grid_for(mm), 256, 0, s>>>(m, w.AV, fa, w.BV, lam, w.G, w.pair);
         FEAST_LAUNCH_CHECK();
         if ((e = mul32(0, m, m, m, fone, w.L, m, w.G, m, fzero, w.W, m))) return e;
         FEAST_CUDA_TRY(cudaMemsetAsync(w.st, 0, sizeof(RefineStat), s));
@@ -631,7 +667,7 @@ static int refined_attempt(cudaStream_t s, int m, const zd *A, const zd *Bt, zd 
         res->resid = left;
         if (!hs.paired && left <= (ever ? 0.25 : 1.0) * prm.target && (!oz || prm.target > 1e-10 || last64)) {
             if ((e = normalise_cols(s, m, V))) return e;
-            k_rf_out<<<cdiv(m, 128), 128, 0, s>>>(m, lam, alpha, beta);
+            k_rf_out<<<cdiv(m, 128), 128, 0, s>>>(m, lam, fl, alpha, beta);
             FEAST_LAUNCH_CHECK();
             res->accepted = 1;
             return FEAST_OK;
