@@ -48,13 +48,17 @@ constexpr int RF_STEPS = 10;          // most steps
 // 640 passes 3 on are warm with 1e-3 and 1e-2 alike (5-9 ms against ~130 ms
 // cold), from pass 5 with 3e-6; a start that does not contract runs cold.
 constexpr float RF_TAU = 3e-3f;
+constexpr double RF_BERR = 0x1p-52;   // residual column at rounding level: <= RF_BERR m (1 + |lambda'|) (entries of
+                                      // A', B' below 1; it measures 6 x 2^-53 at m = 300)
 constexpr int RF_PART = 64;           // partial sums of the defect norm
 
 struct RefineStat {
     unsigned gm;                      // bits of max |G|^2 (non-negative floats order like their bits)
     int bad, paired;
     unsigned wm;                      // the same of max |W_ij|^2, i != j
-    int tiny, pad[3];                 // a close pair's coupling at rounding level was seen
+    int tiny;                         // a close pair's coupling at rounding level was seen
+    unsigned rm;                      // bits of max_j (|R_j| / (1 + |lambda'_j|))^2
+    int pad[2];
 };
 
 // Sizes: the iteration runs on A' = 2^-ea A and B' = 2^-eb B, whose largest
@@ -262,19 +266,30 @@ __global__ void k_rf_lam(int m, const cf *__restrict__ T, zd *__restrict__ lam)
     if (i < m) lam[i] = zmake((double)T[i + (int64_t)i * m].x, (double)T[i + (int64_t)i * m].y);
 }
 
-// R32 = A' V - (B' V) Lambda', rounded to FP32 (fa: A' = fa A); part and near
-// (the m after it) = -1.
+// R32 = A' V - (B' V) Lambda', rounded to FP32 (fa: A' = fa A), and its largest
+// column against the column's own scale; part and near (the m after it) = -1.
+// Warp per column.
 __global__ void k_rf_resid(int m, const zd *__restrict__ AV, double fa, const zd *__restrict__ BV,
-                           const zd *__restrict__ lam, cf *__restrict__ R32, int *__restrict__ part)
+                           const zd *__restrict__ lam, cf *__restrict__ R32, int *__restrict__ part,
+                           RefineStat *__restrict__ st)
 {
-    const int64_t total = (int64_t)m * m;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int j = (int)(e / m);
-        const zd r = zsub(zscale(AV[e], fa), zmul(lam[j], BV[e]));
-        R32[e] = cmakef((float)r.x, (float)r.y);
-        if (e % m == 0) part[j] = part[m + j] = -1;
+    const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (j >= m) return;
+    const zd l = lam[j];
+    float s = 0.f;
+    for (int i = lane; i < m; i += 32) {
+        const int64_t e = i + (int64_t)j * m;
+        const zd r = zsub(zscale(AV[e], fa), zmul(l, BV[e]));
+        const cf rf = cmakef((float)r.x, (float)r.y);
+        R32[e] = rf;
+        s += cabs2(rf);
     }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (lane != 0) return;
+    part[j] = part[m + j] = -1;
+    const float d = 1.f + hypotf((float)l.x, (float)l.y), q = s / (d * d);
+    atomicMax(&st->rm, __float_as_uint(q == q ? q : __int_as_float(0x7f800000)));
 }
 
 // G from W (off the diagonal): see the file comment.  tiny: couplings at
@@ -610,12 +625,13 @@ static int refined_attempt(cudaStream_t s, int m, const zd *A, const zd *Bt, zd 
     dl = sqrt(dl);
     if (qfail || !(dl < 0.1)) return FEAST_OK;
     double gprev = 0.0, wprev = 0.0;
-    bool last64 = false, ever = false;
+    bool last64 = false, only64 = false, ever = false;
     zd *lam = w.lam, *lam2 = w.lam2;
     for (int step = 0; step < RF_STEPS; ++step) {
         // the digit-sliced products while what they leave (about 1e-13 of
         // max|C| over a gap) is not yet what limits the result
-        const bool use_oz = oz && (prm.target > 1e-10 || (!last64 && (step == 0 || gprev == 0.0 || gprev > 1e-6)));
+        const bool use_oz = oz && !only64 &&
+                            (prm.target > 1e-10 || (!last64 && (step == 0 || gprev == 0.0 || gprev > 1e-6)));
         last64 = !use_oz;
         const bool timed = gt && !use_oz && gt->used + 2 <= GemmTimer::kMax;
         if (timed) FEAST_CUDA_TRY(cudaEventRecord(gt->ev[gt->used++], s));
@@ -633,10 +649,10 @@ static int refined_attempt(cudaStream_t s, int m, const zd *A, const zd *Bt, zd 
             FEAST_CUDA_TRY(cudaEventRecord(gt->ev[gt->used++], s));
             gt->flops += 12.0 * (double)m * m * m;
         }
-        k_rf_resid<<<grid_for(mm), 256, 0, s>>>(m, w.AV, fa, w.BV, lam, w.G, w.pair);
+        FEAST_CUDA_TRY(cudaMemsetAsync(w.st, 0, sizeof(RefineStat), s));
+        k_rf_resid<<<cdiv((size_t)m * 32, 256), 256, 0, s>>>(m, w.AV, fa, w.BV, lam, w.G, w.pair, w.st);
         FEAST_LAUNCH_CHECK();
         if ((e = mul32(0, m, m, m, fone, w.L, m, w.G, m, fzero, w.W, m))) return e;
-        FEAST_CUDA_TRY(cudaMemsetAsync(w.st, 0, sizeof(RefineStat), s));
         k_rf_g<<<grid_for(mm), 256, 0, s>>>(m, w.W, lam, (use_oz ? 1e-12f : 1e-14f) * cn, w.G, w.pair, w.near, w.st);
         FEAST_LAUNCH_CHECK();
         k_rf_lambda<<<cdiv(m, 128), 128, 0, s>>>(m, w.W, lam, lam2, w.pair, w.near, w.eff, w.G, w.pu, w.pd, w.st);
@@ -646,9 +662,10 @@ static int refined_attempt(cudaStream_t s, int m, const zd *A, const zd *Bt, zd 
         FEAST_CUDA_TRY(cudaMemcpyAsync(&hs, w.st, sizeof(hs), cudaMemcpyDeviceToHost, s));
         FEAST_CUDA_TRY(cudaStreamSynchronize(s));
         if (hs.bad) return FEAST_OK;
-        float g2, w2;
+        float g2, w2, r2;
         memcpy(&g2, &hs.gm, sizeof(float));
         memcpy(&w2, &hs.wm, sizeof(float));
+        memcpy(&r2, &hs.rm, sizeof(float));
         const double gm = sqrt((double)g2), wm = sqrt((double)w2);
         k_rf_update<<<grid_for(mm), 256, 0, s>>>(m, w.Y, w.eff, w.pu, hs.paired || hs.tiny, V, w.V32);
         FEAST_LAUNCH_CHECK();
@@ -657,15 +674,20 @@ static int refined_attempt(cudaStream_t s, int m, const zd *A, const zd *Bt, zd 
         lam2 = t;
         // what the step leaves: by the bound on delta, or by the contraction
         // seen (|G| over the step before's, at least delta); a pair's block is
-        // followed by another step, and |G| that no longer falls is rounding
-        // (when |W| does not either: a close pair's G can stand still while
-        // the others still converge)
+        // followed by another step.  |G| that no longer falls (nor |W|: a close
+        // pair's G can stand still while the others still converge) is either
+        // the residual's rounding or a slow contraction (delta is let in up to
+        // 0.1), and the residual that the step began with tells them apart: the
+        // pairs are accepted when its backward error is that of an FP64 QZ
         const double ratio = gprev > 0.0 ? gm / gprev : 1e300;
-        double left = gm * fmin(8.0 * fmax(gm, ratio), (double)m * gm + dl);
-        if (gm <= 1e-8 && step > 0 && ratio > 0.1 && ratio < 1e200 && wm > 0.1 * wprev) left = 0.0;
+        const double left = gm * fmin(8.0 * fmax(gm, ratio), (double)m * gm + dl);
+        const bool still = gm <= 1e-8 && step > 0 && ratio > 0.1 && ratio < 1e200 && wm > 0.1 * wprev;
+        const bool exact = still && sqrt((double)r2) <= RF_BERR * (double)m;
+        only64 = only64 || (still && !exact);
         res->steps = step + 1;
-        res->resid = left;
-        if (!hs.paired && left <= (ever ? 0.25 : 1.0) * prm.target && (!oz || prm.target > 1e-10 || last64)) {
+        res->resid = exact ? gm : left;
+        if (!hs.paired && (exact || left <= (ever ? 0.25 : 1.0) * prm.target) &&
+            (!oz || prm.target > 1e-10 || last64)) {
             if ((e = normalise_cols(s, m, V))) return e;
             k_rf_out<<<cdiv(m, 128), 128, 0, s>>>(m, lam, fl, alpha, beta);
             FEAST_LAUNCH_CHECK();

@@ -356,6 +356,7 @@ constexpr int EZ_MIN_M = 3;          // smallest pencil
 constexpr int EZ_STEPS = 10;         // most Newton steps
 constexpr float EZ_PAIR = 1.f / 16;  // largest G_ij of a Newton step
 constexpr double EZ_DONE = 4e-15;    // error bound at which the iteration ends
+constexpr float EZ_BERR = 0x1p-52f;  // residual column at rounding level: <= EZ_BERR m (1 + |lambda'|)
 
 __device__ __forceinline__ void ez_bar() { asm volatile("bar.sync 1, %0;" ::"n"(EZ_Q) : "memory"); }
 
@@ -916,6 +917,18 @@ __global__ void __launch_bounds__(EZ_T) k_eig_refined(int m, const zd *__restric
             }
         }
         __syncthreads();
+        // where the iteration may be standing still: is R' at rounding level?
+        bool rough = true;
+        if (gprev > 0.f && gprev <= 1e-7f) {
+            const int c = t >> 2;                   // four threads per column
+            float s = 0.f;
+            if (c < m)
+                for (int r = t & 3; r < m; r += 4) s += cabs2(W[r * ld + c]);
+            s += __shfl_xor_sync(0xffffffffu, s, 1);
+            s += __shfl_xor_sync(0xffffffffu, s, 2);
+            const float d = c < m ? EZ_BERR * (float)m * (1.f + hypotf(lf[4 * c], lf[4 * c + 2])) : 0.f;
+            rough = __syncthreads_or(!(s <= d * d));
+        }
         ez_mul<false>(m, ld, H, W, Z);              // Z = L^H R'
         float gm = 0.f, wm = 0.f;
         bool paired = false;
@@ -1039,9 +1052,11 @@ __global__ void __launch_bounds__(EZ_T) k_eig_refined(int m, const zd *__restric
         // seen (|G| over the step before's, at least delta); a pair's block is
         // followed by another step
         const double seen = 8.0 * fmax((double)gm, (double)gm / (double)gprev), bnd = (double)m * (double)gm + (double)dl;
-        // (|G| that no longer falls is the residual's rounding, when |W| does not
-        // either: a close pair's G can stand still while the others still converge)
-        done = !paired && ((double)gm * fmin(seen, bnd) <= (ever ? 0.25 : 1.0) * EZ_DONE || (gm <= 1e-8f && gprev > 0.f && gm > 0.1f * gprev && wm > 0.1f * wprev));
+        // (|G| that no longer falls, nor |W|: a close pair's G can stand still while
+        // the others still converge, is the residual's rounding when the
+        // residual this step began with shows it; otherwise a slow contraction)
+        const bool still = !rough && gm <= 1e-8f && gprev > 0.f && gm > 0.1f * gprev && wm > 0.1f * wprev;
+        done = !paired && (still || (double)gm * fmin(seen, bnd) <= (ever ? 0.25 : 1.0) * EZ_DONE);
         // (after a pair's block neither size says how the iteration contracts)
         gprev = paired ? 0.f : gm;
         wprev = wm;

@@ -20,3 +20,29 @@ def test_scaled(m, ea, eb):
     lam = 2 * np.sqrt(rng.random(m)) * np.exp(2j * np.pi * rng.random(m))
     A, B = _pencil(rng, m, lam)
     _check(A * 2.0 ** ea, B * 2.0 ** eb, lam * 2.0 ** (ea - eb), 32 * m * 2.0 ** -53)
+
+
+def _chain(rng, m, p):
+    """Well separated eigenvalues with a few large couplings (eigenvector condition up to ~1e4 at p = 4.5)."""
+    lam = (np.arange(1, m + 1) + 0.3j * rng.random(m)) / m
+    B = np.eye(m) + 0.1 * np.triu(inputs.complex_normal(rng, (m, m))) / np.sqrt(m)
+    W = np.linalg.qr(inputs.complex_normal(rng, (m, m)))[0]
+    T = np.diag(lam) + 10 ** (p / 2) * np.triu(inputs.complex_normal(rng, (m, m)), 1) * (rng.random((m, m)) < 1.5 / m) / m
+    return B @ W @ T @ W.conj().T, B
+
+
+@pytest.mark.parametrize("m,p,nb", [(3, 4.5, 400), (6, 3.5, 300), (10, 3.0, 200), (24, 3.5, 100), (66, 3.5, 4), (100, 3.0, 3)])
+def test_slow_contraction(m, p, nb):
+    """Left vectors that FP32 only has to a few per cent, so that the Newton
+    steps gain little each: the backward error is still that of an FP64 QZ (4 m
+    roundings; above 64 rows the double-single QR's 2^-44 of C for what is left
+    to it, on top of B's condition of 2)."""
+    import paper_1404_1768_gb300 as fg
+    P = [_chain(np.random.default_rng([1, m, int(10 * p), s]), m, p) for s in range(nb)]
+    al, be, V, fail = fg.zqz_batched([a for a, _ in P], [b for _, b in P])
+    assert fail == 0
+    for (A, B), a, b, v in zip(P, al, be, V):
+        B = np.triu(B)
+        r = np.linalg.norm(A @ (v * b) - B @ (v * a), axis=0)
+        scale = np.abs(b) * np.linalg.norm(A) + np.abs(a) * np.linalg.norm(B)
+        assert np.max(r / scale) <= 4 * m * (2.0 ** -53 if m <= 64 else 2.0 ** -47)
