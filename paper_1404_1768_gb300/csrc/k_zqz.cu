@@ -859,9 +859,8 @@ __global__ void __launch_bounds__(EZ_T) k_eig_refined(int m, const zd *__restric
             part[j] = near[j] = -1;
         }
         // R' = 2^-ea (A V - B V Lambda), a 4 x 4 tile per thread, into W (FP32):
-        // in double-single for the first step (whose V and Lambda are FP32;
-        // what 46 bits do not see is below what that step leaves), in FP64
-        // from then on
+        // in double-single for the first step (whose V and Lambda are FP32), in
+        // FP64 from then on
         if (step == 0) {
             __syncthreads();
             ez_resid_first(m, ld, A, lda, fa, B, ldb, fb, L, lf, (float4 *)Vd, Z, W);
@@ -1055,8 +1054,9 @@ __global__ void __launch_bounds__(EZ_T) k_eig_refined(int m, const zd *__restric
         // (|G| that no longer falls, nor |W|: a close pair's G can stand still while
         // the others still converge, is the residual's rounding when the
         // residual this step began with shows it; otherwise a slow contraction)
+        // (the first step's residual has 46 bits: a later one in FP64 always follows)
         const bool still = !rough && gm <= 1e-8f && gprev > 0.f && gm > 0.1f * gprev && wm > 0.1f * wprev;
-        done = !paired && (still || (double)gm * fmin(seen, bnd) <= (ever ? 0.25 : 1.0) * EZ_DONE);
+        done = !paired && step > 0 && (still || (double)gm * fmin(seen, bnd) <= (ever ? 0.25 : 1.0) * EZ_DONE);
         // (after a pair's block neither size says how the iteration contracts)
         gprev = paired ? 0.f : gm;
         wprev = wm;

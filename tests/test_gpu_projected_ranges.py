@@ -46,3 +46,19 @@ def test_slow_contraction(m, p, nb):
         r = np.linalg.norm(A @ (v * b) - B @ (v * a), axis=0)
         scale = np.abs(b) * np.linalg.norm(A) + np.abs(a) * np.linalg.norm(B)
         assert np.max(r / scale) <= 4 * m * (2.0 ** -53 if m <= 64 else 2.0 ** -47)
+
+
+@pytest.mark.parametrize("m", [3, 8, 33, 64])
+def test_diagonal(m):
+    """Nothing couples the pairs, so the first step already finds nothing to
+    correct but the eigenvalues: all 53 bits of them must come back (one rounding
+    of the sum, one of the scale)."""
+    import paper_1404_1768_gb300 as fg
+    rng = np.random.default_rng(m)
+    lam = 2 * np.sqrt(rng.random(m)) * np.exp(2j * np.pi * rng.random(m))
+    for d in (lam, lam.real + 0j):
+        al, be, V, fail = fg.zqz_batched([np.diag(d)], [np.eye(m, dtype=complex)])
+        assert fail == 0
+        got = al[0] / be[0]
+        err = np.abs(got[:, None] - d[None, :]).min(1)
+        assert np.max(err / np.abs(got)) <= 2 * np.sqrt(2) * 2.0 ** -53
