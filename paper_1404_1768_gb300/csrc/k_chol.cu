@@ -28,6 +28,15 @@ constexpr int CB = 32;  // Cholesky block
 // block alone does not pay for the scaling and the copy of V
 constexpr int kChol32MinM = 33;
 constexpr double kChol32Tol = 1e-4;   // its pivots against the unit diagonal
+constexpr double kSeriesLast = 1e-4;  // largest Gram defect that the last series round takes on
+// ... after an FP32 first factorisation of fewer than kWideM columns, which
+// leaves such defects at ordinary conditions: what the round leaves is about 7
+// E^3, 7e-12 of Q's orthonormality from 1e-4 (250 columns, cond(V) = 300), 2e-14
+// -- the digit slices' own level -- from here.  Wider blocks keep 1e-4: the
+// further rounds cost 1.6 % of a solve at n = 2048, m0 = 640, whose eigenvalues
+// are the same 8e-14 off with either.
+constexpr double kSeriesLast32 = 1.5e-5;
+constexpr int64_t kWideM = 256;
 constexpr double kSeriesMax = 1e-2;   // largest Gram defect repeated series rounds take on (no R)
 
 __global__ void k_diag_copy(int m, const zd *__restrict__ G, double *__restrict__ d)
@@ -548,14 +557,15 @@ int zorth_chol(cudaStream_t s, int64_t n, int64_t m, zd *V, int64_t ldv, zd *R, 
         if ((e = gram_defect(s, oz, n, m, V, ldv, F1, emax, &hemax))) return e;
         if (use32 && !(hemax <= 0.5)) continue;
         // Series rounds, each taking a defect E to O(|E|^3): one when max|E|
-        // <= 1e-4 (R = (I + S) R_a then holds to O(|E|^3) as well).  Without
-        // R (only Q's span and orthonormality wanted, and every round is an
-        // upper triangular map with a positive diagonal, so Q is still the
+        // is at most last_max (R = (I + S) R_a then holds to O(|E|^3) as well).
+        // Without R (only Q's span and orthonormality wanted, and every round is
+        // an upper triangular map with a positive diagonal, so Q is still the
         // unique factor) up to three from max|E| <= kSeriesMax, the Gram
         // matrix and its defect measured again after each round that started
-        // above 1e-4.  A defect out of their reach gets a second Cholesky and
-        // inverse instead.
-        const double series_max = R ? 1e-4 : kSeriesMax;
+        // above last_max.  A defect out of their reach gets a second Cholesky
+        // and inverse instead.
+        const double last_max = use32 && m < kWideM ? kSeriesLast32 : kSeriesLast;
+        const double series_max = R ? last_max : kSeriesMax;
         bool finished = false;
         int rounds = 0;
         while (hemax <= series_max && rounds < 3) {
@@ -580,7 +590,7 @@ int zorth_chol(cudaStream_t s, int64_t n, int64_t m, zd *V, int64_t ldv, zd *R, 
                 if ((e = oz_mm(s, oz, 0, m, m, m, one, S, m, F0, m, one, R, ldr))) return e;
             }
             ++rounds;
-            if (hemax <= 1e-4) {
+            if (hemax <= last_max) {
                 finished = true;
                 break;
             }
