@@ -59,6 +59,8 @@ constexpr int OZ_GM = 8;                     // row tiles per raster group
 constexpr int OZ_READ = 256;                 // read-out threads
 constexpr int OZ_THREADS = OZ_READ + 64;
 constexpr int OZ_SMAX = 8;                   // most CTAs that share a tile's K
+// most complex K of one launch: its int64 sums gain up to 2^44.1 per chunk (2^18.9 chunks)
+constexpr int64_t OZ_KMAX = 1 << 26;
 constexpr int OZ_COL1_MAX = 2048;            // longest column of a one-launch right operand
 constexpr int OZ_A_TILE = OZ_BM * OZ_BK * 2; // 8 KiB per slice
 constexpr int OZ_B_TILE = OZ_BN * OZ_BK * 2; // 4 KiB per slice
@@ -195,35 +197,38 @@ __global__ void __launch_bounds__(256) k_oz_slice_rows(int64_t M, int64_t K, con
     __shared__ zd tile[32][33];
     const int64_t half = kp / 2, plane = M * kp;   // in 32-bit words
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t i0 = (int64_t)blockIdx.x * 32, k0 = (int64_t)blockIdx.y * 32;
-    for (int r = w; r < 32; r += 8) {
-        const int64_t a = ct ? k0 + lane : i0 + lane, b = ct ? i0 + r : k0 + r;   // stored row, column
-        const bool in = ct ? (a < K && b < M) : (a < M && b < K);
-        zd v = in ? A[a + b * lda] : zmake(0.0, 0.0);
-        if (ct) tile[r][lane] = zconj(v);
-        else tile[lane][r] = v;
-    }
-    __syncthreads();
-    const int64_t kc = k0 + lane;
-    if (kc >= half) return;
-    for (int r = w; r < 32; r += 8) {
-        const int64_t i = i0 + r;
-        if (i >= M) break;
-        const int ei = e[i];
-        float dr[OZ_S], di[OZ_S];
-        if (kc < K && ei != OZ_NONFINITE) {
-            const zd v = tile[r][lane];
-            digits((unsigned long long)__double_as_longlong(v.x), ei, dr);
-            digits((unsigned long long)__double_as_longlong(v.y), ei, di);
-        } else {
-#pragma unroll
-            for (int s = 0; s < OZ_S; ++s) { dr[s] = 0.f; di[s] = 0.f; }
+    const int64_t i0 = (int64_t)blockIdx.x * 32;
+    for (int64_t k0 = (int64_t)blockIdx.y * 32; k0 < half; k0 += (int64_t)gridDim.y * 32) {   // (once up to half = 32 x 65535)
+        if (k0 != (int64_t)blockIdx.y * 32) __syncthreads();
+        for (int r = w; r < 32; r += 8) {
+            const int64_t a = ct ? k0 + lane : i0 + lane, b = ct ? i0 + r : k0 + r;   // stored row, column
+            const bool in = ct ? (a < K && b < M) : (a < M && b < K);
+            zd v = in ? A[a + b * lda] : zmake(0.0, 0.0);
+            if (ct) tile[r][lane] = zconj(v);
+            else tile[lane][r] = v;
         }
-        const int64_t o = 2 * i * half + kc;
+        __syncthreads();
+        const int64_t kc = k0 + lane;
+        if (kc >= half) continue;
+        for (int r = w; r < 32; r += 8) {
+            const int64_t i = i0 + r;
+            if (i >= M) break;
+            const int ei = e[i];
+            float dr[OZ_S], di[OZ_S];
+            if (kc < K && ei != OZ_NONFINITE) {
+                const zd v = tile[r][lane];
+                digits((unsigned long long)__double_as_longlong(v.x), ei, dr);
+                digits((unsigned long long)__double_as_longlong(v.y), ei, di);
+            } else {
 #pragma unroll
-        for (int s = 0; s < OZ_S; ++s) {
-            planes[(int64_t)s * plane + o] = pack_bf16x2(dr[s], -di[s]);
-            planes[(int64_t)s * plane + o + half] = pack_bf16x2(di[s], dr[s]);
+                for (int s = 0; s < OZ_S; ++s) { dr[s] = 0.f; di[s] = 0.f; }
+            }
+            const int64_t o = 2 * i * half + kc;
+#pragma unroll
+            for (int s = 0; s < OZ_S; ++s) {
+                planes[(int64_t)s * plane + o] = pack_bf16x2(dr[s], -di[s]);
+                planes[(int64_t)s * plane + o + half] = pack_bf16x2(di[s], dr[s]);
+            }
         }
     }
 }
@@ -255,8 +260,8 @@ __global__ void __launch_bounds__(256) k_oz_slice_cols(int64_t K, int64_t N, con
     const int lane = threadIdx.x & 31;
     const int64_t j = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (j >= N) return;
-    const int64_t k1 = ((int64_t)blockIdx.y + 1) * 256 < half ? ((int64_t)blockIdx.y + 1) * 256 : half;
-    slice_col(K, half, N * half, j, B + j * ldb, f[j], (int64_t)blockIdx.y * 256 + lane, k1, 32, planes);
+    for (int64_t k0 = (int64_t)blockIdx.y * 256; k0 < half; k0 += (int64_t)gridDim.y * 256)   // (once up to 256 x 65535 rows)
+        slice_col(K, half, N * half, j, B + j * ldb, f[j], k0 + lane, k0 + 256 < half ? k0 + 256 : half, 32, planes);
 }
 
 // The columns' exponents and digits in one launch (K <= OZ_COL1_MAX): w warps
@@ -321,12 +326,12 @@ __device__ __forceinline__ long long oz_peer(const long long *p, int rank)
     return v;
 }
 
-// splits CTAs (a cluster, 1 to OZ_SMAX) share a tile: CTA r takes K-blocks
-// [r kbs, (r + 1) kbs), then finishes 64 / splits of the tile's columns from
+// K-blocks from kfirst on, of kr real terms.  splits CTAs (a cluster, 1 to
+// OZ_SMAX) share a tile: CTA r takes K-blocks [r kbs, (r + 1) kbs) of them, then finishes 64 / splits of the tile's columns from
 // all of their sums.
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     k_oz_gemm(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tB, int mr, int n,
-              int kr, int splits, int kbs, const int *__restrict__ ea, const int *__restrict__ fb, OzOut out,
+              int kfirst, int kr, int splits, int kbs, const int *__restrict__ ea, const int *__restrict__ fb, OzOut out,
               int *err)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -385,7 +390,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                 if (!mbar_wait(&empty[s], ph ^ 1u) || *(volatile int *)&s_fail) { s_fail = 1; break; }
                 unsigned char *st = base + s * OZ_STAGE;
                 mbar_expect_tx(&full[s], OZ_STAGE);
-                const int kx = (kb0 + kb) * OZ_BK;
+                const int kx = (kfirst + kb0 + kb) * OZ_BK;
 #pragma unroll 1
                 for (int sl = 0; sl < OZ_S; ++sl) {
                     tma_load_3d(st + sl * OZ_A_TILE, &tA, &full[s], kx, row0, sl);
@@ -571,8 +576,8 @@ int oz_prepare_rows(cudaStream_t s, int64_t M, int64_t K, const zd *A, int64_t l
     if (ct) k_oz_colexp<<<cdiv((size_t)M * 32, 256), 256, 0, s>>>(K, M, A, lda, e);
     else k_oz_rowexp<<<cdiv((size_t)M, 32), 32 * RE_W, 0, s>>>(M, K, A, lda, e);
     FEAST_LAUNCH_CHECK();
-    if (cdiv((size_t)kp / 2, 32) > 65535) return FEAST_EINVAL;
-    k_oz_slice_rows<<<dim3(cdiv((size_t)M, 32), cdiv((size_t)kp / 2, 32)), 256, 0, s>>>(M, K, A, lda, ct, e, planes, kp);
+    const unsigned gk = cdiv((size_t)kp / 2, 32);
+    k_oz_slice_rows<<<dim3(cdiv((size_t)M, 32), gk > 65535 ? 65535 : gk), 256, 0, s>>>(M, K, A, lda, ct, e, planes, kp);
     FEAST_LAUNCH_CHECK();
     return FEAST_OK;
 }
@@ -584,7 +589,6 @@ int oz_prepare_cols(cudaStream_t s, int64_t K, int64_t N, const zd *B, int64_t l
     const int64_t kp = oz_kp(K);
     uint32_t *planes = (uint32_t *)work;
     int *f = (int *)((char *)work + (size_t)OZ_S * N * kp * 2 + 256);
-    if (cdiv((size_t)kp / 2, 256) > 65535) return FEAST_EINVAL;
     // one launch while a column is a few loads a thread; longer columns spread
     // their slicing over more CTAs than there are columns
     if (K <= OZ_COL1_MAX) {
@@ -596,7 +600,8 @@ int oz_prepare_cols(cudaStream_t s, int64_t K, int64_t N, const zd *B, int64_t l
     }
     k_oz_colexp<<<cdiv((size_t)N * 32, 256), 256, 0, s>>>(K, N, B, ldb, f);
     FEAST_LAUNCH_CHECK();
-    k_oz_slice_cols<<<dim3(cdiv((size_t)N, 8), cdiv((size_t)kp / 2, 256)), 256, 0, s>>>(K, N, B, ldb, f, planes, kp);
+    const unsigned gk = cdiv((size_t)kp / 2, 256);
+    k_oz_slice_cols<<<dim3(cdiv((size_t)N, 8), gk > 65535 ? 65535 : gk), 256, 0, s>>>(K, N, B, ldb, f, planes, kp);
     FEAST_LAUNCH_CHECK();
     return FEAST_OK;
 }
@@ -626,7 +631,8 @@ int oz_gemm(cudaStream_t s, int64_t M, int64_t N, int64_t K, const void *Arows, 
     // K split over a cluster: the split with the least waves x (its K-blocks at
     // 2 x 28 x 48 clocks + the fixed cost of a CTA: pipeline fill, read-out,
     // result, and the exchange when it shares its tile)
-    const int kb = (int)((2 * K + OZ_BK - 1) / OZ_BK);
+    const int64_t kpiece = K < OZ_KMAX ? K : OZ_KMAX;
+    const int kb = (int)((2 * kpiece + OZ_BK - 1) / OZ_BK);
     int splits = 1;
     double best = 0.0;
     for (int x = 1; x <= OZ_SMAX; x *= 2) {
@@ -639,7 +645,6 @@ int oz_gemm(cudaStream_t s, int64_t M, int64_t N, int64_t K, const void *Arows, 
         }
     }
     if (tiles * splits > 0x7fffffff) return FEAST_EINVAL;
-    OzOut o{C, ldc, alpha, zcol, cblk > 0 ? cblk : 1, beta};
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -652,9 +657,13 @@ int oz_gemm(cudaStream_t s, int64_t M, int64_t N, int64_t K, const void *Arows, 
     cfg.stream = s;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    FEAST_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_oz_gemm, mA, mB, (int)mr, (int)N, (int)(2 * K), splits,
-                                      (kb + splits - 1) / splits, ea, fb, o, err));
-    FEAST_LAUNCH_CHECK();
+    for (int64_t k0 = 0; k0 < K; k0 += kpiece) {
+        OzOut o{C, ldc, alpha, zcol, cblk > 0 ? cblk : 1, k0 ? zmake(1.0, 0.0) : beta};
+        const int64_t kn = K - k0 < kpiece ? K - k0 : kpiece;
+        FEAST_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_oz_gemm, mA, mB, (int)mr, (int)N, (int)(2 * k0 / OZ_BK), (int)(2 * kn),
+                                          splits, (kb + splits - 1) / splits, ea, fb, o, err));
+        FEAST_LAUNCH_CHECK();
+    }
     return FEAST_OK;
 }
 

@@ -322,22 +322,25 @@ __global__ void __launch_bounds__(256) k_realify_split(int m, int k, const float
 {
     __shared__ float2 tile[32][33];
     const int b = blockIdx.z, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int i0 = blockIdx.x * 32, p0 = blockIdx.y * 32;
+    const int i0 = blockIdx.x * 32;
     const float2 *Ab = A + (int64_t)b * sA;
-    for (int p = w; p < 32; p += 8)
-        if (i0 + lane < m && p0 + p < k) tile[lane][p] = Ab[i0 + lane + (int64_t)(p0 + p) * lda];
-    __syncthreads();
-    if (p0 + lane >= k) return;
-    for (int i = w; i < 32; i += 8) {
-        if (i0 + i >= m) break;
-        const float2 a = tile[i][lane];
-        const float2 h = make_float2(tf32_head(a.x), tf32_head(a.y));
-        const float2 t = make_float2(a.x - h.x, a.y - h.y);
-        const int64_t o = (int64_t)b * sR + (int64_t)(2 * (i0 + i)) * ldr + 2 * (p0 + lane);
-        *(float2 *)(head + o) = make_float2(h.x, -h.y);          // (2i, 2p), (2i, 2p + 1)
-        *(float2 *)(tail + o) = make_float2(t.x, -t.y);
-        *(float2 *)(head + o + ldr) = make_float2(h.y, h.x);     // (2i + 1, ..)
-        *(float2 *)(tail + o + ldr) = make_float2(t.y, t.x);
+    for (int64_t p0 = (int64_t)blockIdx.y * 32; p0 < k; p0 += (int64_t)gridDim.y * 32) {   // (once up to k = 32 x 65535)
+        if (p0 != (int64_t)blockIdx.y * 32) __syncthreads();
+        for (int p = w; p < 32; p += 8)
+            if (i0 + lane < m && p0 + p < k) tile[lane][p] = Ab[i0 + lane + (p0 + p) * lda];
+        __syncthreads();
+        if (p0 + lane >= k) continue;
+        for (int i = w; i < 32; i += 8) {
+            if (i0 + i >= m) break;
+            const float2 a = tile[i][lane];
+            const float2 h = make_float2(tf32_head(a.x), tf32_head(a.y));
+            const float2 t = make_float2(a.x - h.x, a.y - h.y);
+            const int64_t o = (int64_t)b * sR + (int64_t)(2 * (i0 + i)) * ldr + 2 * (p0 + lane);
+            *(float2 *)(head + o) = make_float2(h.x, -h.y);          // (2i, 2p), (2i, 2p + 1)
+            *(float2 *)(tail + o) = make_float2(t.x, -t.y);
+            *(float2 *)(head + o + ldr) = make_float2(h.y, h.x);     // (2i + 1, ..)
+            *(float2 *)(tail + o + ldr) = make_float2(t.y, t.x);
+        }
     }
 }
 
@@ -352,15 +355,16 @@ __global__ void __launch_bounds__(256) k_split_tf32(int64_t k, int n, const floa
     if (c >= n) return;
     const float2 *x = X + (int64_t)b * sX + c * ldx;
     float2 *h = (float2 *)(head + (int64_t)b * sH + c * ldh2), *t = (float2 *)(tail + (int64_t)b * sH + c * ldh2);
-    const int64_t r0 = (int64_t)blockIdx.y * 256;
+    for (int64_t r0 = (int64_t)blockIdx.y * 256; r0 < k; r0 += (int64_t)gridDim.y * 256) {   // (once up to k = 256 x 65535)
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-        const int64_t r = r0 + 32 * u + lane;
-        if (r >= k) continue;
-        const float2 v = x[r];
-        const float2 hv = make_float2(tf32_head(v.x), tf32_head(v.y));
-        h[r] = hv;
-        t[r] = make_float2(v.x - hv.x, v.y - hv.y);
+        for (int u = 0; u < 8; ++u) {
+            const int64_t r = r0 + 32 * u + lane;
+            if (r >= k) continue;
+            const float2 v = x[r];
+            const float2 hv = make_float2(tf32_head(v.x), tf32_head(v.y));
+            h[r] = hv;
+            t[r] = make_float2(v.x - hv.x, v.y - hv.y);
+        }
     }
 }
 
@@ -468,8 +472,9 @@ int tc_prepare_A(cudaStream_t s, int64_t m, int64_t k, const cf *A, int64_t lda,
     const int64_t mr = 2 * m;
     float *Ah = Aprep, *At = Ah + (size_t)batch * mr * kr;
     if (kr != 2 * k) FEAST_CUDA_TRY(cudaMemsetAsync(Ah, 0, sizeof(float) * 2 * (size_t)batch * mr * kr, s));
-    if (cdiv(k, 32) > 65535 || batch > 65535) return FEAST_EINVAL;
-    k_realify_split<<<dim3(cdiv(m, 32), cdiv(k, 32), batch), 256, 0, s>>>((int)m, (int)k, A, lda, sA, Ah, At, kr, mr * kr);
+    if (batch > 65535) return FEAST_EINVAL;
+    const unsigned gk = cdiv(k, 32);
+    k_realify_split<<<dim3(cdiv(m, 32), gk > 65535 ? 65535 : gk, batch), 256, 0, s>>>((int)m, (int)k, A, lda, sA, Ah, At, kr, mr * kr);
     FEAST_LAUNCH_CHECK();
     return FEAST_OK;
 }
@@ -486,8 +491,9 @@ int tc_cgemm_prepA(cudaStream_t s, int64_t m, int64_t n, int64_t k, cf alpha, co
     const float *Ah = Aprep, *At = Ah + (size_t)batch * mr * kr;
     float *Xh = scratch, *Xt = Xh + (size_t)batch * kr * n;
     if (kr != 2 * k) FEAST_CUDA_TRY(cudaMemsetAsync(Xh, 0, sizeof(float) * 2 * (size_t)batch * kr * n, s));
-    if (cdiv(k, 256) > 65535 || batch > 65535) return FEAST_EINVAL;
-    k_split_tf32<<<dim3(cdiv(n, 8), cdiv(k, 256), batch), 256, 0, s>>>(k, (int)n, X, ldx, sX, Xh, Xt, kr, kr * n);
+    if (batch > 65535) return FEAST_EINVAL;
+    const unsigned gk = cdiv(k, 256);
+    k_split_tf32<<<dim3(cdiv(n, 8), gk > 65535 ? 65535 : gk, batch), 256, 0, s>>>(k, (int)n, X, ldx, sX, Xh, Xt, kr, kr * n);
     FEAST_LAUNCH_CHECK();
     CUtensorMap mAh, mAt, mXh, mXt;
     int e;
