@@ -401,10 +401,11 @@ int zqz_batched(cudaStream_t s, int m, int batch, zd *A, int64_t lda, int64_t sA
                 void *work, int *fail, int *timeout, int *stats = nullptr, double defl = 0.0);
 
 // The same for 3 <= m <= 64 by an FP32 Schur form and an FP64 Newton
-// iteration alone (A, B kept): the int at work + 16 b m^2 bytes is 0 when
-// pencil b was solved (beta = 1), 1 when it needs another method (its
-// alpha, beta and V are then not written).
-int zeig_refined(cudaStream_t s, int m, int batch, const zd *A, int64_t lda, int64_t sA, const zd *B, int64_t ldb,
+// iteration alone (B kept, A kept or shifted): the int at work + 16 b m^2
+// bytes is 0 when pencil b was solved (beta = 1), 1 when it needs another method
+// (its alpha, beta and V are then not written); the complex128 after that
+// first one is sigma when A was replaced by A - sigma B, else 0.
+int zeig_refined(cudaStream_t s, int m, int batch, zd *A, int64_t lda, int64_t sA, const zd *B, int64_t ldb,
                  int64_t sB, zd *alpha, zd *beta, zd *V, int64_t ldv, int64_t sV, void *work);
 
 // Large projected problems (k_zeig.cu): standard form, Hessenberg
@@ -453,6 +454,7 @@ int rrqr_basis(cudaStream_t s, int64_t n, int m, const zd *U, zd *Q, double rank
 struct RefineParams {
     int warm;           // 1: C's leading columns may have converged (ordered Ritz pairs)
     double target;      // error of the eigenvectors at which the iteration may end
+    int find;           // 1: end at once (narrow, sigma) where A is nearly sigma B
 };
 struct RefineResult {
     int accepted;   // 1: alpha, beta, V hold the eigenpairs
@@ -460,7 +462,13 @@ struct RefineResult {
     int tail;       // rows of the block given to the QR
     int steps;      // Newton steps taken
     double resid;   // estimated error left by the last step
+    int narrow;     // prm.find: A - sigma B is below 1/16 of A: nothing was solved
+    zd sigma;
 };
+// A spectrum narrow against its distance from the origin is solved as that of
+// (A - sigma B, B): A <- A - sigma triu(B), alpha <- alpha + sigma beta.
+int shift_pencil(cudaStream_t s, int m, zd *A, const zd *Bt, zd sigma);
+int shift_values(cudaStream_t s, int m, zd *alpha, const zd *beta, zd sigma);
 size_t zeig_refined_large_work_bytes(int m);
 // Events around the projected solve's FP64 product segments, for the
 // per-kernel roofline: pairs (begin, end) in

@@ -137,6 +137,13 @@ namespace {
 // ordered its Ritz pairs.
 constexpr int kWarmMinM = 96;
 constexpr double kWarmAccMin = 1e-12;  // the double-single QR's own backward error (2^-44 of ||H||)
+// A contour this narrow against its centre c has line 6 solve (A~ - c B~, B~):
+// FP32 would round away the gaps between the eigenvalues inside, and the warm
+// start's converged columns, told by max|C| ~ |c|, would be all of them.  n =
+// 800, m0 = 128, radius 1e-4 around 1: passes of 35 ms unshifted (the double-single
+// QR after two refused attempts), 6.5 ms cold and 1 ms warm shifted; the
+// unshifted solve was refused from 1e-4 (100 rows) or 1e-3 (300) on.
+constexpr double kNarrow = 1.0 / 16;
 constexpr int kZeigMinM = 8;         // smallest projected problem on the standard-form QR
 // banded precision form: the n x m0 products go to the digit-sliced
 // tensor-core GEMM from this width on (below it the FP64 GEMMs of the tall,
@@ -885,6 +892,15 @@ static int iterate_impl(feast_ctx *c, feast_iter_info *info)
     // accuracy, as at any pass that may stop)
     const bool final_pass = c->k >= c->max_iter && !c->no_stop;
     const double acc = final_pass ? kWarmAccMin : fmax(kWarmAccMin, 1e-3 * eref);
+    const zd centre = zmake(c->contour.center_re, c->contour.center_im);
+    const bool narrow = fmax(c->contour.a, c->contour.b) <= kNarrow * hypot(centre.x, centre.y);
+    // [A~ | B~] into Q, B~ triangular, A~ shifted where the contour is narrow
+    auto pencil_to_q = [&]() -> int {
+        FEAST_CUDA_TRY(cudaMemcpyAsync(c->Q, c->P, sizeof(zd) * 2 * m * m, cudaMemcpyDeviceToDevice, s));
+        int er;
+        if (rr && (er = triangularise_bt(c))) return er;
+        return narrow ? shift_pencil(s, (int)m, c->Q, c->Q + m * m, centre) : FEAST_OK;
+    };
     if (m > 64) {
         // FP32 Schur form (of the unconverged trailing block, when the
         // previous pass filtered its ordered Ritz vectors) and Newton steps
@@ -892,13 +908,12 @@ static int iterate_impl(feast_ctx *c, feast_iter_info *info)
         // residuals' products run on the digit-sliced tensor-core GEMM where
         // the context has its scratch, as far as its resolution goes
         const zd *Ap = c->P, *Bp = c->P + m * m;
-        if (rr) {
-            FEAST_CUDA_TRY(cudaMemcpyAsync(c->Q, c->P, sizeof(zd) * 2 * m * m, cudaMemcpyDeviceToDevice, s));
-            if ((e = triangularise_bt(c))) return e;
+        if (rr || narrow) {
+            if ((e = pencil_to_q())) return e;
             Ap = c->Q;
             Bp = c->Q + m * m;
         }
-        const RefineParams prm{c->warm_ready, 1e-2 * acc};
+        const RefineParams prm{c->warm_ready, 1e-2 * acc, 0};
         if ((e = zeig_refined_large(s, (int)m, Ap, Bp, c->alpha, c->beta, c->Yv, c->warm_work, prm, &c->last_warm,
                                     &c->st->timeout, &c->st->qz_sweeps, &c->gt, orth_oz(c))))
             return e;
@@ -913,8 +928,7 @@ static int iterate_impl(feast_ctx *c, feast_iter_info *info)
         // pass that may stop deflates at the double-single floor, so that
         // its pairs reach eps.
         const double defl = (c->c_prev > 0 || final_pass) ? 0.0 : 1e-8;
-        FEAST_CUDA_TRY(cudaMemcpyAsync(c->Q, c->P, sizeof(zd) * 2 * m * m, cudaMemcpyDeviceToDevice, s));
-        if (rr && (e = triangularise_bt(c))) return e;
+        if ((e = pencil_to_q())) return e;
         // B~ is upper triangular here (R2, or made so for Rayleigh-Ritz).
         // Up to 64 rows one CTA solves the pencil to FP64 accuracy (an FP32
         // Schur form and an FP64 Newton iteration, k_zqz.cu: 2.5 ms at m0 =
@@ -924,11 +938,13 @@ static int iterate_impl(feast_ctx *c, feast_iter_info *info)
         // that e(k) can still fall below eps
         zd *Bq = c->Q + m * m;
         int left = 1;
+        zd hw[2] = {};   // (the flag, and the shift that zeig_refined made by itself)
         if (m >= 3 && m <= 64) {
             if ((e = zeig_refined(s, (int)m, 1, c->Q, m, 0, Bq, m, 0, c->alpha, c->beta, c->Yv, m, 0, c->qz_work)))
                 return e;
-            FEAST_CUDA_TRY(cudaMemcpyAsync(&left, c->qz_work, sizeof(int), cudaMemcpyDeviceToHost, s));
+            FEAST_CUDA_TRY(cudaMemcpyAsync(hw, c->qz_work, sizeof(hw), cudaMemcpyDeviceToHost, s));
             FEAST_CUDA_TRY(cudaStreamSynchronize(s));
+            memcpy(&left, hw, sizeof(int));
         }
         if (!left)
             e = FEAST_OK;
@@ -939,7 +955,9 @@ static int iterate_impl(feast_ctx *c, feast_iter_info *info)
             e = zqz_batched(s, (int)m, 1, c->Q, m, 0, Bq, m, 0, c->alpha, c->beta, c->Yv, m, 0, c->qz_work,
                             &c->st->qz_fail, &c->st->timeout, &c->st->qz_sweeps, defl);
         if (e) return e;
+        if (left && (hw[1].x != 0.0 || hw[1].y != 0.0) && (e = shift_values(s, (int)m, c->alpha, c->beta, hw[1]))) return e;
     }
+    if (narrow && (e = shift_values(s, (int)m, c->alpha, c->beta, centre))) return e;
     FEAST_CUDA_TRY(cudaEventRecord(c->ev[2], s));
     if (use_oz_small(c)) {
         // x_i = U1 y_i, A x_i = (A U1) y_i, B x_i = (B U1) y_i with Y's digits made once

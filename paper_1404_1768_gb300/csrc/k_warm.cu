@@ -40,6 +40,7 @@
 namespace feast {
 namespace {
 
+constexpr double RF_NARROW = 1.0 / 16;  // |A - sigma B| / |A| from which A is shifted (prm.find)
 constexpr float RF_PAIR = 1.f / 16;   // largest G_ij of a step (beyond: the pair's own block)
 constexpr int RF_STEPS = 10;          // most steps
 // converged column: strictly lower part <= RF_TAU max|C|.  The iteration
@@ -102,21 +103,62 @@ __device__ __forceinline__ double rf_scale(unsigned ext)   // 2^-e (1 where the 
 }
 
 // X = [C | I], both m x m: C = A' and the identity in FP32; B32 = the upper
-// triangle of B', Bu the same in FP64.
-__global__ void k_rf_cast(int m, const zd *__restrict__ A, const zd *__restrict__ Bt, cf *__restrict__ X,
-                          cf *__restrict__ B32, zd *__restrict__ Bu, const unsigned *__restrict__ ext)
+// triangle of B', Bu the same in FP64.  mom (may be null): per block (at most
+// RF_MOM of 256 threads) the sums of conj(b) a, |a|^2 and |b|^2.
+constexpr int RF_MOM = 256;
+__global__ void __launch_bounds__(256) k_rf_cast(int m, const zd *__restrict__ A, const zd *__restrict__ Bt,
+                                                 cf *__restrict__ X, cf *__restrict__ B32, zd *__restrict__ Bu,
+                                                 const unsigned *__restrict__ ext, float4 *__restrict__ mom)
 {
+    float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
     const int64_t total = (int64_t)m * m;
     const double fa = rf_scale(ext[0]), fb = rf_scale(ext[1]);
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
          e += (int64_t)gridDim.x * blockDim.x) {
         const int i = (int)(e % m), j = (int)(e / m);
         const zd a = A[e], b = (i <= j) ? zscale(Bt[e], fb) : zmake(0.0, 0.0);
-        X[e] = cmakef((float)(a.x * fa), (float)(a.y * fa));
+        const cf af = cmakef((float)(a.x * fa), (float)(a.y * fa)), bf = cmakef((float)b.x, (float)b.y);
+        X[e] = af;
         X[total + e] = cmakef(i == j ? 1.f : 0.f, 0.f);
-        B32[e] = cmakef((float)b.x, (float)b.y);
+        B32[e] = bf;
         Bu[e] = b;
+        q.x += bf.x * af.x + bf.y * af.y;
+        q.y += bf.x * af.y - bf.y * af.x;
+        q.z += cabs2(af);
+        q.w += cabs2(bf);
     }
+    if (!mom) return;
+    __shared__ float4 red[8];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        q.x += __shfl_xor_sync(0xffffffffu, q.x, off);
+        q.y += __shfl_xor_sync(0xffffffffu, q.y, off);
+        q.z += __shfl_xor_sync(0xffffffffu, q.z, off);
+        q.w += __shfl_xor_sync(0xffffffffu, q.w, off);
+    }
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = q;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    for (int w = 1; w < 8; ++w) {
+        q.x += red[w].x;
+        q.y += red[w].y;
+        q.z += red[w].z;
+        q.w += red[w].w;
+    }
+    mom[blockIdx.x] = q;
+}
+
+__global__ void k_shift_pencil(int m, zd *__restrict__ A, const zd *__restrict__ Bt, zd sigma)
+{
+    const int64_t total = (int64_t)m * m;
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
+         e += (int64_t)gridDim.x * blockDim.x)
+        if (e % m <= e / m) A[e] = zsub(A[e], zmul(sigma, Bt[e]));
+}
+__global__ void k_shift_values(int m, zd *__restrict__ alpha, const zd *__restrict__ beta, zd sigma)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < m) alpha[i] = zadd(alpha[i], zmul(sigma, beta[i]));
 }
 
 // Per column j of C: ||C[j+1:m, j]||_2 and max_i |C_ij| (Inf for a NaN).  Warp per column.
@@ -460,6 +502,7 @@ struct RefineCarve {
     float *lower, *cmax, *nv, *part;
     int *pair, *near, *eff, *fail;
     unsigned *ext;
+    float4 *mom;
     RefineStat *st;
     void *schur;
     size_t bytes;
@@ -494,6 +537,7 @@ RefineCarve refine_carve(void *work, int m)
     w.eff = w.near + m;
     w.fail = (int *)take(sizeof(int));
     w.ext = (unsigned *)take(8);
+    w.mom = (float4 *)take(RF_MOM * sizeof(float4));
     w.st = (RefineStat *)take(sizeof(RefineStat));
     w.schur = take(schur32_work_bytes(m));
     w.bytes = off;
@@ -509,6 +553,20 @@ unsigned grid_for(size_t count)
 }  // namespace
 
 size_t zeig_refined_large_work_bytes(int m) { return refine_carve(nullptr, m).bytes + 256; }
+
+int shift_pencil(cudaStream_t s, int m, zd *A, const zd *Bt, zd sigma)
+{
+    k_shift_pencil<<<grid_for((size_t)m * m), 256, 0, s>>>(m, A, Bt, sigma);
+    FEAST_LAUNCH_CHECK();
+    return FEAST_OK;
+}
+
+int shift_values(cudaStream_t s, int m, zd *alpha, const zd *beta, zd sigma)
+{
+    k_shift_values<<<cdiv(m, 128), 128, 0, s>>>(m, alpha, beta, sigma);
+    FEAST_LAUNCH_CHECK();
+    return FEAST_OK;
+}
 
 int permute_cols(cudaStream_t s, int64_t rows, int m, const int *perm, const zd *Vin, zd *Vout)
 {
@@ -537,15 +595,18 @@ static int refined_attempt(cudaStream_t s, int m, const zd *A, const zd *Bt, zd 
     FEAST_CUDA_TRY(cudaMemsetAsync(w.ext, 0, 8, s));
     k_rf_extent<<<grid_for(mm), 256, 0, s>>>(m, A, Bt, w.ext);
     FEAST_LAUNCH_CHECK();
-    k_rf_cast<<<grid_for(mm), 256, 0, s>>>(m, A, Bt, w.X, w.B32, w.Bu, w.ext);
+    const unsigned gc = prm.find && grid_for(mm) > RF_MOM ? RF_MOM : grid_for(mm);
+    k_rf_cast<<<gc, 256, 0, s>>>(m, A, Bt, w.X, w.B32, w.Bu, w.ext, prm.find ? w.mom : nullptr);
     FEAST_LAUNCH_CHECK();
     if ((e = trsm_upper_batched<cf>(s, m, 2 * m, 1, w.B32, m, 0, w.X, m, 0))) return e;
     cf *C = w.X, *Bi = w.X + mm;
     k_col_stats32<<<cdiv((size_t)m * 32, 256), 256, 0, s>>>(m, C, w.lower, w.cmax);
     FEAST_LAUNCH_CHECK();
-    float *h = (float *)malloc(sizeof(float) * (2 * (size_t)m + RF_PART));
-    if (!h) return FEAST_ENOMEM;
     unsigned ext[2] = {0, 0};
+    float4 mom[RF_MOM];
+    if (prm.find) FEAST_CUDA_TRY(cudaMemcpyAsync(mom, w.mom, gc * sizeof(float4), cudaMemcpyDeviceToHost, s));
+    float *h = (float *)malloc(sizeof(float) * 2 * (size_t)m);
+    if (!h) return FEAST_ENOMEM;
     if (cudaMemcpyAsync(h, w.lower, sizeof(float) * 2 * (size_t)m, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaMemcpyAsync(ext, w.ext, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess) {
@@ -554,14 +615,28 @@ static int refined_attempt(cudaStream_t s, int m, const zd *A, const zd *Bt, zd 
     }
     float cn = 0.f;
     for (int j = 0; j < m; ++j) cn = h[m + j] > cn ? h[m + j] : cn;
+    const int xa = (int)(ext[0] >> 20) - 1022, xb = (int)(ext[1] >> 20) - 1022;
     int k = 0;
     while (k < m && h[k] <= RF_TAU * cn) ++k;
     res->k = k;
     free(h);
     // (zero, non-finite or far out of range; B singular shows as a non-finite C)
     if (!rf_exp_ok(ext[0]) || !rf_exp_ok(ext[1]) || !(cn > 0.f && cn < 1e14f)) return FEAST_OK;
-    const int xa = (int)(ext[0] >> 20) - 1022, xb = (int)(ext[1] >> 20) - 1022;
     const double fa = ldexp(1.0, -xa), fl = ldexp(1.0, xa - xb);
+    if (prm.find) {
+        double x = 0.0, y = 0.0, aa = 0.0, bb = 0.0;
+        for (unsigned i = 0; i < gc; ++i) {
+            x += mom[i].x;
+            y += mom[i].y;
+            aa += mom[i].z;
+            bb += mom[i].w;
+        }
+        if (aa * bb - (x * x + y * y) <= RF_NARROW * RF_NARROW * aa * bb) {
+            res->narrow = 1;
+            res->sigma = zmake(x / bb * fl, y / bb * fl);
+            return FEAST_OK;
+        }
+    }
     if (k > m - 8) k = m - 8;
     if (!prm.warm || k < m / 4) k = 0;               // too little has converged: the whole matrix
     const int mb = m - k;
@@ -719,7 +794,7 @@ int zeig_refined_large(cudaStream_t s, int m, const zd *A, const zd *Bt, zd *alp
                        const OzScratch *oz)
 {
     int e = refined_attempt(s, m, A, Bt, alpha, beta, V, work, prm, res, timeout, stats, gt, oz);
-    if (e || res->accepted || res->tail == m || !prm.warm) return e;
+    if (e || res->accepted || res->narrow || res->tail == m || !prm.warm) return e;
     RefineParams cold = prm;   // the warm start did not contract: the whole matrix
     cold.warm = 0;
     const int k = res->k;

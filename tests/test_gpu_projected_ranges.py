@@ -62,3 +62,80 @@ def test_diagonal(m):
         got = al[0] / be[0]
         err = np.abs(got[:, None] - d[None, :]).min(1)
         assert np.max(err / np.abs(got)) <= 2 * np.sqrt(2) * 2.0 ** -53
+
+
+@pytest.mark.parametrize("m", [3, 24, 64, 100, 300])
+@pytest.mark.parametrize("ratio", [3e-2, 1e-3, 1e-4, 1e-5, 1e-6])
+@pytest.mark.parametrize("ea", [0, 70])
+def test_narrow_spectrum(m, ratio, ea):
+    """Eigenvalues in a disk of that radius around 1: the bounds of the general
+    pencil, relative to |lambda|."""
+    rng = np.random.default_rng(m)
+    lam = 1 + ratio * 2 * np.sqrt(rng.random(m)) * np.exp(2j * np.pi * rng.random(m))
+    A, B = _pencil(rng, m, lam)
+    _check(A * 2.0 ** ea, B, lam * 2.0 ** ea, 32 * m * 2.0 ** -53)
+
+
+def test_narrow_spectrum_left_to_qz():
+    """A shifted pencil that goes on to QZ: three equal eigenvalues, one of them defective."""
+    import paper_1404_1768_gb300 as fg
+    rng = np.random.default_rng(2)
+    m = 12
+    T = np.diag(1 + 1e-5 * np.concatenate([[0.5, 0.5, 0.5], np.arange(1, m - 2)])).astype(complex)
+    T[0, 1] = 1e-5
+    W = np.linalg.qr(inputs.complex_normal(rng, (m, m)))[0]
+    B = np.eye(m) + 0.1 * np.triu(inputs.complex_normal(rng, (m, m))) / np.sqrt(m)
+    A = B @ W @ T @ W.conj().T
+    al, be, V, fail = fg.zqz_batched([A], [B])
+    assert fail == 0
+    r = np.linalg.norm(A @ (V[0] * be[0]) - B @ (V[0] * al[0]), axis=0)
+    assert np.max(r / (np.abs(be[0]) * np.linalg.norm(A) + np.abs(al[0]) * np.linalg.norm(B))) <= 4 * m * 2.0 ** -53
+    got = al[0] / be[0]
+    # (the defective pair splits by the square root of the backward error over its coupling)
+    assert np.abs(np.sort(got.real) - np.sort(np.diag(T).real)).max() <= 1e-5 * np.sqrt(32 * m * 2.0 ** -53 / 1e-5)
+
+
+def _narrow_pencil(rng, n, nin, ratio, far):
+    lin = 1 + ratio * 0.95 * np.sqrt(rng.random(nin)) * np.exp(2j * np.pi * rng.random(nin))
+    if far:
+        lout = 4 + np.sqrt(rng.random(n - nin)) * np.exp(2j * np.pi * rng.random(n - nin))
+    else:
+        rad = 1.05 * np.sqrt(1 + (n - nin) / nin * rng.random(n - nin))
+        lout = 1 + ratio * rad * np.exp(2j * np.pi * rng.random(n - nin))
+    P, Q = (np.eye(n) + 0.1 * inputs.complex_normal(rng, (n, n)) / np.sqrt(n) for _ in range(2))
+    return (P * np.concatenate([lin, lout])) @ Q, P @ Q, lin
+
+
+@pytest.mark.parametrize("ratio", [1e-3, 1e-4, 1e-5])
+@pytest.mark.parametrize("prec", [0, 1])
+def test_narrow_contour_warm(ratio, prec):
+    """A contour that is narrow against its centre, in a spectrum of the same
+    density around it: every pass is solved by the FP32 Schur form and its
+    iteration, and warm once columns have converged."""
+    import paper_1404_1768_gb300 as fg
+    rng = np.random.default_rng(11)
+    A, B, _ = _narrow_pencil(rng, 600, 80, ratio, False)
+    g = fg.Feast(A, B, inputs.complex_normal(rng, (600, 112)), center=1 + 0j, a=ratio, q=16, prec=prec, eps=1e-12, max_iter=7)
+    infos = g.run()
+    g.close()
+    assert all(i["qz_cold_fp32"] >= 0 for i in infos)
+    assert infos[-1]["qz_warm"] == 1
+
+
+@pytest.mark.parametrize("m0", [56, 112])
+@pytest.mark.parametrize("ratio", [1e-2, 1e-4])
+@pytest.mark.parametrize("prec", [0, 1])
+def test_narrow_contour_eigenvalues(m0, ratio, prec):
+    """The same with the rest of the spectrum far away: residuals below eps bound
+    the eigenvalues' errors by eps (|A| + |lambda| |B|) times the pairs' condition (< 3)."""
+    import paper_1404_1768_gb300 as fg
+    rng = np.random.default_rng(12)
+    A, B, lin = _narrow_pencil(rng, 400, int(m0 / 1.4), ratio, True)
+    eps = 1e-11
+    g = fg.Feast(A, B, inputs.complex_normal(rng, (400, m0)), center=1 + 0j, a=ratio, q=16, prec=prec, eps=eps, max_iter=12)
+    infos = g.run()
+    lam = np.asarray(g.eigs(False)["lam"])
+    g.close()
+    assert infos[-1]["flag"] == 1 and lam.size == lin.size
+    d = np.abs(lam[:, None] - lin[None, :])
+    assert max(d.min(0).max(), d.min(1).max()) <= 3 * eps * (np.linalg.norm(A, 2) + np.linalg.norm(B, 2))
