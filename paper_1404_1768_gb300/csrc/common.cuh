@@ -407,6 +407,10 @@ int zqz_batched(cudaStream_t s, int m, int batch, zd *A, int64_t lda, int64_t sA
 // first one is sigma when A was replaced by A - sigma B, else 0.
 int zeig_refined(cudaStream_t s, int m, int batch, zd *A, int64_t lda, int64_t sA, const zd *B, int64_t ldb,
                  int64_t sB, zd *alpha, zd *beta, zd *V, int64_t ldv, int64_t sV, void *work);
+// QZ (m <= 64; A, B overwritten by their Schur form) of the pencils that it left
+// (refined 1: work as zeig_refined wrote it, its shift added back), or of all (0).
+int zqz_left(cudaStream_t s, int m, int batch, zd *A, int64_t lda, int64_t sA, zd *B, int64_t ldb, int64_t sB, zd *alpha,
+             zd *beta, zd *V, int64_t ldv, int64_t sV, void *work, int *fail, int refined);
 
 // Large projected problems (k_zeig.cu): standard form, Hessenberg
 // reduction and chunked QR; alpha = eigenvalue, beta = 1.

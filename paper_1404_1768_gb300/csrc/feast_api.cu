@@ -946,16 +946,18 @@ static int iterate_impl(feast_ctx *c, feast_iter_info *info)
             FEAST_CUDA_TRY(cudaStreamSynchronize(s));
             memcpy(&left, hw, sizeof(int));
         }
-        if (!left)
+        if (!left) {
             e = FEAST_OK;
-        else if (m > 64 || (m >= kZeigMinM && c->eps >= kZeigSmallEpsMin))
-            e = zeig_large(s, (int)m, c->Q, Bq, c->alpha, c->beta, c->Yv, c->qz_work, &c->st->qz_fail,
-                           &c->st->timeout, &c->st->qz_sweeps, defl);
-        else
-            e = zqz_batched(s, (int)m, 1, c->Q, m, 0, Bq, m, 0, c->alpha, c->beta, c->Yv, m, 0, c->qz_work,
-                            &c->st->qz_fail, &c->st->timeout, &c->st->qz_sweeps, defl);
+        } else if (m > 64 || (m >= kZeigMinM && c->eps >= kZeigSmallEpsMin)) {
+            if ((e = zeig_large(s, (int)m, c->Q, Bq, c->alpha, c->beta, c->Yv, c->qz_work, &c->st->qz_fail,
+                                &c->st->timeout, &c->st->qz_sweeps, defl)))
+                return e;
+            if (hw[1].x != 0.0 || hw[1].y != 0.0) e = shift_values(s, (int)m, c->alpha, c->beta, hw[1]);
+        } else {
+            e = zqz_left(s, (int)m, 1, c->Q, m, 0, Bq, m, 0, c->alpha, c->beta, c->Yv, m, 0, c->qz_work, &c->st->qz_fail,
+                         m >= 3);
+        }
         if (e) return e;
-        if (left && (hw[1].x != 0.0 || hw[1].y != 0.0) && (e = shift_values(s, (int)m, c->alpha, c->beta, hw[1]))) return e;
     }
     if (narrow && (e = shift_values(s, (int)m, c->alpha, c->beta, centre))) return e;
     FEAST_CUDA_TRY(cudaEventRecord(c->ev[2], s));

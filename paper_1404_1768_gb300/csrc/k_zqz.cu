@@ -1152,13 +1152,22 @@ int zeig_refined(cudaStream_t s, int m, int batch, zd *A, int64_t lda, int64_t s
     return FEAST_OK;
 }
 
+int zqz_left(cudaStream_t s, int m, int batch, zd *A, int64_t lda, int64_t sA, zd *B, int64_t ldb, int64_t sB, zd *alpha,
+             zd *beta, zd *V, int64_t ldv, int64_t sV, void *work, int *fail, int refined)
+{
+    const size_t sm = 3 * (size_t)m * m * sizeof(zd);
+    FEAST_CUDA_TRY(ensure_dyn_smem(k_qz<128>, sm));
+    k_qz<128><<<batch, 128, sm, s>>>(m, A, lda, sA, B, ldb, sB, alpha, beta, V, ldv, sV, (zd *)work, 1, fail, refined);
+    FEAST_LAUNCH_CHECK();
+    return FEAST_OK;
+}
+
 int zqz_batched(cudaStream_t s, int m, int batch, zd *A, int64_t lda, int64_t sA, zd *B,
                 int64_t ldb, int64_t sB, zd *alpha, zd *beta, zd *V, int64_t ldv, int64_t sV,
                 void *work, int *fail, int *timeout, int *stats, double defl)
 {
     if (m <= 0 || batch <= 0) return FEAST_OK;
     if (m <= 64) {
-        size_t sm = 3 * (size_t)m * m * sizeof(zd);
         // refined FP32 Schur form first (GB300, one pencil per SM: 0.41 ms at
         // m = 24 and 2.5 ms at m = 64, against 10.5 and 67 ms for k_qz, whose
         // every rotation is a chain of FP64 instructions); k_qz then solves
@@ -1167,11 +1176,7 @@ int zqz_batched(cudaStream_t s, int m, int batch, zd *A, int64_t lda, int64_t sA
         const int refined = m >= EZ_MIN_M;
         int e;
         if (refined && (e = zeig_refined(s, m, batch, A, lda, sA, B, ldb, sB, alpha, beta, V, ldv, sV, work))) return e;
-        FEAST_CUDA_TRY(ensure_dyn_smem(k_qz<128>, sm));
-        k_qz<128><<<batch, 128, sm, s>>>(m, A, lda, sA, B, ldb, sB, alpha, beta, V, ldv, sV, (zd *)work, 1, fail,
-                                         refined);
-        FEAST_LAUNCH_CHECK();
-        return FEAST_OK;
+        return zqz_left(s, m, batch, A, lda, sA, B, ldb, sB, alpha, beta, V, ldv, sV, work, fail, refined);
     }
     if (lda != m || ldb != m || ldv != m) return FEAST_EINVAL;
     const size_t wb = zqz_work_bytes(m);

@@ -139,3 +139,33 @@ def test_narrow_contour_eigenvalues(m0, ratio, prec):
     assert infos[-1]["flag"] == 1 and lam.size == lin.size
     d = np.abs(lam[:, None] - lin[None, :])
     assert max(d.min(0).max(), d.min(1).max()) <= 3 * eps * (np.linalg.norm(A, 2) + np.linalg.norm(B, 2))
+
+
+def _pass_launches(A, B, Y, passes, **kw):
+    import paper_1404_1768_gb300 as fg
+    g = fg.Feast(A, B, Y, max_iter=passes + 2, **kw)
+    out = []
+    for _ in range(passes):
+        n0 = fg.kernel_launches()
+        info = g.iterate()
+        out.append((fg.kernel_launches() - n0, info))
+        if info["flag"] != 2:
+            break
+    g.close()
+    return out
+
+
+def test_refused_small_pencil_is_tried_once():
+    """A cluster of three that goes to QZ: one launch more than the pass of an easy
+    pencil of the same sizes (k_qz), not a second attempt before it."""
+    rng = np.random.default_rng(21)
+    n, m0 = 64, 16
+    P, Q = (np.eye(n) + 0.1 * inputs.complex_normal(rng, (n, n)) / np.sqrt(n) for _ in range(2))
+    Y = inputs.complex_normal(rng, (n, m0))
+    lam = np.concatenate([0.9 * (np.arange(1, 13) / 13) * np.exp(1j * np.arange(12)), 3 + np.arange(n - 12) / n])
+    hard = lam.copy()
+    hard[1:3] = hard[0]
+    kw = dict(center=0j, a=1.0, q=16, prec=0, eps=1e-13)
+    easy_n = _pass_launches((P * lam) @ Q, P @ Q, Y, 1, **kw)[0][0]
+    hard_n = _pass_launches((P * hard) @ Q, P @ Q, Y, 1, **kw)[0][0]
+    assert hard_n == easy_n + 1
