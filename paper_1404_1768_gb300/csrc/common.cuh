@@ -468,7 +468,6 @@ struct RefineResult {
     double resid;   // estimated error left by the last step
     int narrow;     // prm.find: A - sigma B is below 1/16 of A: nothing was solved
     zd sigma;
-    int cluster;    // eigenvalues closer than FP32 resolves ended it: no other start would do
 };
 // A spectrum narrow against its distance from the origin is solved as that of
 // (A - sigma B, B): A <- A - sigma triu(B), alpha <- alpha + sigma beta.

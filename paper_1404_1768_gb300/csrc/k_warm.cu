@@ -619,8 +619,6 @@ static int refined_attempt(cudaStream_t s, int m, const zd *A, const zd *Bt, zd 
     int k = 0;
     while (k < m && h[k] <= RF_TAU * cn) ++k;
     res->k = k;
-    float rem = 0.f;                                 // what the leading columns have left below the diagonal
-    for (int j = 0; j < k; ++j) rem = h[j] > rem ? h[j] : rem;
     free(h);
     // (zero, non-finite or far out of range; B singular shows as a non-finite C)
     if (!rf_exp_ok(ext[0]) || !rf_exp_ok(ext[1]) || !(cn > 0.f && cn < 1e14f)) return FEAST_OK;
@@ -738,10 +736,7 @@ static int refined_attempt(cudaStream_t s, int m, const zd *A, const zd *Bt, zd 
         RefineStat hs;
         FEAST_CUDA_TRY(cudaMemcpyAsync(&hs, w.st, sizeof(hs), cudaMemcpyDeviceToHost, s));
         FEAST_CUDA_TRY(cudaStreamSynchronize(s));
-        if (hs.bad) {
-            res->cluster = rem <= 5e-7f * cn;        // (nothing above FP32's own rounding was left out)
-            return FEAST_OK;
-        }
+        if (hs.bad) return FEAST_OK;
         float g2, w2, r2;
         memcpy(&g2, &hs.gm, sizeof(float));
         memcpy(&w2, &hs.wm, sizeof(float));
@@ -799,7 +794,7 @@ int zeig_refined_large(cudaStream_t s, int m, const zd *A, const zd *Bt, zd *alp
                        const OzScratch *oz)
 {
     int e = refined_attempt(s, m, A, Bt, alpha, beta, V, work, prm, res, timeout, stats, gt, oz);
-    if (e || res->accepted || res->narrow || res->cluster || res->tail == m || !prm.warm) return e;
+    if (e || res->accepted || res->narrow || res->tail == m || !prm.warm) return e;
     RefineParams cold = prm;   // the warm start did not contract: the whole matrix
     cold.warm = 0;
     const int k = res->k;

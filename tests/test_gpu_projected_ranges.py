@@ -169,23 +169,3 @@ def test_refused_small_pencil_is_tried_once():
     easy_n = _pass_launches((P * lam) @ Q, P @ Q, Y, 1, **kw)[0][0]
     hard_n = _pass_launches((P * hard) @ Q, P @ Q, Y, 1, **kw)[0][0]
     assert hard_n == easy_n + 1
-
-
-def _clustered(gaps, passes, m0=104):
-    """72 eigenvalues inside, the first three those gaps apart, the others far outside."""
-    rng = np.random.default_rng(22)
-    n, nin = 300, 72
-    P, Q = (np.eye(n) + 0.1 * inputs.complex_normal(rng, (n, n)) / np.sqrt(n) for _ in range(2))
-    lam = np.concatenate([0.9 * np.sqrt(rng.random(nin)) * np.exp(2j * np.pi * rng.random(nin)), 4 + rng.random(n - nin)])
-    lam[1:3] = lam[0] + np.array(gaps)
-    return _pass_launches((P * lam) @ Q, P @ Q, inputs.complex_normal(rng, (n, m0)), passes, center=0j, a=1.0, q=16, prec=0,
-                          eps=1e-30, converged_only=True)
-
-
-def test_refused_cluster_is_not_tried_cold():
-    """Above 64 rows: once the columns have converged, a cluster that ends the warm
-    attempt is not met again by a cold one (which takes more than 30 launches)
-    before the double-single QR."""
-    out = _clustered([1e-8, 2e-8], 2)
-    assert out[1][1]["qz_warm"] == 0 and out[1][1]["qz_warm_k"] >= 72   # (a warm attempt was made, and refused)
-    assert out[1][0] <= out[0][0] + 20
