@@ -458,11 +458,13 @@ int rrqr_basis(cudaStream_t s, int64_t n, int m, const zd *U, zd *Q, double rank
 struct RefineParams {
     int warm;           // 1: C's leading columns may have converged (ordered Ritz pairs)
     double target;      // error of the eigenvectors at which the iteration may end
+    float tau;          // column of C counted converged: strictly lower part <= tau max|C| (0: the usual line)
     int find;           // 1: end at once (narrow, sigma) where A is nearly sigma B
 };
 struct RefineResult {
     int accepted;   // 1: alpha, beta, V hold the eigenpairs
     int k;          // converged leading columns found
+    int k_tight;    // the same by the tighter line of a second warm attempt
     int tail;       // rows of the block given to the QR
     int steps;      // Newton steps taken
     double resid;   // estimated error left by the last step

@@ -913,7 +913,7 @@ static int iterate_impl(feast_ctx *c, feast_iter_info *info)
             Ap = c->Q;
             Bp = c->Q + m * m;
         }
-        const RefineParams prm{c->warm_ready, 1e-2 * acc, 0};
+        const RefineParams prm{c->warm_ready, 1e-2 * acc, 0.f, 0};
         if ((e = zeig_refined_large(s, (int)m, Ap, Bp, c->alpha, c->beta, c->Yv, c->warm_work, prm, &c->last_warm,
                                     &c->st->timeout, &c->st->qz_sweeps, &c->gt, orth_oz(c))))
             return e;

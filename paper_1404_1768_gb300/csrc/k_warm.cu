@@ -47,8 +47,12 @@ constexpr int RF_STEPS = 10;          // most steps
 // removes the remainder as it removes FP32's error (a step squares it over a
 // gap), so the line is where its first step still contracts: at n = 2048, m0 =
 // 640 passes 3 on are warm with 1e-3 and 1e-2 alike (5-9 ms against ~130 ms
-// cold), from pass 5 with 3e-6; a start that does not contract runs cold.
-constexpr float RF_TAU = 3e-3f;
+// cold), from pass 5 with 3e-6.  A start that does not contract is tried again
+// from the columns below RF_TIGHT (pairs outside the contour can pass the first
+// line while they are still further off than their gaps: n = 300, 72 pairs
+// inside, m0 = 104: 1.1 ms where the cold solve takes 4.6, and 22 if a cluster
+// sends that one to the double-single QR), then cold.
+constexpr float RF_TAU = 3e-3f, RF_TIGHT = 1e-5f;
 constexpr double RF_BERR = 0x1p-52;   // residual column at rounding level: <= RF_BERR m (1 + |lambda'|) (entries of
                                       // A', B' below 1; it measures 6 x 2^-53 at m = 300)
 constexpr int RF_PART = 64;           // partial sums of the defect norm
@@ -616,9 +620,11 @@ static int refined_attempt(cudaStream_t s, int m, const zd *A, const zd *Bt, zd 
     float cn = 0.f;
     for (int j = 0; j < m; ++j) cn = h[m + j] > cn ? h[m + j] : cn;
     const int xa = (int)(ext[0] >> 20) - 1022, xb = (int)(ext[1] >> 20) - 1022;
+    const float tau = prm.tau > 0.f ? prm.tau : RF_TAU;
     int k = 0;
-    while (k < m && h[k] <= RF_TAU * cn) ++k;
+    while (k < m && h[k] <= tau * cn) ++k;
     res->k = k;
+    while (res->k_tight < m && h[res->k_tight] <= RF_TIGHT * cn) ++res->k_tight;
     free(h);
     // (zero, non-finite or far out of range; B singular shows as a non-finite C)
     if (!rf_exp_ok(ext[0]) || !rf_exp_ok(ext[1]) || !(cn > 0.f && cn < 1e14f)) return FEAST_OK;
@@ -795,10 +801,16 @@ int zeig_refined_large(cudaStream_t s, int m, const zd *A, const zd *Bt, zd *alp
 {
     int e = refined_attempt(s, m, A, Bt, alpha, beta, V, work, prm, res, timeout, stats, gt, oz);
     if (e || res->accepted || res->narrow || res->tail == m || !prm.warm) return e;
-    RefineParams cold = prm;   // the warm start did not contract: the whole matrix
-    cold.warm = 0;
     const int k = res->k;
-    e = refined_attempt(s, m, A, Bt, alpha, beta, V, work, cold, res, timeout, stats, gt, oz);
+    RefineParams next = prm;
+    if (res->k_tight >= m / 4 && res->k_tight < m - res->tail) {   // (m - tail: the columns that it started from)
+        next.tau = RF_TIGHT;
+        e = refined_attempt(s, m, A, Bt, alpha, beta, V, work, next, res, timeout, stats, gt, oz);
+        res->k = k;
+        if (e || res->accepted) return e;
+    }
+    next.warm = 0;   // the warm start does not contract: the whole matrix
+    e = refined_attempt(s, m, A, Bt, alpha, beta, V, work, next, res, timeout, stats, gt, oz);
     res->k = k;
     return e;
 }

@@ -1187,7 +1187,7 @@ int zqz_batched(cudaStream_t s, int m, int batch, zd *A, int64_t lda, int64_t sA
         zd *Ab = A + (int64_t)b * sA, *Bb = B + (int64_t)b * sB, *al = alpha + (int64_t)b * m, *be = beta + (int64_t)b * m;
         zd *Vb = V + (int64_t)b * sV, sigma = zmake(0.0, 0.0);
         char *wk = (char *)work + b * wb;
-        RefineParams prm{0, EZ_DONE, 1};
+        RefineParams prm{0, EZ_DONE, 0.f, 1};
         int e = zeig_refined_large(s, m, Ab, Bb, al, be, Vb, wk, prm, &rr, timeout, stats);
         if (e) return e;
         if (rr.narrow) {

@@ -169,3 +169,23 @@ def test_refused_small_pencil_is_tried_once():
     easy_n = _pass_launches((P * lam) @ Q, P @ Q, Y, 1, **kw)[0][0]
     hard_n = _pass_launches((P * hard) @ Q, P @ Q, Y, 1, **kw)[0][0]
     assert hard_n == easy_n + 1
+
+
+def _clustered(gaps, passes, m0=104):
+    """72 eigenvalues inside, the first three those gaps apart, the others far outside."""
+    rng = np.random.default_rng(22)
+    n, nin = 300, 72
+    P, Q = (np.eye(n) + 0.1 * inputs.complex_normal(rng, (n, n)) / np.sqrt(n) for _ in range(2))
+    lam = np.concatenate([0.9 * np.sqrt(rng.random(nin)) * np.exp(2j * np.pi * rng.random(nin)), 4 + rng.random(n - nin)])
+    lam[1:3] = lam[0] + np.array(gaps)
+    return _pass_launches((P * lam) @ Q, P @ Q, inputs.complex_normal(rng, (n, m0)), passes, center=0j, a=1.0, q=16, prec=0,
+                          eps=1e-30, converged_only=True)
+
+
+@pytest.mark.parametrize("gaps", [(2e-7, 3.5e-7j), (1e-5, 2e-5j), (0.1, 0.2j)])
+def test_warm_after_convergence(gaps):
+    """Passes after the pairs inside have converged stay warm, whatever the extra
+    directions of the subspace look like: their columns pass for converged
+    before their couplings are below their gaps."""
+    out = _clustered(gaps, 5)
+    assert [i["qz_warm"] for _, i in out[2:]] == [1] * (len(out) - 2)
