@@ -437,8 +437,9 @@ int feast_grad_abs2(feast_ctx *right, feast_ctx *left, void *gA, void *gB, int64
  * column of B is scaled by a power of two and written as 7 base-128 digits;
  * digit products and their sums over K-chunks of 512 are exact in the tensor
  * cores' FP32 accumulators, and the chunk sums are combined as 64-bit integers.
- * Error: about 2^-48 times max_k|A_ik| * max_k|B_kj| * k per entry (not
- * relative to |C|).  work: device, >= feast_zgemm_oz_work_bytes bytes, 256-
+ * Error: at most 2^-44 times max_k|A_ik| * max_k|B_kj| * k per entry, maxima
+ * over real and imaginary parts (not relative to |C|); random data stay near
+ * 2^-49 sqrt(k).  work: device, >= feast_zgemm_oz_work_bytes bytes, 256-
  * byte aligned (digit planes).  err: device int32, set non-zero (0x400) if
  * a bounded pipeline wait (4 s of device time) gave up (C is then
  * unspecified).  Asynchronous. */

@@ -655,7 +655,7 @@ def cgemm_tc(A_list, X_list, C_list=None, alpha=1.0, beta=0.0, stream=None):
 
 def zgemm_oz(A, Bm, Cm=None, alpha=1.0, beta=0.0, stream=None):
     """complex128 C = beta C + alpha A B on the bf16 tensor cores with exact
-    digit slicing (FP64-accurate to ~2^-47 of max|A| max|B| k)."""
+    digit slicing (FP64-accurate: at most 2^-44 of max|A| max|B| k, near 2^-49 sqrt(k) on random data)."""
     torch = _torch()
     lib = load()
     A = np.asarray(A, np.complex128)

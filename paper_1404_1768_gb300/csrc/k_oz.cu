@@ -1,6 +1,6 @@
 // FP64-accurate complex GEMM on the bf16 tensor cores (tcgen05, kind::f16)
 // by exact integer slicing, for the refinement residual of the precision
-// form (and any FP64 product that tolerates ~2^-47 relative to |A||B|).
+// form (and any FP64 product that tolerates 2^-44 K relative to max|A| max|B|).
 //
 //   C = beta C + alpha_c A B       A: M x K, B: K x N complex128, column-major
 //
@@ -15,19 +15,22 @@
 // g = s + t over a K-chunk of OZ_KC terms while it stays below 2^24 (all but
 // the last class always do; it can pass it only by a factor 1.13 at worst, and
 // rounds then at a weight below 2^-60).  The kernel keeps one tensor-memory
-// accumulator per class g = 2..8 (all products with s + t <= OZ_S + 1; the
-// rest weigh < 2^-50), reads the classes out after each K-chunk and adds them
+// accumulator per class g = 2..8 (all products with s + t <= OZ_S + 1), reads the classes out after each K-chunk and adds them
 // on the integer pipe into two exact int64 sums per entry,
 //     hi = sum_(g<=5) 128^(5-g) S_g ,   lo = sum_(g>=6) 128^(8-g) S_g ;
 // FP64 enters once per entry, at the end: C gets alpha_c 2^(e_i + f_j - 14)
 // 2^-21 (hi + 2^-21 lo).  Integer sums do not depend on their order, so K is
 // split over the CTAs of a cluster where the tiles do not fill the GPU evenly,
 // with the same result.
-// Representation and truncation error: ~2^-49 relative to
-// max_k |A'_ik| * max_k |B'_kj| per entry, K-fold at most.
+// Error, in units of 2^(e_i + f_j) per real product: 2^-50 for each operand's
+// digits beyond the seventh and 6 x 64 x 64 x 128^-9 = 1.5 x 2^-49 for class 9,
+// 2.5 x 2^-49 in all.  A complex entry sums 2 K of them, and a maximum may be
+// just above half of its power of two (a factor 4): at most 1.25 x 2^-45 K
+// max_k|A'_ik| max_k|B'_kj| in each component, below 2^-44 K in modulus; random
+// data stay near 2^-49 sqrt(K).
 //
-// Seven base-128 digits are 28 slice products and 49 bits; the eight base-64
-// digits before them were 36 products and 48 bits, with an FP64 sum per chunk
+// Seven base-128 digits are 28 slice products; the eight base-64 digits before
+// them were 36 products and left 2.2 times the error, with an FP64 sum per chunk
 // that the shorter chunks (512 instead of 2048 terms) would have made a third
 // of the time: an FP64 instruction takes 64 clocks of an SM quarter here.
 //
