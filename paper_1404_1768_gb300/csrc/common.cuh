@@ -252,6 +252,12 @@ __device__ __forceinline__ double peer_load(const double *p, unsigned rank)
     asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(peer_addr(p, rank)) : "memory");
     return v;
 }
+__device__ __forceinline__ long long peer_load(const long long *p, unsigned rank)
+{
+    long long v;
+    asm volatile("ld.shared::cluster.s64 %0, [%1];" : "=l"(v) : "r"(peer_addr(p, rank)) : "memory");
+    return v;
+}
 __device__ __forceinline__ unsigned long long peer_load(const unsigned long long *p, unsigned rank)
 {
     unsigned long long v;

@@ -619,16 +619,6 @@ __global__ void k_gb_matmul(int64_t n, int64_t kl, int64_t ku, const zd *M, int6
 constexpr int GL_T = 256;
 constexpr int GL_C = 8;          // CTAs per node (a portable cluster)
 constexpr int GL_NB = 32;
-__device__ __forceinline__ unsigned gl_rank()
-{
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void gl_cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 // Order of the pivot search: 0 no candidate, 1 a NaN on the diagonal (taken
 // when there is nothing else), 2 zero, then by magnitude.
 __device__ __forceinline__ unsigned gl_key(cf v, bool diag)
@@ -647,7 +637,7 @@ __global__ void __launch_bounds__(GL_T) k_gb_lu_fused(int64_t n, int kl, int ku,
     __shared__ int s_pos[2][NW];
     __shared__ int s_piv[NB];
     const int kv = kl + ku, ldd = NB + kl, ldu = tc + 2;
-    const int rank = (int)gl_rank(), kvs = (kv + GL_C - 1) / GL_C;
+    const int rank = (int)cluster_rank_id(), kvs = (kv + GL_C - 1) / GL_C;
     const int cb = rank * kvs, ce = (cb + kvs < kv) ? cb + kvs : kv;   // this CTA's columns [cb, ce) right of a panel
     cf *D = reinterpret_cast<cf *>(sm_raw);          // the factored panel by final position, column-major
     cf *U = D + (size_t)ldd * NB;                     // NB x tc slice of U12, row-major
@@ -688,7 +678,7 @@ __global__ void __launch_bounds__(GL_T) k_gb_lu_fused(int64_t n, int kl, int ku,
         }
         if (cb < ce) gather(cb);
         // every CTA holds the panel before any of it is written back
-        gl_cluster_sync();
+        cluster_barrier();
 #pragma unroll
         for (int j = 0; j < NB; ++j) {
             if (j >= nb) break;
@@ -822,7 +812,7 @@ __global__ void __launch_bounds__(GL_T) k_gb_lu_fused(int64_t n, int kl, int ku,
         }
         // every CTA's updates (and the panel) are in memory before any
         // CTA reads the next panel
-        gl_cluster_sync();
+        cluster_barrier();
     }
 }
 

@@ -30,34 +30,6 @@ __device__ __forceinline__ void atomic_cadd(float2 *p, float2 v)
     atomicAdd(&p->y, v.y);
 }
 
-__device__ __forceinline__ unsigned gb_cluster_rank()
-{
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void gb_cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// Load 2 (float2) or 4 (double2) words of shared memory from CTA `rank`.
-__device__ __forceinline__ float2 gb_dsmem_load(const float2 *p, unsigned rank)
-{
-    uint32_t a;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-    float2 v;
-    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
-    return v;
-}
-__device__ __forceinline__ double2 gb_dsmem_load(const double2 *p, unsigned rank)
-{
-    uint32_t a;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-    double2 v;
-    asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(a) : "memory");
-    return v;
-}
-
 // splits > 1: blockIdx.z = batch * splits + s takes the s-th slice of K.
 // Up to GB_SMAX slices the launch groups a tile's slices into one cluster
 // (s = the CTA's rank in it) and CTA 0 sums the slices' tiles in rank order
@@ -142,20 +114,20 @@ __global__ void __launch_bounds__(GB_T) k_gemm(int conj_a, int64_t m, int64_t n,
         // others' in rank order (distributed shared memory), then all wait
         // until it has read them
         T *red = reinterpret_cast<T *>(gb_red_raw);
-        const unsigned rank = gb_cluster_rank();
+        const unsigned rank = cluster_rank_id();
 #pragma unroll
         for (int a = 0; a < TM; ++a)
 #pragma unroll
             for (int c = 0; c < TM; ++c) red[(a * TM + c) * GB_T + threadIdx.x] = acc[a][c];
-        gb_cluster_sync();
+        cluster_barrier();
         if (rank == 0)
             for (int r = 1; r < splits; ++r)
 #pragma unroll
                 for (int a = 0; a < TM; ++a)
 #pragma unroll
                     for (int c = 0; c < TM; ++c)
-                        acc[a][c] = cadd(acc[a][c], gb_dsmem_load(red + (a * TM + c) * GB_T + threadIdx.x, r));
-        gb_cluster_sync();
+                        acc[a][c] = cadd(acc[a][c], peer_load(red + (a * TM + c) * GB_T + threadIdx.x, r));
+        cluster_barrier();
         if (rank != 0) return;
     }
     const bool beta0 = cis_zero(beta);

@@ -40,8 +40,10 @@
 // products per K-step of 16 into the seven accumulators (7 x 64 TMEM columns)
 // and commits each stage and each K-chunk; warps 0-7 read the chunks out (TMEM
 // lane quarter = warp % 4, columns 0-31 or 32-63) and write the result.  What
-// bounds it: shared-memory reads of the A slices (4 KB per 128 x 64 x 16
-// product, 48 clocks for 32 of MMA).  All waits are bounded; on expiry the CTA
+// bounds it: the A slices are read from shared memory for every product (4 KB
+// per 128 x 64 x 16, 48 clocks for 32 of MMA), which accounts for 0.35 of the
+// 0.65 ms that 2048 x 640 x 2048 takes; the rest is not separated yet (the ring
+// holds two stages, the read-out of a chunk overlaps nothing).  All waits are bounded; on expiry the CTA
 // raises *err and finishes.
 #include "tcgen05.cuh"
 
@@ -270,7 +272,7 @@ __global__ void __launch_bounds__(256) k_oz_slice_cols(int64_t K, int64_t N, con
 // The columns' exponents and digits in one launch (K <= OZ_COL1_MAX): w warps
 // (1, 2, 4 or 8) per column, which is read a second time from L1.  A small product
 // is bound by its launches, and a column's digits waited for all columns' exponents
-// (2048 x 640: two launches of 20 and 34 us; the whole product 831 -> 813 us).
+// (2048 x 640: one launch of 38 us for two of 20 and 34; the whole product 831 -> 813 us).
 __global__ void __launch_bounds__(256) k_oz_cols(int64_t K, int64_t N, int w, const zd *__restrict__ B, int64_t ldb,
                                                  int *__restrict__ f, uint32_t *__restrict__ planes, int64_t kp)
 {
@@ -315,23 +317,9 @@ struct OzOut {
     zd beta;
 };
 
-__device__ __forceinline__ void oz_cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// 64-bit word at p's place in the shared memory of CTA rank of the cluster.
-__device__ __forceinline__ long long oz_peer(const long long *p, int rank)
-{
-    uint32_t a;
-    long long v;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
-    asm volatile("ld.shared::cluster.s64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
-    return v;
-}
-
 // K-blocks from kfirst on, of kr real terms.  splits CTAs (a cluster, 1 to
-// OZ_SMAX) share a tile: CTA r takes K-blocks [r kbs, (r + 1) kbs) of them, then finishes 64 / splits of the tile's columns from
-// all of their sums.
+// OZ_SMAX) share a tile: CTA r takes K-blocks [r kbs, (r + 1) kbs) of them, then
+// finishes 64 / splits of the tile's columns from all of their sums.
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     k_oz_gemm(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tB, int mr, int n,
               int kfirst, int kr, int splits, int kbs, const int *__restrict__ ea, const int *__restrict__ fb, OzOut out,
@@ -499,7 +487,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             q[OZ_BM] = lo[j];
         }
     }
-    if (splits > 1) oz_cluster_sync();
+    if (splits > 1) cluster_barrier();
     else __syncthreads();
     if (threadIdx.x < OZ_READ && !s_fail) {
         const int r = row0 + quarter * 32 + lane;            // real row
@@ -522,8 +510,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                 long long h = q[0], l = q[OZ_BM];
                 for (int x = 1; x < splits; ++x) {
                     const int pr = (rank + x) % splits;
-                    h += oz_peer(q, pr);
-                    l += oz_peer(q + OZ_BM, pr);
+                    h += peer_load(q, pr);
+                    l += peer_load(q + OZ_BM, pr);
                 }
                 v[t] = fma((double)l, 0x1p-21, (double)h);
             }
@@ -556,7 +544,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         }
     }
     __syncthreads();
-    if (splits > 1) oz_cluster_sync();   // no CTA leaves while a peer reads its sums
+    if (splits > 1) cluster_barrier();   // no CTA leaves while a peer reads its sums
     if (threadIdx.x == 0 && s_fail) atomicOr(err, TO_OZ);
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
 }
@@ -593,7 +581,11 @@ int oz_prepare_cols(cudaStream_t s, int64_t K, int64_t N, const zd *B, int64_t l
     uint32_t *planes = (uint32_t *)work;
     int *f = (int *)((char *)work + (size_t)OZ_S * N * kp * 2 + 256);
     // one launch while a column is a few loads a thread; longer columns spread
-    // their slicing over more CTAs than there are columns
+    // their slicing over more CTAs than there are columns.  Whole products with
+    // one / two launches, us: K = 2048, N = 16 84 / 91, N = 640 147 / 166; K =
+    // 16384, N = 16 641 / 684, N = 640 1081 / 1132 (128 rows); two win only where
+    // columns are few and long (N = 1, K = 16384 431 / 404, 32768 840 / 768; 16
+    // rows), so the line could lie higher
     if (K <= OZ_COL1_MAX) {
         int w = 1;
         while (w < 8 && w * 64 < K) w *= 2;

@@ -54,23 +54,6 @@ constexpr int K2_TILE_BYTES = K2_BM * K2_BK * 4;        // 8 KiB: one plane of A
 constexpr int K2_STAGE_BYTES = 4 * K2_TILE_BYTES;      // Ah, At, Xh, Xt
 constexpr size_t K2_SMEM = (size_t)K2_STAGES * K2_STAGE_BYTES + 1024;
 
-__device__ __forceinline__ uint32_t cluster_rank()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-// Shared-memory address of the same variable in CTA `rank` of the cluster.
-__device__ __forceinline__ uint32_t map_to_rank(const void *p, uint32_t rank)
-{
-    uint32_t out;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(out) : "r"(smem_u32(p)), "r"(rank));
-    return out;
-}
-__device__ __forceinline__ void cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 // Bounded wait that also gives up once any thread has raised *err (unless
 // it waits for this CTA's own copies or MMAs in flight: those are waited
 // out, up to the time bound); a wait that runs out itself raises the
@@ -138,7 +121,7 @@ __global__ void __launch_bounds__(K2_THREADS, 1)
     __shared__ uint32_t tmem_base;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t rank = cluster_rank();
+    const uint32_t rank = cluster_rank_id();
     const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
     const int mt = (mr + 2 * K2_BM - 1) / (2 * K2_BM), nt = (n + K2_BN - 1) / K2_BN;
     const long long tiles = (long long)batch * mt * nt;
@@ -164,13 +147,13 @@ __global__ void __launch_bounds__(K2_THREADS, 1)
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
-    cluster_sync();                           // the peer's barriers exist before anyone signals them
+    cluster_barrier();                           // the peer's barriers exist before anyone signals them
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = tmem_base;
 
     if (warp == 0 && lane == 0) {
         // TMA producer (both CTAs): this CTA's 128 rows of A', 128 columns of X'
-        const uint32_t full0 = map_to_rank(&full[0], 0);
+        const uint32_t full0 = peer_addr(&full[0], 0);
         long long it = 0;
         bool ok = true;
         for (long long t = pair; t < tiles && ok; t += npairs) {
@@ -240,7 +223,7 @@ __global__ void __launch_bounds__(K2_THREADS, 1)
     } else if (warp >= 2) {
         // epilogue: TMEM lanes 32 (warp % 4) .. +31 of this CTA's 128 rows
         const int quarter = warp & 3;
-        const uint32_t tempty0 = map_to_rank(&tempty[0], 0);
+        const uint32_t tempty0 = peer_addr(&tempty[0], 0);
         const bool rd = (beta.x != 0.f || beta.y != 0.f);
         int tl = 0;
         for (long long t = pair; t < tiles; t += npairs, ++tl) {
@@ -300,7 +283,7 @@ __global__ void __launch_bounds__(K2_THREADS, 1)
     __syncwarp();
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
-    cluster_sync();                           // no CTA leaves while its peer may still signal it
+    cluster_barrier();                           // no CTA leaves while its peer may still signal it
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
 }

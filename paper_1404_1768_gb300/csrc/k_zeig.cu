@@ -726,6 +726,7 @@ __device__ __forceinline__ void win_rot(const RotDS &gr, int k, int c0, int r1, 
     __syncthreads();
 }
 
+#if !FEAST_QR_FP32
 // Schur form of the w x w upper Hessenberg T (in place) with Schur vectors
 // accumulated into V (which starts as I): single-shift QR with full window
 // updates.  Whole CTA; false if the iteration budget runs out.
@@ -774,6 +775,7 @@ __device__ bool win_schur(int w, cds (*T)[NWP], cds (*V)[NWP], float tol_rel, fl
     __syncthreads();
     return true;
 }
+#endif
 
 #if FEAST_QR_FP32
 // FP32 build: the same single-shift QR on complex64 copies of T and V
@@ -1198,6 +1200,7 @@ __global__ void __launch_bounds__(QT, 1) k_hqr(int m, dsv *H, dsv *Z, int ld, Ro
             continue;
         }
 #endif
+#if !FEAST_QR_FP32
         if (L <= NW) {
             // the whole active block fits a window: its Schur form at once
             if (blockIdx.x == 0) {
@@ -1215,6 +1218,7 @@ __global__ void __launch_bounds__(QT, 1) k_hqr(int m, dsv *H, dsv *Z, int ld, Ro
             }
             // (window iteration budget ran out: fall through to a single-shift sweep)
         }
+#endif
         if (ns > 1) {
             // ------------------------------------------------ multishift sweep
             // aggressive early deflation on the bottom NW rows first; its
