@@ -644,16 +644,25 @@ __global__ void __launch_bounds__(LC_T) k_lu_panel_cl(int64_t n, int64_t k0, int
 // The panel [k0, k0 + nb) of every batch member: the cluster form while its
 // CTAs' rows fit shared memory (200 KB: n - k0 <= 3096 in FP64, 6200 in
 // complex64), the one-CTA form on global memory beyond.  At least 16 rows a CTA:
-// below that the barrier costs more than the rows.
+// below that the barrier costs more than the rows.  In FP64 a larger batch fills
+// the SMs by itself, and then the columns' barriers and repeated searches cost
+// more than the split gives: 8 CTAs a matrix up to 8 matrices, 4 up to 32, 2 up
+// to 64, 1 beyond (whole LU of 200 rows with 1 / 2 / 4 / 8, us: 8 matrices 1245 /
+// 1142 / 1049 / 1021, 16 1446 / 1344 / 1252 / 1379, 48 2265 / 2163 / 2360 / 2445,
+// 96 3446 / 3747 / 3868 / 4426, 256 8625 / 9272 / 10044 / 11311, and 10475 by the
+// one-CTA form on global memory).
 template <typename T>
 int lu_panel(cudaStream_t s, int64_t n, int64_t k0, int nb, int batch, T *F, int64_t ldf, int64_t sF, int *piv,
              int64_t pstride, int *info, int *row)
 {
     const int64_t total = n - k0;
+    const int most = sizeof(T) == sizeof(cf) || batch <= 8 ? LC_MAX : batch <= 32 ? 4 : batch <= 64 ? 2 : 1;
+    auto rows_of = [&](int c) { return (total + c - 1) / c; };
+    auto smem_of = [&](int c) { return (size_t)rows_of(c) * (LU_NB + 1) * sizeof(T); };
     int C = 1;
-    while (C < LC_MAX && 32 * C <= total) C *= 2;
-    const int64_t rp = (total + C - 1) / C;
-    const size_t sm = (size_t)rp * (LU_NB + 1) * sizeof(T);
+    while (C < LC_MAX && 32 * C <= total && (C < most || smem_of(C) > 200 * 1024)) C *= 2;
+    const int64_t rp = rows_of(C);
+    const size_t sm = smem_of(C);
     if (sm > 200 * 1024 || (int64_t)batch * C > 0x7fffffff) {
         k_lu_panel<T><<<batch, LU_PT, 0, s>>>(n, k0, nb, F, ldf, sF, piv, pstride, info, row);
         FEAST_LAUNCH_CHECK();

@@ -56,3 +56,17 @@ def test_sliced_columns(n):
     ref = A @ B
     bound = 2.0 ** -44 * 2048 * np.abs(A).max(1)[:, None] * np.abs(B).max(0)[None, :]
     assert np.all(np.abs(one - ref) <= bound)
+
+
+@pytest.mark.parametrize("batch", [8, 9, 32, 33, 64, 65])
+@pytest.mark.parametrize("n", [40, 140, 420])
+def test_lu_batches(n, batch):
+    """8, 4, 2 and 1 CTAs a matrix by the batch's size (more where the panel's rows need them)."""
+    import paper_1404_1768_gb300 as fg
+    rng = np.random.default_rng(n + batch)
+    M = [inputs.complex_normal(rng, (n, n)) + 3 * np.sqrt(n) * np.eye(n) for _ in range(batch)]
+    R = [inputs.complex_normal(rng, (n, 2)) for _ in range(batch)]
+    F, piv, info = fg.zgetrf_batched(M)
+    assert info == 0
+    for m, r, x in zip(M, R, fg.zgetrs_batched(F, piv, R)):
+        assert np.linalg.norm(m @ x - r) <= 4 * n * 2.0 ** -53 * np.linalg.norm(m) * np.linalg.norm(x)
