@@ -167,9 +167,12 @@ __global__ void __launch_bounds__(NT) k_qz(int m, zd *A, int64_t lda, int64_t sA
     beta += (int64_t)b * m;
     zd *Wk = work + (int64_t)b * m * m;
     const int tid = threadIdx.x;
-    if (only_redo && *(volatile int *)Wk == 0) return;   // k_eig_refined has solved this pencil
-    const zd sigma = only_redo ? zmake(((volatile double *)Wk)[2], ((volatile double *)Wk)[3]) : zmake(0.0, 0.0);
-    Team<NT>::bar();
+    zd sigma = zmake(0.0, 0.0);
+    if (only_redo) {
+        if (*(volatile int *)Wk == 0) return;        // k_eig_refined has solved this pencil
+        sigma = zmake(((volatile double *)Wk)[2], ((volatile double *)Wk)[3]);
+        Team<NT>::bar();
+    }
     const double eps = 2.220446049250313e-16;
 
     Mat H, T, Z, Yh;
@@ -275,7 +278,7 @@ __global__ void __launch_bounds__(NT) k_qz(int m, zd *A, int64_t lda, int64_t sA
     if (failed && tid == 0 && fail) atomicAdd(fail, 1);
     // eigenvalues
     for (int k = tid; k < m; k += NT) {
-        alpha[k] = zadd(H(k, k), zmul(sigma, T(k, k)));     // (A was shifted by sigma B)
+        alpha[k] = only_redo ? zadd(H(k, k), zmul(sigma, T(k, k))) : H(k, k);   // (A was shifted by sigma B)
         beta[k] = T(k, k);
     }
     // y_hat_k by back-substitution, one thread per eigenvector
