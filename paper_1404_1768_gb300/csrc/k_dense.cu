@@ -644,19 +644,22 @@ __global__ void __launch_bounds__(LC_T) k_lu_panel_cl(int64_t n, int64_t k0, int
 // The panel [k0, k0 + nb) of every batch member: the cluster form while its
 // CTAs' rows fit shared memory (200 KB: n - k0 <= 3096 in FP64, 6200 in
 // complex64), the one-CTA form on global memory beyond.  At least 16 rows a CTA:
-// below that the barrier costs more than the rows.  In FP64 a larger batch fills
-// the SMs by itself, and then the columns' barriers and repeated searches cost
-// more than the split gives: 8 CTAs a matrix up to 8 matrices, 4 up to 32, 2 up
+// below that the barrier costs more than the rows.  A larger batch fills the SMs
+// by itself, and then the columns' barriers and repeated searches cost more than
+// the split gives.  FP64: 8 CTAs a matrix up to 8 matrices, 4 up to 32, 2 up
 // to 64, 1 beyond (whole LU of 200 rows with 1 / 2 / 4 / 8, us: 8 matrices 1245 /
 // 1142 / 1049 / 1021, 16 1446 / 1344 / 1252 / 1379, 48 2265 / 2163 / 2360 / 2445,
 // 96 3446 / 3747 / 3868 / 4426, 256 8625 / 9272 / 10044 / 11311, and 10475 by the
-// one-CTA form on global memory).
+// one-CTA form on global memory).  complex64: 8 up to 32 matrices, 1 beyond (LU
+// of 200 rows with 1 / 8, us: 128 matrices 997 / 1405, 256 1317 / 2162, 1670 by
+// the form on global memory; 48 of 800 rows 6547 / 6790, 32 5413 / 5469).
 template <typename T>
 int lu_panel(cudaStream_t s, int64_t n, int64_t k0, int nb, int batch, T *F, int64_t ldf, int64_t sF, int *piv,
              int64_t pstride, int *info, int *row)
 {
     const int64_t total = n - k0;
-    const int most = sizeof(T) == sizeof(cf) || batch <= 8 ? LC_MAX : batch <= 32 ? 4 : batch <= 64 ? 2 : 1;
+    const int most = sizeof(T) == sizeof(cf) ? (batch <= 32 ? LC_MAX : 1)
+                     : batch <= 8 ? LC_MAX : batch <= 32 ? 4 : batch <= 64 ? 2 : 1;
     auto rows_of = [&](int c) { return (total + c - 1) / c; };
     auto smem_of = [&](int c) { return (size_t)rows_of(c) * (LU_NB + 1) * sizeof(T); };
     int C = 1;

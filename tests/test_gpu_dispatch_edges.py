@@ -70,3 +70,20 @@ def test_lu_batches(n, batch):
     assert info == 0
     for m, r, x in zip(M, R, fg.zgetrs_batched(F, piv, R)):
         assert np.linalg.norm(m @ x - r) <= 4 * n * 2.0 ** -53 * np.linalg.norm(m) * np.linalg.norm(x)
+
+
+@pytest.mark.parametrize("q", [32, 33])
+@pytest.mark.parametrize("n", [70, 330])
+def test_complex64_lu_batches(n, q):
+    """The node-batched complex64 LU with 8 CTAs a matrix and with one, through the
+    filter of the precision form refined to FP64."""
+    import oracle
+    import paper_1404_1768_gb300 as fg
+    p = inputs.prescribed_pencil(n, n // 4, seed=n)
+    Y = inputs.complex_normal(np.random.default_rng(q), (n, 5))
+    kw = dict(contour_kind=0, rule=0, q=q, center=0j, a=1.0)
+    g = fg.Feast(p.A, p.B, Y, prec=fg.FEAST_C64_REFINE, refine_tol=1e-14, max_refine=6, **kw)
+    o = oracle.Feast(p.A, p.B, Y, **kw)
+    Ug, Uo = g.filter(Y), o.filter(Y)
+    g.close(); o.close()
+    assert np.abs(Ug - Uo).max() <= 1e-10 * np.abs(Uo).max()
